@@ -36,7 +36,8 @@ BYTES_PER_UPDATE = {"fp64": 2 * 41 * 8, "fp32": 2 * 41 * 4, "fp16_shifted": 2 * 
 DTYPE = {"fp64": "f64", "fp32": "f32", "fp16_shifted": "f16 storage / f32 math",
          "bf16_shifted": "bf16 storage / f32 math"}
 PROFILE_FILE = os.path.join(ROOT, "profiles", "k_step_split_fp32_cyl64x4x256_b24.md")
-KERNEL_SOURCES = ["paper_1411_3133_gb300/csrc/lbm_device.cuh", "paper_1411_3133_gb300/csrc/kernels.cuh",
+KERNEL_SOURCES = ["paper_1411_3133_gb300/csrc/collision.cuh", "paper_1411_3133_gb300/csrc/lbm_device.cuh",
+                  "paper_1411_3133_gb300/csrc/kernels.cuh",
                   "paper_1411_3133_gb300/csrc/step_launch.cuh", "paper_1411_3133_gb300/csrc/step_f32.cu",
                   "paper_1411_3133_gb300/csrc/lattice.cuh"]
 METRIC = "MLUPS and % of HBM roofline at 1 GB300"
@@ -45,7 +46,8 @@ METRIC = "MLUPS and % of HBM roofline at 1 GB300"
 FP64_PROFILE_FILE = os.path.join(ROOT, "profiles", "k_step_fp64_cyl64x4x256_b24.md")
 # the FP64 step is the plain k_step; its instruction counts depend on the
 # kernel body alone
-FP64_KERNEL_SOURCES = ["paper_1411_3133_gb300/csrc/lbm_device.cuh", "paper_1411_3133_gb300/csrc/kernels.cuh",
+FP64_KERNEL_SOURCES = ["paper_1411_3133_gb300/csrc/collision.cuh", "paper_1411_3133_gb300/csrc/lbm_device.cuh",
+                  "paper_1411_3133_gb300/csrc/kernels.cuh",
                        "paper_1411_3133_gb300/csrc/step_f64.cu", "paper_1411_3133_gb300/csrc/lattice.cuh"]
 
 
@@ -78,7 +80,8 @@ def measured_traffic():
 
 # ncu summaries of the other timed configurations: DRAM bytes of one whole
 # step (all its kernels), valid for the step sources of that storage type
-STEP_SOURCES = {p: ["paper_1411_3133_gb300/csrc/lbm_device.cuh", "paper_1411_3133_gb300/csrc/kernels.cuh",
+STEP_SOURCES = {p: ["paper_1411_3133_gb300/csrc/collision.cuh", "paper_1411_3133_gb300/csrc/lbm_device.cuh",
+                  "paper_1411_3133_gb300/csrc/kernels.cuh",
                     "paper_1411_3133_gb300/csrc/step_launch.cuh", f"paper_1411_3133_gb300/csrc/step_{t}.cu",
                     "paper_1411_3133_gb300/csrc/lattice.cuh"]
                 for p, t in (("fp32", "f32"), ("fp16_shifted", "h16"), ("bf16_shifted", "b16"))}

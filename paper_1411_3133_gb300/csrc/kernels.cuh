@@ -53,7 +53,7 @@ __device__ __forceinline__ void collide_store(Real (&f)[Q], S* __restrict__ fout
     store_raw<S>(fout, p, d, f);
     return;
   }
-  const Moments<Real> m = moments(f);
+  const Moments<Real> m = step_moments(f);
   if (!finite_v(m.rho)) {  // NaN or Inf
     if (*flag == 0) atomicExch(flag, 1);
   }
@@ -538,15 +538,39 @@ __global__ void __launch_bounds__(128) k_stream_table(float4* __restrict__ st, c
     tl[L] = (double(om1) * r - double(rb[ref_index<K>(d, L, own)])) / WeightOf<L>::w;
   });
   float4* out = st + size_t(b) * ST_K * nrows + uint32_t(srow);
+  // even and odd parts of t per pair, then each shell's transform to the
+  // coefficients its pairs are evaluated from (update_face, update_body)
+  double te[NPAIR], to[NPAIR];
+#pragma unroll
+  for (int P = 0; P < NPAIR; ++P) {
+    te[P] = 0.5 * (tl[2 * P + 1] + tl[2 * P + 2]);
+    to[P] = 0.5 * (tl[2 * P + 1] - tl[2 * P + 2]);
+  }
+  auto face = [](double* v) {
+    const double a = v[0], b2 = v[1];
+    v[0] = 0.5 * (a + b2);
+    v[1] = 0.5 * (a - b2);
+  };
+  auto body = [](double* v) {
+    const double p2 = v[0] + v[1], q = v[2] + v[3], r = v[0] - v[1], s = v[2] - v[3];
+    v[0] = 0.25 * (p2 + q);
+    v[1] = 0.25 * (p2 - q);
+    v[2] = 0.25 * (r + s);
+    v[3] = 0.25 * (r - s);
+  };
+  for (double* v : {te, to}) {
+    face(v + 3);
+    face(v + 5);
+    face(v + 7);
+    body(v + 9);
+    body(v + 16);
+  }
   out[0] = make_float4(float(m[0]), float(m[1]), float(m[2]), float(m[3]));
   out[nrows] = make_float4(float(m[4]), float(m[5]), float(m[6]), float(m[7]));
   out[2 * nrows] = make_float4(float(m[8]), float(m[9]), float(tl[0]), 0.0f);
 #pragma unroll
-  for (int j = 0; j < NPAIR / 2; ++j) {
-    const double tp0 = tl[4 * j + 1], tm0 = tl[4 * j + 2], tp1 = tl[4 * j + 3], tm1 = tl[4 * j + 4];
-    out[(3 + j) * nrows] = make_float4(float(0.5 * (tp0 + tm0)), float(0.5 * (tp0 - tm0)),
-                                       float(0.5 * (tp1 + tm1)), float(0.5 * (tp1 - tm1)));
-  }
+  for (int j = 0; j < NPAIR / 2; ++j)
+    out[(3 + j) * nrows] = make_float4(float(te[2 * j]), float(to[2 * j]), float(te[2 * j + 1]), float(to[2 * j + 1]));
 }
 
 }  // namespace lbgm

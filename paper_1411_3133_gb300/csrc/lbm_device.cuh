@@ -13,14 +13,9 @@
 #include <cstdint>
 #include <type_traits>
 
-#include "lattice.cuh"
+#include "collision.cuh"
 
 namespace lbgm {
-
-// KELT: the theta-resolved double-curved channel -- the ellipsoidal metric
-// of each theta node (full Delta^ij, body force with r and phi components),
-// the frozen channel's Christoffel symbols, one geometry row per node.
-enum MetricKind { KFLAT = 0, KCYL = 1, KELL = 2, KELT = 3 };
 
 // ---------------------------------------------------------------------------
 // launch geometry
@@ -121,8 +116,12 @@ __device__ __forceinline__ int stream_row(const Dims& d, int ir, int i3) {
 //   k = 0: sum rho_l, sum c^x rho_l, sum c^y rho_l, sum c^z rho_l
 //   k = 1: sum c^x c^x rho_l, c^y c^y, c^z c^z, c^x c^y
 //   k = 2: sum c^x c^z rho_l, sum c^y c^z rho_l, t_0, 0
-//   k = 3 + j, j = 0..9: (t_+ + t_-) / 2 and (t_+ - t_-) / 2 of pair 2 j,
-//           then of pair 2 j + 1 (t_+ of population 2 P + 1, t_- of 2 P + 2)
+//   k = 3 + j, j = 0..9: E and O of slot 2 j, then of slot 2 j + 1. A slot
+//           belongs to a pair (t_+ of population 2 P + 1, t_- of 2 P + 2) and
+//           E, O hold te = (t_+ + t_-) / 2 and to = (t_+ - t_-) / 2 in
+//           the coefficient space of the pair's shell: te, to themselves on
+//           the axes; half sum and half difference of a face's two pairs; the
+//           4-point Hadamard transform over 4 of a body shell's four
 constexpr int ST_K = 13;
 __device__ __forceinline__ const float4* stream_of(const Dims& d, int b) {
   return d.st + size_t(b) * ST_K * size_t(d.nr) * size_t(d.st_rows3);
@@ -182,29 +181,6 @@ __device__ __forceinline__ CellPos locate(const Dims& d, uint32_t t) {
   p.it = int(row) - p.ir * d.nt;
   return p;
 }
-
-// ---------------------------------------------------------------------------
-// compile-time loops
-// ---------------------------------------------------------------------------
-template <int I, int N, typename F>
-__device__ __forceinline__ void static_for(F&& f) {
-  if constexpr (I < N) {
-    f(std::integral_constant<int, I>{});
-    static_for<I + 1, N>(f);
-  }
-}
-
-template <int P>
-struct Pair {
-  static constexpr int x = PAIRS[P].x, y = PAIRS[P].y, z = PAIRS[P].z;
-  static constexpr double w = PAIRS[P].w;
-  static constexpr int s = (x != 0 ? (x < 0 ? -x : x) : (y != 0 ? (y < 0 ? -y : y) : (z < 0 ? -z : z)));
-};
-
-template <int L>
-struct WeightOf {
-  static constexpr double w = L == 0 ? W_REST : PAIRS[(L - 1) / 2].w;
-};
 
 // ---------------------------------------------------------------------------
 // population storage
@@ -612,159 +588,8 @@ __device__ __forceinline__ void store_node(S* __restrict__ out, const float* ref
 }
 
 // ---------------------------------------------------------------------------
-// arithmetic types
+// geometry and stream-table rows
 // ---------------------------------------------------------------------------
-// The update is written once for an arithmetic type V: double, float, or PF2
-// -- two nodes per thread in packed FP32x2 instructions (FFMA2/FADD2/FMUL2 of
-// sm_100 and later), one node per lane, each lane rounded exactly like the
-// scalar float instruction. Multiplications by the lattice's integer
-// velocity components are spelled out with compile-time helpers (mac, dot3)
-// so that no multiplication by 0 or +-1 is issued for any type.
-// Every multiply-add is an explicit fmav and the library is compiled with
-// -fmad=false, so the compiler fuses no other product into an add: every
-// kernel that inlines these functions (plain, TMA, work-list) rounds alike.
-struct PF2 {
-  float2 v;
-  PF2() = default;
-  __device__ __forceinline__ PF2(float2 a) : v(a) {}
-  __device__ __forceinline__ PF2(float a, float b) : v(make_float2(a, b)) {}
-  __device__ __forceinline__ explicit PF2(double c) : v(make_float2(float(c), float(c))) {}
-};
-__device__ __forceinline__ PF2 operator+(PF2 a, PF2 b) { return PF2(__fadd2_rn(a.v, b.v)); }
-__device__ __forceinline__ PF2 operator*(PF2 a, PF2 b) { return PF2(__fmul2_rn(a.v, b.v)); }
-__device__ __forceinline__ PF2 operator-(PF2 a, PF2 b) {
-  return PF2(__ffma2_rn(b.v, make_float2(-1.f, -1.f), a.v));
-}
-__device__ __forceinline__ PF2 fmav(PF2 a, PF2 b, PF2 c) { return PF2(__ffma2_rn(a.v, b.v, c.v)); }
-__device__ __forceinline__ float fmav(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fmav(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ PF2 rcpv(PF2 a) { return PF2(__frcp_rn(a.v.x), __frcp_rn(a.v.y)); }
-__device__ __forceinline__ float rcpv(float a) { return 1.0f / a; }
-__device__ __forceinline__ double rcpv(double a) { return 1.0 / a; }
-__device__ __forceinline__ bool finite_v(PF2 a) { return fabsf(a.v.x) < 1e30f && fabsf(a.v.y) < 1e30f; }
-__device__ __forceinline__ bool finite_v(float a) { return fabsf(a) < 1e30f; }
-__device__ __forceinline__ bool finite_v(double a) { return fabs(a) < 1e300; }
-
-// acc + C x, compile-time integer C
-template <int C, class V>
-__device__ __forceinline__ V mac(const V& acc, const V& x) {
-  if constexpr (C == 0) return acc;
-  else if constexpr (C == 1) return acc + x;
-  else if constexpr (C == -1) return acc - x;
-  else return fmav(V(double(C)), x, acc);
-}
-// C x, compile-time integer C != 0
-template <int C, class V>
-__device__ __forceinline__ V mulc(const V& x) {
-  static_assert(C != 0, "mulc by zero");
-  if constexpr (C == 1) return x;
-  else return V(double(C)) * x;
-}
-// cx ax + cy ay + cz az; the first non-zero component of every pair's
-// representative velocity is positive
-template <int CX, int CY, int CZ, class V>
-__device__ __forceinline__ V dot3(const V& ax, const V& ay, const V& az) {
-  if constexpr (CX != 0) return mac<CZ>(mac<CY>(mulc<CX>(ax), ay), az);
-  else if constexpr (CY != 0) return mac<CZ>(mulc<CY>(ay), az);
-  else return mulc<CZ>(az);
-}
-
-// ---------------------------------------------------------------------------
-// moments and collision
-// ---------------------------------------------------------------------------
-template <typename V>
-struct Moments {
-  V rho, jx, jy, jz;
-  V sxx, syy, szz, sxy, sxz, syz;  // sum_l c^i c^j f_l
-};
-
-template <typename V>
-__device__ __forceinline__ Moments<V> moments(const V (&f)[Q]) {
-  Moments<V> m;
-  const V z = V(0.0);
-  m.rho = f[0];
-  m.jx = m.jy = m.jz = z;
-  m.sxx = m.syy = m.szz = m.sxy = m.sxz = m.syz = z;
-  static_for<0, NPAIR>([&](auto P_) {
-    constexpr int P = decltype(P_)::value;
-    using C = Pair<P>;
-    const V s = f[2 * P + 1] + f[2 * P + 2];
-    const V df = f[2 * P + 1] - f[2 * P + 2];
-    m.rho = m.rho + s;
-    m.jx = mac<C::x>(m.jx, df);
-    m.jy = mac<C::y>(m.jy, df);
-    m.jz = mac<C::z>(m.jz, df);
-    m.sxx = mac<C::x * C::x>(m.sxx, s);
-    m.syy = mac<C::y * C::y>(m.syy, s);
-    m.szz = mac<C::z * C::z>(m.szz, s);
-    m.sxy = mac<C::x * C::y>(m.sxy, s);
-    m.sxz = mac<C::x * C::z>(m.sxz, s);
-    m.syz = mac<C::y * C::z>(m.syz, s);
-  });
-  return m;
-}
-
-// acc + (C w_P) x: a lattice-integer coefficient times pair P's weight
-template <int C, int P, class V>
-__device__ __forceinline__ V macw(const V& acc, const V& x) {
-  if constexpr (C == 0) return acc;
-  else return fmav(V(double(C) * Pair<P>::w), x, acc);
-}
-
-// Moments of the streamed populations f_l = w_l g_l + rho_l from the stored
-// deviations g of 2-byte storage: the streamed references' moments (stream
-// table entries a, b, c) start the sums, and every weight is folded into the
-// multiply-add that accumulates it.
-template <typename V>
-__device__ __forceinline__ Moments<V> moments_dev(const V (&g)[Q], const float4& a, const float4& b,
-                                                  const float4& c) {
-  Moments<V> m;
-  m.rho = fmav(V(W_REST), g[0], V(a.x));
-  m.jx = V(a.y);
-  m.jy = V(a.z);
-  m.jz = V(a.w);
-  m.sxx = V(b.x);
-  m.syy = V(b.y);
-  m.szz = V(b.z);
-  m.sxy = V(b.w);
-  m.sxz = V(c.x);
-  m.syz = V(c.y);
-  static_for<0, NPAIR>([&](auto P_) {
-    constexpr int P = decltype(P_)::value;
-    using C = Pair<P>;
-    const V s = g[2 * P + 1] + g[2 * P + 2];
-    const V df = g[2 * P + 1] - g[2 * P + 2];
-    m.rho = macw<1, P>(m.rho, s);
-    m.jx = macw<C::x, P>(m.jx, df);
-    m.jy = macw<C::y, P>(m.jy, df);
-    m.jz = macw<C::z, P>(m.jz, df);
-    m.sxx = macw<C::x * C::x, P>(m.sxx, s);
-    m.syy = macw<C::y * C::y, P>(m.syy, s);
-    m.szz = macw<C::z * C::z, P>(m.szz, s);
-    m.sxy = macw<C::x * C::y, P>(m.sxy, s);
-    m.sxz = macw<C::x * C::z, P>(m.sxz, s);
-    m.syz = macw<C::y * C::z, P>(m.syz, s);
-  });
-  return m;
-}
-
-// Geometry of one node, read for the metric kind K. The Christoffel symbols
-// are kept with a minus sign (F^i = F_ext^i - Gamma^i_jk c^j c^k).
-template <typename V, int K>
-struct NodeGeo {
-  V dtt = V(0.0), dpp = V(0.0);
-  V n_rtt = V(0.0), n_rpp = V(0.0), n_trt = V(0.0), n_prp = V(0.0), n_ttp = V(0.0), n_ptt = V(0.0);
-  V fth = V(1.0);
-};
-
-// The theta-resolved ellipsoid adds the off-diagonal and r r components of
-// Delta and the r and x3 components of the body force direction.
-template <typename V>
-struct NodeGeo<V, KELT> : NodeGeo<V, KELL> {
-  V drr = V(0.0), drt = V(0.0), drp = V(0.0), dtp = V(0.0);
-  V fr = V(0.0), fp = V(0.0);
-};
-
 template <typename Real, int K>
 __device__ __forceinline__ NodeGeo<Real, K> load_geo(const GeoDev<Real>& g, int row) {
   NodeGeo<Real, K> n;
@@ -791,279 +616,6 @@ __device__ __forceinline__ NodeGeo<Real, K> load_geo(const GeoDev<Real>& g, int 
     n.fp = __ldg(e + 5 * g.ext_stride);
   }
   return n;
-}
-
-// two nodes' rows into the lanes of a PF2 geometry
-template <int K>
-__device__ __forceinline__ NodeGeo<PF2, K> load_geo2(const GeoDev<float>& g, int row0, int row1) {
-  const NodeGeo<float, K> a = load_geo<float, K>(g, row0);
-  const NodeGeo<float, K> b = row1 == row0 ? a : load_geo<float, K>(g, row1);
-  NodeGeo<PF2, K> n;
-  n.dtt = PF2(a.dtt, b.dtt);
-  n.dpp = PF2(a.dpp, b.dpp);
-  n.n_rtt = PF2(a.n_rtt, b.n_rtt);
-  n.n_rpp = PF2(a.n_rpp, b.n_rpp);
-  n.n_trt = PF2(a.n_trt, b.n_trt);
-  n.n_prp = PF2(a.n_prp, b.n_prp);
-  n.n_ttp = PF2(a.n_ttp, b.n_ttp);
-  n.n_ptt = PF2(a.n_ptt, b.n_ptt);
-  n.fth = PF2(a.fth, b.fth);
-  return n;
-}
-
-// Per-node coefficients of the equilibrium and of the forcing term.
-//   f^eq(+-c) = w (E +- O), forcing(+-c) = w (Fe +- Fo), with
-//   E  = e0 + eA c.Delta.c + eB (u.c)^2
-//   O  = u.c (oA + eB c.Delta.c + oC (u.c)^2) - Vs.c
-//   Fe = fA (u.c)(F.c) - fB (u.F)
-//   Fo = (F.c)(t0 + (c.A2s.c) / (2 cs^2)) - F.(A2s c)
-// where, from Sec. II,
-//   a2 = rho (cs^2 Delta + u u),  tr a2 = rho (cs^2 tr Delta + |u|^2),
-//   V^k = a3^{iik} = rho (cs^2 (tr Delta u^k + 2 (Delta u)^k) + |u|^2 u^k),
-//   A2 = a2 + kappa Pi,  Pi = sum c c f - rho (cs^2 g^-1 + u u)
-//   (sum c c f^eq = rho cs^2 g^ij + rho u^i u^j by the lattice's 4th-moment
-//   identity), A2s = A2 / cs^4, F^i = F_ext^i - Gamma^i_jk c^j c^k.
-// Stored with signs chosen so that every term is one multiply-add:
-// nv = -Vs, nfB = -fB, na = -A2s, and eAt = eA Delta^thth etc.
-template <typename V>
-struct Coef {
-  V ux, uy, uz;
-  V e0, eB, oA, oC;
-  V eAt, eAp, eBt, eBp;     // eA dtt, eA dpp, eB dtt, eB dpp
-  V nvx, nvy, nvz;
-  V fA, nfB, t0;
-  V naxx, nayy, nazz, naxy, naxz, nayz;
-  V fext_t;
-  // theta-resolved ellipsoid: eA and eB times Delta^rr, Delta^{r theta},
-  // Delta^{r 3}, Delta^{theta 3}; the body force's r and x3 components
-  V eArr, eArt, eArp, eAtp, eBrr, eBrt, eBrp, eBtp;
-  V fext_r, fext_p;
-};
-
-template <typename V, int K>
-__device__ __forceinline__ Coef<V> coefficients(const Moments<V>& m, const NodeGeo<V, K>& g, const V& kappa,
-                                                const V& G) {
-  const V cs2 = V(CS2);
-  const V inv_cs2 = V(1.0 / CS2);
-  const V inv_cs4 = V(1.0 / (CS2 * CS2));
-  Coef<V> c;
-  const V rho = m.rho;
-  const V irho = rcpv(rho);
-  const V ux = m.jx * irho, uy = m.jy * irho, uz = m.jz * irho;
-  c.ux = ux;
-  c.uy = uy;
-  c.uz = uz;
-  const V uu = fmav(uz, uz, fmav(uy, uy, ux * ux));
-  V trD = g.dtt + g.dpp;
-  if constexpr (K == KELT) trD = trD + g.drr;
-  const V tra2 = rho * fmav(cs2, trD, uu);
-  c.e0 = fmav(V(-0.5 / CS2), tra2, rho);
-  const V eA = rho * V(0.5 / CS2);
-  c.eB = rho * V(0.5 / (CS2 * CS2));
-  c.eAt = eA * g.dtt;
-  c.eAp = eA * g.dpp;
-  c.eBt = c.eB * g.dtt;
-  c.eBp = c.eB * g.dpp;
-  c.oA = rho * inv_cs2;
-  c.oC = rho * V(1.0 / (6.0 * CS2 * CS2 * CS2));
-  // -V / (2 cs^4), Delta diagonal (dtt on theta, dpp on x3)
-  const V nvs = V(-0.5 / (CS2 * CS2)) * rho;
-  const V trDc = cs2 * trD;
-  if constexpr (K == KELT) {
-    // full Delta: V^k / rho = cs^2 (tr Delta u^k + 2 (Delta u)^k) + |u|^2 u^k
-    const V c2 = V(2.0 * CS2);
-    const V dux = fmav(g.drr, ux, fmav(g.drt, uy, g.drp * uz));
-    const V duy = fmav(g.drt, ux, fmav(g.dtt, uy, g.dtp * uz));
-    const V duz = fmav(g.drp, ux, fmav(g.dtp, uy, g.dpp * uz));
-    c.nvx = nvs * fmav(c2, dux, fmav(trDc, ux, uu * ux));
-    c.nvy = nvs * fmav(c2, duy, fmav(trDc, uy, uu * uy));
-    c.nvz = nvs * fmav(c2, duz, fmav(trDc, uz, uu * uz));
-    c.eArr = eA * g.drr;
-    c.eArt = eA * g.drt;
-    c.eArp = eA * g.drp;
-    c.eAtp = eA * g.dtp;
-    c.eBrr = c.eB * g.drr;
-    c.eBrt = c.eB * g.drt;
-    c.eBrp = c.eB * g.drp;
-    c.eBtp = c.eB * g.dtp;
-  } else {
-    c.nvx = nvs * (fmav(trDc, ux, uu * ux));
-    c.nvy = nvs * (fmav(fmav(V(2.0 * CS2), g.dtt, trDc), uy, uu * uy));
-    c.nvz = nvs * (fmav(fmav(V(2.0 * CS2), g.dpp, trDc), uz, uu * uz));
-  }
-  c.fA = rho * inv_cs4;
-  c.nfB = rho * V(-1.0 / CS2);
-  // A2 = (1 - kappa) rho (cs^2 Delta + u u) + kappa (S - rho cs^2 delta)
-  const V k1 = V(1.0) - kappa;
-  const V rc = rho * cs2;
-  const V rk = rho * k1;
-  V axx, axy, axz, ayz;
-  if constexpr (K == KELT) {
-    axx = fmav(rk, fmav(cs2, g.drr, ux * ux), kappa * (m.sxx - rc));
-    axy = fmav(rk, fmav(cs2, g.drt, ux * uy), kappa * m.sxy);
-    axz = fmav(rk, fmav(cs2, g.drp, ux * uz), kappa * m.sxz);
-    ayz = fmav(rk, fmav(cs2, g.dtp, uy * uz), kappa * m.syz);
-  } else {
-    axx = fmav(rk, ux * ux, kappa * (m.sxx - rc));
-    axy = fmav(rk, ux * uy, kappa * m.sxy);
-    axz = fmav(rk, ux * uz, kappa * m.sxz);
-    ayz = fmav(rk, uy * uz, kappa * m.syz);
-  }
-  const V ayy = fmav(rk, fmav(cs2, g.dtt, uy * uy), kappa * (m.syy - rc));
-  const V azz = fmav(rk, fmav(cs2, g.dpp, uz * uz), kappa * (m.szz - rc));
-  const V trA2 = axx + ayy + azz;
-  c.t0 = fmav(V(-0.5 / (CS2 * CS2)), trA2, rho * inv_cs2);
-  const V nic4 = V(-1.0 / (CS2 * CS2));
-  c.naxx = axx * nic4;
-  c.nayy = ayy * nic4;
-  c.nazz = azz * nic4;
-  c.naxy = axy * nic4;
-  c.naxz = axz * nic4;
-  c.nayz = ayz * nic4;
-  c.fext_t = G * g.fth;
-  if constexpr (K == KELT) {
-    c.fext_r = G * g.fr;
-    c.fext_p = G * g.fp;
-  }
-  return c;
-}
-
-// E += eA c.Delta.c and X += eB c.Delta.c for velocity (cx, cy, cz): the
-// diagonal theta and x3 terms of every curved metric, and the theta-resolved
-// ellipsoid's r r and off-diagonal terms.
-template <int K, int cx, int cy, int cz, class V>
-__device__ __forceinline__ void add_cdc(V& E, V& X, const Coef<V>& k) {
-  constexpr bool curv = K != KFLAT;
-  constexpr bool ell = K == KELL || K == KELT;
-  if constexpr (curv && cy != 0) {
-    E = mac<cy * cy>(E, k.eAt);
-    X = mac<cy * cy>(X, k.eBt);
-  }
-  if constexpr (ell && cz != 0) {
-    E = mac<cz * cz>(E, k.eAp);
-    X = mac<cz * cz>(X, k.eBp);
-  }
-  if constexpr (K == KELT) {
-    if constexpr (cx != 0) {
-      E = mac<cx * cx>(E, k.eArr);
-      X = mac<cx * cx>(X, k.eBrr);
-    }
-    if constexpr (cx * cy != 0) {
-      E = mac<2 * cx * cy>(E, k.eArt);
-      X = mac<2 * cx * cy>(X, k.eBrt);
-    }
-    if constexpr (cx * cz != 0) {
-      E = mac<2 * cx * cz>(E, k.eArp);
-      X = mac<2 * cx * cz>(X, k.eBrp);
-    }
-    if constexpr (cy * cz != 0) {
-      E = mac<2 * cy * cz>(E, k.eAtp);
-      X = mac<2 * cy * cz>(X, k.eBtp);
-    }
-  }
-}
-
-// BGK collision with the forcing term for the pair (c, -c), in place:
-//   f* = (1 - omega) f + omega f^eq + F
-//      = (1 - omega) f + w (omega E + Fe) +- w (omega O + Fo)
-//
-// DEV (2-byte storage): fp, fm are the stored deviations g = (f - r) / w and
-// the result is the post-collision deviation
-//   g* = (1 - omega) g + (omega E + Fe + te) +- (omega O + Fo + to)
-// with te, to the even and odd parts of t = ((1 - omega) rho - r) / w from the
-// stream table; te and to start the sums of Fe and Fo, so they cost no
-// instruction, and the weight multiply of the pair drops out.
-template <typename V, int K, int P, bool DEV = false>
-__device__ __forceinline__ void collide_pair(V& fp, V& fm, const Coef<V>& k, const NodeGeo<V, K>& g,
-                                             const V& omega, const V& om1, const V& te = V(0.0),
-                                             const V& to = V(0.0)) {
-  using C = Pair<P>;
-  constexpr int cx = C::x, cy = C::y, cz = C::z;
-  constexpr bool curv = K != KFLAT;
-  constexpr bool ell = K == KELL || K == KELT;
-  constexpr bool gen = K == KELT;
-  const V uc = dot3<cx, cy, cz>(k.ux, k.uy, k.uz);
-  const V uc2 = uc * uc;
-  V E = fmav(k.eB, uc2, k.e0);
-  V X = fmav(k.oC, uc2, k.oA);
-  add_cdc<K, cx, cy, cz>(E, X, k);
-  const V O = fmav(uc, X, dot3<cx, cy, cz>(k.nvx, k.nvy, k.nvz));
-  // F = F_ext - Gamma(c, c), even in c; which components exist is known here
-  // (the theta-resolved ellipsoid's body force has all three)
-  constexpr bool hasFr = gen || (curv && (cy != 0 || (ell && cz != 0)));
-  constexpr bool hasFz = gen || (ell && (cx * cz != 0 || cy != 0));
-  V Fr = V(0.0), Fz = V(0.0);
-  if constexpr (gen) {
-    Fr = k.fext_r;
-    if constexpr (cy != 0) Fr = mac<cy * cy>(Fr, g.n_rtt);
-    if constexpr (cz != 0) Fr = mac<cz * cz>(Fr, g.n_rpp);
-    Fz = k.fext_p;
-    if constexpr (cy != 0) Fz = mac<cy * cy>(Fz, g.n_ptt);
-    if constexpr (cx * cz != 0) Fz = mac<2 * cx * cz>(Fz, g.n_prp);
-  } else {
-    if constexpr (curv && cy != 0) Fr = mulc<cy * cy>(g.n_rtt);
-    if constexpr (ell && cz != 0) Fr = (cy != 0) ? mac<cz * cz>(Fr, g.n_rpp) : mulc<cz * cz>(g.n_rpp);
-    if constexpr (ell && cx * cz != 0 && cy != 0) Fz = mac<2 * cx * cz>(mulc<cy * cy>(g.n_ptt), g.n_prp);
-    else if constexpr (ell && cx * cz != 0) Fz = mulc<2 * cx * cz>(g.n_prp);
-    else if constexpr (ell && cy != 0) Fz = mulc<cy * cy>(g.n_ptt);
-  }
-  V Ft = k.fext_t;
-  if constexpr (curv && cx * cy != 0) Ft = mac<2 * cx * cy>(Ft, g.n_trt);
-  if constexpr (ell && cy * cz != 0) Ft = mac<2 * cy * cz>(Ft, g.n_ttp);
-  // F.c and u.F
-  constexpr bool hasFc = cy != 0 || (cx != 0 && hasFr) || (cz != 0 && hasFz);
-  V Fc = V(0.0);
-  if constexpr (hasFc) {
-    constexpr int ax_ = hasFr ? cx : 0, az_ = hasFz ? cz : 0;
-    Fc = dot3<ax_, cy, az_>(Fr, Ft, Fz);
-  }
-  V uF = k.uy * Ft;
-  if constexpr (hasFr) uF = fmav(k.ux, Fr, uF);
-  if constexpr (hasFz) uF = fmav(k.uz, Fz, uF);
-  // -A2s c, its quadratic form, and F.(-A2s c)
-  const V nax = dot3<cx, cy, cz>(k.naxx, k.naxy, k.naxz);
-  const V nay = dot3<cx, cy, cz>(k.naxy, k.nayy, k.nayz);
-  const V naz = dot3<cx, cy, cz>(k.naxz, k.nayz, k.nazz);
-  V FnA;
-  if constexpr (DEV) FnA = fmav(Ft, nay, to);
-  else FnA = Ft * nay;
-  if constexpr (hasFr) FnA = fmav(Fr, nax, FnA);
-  if constexpr (hasFz) FnA = fmav(Fz, naz, FnA);
-  // Fe = fA uc Fc - fB uF,  Fo = Fc (t0 + cAc / (2 cs^2)) - F.A2s c
-  V Fe;
-  if constexpr (DEV) Fe = fmav(k.nfB, uF, te);
-  else Fe = k.nfB * uF;
-  V Fo = FnA;
-  if constexpr (hasFc) {
-    Fe = fmav(k.fA * uc, Fc, Fe);
-    const V ncAc = dot3<cx, cy, cz>(nax, nay, naz);
-    Fo = fmav(Fc, fmav(V(-0.5 / CS2), ncAc, k.t0), FnA);
-  }
-  if constexpr (DEV) {
-    const V B = fmav(omega, O, Fo);
-    const V a = fmav(omega, E, Fe);
-    fp = fmav(om1, fp, a + B);
-    fm = fmav(om1, fm, a - B);
-  } else {
-    const V w = V(C::w);
-    const V Bw = fmav(omega, O, Fo) * w;
-    const V a = fmav(omega, E, Fe);
-    fp = fmav(om1, fp, fmav(a, w, Bw));
-    fm = fmav(om1, fm, fmav(a, w, -Bw));
-  }
-}
-
-template <typename V, int K>
-__device__ __forceinline__ void collide(V (&f)[Q], const Coef<V>& k, const NodeGeo<V, K>& g, const V& omega) {
-  const V om1 = V(1.0) - omega;
-  // rest velocity: f^eq = w0 e0, forcing = -w0 fB (u . F_ext)
-  V uF0 = k.uy * k.fext_t;
-  if constexpr (K == KELT) uF0 = fmav(k.ux, k.fext_r, fmav(k.uz, k.fext_p, uF0));
-  f[0] = fmav(om1, f[0], fmav(omega, k.e0, k.nfB * uF0) * V(W_REST));
-  static_for<0, NPAIR>([&](auto P_) {
-    constexpr int P = decltype(P_)::value;
-    collide_pair<V, K, P>(f[2 * P + 1], f[2 * P + 2], k, g, omega, om1);
-  });
 }
 
 // A node's stream-table row: entry k of the table in global memory (st the
@@ -1102,79 +654,23 @@ __device__ __forceinline__ void stage_table(float4* dst, int step, const float4*
 }
 __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
+// Moments of the streamed populations f_l = w_l g_l + rho_l from the stored
+// deviations g of 2-byte storage: the streamed references' moments (stream
+// table entries a, b, c) start the sums, and every weight is folded into the
+// multiply-add that accumulates it.
+template <typename V>
+__device__ __forceinline__ Moments<V> moments_dev(const V (&g)[Q], const float4& a, const float4& b,
+                                                  const float4& c) {
+  const Moments<V> m0 = {V(a.x), V(a.y), V(a.z), V(a.w), V(b.x), V(b.y), V(b.z), V(b.w), V(c.x), V(c.y)};
+  return moments_shells<true>(g, m0);
+}
+
 // BGK collision with forcing on the stored deviations g of 2-byte storage,
-// in place (collide_pair with DEV), with the node's stream-table row tab.
+// in place, with the node's stream-table row tab.
 template <int K, class Tab>
 __device__ __forceinline__ void collide_dev(float (&g)[Q], const Coef<float>& k, const NodeGeo<float, K>& geo,
                                             float omega, const Tab& tab, float t0) {
-  const float om1 = 1.0f - omega;
-  g[0] = fmaf(om1, g[0], fmaf(omega, k.e0, fmaf(k.nfB, k.uy * k.fext_t, t0)));
-  // each table entry is requested one pair group ahead of its use, so a
-  // global load overlaps the arithmetic of the group before
-  float4 t = tab.at(3);
-  static_for<0, NPAIR / 2>([&](auto J_) {
-    constexpr int J = decltype(J_)::value;
-    float4 tn = t;
-    if constexpr (J + 1 < NPAIR / 2) tn = tab.at(4 + J);
-    collide_pair<float, K, 2 * J, true>(g[4 * J + 1], g[4 * J + 2], k, geo, omega, om1, t.x, t.y);
-    collide_pair<float, K, 2 * J + 1, true>(g[4 * J + 3], g[4 * J + 4], k, geo, omega, om1, t.z, t.w);
-    t = tn;
-  });
-}
-
-// f^eq(rho, u) for all 41 velocities (initial state, Sec. II).
-template <typename V, int K>
-__device__ __forceinline__ void equilibrium(const V& rho, const V& ux, const V& uy, const V& uz,
-                                            const NodeGeo<V, K>& g, V (&f)[Q]) {
-  Moments<V> m;
-  m.rho = rho;
-  m.jx = rho * ux;
-  m.jy = rho * uy;
-  m.jz = rho * uz;
-  m.sxx = m.syy = m.szz = m.sxy = m.sxz = m.syz = V(0.0);  // unused with kappa = 0
-  Coef<V> k = coefficients<V, K>(m, g, V(0.0), V(0.0));
-  k.ux = ux;
-  k.uy = uy;
-  k.uz = uz;
-  f[0] = k.e0 * V(W_REST);
-  static_for<0, NPAIR>([&](auto P_) {
-    constexpr int P = decltype(P_)::value;
-    using C = Pair<P>;
-    constexpr int cx = C::x, cy = C::y, cz = C::z;
-    const V uc = dot3<cx, cy, cz>(ux, uy, uz);
-    const V uc2 = uc * uc;
-    V E = fmav(k.eB, uc2, k.e0);
-    V X = fmav(k.oC, uc2, k.oA);
-    if constexpr (cy != 0) {
-      E = mac<cy * cy>(E, k.eAt);
-      X = mac<cy * cy>(X, k.eBt);
-    }
-    if constexpr (cz != 0) {
-      E = mac<cz * cz>(E, k.eAp);
-      X = mac<cz * cz>(X, k.eBp);
-    }
-    if constexpr (K == KELT) {
-      if constexpr (cx != 0) {
-        E = mac<cx * cx>(E, k.eArr);
-        X = mac<cx * cx>(X, k.eBrr);
-      }
-      if constexpr (cx * cy != 0) {
-        E = mac<2 * cx * cy>(E, k.eArt);
-        X = mac<2 * cx * cy>(X, k.eBrt);
-      }
-      if constexpr (cx * cz != 0) {
-        E = mac<2 * cx * cz>(E, k.eArp);
-        X = mac<2 * cx * cz>(X, k.eBrp);
-      }
-      if constexpr (cy * cz != 0) {
-        E = mac<2 * cy * cz>(E, k.eAtp);
-        X = mac<2 * cy * cz>(X, k.eBtp);
-      }
-    }
-    const V O = fmav(uc, X, dot3<cx, cy, cz>(k.nvx, k.nvy, k.nvz));
-    f[2 * P + 1] = (E + O) * V(C::w);
-    f[2 * P + 2] = (E - O) * V(C::w);
-  });
+  collide_shells<float, K>(g, k, geo, omega, tab, t0);
 }
 
 }  // namespace lbgm

@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(KBounds<S, Real, K>::maxt, KBounds<S, Real, K>
   const InstParams<Real>& ip = inst[b];
   Real f[Q];
   gather<K, S, Real, 2>(fin + base, ref, p, d, f);
-  const Moments<Real> m = moments(f);
+  const Moments<Real> m = step_moments(f);
   if (!finite_v(m.rho)) {
     if (*flag == 0) atomicExch(flag, 1);
   }

@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(NX, 512 / NX) k_step_tma(const __grid_constant
       fence_proxy_async_smem();
       issue_tile<NX>(&map, stages + s * Q * NX, &full[s], tile + 2 * G, d, vel, lane);
     }
-    const Moments<float> m = moments(f);
+    const Moments<float> m = step_moments(f);
     if (!finite_v(m.rho)) {
       if (*flag == 0) atomicOr(flag, 1);
     }
