@@ -3,6 +3,7 @@
 // point. All numerical work runs in the kernels of kernels.cuh / aux.cu.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -238,16 +239,6 @@ cudaError_t launch_split(lb_ctx* c, int src, int dst) {
   if (e == cudaSuccess) e = cudaStreamWaitEvent(c->aux, c->ev_fork, 0);
   if (e != cudaSuccess) return e;
   switch (c->prec) {
-    case LB_FP64:
-      e = launch_step_split_f64(c->K, static_cast<const double*>(c->f[src]), static_cast<double*>(c->f[dst]),
-                                c->geo_d, static_cast<const InstParams<double>*>(c->inst), c->dims, c->flag,
-                                c->block_threads, c->stream, c->aux);
-      break;
-    case LB_FP32:
-      e = launch_step_split_f32(c->K, static_cast<const float*>(c->f[src]), static_cast<float*>(c->f[dst]),
-                                c->geo_f, static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag,
-                                c->block_threads, c->stream, c->aux);
-      break;
     case LB_FP16_SHIFTED:
       e = launch_step_split_h16(c->K, static_cast<const __half*>(c->f[src]), static_cast<__half*>(c->f[dst]),
                                 c->geo_f, static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag,
@@ -265,14 +256,22 @@ cudaError_t launch_split(lb_ctx* c, int src, int dst) {
   return e != cudaSuccess ? e : e2;
 }
 
-// LB_OPT_STEP_KERNEL 0 (auto): the region split where x3 is periodic and the
-// arithmetic is FP32 (measured fastest there), the one-kernel step otherwise.
+// The step kernel of the context: the TMA kernel (2) where it was asked for;
+// the region split (4) of 2-byte storage where it applies -- flat and
+// cylinder, periodic x3, bounce-back walls, blocks within an i_r layer -- and
+// neither kernel 1 nor the work list (5) was asked for (measured on 24
+// 64 x 4 x 256 cylinders, FP16: 74.4 us a step against 91.6); else the
+// one-kernel step (1): in FP32 82.4 us against 84.9 for a region split and
+// 103.6 for the work list, 87.0 against 92.1 on 24 four-wall ellipsoids.
 int resolved_kernel(const lb_ctx* c) {
   if (c->any_shift) return 1;  // the half-force variant runs in the plain kernel only
-  if (c->K == KELT) return 1;   // the theta-resolved ellipsoid too
-  if (c->step_kernel != 0) return c->step_kernel;
-  if (c->prec == LB_FP64) return 1;
-  return (c->geom.periodic3 && c->geom.wall == LB_WALL_BOUNCEBACK) ? 4 : 5;
+  if (use_tma(c)) return 2;
+  const int threads = std::min(c->block_threads, 128);
+  if (c->elem_bytes == 2 && (c->step_kernel == 0 || c->step_kernel == 4) && c->geom.periodic3 &&
+      c->geom.wall == LB_WALL_BOUNCEBACK && (c->K == KFLAT || c->K == KCYL) &&
+      (c->dims.nt * c->dims.n3) % threads == 0)
+    return 4;
+  return 1;
 }
 
 lb_status launch_step_once(lb_ctx* c) {
@@ -281,12 +280,6 @@ lb_status launch_step_once(lb_ctx* c) {
   cudaError_t e;
   if (kern == 4)
     e = launch_split(c, src, dst);
-  else if (kern == 5) {
-    lb_status st = ctx_tiled_prepare(c);  // a no-op once the tiles are current
-    if (st == LB_OK) st = ctx_tiled_launch(c);
-    if (st != LB_OK) return st;
-    e = cudaSuccess;
-  }
   else if (c->any_shift && c->prec == LB_FP64)
     e = launch_step_shift_f64(c->K, static_cast<const double*>(c->f[src]), static_cast<double*>(c->f[dst]),
                               c->geo_d, static_cast<const InstParams<double>*>(c->inst), c->dims, c->flag,
@@ -295,7 +288,7 @@ lb_status launch_step_once(lb_ctx* c) {
     e = launch_step_shift_f32(c->K, static_cast<const float*>(c->f[src]), static_cast<float*>(c->f[dst]),
                               c->geo_f, static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag,
                               c->block_threads, c->stream);
-  else if (use_tma(c))
+  else if (kern == 2)
     e = launch_step_tma_f32(c->K, c->tmap[src], static_cast<const float*>(c->f[src]),
                             static_cast<float*>(c->f[dst]), c->geo_f,
                             static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag, c->stream);
@@ -493,6 +486,11 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
   c->partial = static_cast<double*>(dalloc(c, size_t(batch) * c->nblk * DIAG_NQ * sizeof(double)));
   c->diag_out = static_cast<double*>(dalloc(c, size_t(batch) * DIAG_NQ * sizeof(double)));
   c->flag = static_cast<int*>(dalloc(c, sizeof(int)));
+  d.src_nt = axis_classes(d.nt);
+  d.src_n3 = axis_classes(d.n3);
+  c->src_tab = static_cast<int4*>(
+      dalloc(c, size_t(axis_classes(d.nr)) * d.src_nt * d.src_n3 * SRC_ROW * sizeof(int4)));
+  d.src = c->src_tab;
   d.st_rows3 = c->K == KELL ? d.geo_rows3 : (d.periodic3 ? 1 : 7);
   if (c->elem_bytes == 2) {
     c->ref_tab = static_cast<float*>(dalloc(c, size_t(batch) * Q * nrows * sizeof(float)));
@@ -503,7 +501,7 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
     d.st = c->st_tab;
   }
   if (!c->f[0] || !c->f[1] || !c->geo_real || !c->geo64 || !c->sqrtg || !c->base_uth || !c->ini ||
-      !c->inst || !c->rho_s || !c->u_s || !c->rowmean || !c->partial || !c->diag_out || !c->flag)
+      !c->inst || !c->rho_s || !c->u_s || !c->rowmean || !c->partial || !c->diag_out || !c->flag || !c->src_tab)
     return bail(LB_ERR_CUDA, "device allocation failed");
 
   // geometry tables
@@ -532,6 +530,7 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
       geo_arrays(static_cast<float*>(c->geo_real), nrows, c->geo_f);
     }
   }
+  if (e == cudaSuccess) e = launch_source_table(c->src_tab, c->f[0], d, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return bail(LB_ERR_CUDA, std::string("geometry upload: ") + cudaGetErrorString(e));
@@ -627,10 +626,6 @@ lb_status lb_step(lb_ctx* c, long long n) {
       if (s != LB_OK) return s;
       ++c->step;
       --n;
-    }
-    if (resolved_kernel(c) == 5) {  // tiles are uploaded outside the capture
-      s = ctx_tiled_prepare(c);
-      if (s != LB_OK) return s;
     }
     // the captured kernels depend on the resolved step kernel and on whether
     // an instance uses the half-force variant (both can change with lb_init)
@@ -928,7 +923,6 @@ lb_status lb_autotune(lb_ctx* c, int steps_per_trial, lb_tune* best, lb_tune* tr
 void lb_destroy(lb_ctx* c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
-  lb_batch_destroy(c->tiles);
   if (c->aux) {
     cudaStreamSynchronize(c->aux);
     cudaStreamDestroy(c->aux);

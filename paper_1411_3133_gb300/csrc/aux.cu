@@ -51,6 +51,28 @@ cudaError_t init_t(int K, S* f, const GeoDev<Real>& geo, const double* sqrtg, co
   return cudaGetLastError();
 }
 
+// Source table (gather_table): one thread per key, from the general source
+// rule at a node of the key's classes. fin is any address: the sources'
+// addresses are formed, never read.
+__global__ void __launch_bounds__(64) k_source_table(int* __restrict__ tab, const float* fin, Dims d) {
+  const int keys = axis_classes(d.nr) * d.src_nt * d.src_n3;
+  const int k = int(blockIdx.x * blockDim.x + threadIdx.x);
+  if (k >= keys) return;
+  const int c3 = k % d.src_n3, ct = (k / d.src_n3) % d.src_nt, cr = k / (d.src_n3 * d.src_nt);
+  CellPos p;
+  p.b = 0;
+  p.ir = axis_class_node(cr, d.nr);
+  p.it = axis_class_node(ct, d.nt);
+  p.i3 = axis_class_node(c3, d.n3);
+  p.cell = (p.ir * d.nt + p.it) * d.n3 + p.i3;
+  int* row = tab + k * 4 * SRC_ROW;
+  auto put = [&](auto L_, const float* src, int, int) { row[decltype(L_)::value] = int(src - fin) - p.cell; };
+  put(std::integral_constant<int, 0>{}, fin + p.cell, 0, 0);
+  if (near_wall(p, d)) for_each_source_wall<KFLAT, float>(fin, p, d, put);
+  else for_each_source_far<KFLAT, float>(fin, p, d, put);
+  for (int j = Q; j < 4 * SRC_ROW; ++j) row[j] = 0;
+}
+
 // weights by population index, for the element-wise conversions
 __constant__ double c_weight[Q];
 
@@ -399,6 +421,12 @@ cudaError_t launch_stream_table(int prec, int K, float4* st, const float* ref, c
   if (prec == 2) return launch_stream_table_t<__half>(K, st, ref, inst, fin, d, s);
   if (prec == 3) return launch_stream_table_t<__nv_bfloat16>(K, st, ref, inst, fin, d, s);
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_source_table(int4* tab, const void* fin, const Dims& d, cudaStream_t s) {
+  const int keys = axis_classes(d.nr) * d.src_nt * d.src_n3;
+  k_source_table<<<(keys + 63) / 64, 64, 0, s>>>(reinterpret_cast<int*>(tab), static_cast<const float*>(fin), d);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_diag(const double* rho, const double* u, double* rowmean, const double* geo64,

@@ -1,14 +1,9 @@
 // Batches of contexts of different geometry (lb_batch_* of include/lbgm.h).
 //
 // Every instance of every member becomes one ListInst record; instances are
-// grouped by metric kind and each group gets four work lists: tiles of
-// interior nodes (instance, first node, count) and, per wall-node class,
-// tiles of wall nodes (instance, first index into a list of wall-node
-// indices, count) -- nodes near an r-wall only, near an x3-wall only, and
-// the rest (corners, equilibrium walls, short axes). One batch step is one
-// k_step_list launch per non-empty list; the lists after the first run on
-// forked streams, so the wall-node kernels (bound by instruction fetch)
-// overlap the interior kernels (bound by memory).
+// grouped by metric kind and each group gets one work list, tiles (instance,
+// first node, count) over all its nodes. One batch step is one k_step_list
+// launch per kind, the kinds after the first on forked streams.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -24,66 +19,15 @@ using namespace lbgm;
 namespace {
 
 constexpr int kMaxGroups = 3;  // flat, cylinder, ellipsoid
-constexpr int kLists = 4;                  // interior tiles, three wall-node classes
-constexpr int kMaxLanes = kLists * kMaxGroups;
 
 struct Group {
   int K = 0;
   int ninst = 0;
-  int nwork[kLists] = {};        // interior tiles, wall-node tiles per class
-  size_t inst_off = 0;           // byte offset of the ListInst records in dmem
-  size_t work_off[kLists] = {};  // byte offsets of the int4 tiles in dmem
-  size_t cells_off = 0;         // byte offset of the wall-node indices in dmem
-  int blocks_per_sm = 0;        // occupancy of the interior kernel at the built block size
+  int nwork = 0;
+  size_t inst_off = 0;     // byte offset of the ListInst records in dmem
+  size_t work_off = 0;     // byte offset of the int4 tiles in dmem
+  int blocks_per_sm = 0;   // occupancy of the kernel at the built block size
 };
-
-// Wall-node class of node (i_r, i_3) near a wall (lists 1..3): 1 within 3
-// layers of an r-wall only, 2 of an x3-wall only -- each with one
-// compile-time fold per layer, which needs bounce-back walls and the walled
-// axis at least 7 nodes long -- and 3 the rest (the general wall rule).
-int wall_class(const Dims& d, int ir, int i3) {
-  const bool near_r = ir < 3 || ir > d.nr - 4;
-  const bool near_3 = !d.periodic3 && (i3 < 3 || i3 > d.n3 - 4);
-  if (d.wall_eq) return 3;
-  if (near_r && !near_3 && d.nr >= 7) return 1;
-  if (near_3 && !near_r && d.n3 >= 7) return 2;
-  return 3;
-}
-
-// Tiles of one instance (group-local index li): runs of interior nodes (no
-// wall within 3 nodes) as (li, first node, count), counts <= tile, into
-// lists[0]; the wall nodes' indices appended to cells[c - 1] by class c and
-// tiled as (li, first index into cells[c - 1], count), counts <= wall_tile,
-// into lists[c].
-void instance_tiles(const Dims& d, int li, int tile, int wall_tile, std::vector<int4> (&lists)[kLists],
-                    std::vector<int> (&cells)[kLists - 1]) {
-  const int nr = d.nr, nt = d.nt, n3 = d.n3;
-  auto inner_r = [&](int ir) { return ir >= 3 && ir <= nr - 4; };
-  auto inner_3 = [&](int i3) { return d.periodic3 || (i3 >= 3 && i3 <= n3 - 4); };
-  int run_start = -1;
-  auto close_run = [&](int end) {
-    for (int a = run_start; a < end; a += tile) lists[0].push_back(make_int4(li, a, std::min(tile, end - a), 0));
-    run_start = -1;
-  };
-  size_t w0[kLists - 1];
-  for (int c = 0; c < kLists - 1; ++c) w0[c] = cells[c].size();
-  for (int ir = 0; ir < nr; ++ir)
-    for (int it = 0; it < nt; ++it)
-      for (int i3 = 0; i3 < n3; ++i3) {
-        const int cell = (ir * nt + it) * n3 + i3;
-        if (inner_r(ir) && inner_3(i3)) {
-          if (run_start < 0) run_start = cell;
-        } else {
-          if (run_start >= 0) close_run(cell);
-          cells[wall_class(d, ir, i3) - 1].push_back(cell);
-        }
-      }
-  if (run_start >= 0) close_run(nr * nt * n3);
-  for (int c = 0; c < kLists - 1; ++c)
-    for (size_t a = w0[c]; a < cells[c].size(); a += size_t(wall_tile))
-      lists[c + 1].push_back(
-          make_int4(li, int(a), int(std::min(size_t(wall_tile), cells[c].size() - a)), 0));
-}
 
 }  // namespace
 
@@ -106,9 +50,9 @@ struct lb_batch {
   void* dmem = nullptr;
   size_t dmem_bytes = 0;
 
-  cudaStream_t aux[kMaxLanes - 1] = {};
+  cudaStream_t aux[kMaxGroups - 1] = {};
   cudaEvent_t ev_fork = nullptr;
-  cudaEvent_t ev_join[kMaxLanes - 1] = {};
+  cudaEvent_t ev_join[kMaxGroups - 1] = {};
 
   int threads = 128;
   int tile_blocks = 1;  // LB_OPT_TILE_BLOCKS: nodes per tile = tile_blocks x threads
@@ -204,8 +148,7 @@ lb_status build(lb_batch* b) {
   drop_graph(b);
   b->built = false;
   std::vector<unsigned char> recs;
-  std::vector<int4> tiles[kMaxGroups][kLists];
-  std::vector<int> cells[kMaxGroups];
+  std::vector<int4> tiles[kMaxGroups];
   b->ngroups = 0;
   for (int K : {int(KCYL), int(KELL), int(KFLAT)}) {
     Group gr;
@@ -220,35 +163,26 @@ lb_status build(lb_batch* b) {
     if (gr.ninst == 0) continue;
     gr.inst_off = before;
     // tiles, instance-major; instance ids are local to the group
-    const int gi = b->ngroups;
+    std::vector<int4>& t = tiles[b->ngroups];
+    const int tile = b->threads * b->tile_blocks;
     int local = 0;
-    std::vector<int> cls[kLists - 1];
     for (const lb_ctx* c : b->m) {
       if (c->K != K) continue;
+      const int n = c->dims.ncell;
       for (int bi = 0; bi < c->batch; ++bi, ++local)
-        instance_tiles(c->dims, local, b->threads * b->tile_blocks, b->threads, tiles[gi], cls);
+        for (int a = 0; a < n; a += tile) t.push_back(make_int4(local, a, std::min(tile, n - a), 0));
     }
-    // one index list per group: the classes one after the other
-    for (int c = 0; c < kLists - 1; ++c) {
-      const int shift = int(cells[gi].size());
-      for (int4& t : tiles[gi][c + 1]) t.y += shift;
-      cells[gi].insert(cells[gi].end(), cls[c].begin(), cls[c].end());
-    }
-    for (int m = 0; m < kLists; ++m) gr.nwork[m] = int(tiles[gi][m].size());
+    gr.nwork = int(t.size());
     cudaError_t e = occupancy(b->prec, K, b->threads, &gr.blocks_per_sm);
     if (e != cudaSuccess) return bcuda(b, e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     b->g[b->ngroups++] = gr;
   }
-  // layout: records | per group: interior tiles, wall tiles, wall-node indices
+  // layout: records | tiles per group
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   size_t off = al(recs.size());
   for (int i = 0; i < b->ngroups; ++i) {
-    for (int m = 0; m < kLists; ++m) {
-      b->g[i].work_off[m] = off;
-      off = al(off + tiles[i][m].size() * sizeof(int4));
-    }
-    b->g[i].cells_off = off;
-    off = al(off + cells[i].size() * sizeof(int));
+    b->g[i].work_off = off;
+    off = al(off + tiles[i].size() * sizeof(int4));
   }
   const size_t need = off;
   if (need > b->dmem_bytes) {
@@ -260,15 +194,9 @@ lb_status build(lb_batch* b) {
   }
   unsigned char* base = static_cast<unsigned char*>(b->dmem);
   LB_BCUDA(b, cudaMemcpyAsync(base, recs.data(), recs.size(), cudaMemcpyHostToDevice, b->stream));
-  for (int i = 0; i < b->ngroups; ++i) {
-    for (int m = 0; m < kLists; ++m)
-      if (!tiles[i][m].empty())
-        LB_BCUDA(b, cudaMemcpyAsync(base + b->g[i].work_off[m], tiles[i][m].data(),
-                                    tiles[i][m].size() * sizeof(int4), cudaMemcpyHostToDevice, b->stream));
-    if (!cells[i].empty())
-      LB_BCUDA(b, cudaMemcpyAsync(base + b->g[i].cells_off, cells[i].data(), cells[i].size() * sizeof(int),
-                                  cudaMemcpyHostToDevice, b->stream));
-  }
+  for (int i = 0; i < b->ngroups; ++i)
+    LB_BCUDA(b, cudaMemcpyAsync(base + b->g[i].work_off, tiles[i].data(), tiles[i].size() * sizeof(int4),
+                                cudaMemcpyHostToDevice, b->stream));
   LB_BCUDA(b, cudaStreamSynchronize(b->stream));  // the host vectors go out of scope
   b->base_cur.resize(b->m.size());
   for (size_t i = 0; i < b->m.size(); ++i) b->base_cur[i] = b->m[i]->cur;
@@ -288,49 +216,32 @@ bool records_current(const lb_batch* b) {
   return true;
 }
 
-// One work list of one group (m = 0: interior tiles, 1..3: wall-node tiles
-// of class m) on stream s.
-cudaError_t launch_lane(const lb_batch* b, const Group& gr, int m, cudaStream_t s) {
+// The work list of one group on stream s.
+cudaError_t launch_group(const lb_batch* b, const Group& gr, cudaStream_t s) {
   const unsigned char* base = static_cast<const unsigned char*>(b->dmem);
   const void* insts = base + gr.inst_off;
-  const int* cells = reinterpret_cast<const int*>(base + gr.cells_off);
   const int grid = b->schedule == 1 ? std::max(1, gr.blocks_per_sm) * b->nsm : 0;
-  const int4* work = reinterpret_cast<const int4*>(base + gr.work_off[m]);
-  const int sel = m | (m == 0 && b->built_tile_blocks > 1 ? 4 : 0);  // list class; multi-block tiles
+  const int4* work = reinterpret_cast<const int4*>(base + gr.work_off);
+  const bool multi = b->built_tile_blocks > 1;
   switch (b->prec) {
-    case LB_FP64:
-      return launch_step_list_f64(gr.K, sel, insts, work, gr.nwork[m], cells, b->threads, grid, b->parity, s);
-    case LB_FP32:
-      return launch_step_list_f32(gr.K, sel, insts, work, gr.nwork[m], cells, b->threads, grid, b->parity, s);
+    case LB_FP64: return launch_step_list_f64(gr.K, multi, insts, work, gr.nwork, b->threads, grid, b->parity, s);
+    case LB_FP32: return launch_step_list_f32(gr.K, multi, insts, work, gr.nwork, b->threads, grid, b->parity, s);
     case LB_FP16_SHIFTED:
-      return launch_step_list_h16(gr.K, sel, insts, work, gr.nwork[m], cells, b->threads, grid, b->parity, s);
-    default:
-      return launch_step_list_b16(gr.K, sel, insts, work, gr.nwork[m], cells, b->threads, grid, b->parity, s);
+      return launch_step_list_h16(gr.K, multi, insts, work, gr.nwork, b->threads, grid, b->parity, s);
+    default: return launch_step_list_b16(gr.K, multi, insts, work, gr.nwork, b->threads, grid, b->parity, s);
   }
 }
 
-// One batch step. Every non-empty work list is a lane of its own: they read
-// the same buffer and write disjoint nodes, so they run side by side -- the
-// wall-node kernels, bound by instruction fetch, beside the interior
-// kernels, bound by memory. The first lane (an interior list) goes on the
-// batch stream first; the others are forked after it, interior lists before
-// wall-node lists, and joined back (measured: +9 % on 24 four-wall
-// double-curved channels; launching the wall-node lists first was slower).
+// One batch step. The metric kinds read the same buffers and write disjoint
+// nodes, so they run side by side: the first on the batch stream, the others
+// forked before it and joined back.
 lb_status step_once(lb_batch* b) {
-  int lg[kMaxLanes], lm[kMaxLanes], n = 0;
-  for (int m = 0; m < kLists; ++m) {
-    for (int i = 0; i < b->ngroups; ++i)
-      if (b->g[i].nwork[m] > 0) {
-        lg[n] = i;
-        lm[n] = m;
-        ++n;
-      }
-  }
+  const int n = b->ngroups;
   if (n > 1) LB_BCUDA(b, cudaEventRecord(b->ev_fork, b->stream));
-  if (n > 0) LB_BCUDA(b, launch_lane(b, b->g[lg[0]], lm[0], b->stream));
+  if (n > 0) LB_BCUDA(b, launch_group(b, b->g[0], b->stream));
   for (int k = 1; k < n; ++k) {
     LB_BCUDA(b, cudaStreamWaitEvent(b->aux[k - 1], b->ev_fork, 0));
-    LB_BCUDA(b, launch_lane(b, b->g[lg[k]], lm[k], b->aux[k - 1]));
+    LB_BCUDA(b, launch_group(b, b->g[k], b->aux[k - 1]));
     LB_BCUDA(b, cudaEventRecord(b->ev_join[k - 1], b->aux[k - 1]));
   }
   for (int k = 1; k < n; ++k) LB_BCUDA(b, cudaStreamWaitEvent(b->stream, b->ev_join[k - 1], 0));
@@ -429,35 +340,6 @@ lb_status run(lb_batch* b, long long n, bool graph) {
 
 }  // namespace
 
-// A context stepped through its own single-member batch (interior and
-// wall-node tiles in separate kernels): build the tiles for the context's
-// current buffer and block size, outside any stream capture.
-lb_status lbgm::ctx_tiled_prepare(lb_ctx* c) {
-  if (!c->tiles) {
-    lb_ctx* one[1] = {c};
-    lb_status s = lb_batch_create(one, 1, &c->tiles);
-    if (s != LB_OK) return ctx_fail(c, s, std::string("tiled step: ") + lb_last_error(nullptr));
-  }
-  lb_batch* b = c->tiles;
-  b->threads = std::min(c->block_threads, max_threads(b->prec));
-  if (!records_current(b)) {
-    lb_status s = build(b);
-    if (s != LB_OK) return ctx_fail(c, s, "tiled step: " + b->err);
-  }
-  return LB_OK;
-}
-
-// One step's launches; the caller flips the context's buffer and counts the
-// step (the batch's parity follows, so its records stay current).
-lb_status lbgm::ctx_tiled_launch(lb_ctx* c) {
-  lb_batch* b = c->tiles;
-  if (!b || !records_current(b) || b->threads != std::min(c->block_threads, max_threads(b->prec)))
-    return ctx_fail(c, LB_ERR_STATE, "tiled step used without preparation");
-  lb_status s = step_once(b);
-  if (s != LB_OK) return ctx_fail(c, s, "tiled step: " + b->err);
-  return LB_OK;
-}
-
 extern "C" {
 
 lb_status lb_batch_create(lb_ctx* const* members, int count, lb_batch** out) {
@@ -491,7 +373,7 @@ lb_status lb_batch_create(lb_ctx* const* members, int count, lb_batch** out) {
   if (e == cudaSuccess && cur_dev != b->device) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, b->device);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
-  for (int i = 0; i < kMaxLanes - 1 && e == cudaSuccess; ++i) {
+  for (int i = 0; i < kMaxGroups - 1 && e == cudaSuccess; ++i) {
     e = cudaStreamCreateWithFlags(&b->aux[i], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_join[i], cudaEventDisableTiming);
   }
@@ -605,7 +487,7 @@ void lb_batch_destroy(lb_batch* b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
   drop_graph(b);
   if (b->dmem) cudaFree(b->dmem);
-  for (int i = 0; i < kMaxLanes - 1; ++i) {
+  for (int i = 0; i < kMaxGroups - 1; ++i) {
     if (b->aux[i]) cudaStreamDestroy(b->aux[i]);
     if (b->ev_join[i]) cudaEventDestroy(b->ev_join[i]);
   }

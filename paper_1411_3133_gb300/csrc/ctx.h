@@ -47,6 +47,7 @@ struct lb_ctx {
   double* dbl_stage = nullptr;     // conversion staging (FP32 populations), lazily allocated
   float* ref_tab = nullptr;        // 2-byte storage: reference populations [batch][Q][rows]
   float4* st_tab = nullptr;        // 2-byte storage: stream table [batch][ST_K][stream rows]
+  int4* src_tab = nullptr;         // source table of the step's gather
   int ref_mode = 1;                // LB_OPT_STORAGE_REFERENCE
   int* flag = nullptr;
   int nblk = 0;
@@ -66,7 +67,6 @@ struct lb_ctx {
   int graph_kernel = -1;             // 2 x resolved step kernel + any_shift of the captured graph
   int step_kernel = 0;               // LB_OPT_STEP_KERNEL
   bool any_shift = false;            // an instance uses the half-force velocity (old_forcing 2)
-  lb_batch* tiles = nullptr;         // private single-member batch of the tiled step
   cudaStream_t aux = nullptr;        // second stream of the region-split step
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool tma_ok = false;               // tensor maps built for both buffers
@@ -80,9 +80,5 @@ namespace lbgm {
 lb_status ctx_fail(lb_ctx* c, lb_status s, const std::string& msg);
 // False (with *s set) unless c is non-NULL, initialised and not poisoned.
 bool ctx_usable(lb_ctx* c, lb_status* s);
-// Tiled step (LB_OPT_STEP_KERNEL 5): prepare the tiles (outside captures),
-// then launch one step of them.
-lb_status ctx_tiled_prepare(lb_ctx* c);
-lb_status ctx_tiled_launch(lb_ctx* c);
 
 }  // namespace lbgm

@@ -70,8 +70,8 @@ __device__ __forceinline__ void collide_store(Real (&f)[Q], S* __restrict__ fout
 }
 
 // Fused time step of one node p of one instance whose state blocks start at
-// fin and fout (reference table ref): pull streaming + walls, then
-// collide_store.
+// fin and fout (reference table ref): pull streaming + walls (gather_step),
+// then collide_store.
 // 2-byte storage of the ellipsoid, whose stream rows are (i_r, i_3) -- one
 // per node: the node's stream-table row is staged into shared memory before
 // the gather (stage_table), so its latency runs under the gather's and no
@@ -82,7 +82,7 @@ __device__ __forceinline__ void collide_store(Real (&f)[Q], S* __restrict__ fout
 #ifndef LBGM_STAGE_TABLE
 #define LBGM_STAGE_TABLE 1
 #endif
-template <typename S, typename Real, int K, int WALLS = 2>
+template <typename S, typename Real, int K>
 __device__ __forceinline__ void step_node(const S* __restrict__ fin, S* __restrict__ fout, const float* ref,
                                           const GeoDev<Real>& geo, const InstParams<Real>& ip, const Dims& d,
                                           const CellPos& p, int* __restrict__ flag) {
@@ -92,11 +92,11 @@ __device__ __forceinline__ void step_node(const S* __restrict__ fin, S* __restri
     const TabStaged tab{s_tab + threadIdx.x, int(blockDim.x)};
     stage_table(s_tab + threadIdx.x, int(blockDim.x), stream_of(d, p.b) + stream_row<K>(d, p.ir, p.i3),
                 uint32_t(d.nr) * uint32_t(d.st_rows3));
-    gather<K, S, Real, WALLS, true>(fin, ref, p, d, f);
+    gather_step<K>(fin, p, d, f);
     stage_wait();
     collide_store<S, Real, K>(f, fout, ref, geo, ip, d, p, flag, &tab);
   } else {
-    gather<K, S, Real, WALLS, Codec<S, Real>::uses_ref>(fin, ref, p, d, f);
+    gather_step<K>(fin, p, d, f);
     collide_store<S, Real, K>(f, fout, ref, geo, ip, d, p, flag);
   }
 }
@@ -162,24 +162,10 @@ __global__ void __launch_bounds__(KBounds<S, Real, K>::maxt, KBounds<S, Real, K>
   step_node<S, Real, K>(fin + base, fout + base, ref_of(d, b), geo, inst[b], d, p, flag);
 }
 
-// The same update split by region for channels periodic in x3, where only
-// the three node layers next to each r-wall need the wall rule: k_step_bulk
-// covers the contiguous interior layers 3 .. nr - 4 with the far-from-wall
-// gather alone, k_step_edge the 6 wall layers with the per-layer constant
-// folds (gather_edge), so neither kernel carries the other's code.
-template <typename S, typename Real, int K>
-__global__ void __launch_bounds__(KBounds<S, Real, K>::maxt, KBounds<S, Real, K>::minb)
-    k_step_bulk(const S* __restrict__ fin, S* __restrict__ fout, GeoDev<Real> geo,
-                const InstParams<Real>* __restrict__ inst, Dims d, int* __restrict__ flag) {
-  const uint32_t layer = uint32_t(d.nt) * uint32_t(d.n3);
-  const uint32_t cell = 3u * layer + blockIdx.x * blockDim.x + threadIdx.x;
-  if (cell >= uint32_t(d.nr - 3) * layer) return;
-  const int b = int(blockIdx.y);
-  const CellPos p = locate_cell(d, b, cell);
-  const size_t base = size_t(b) * Q * uint32_t(d.ncell);
-  step_node<S, Real, K, 0>(fin + base, fout + base, ref_of(d, b), geo, inst[b], d, p, flag);
-}
-
+// Region split of 2-byte storage for channels periodic in x3: the contiguous
+// interior layers 3 .. nr - 4 in k_step_bulk_rowsm with the far-from-wall
+// gather alone, the 6 wall layers in k_step_edge_rowsm with the per-layer
+// constant folds (gather_edge).
 // 2-byte storage for metrics whose geometry and stream rows are i_r alone
 // (flat, cylinder), with blocks that never straddle an i_r layer (nt n3 a
 // multiple of blockDim.x): the block's nodes share one geometry row, one
@@ -269,27 +255,6 @@ __global__ void __launch_bounds__(KBounds<S, float, K>::maxt, LBGM_EDGE_ROWSM_MI
                         [&](float (&f)[Q]) { gather_edge<K, S, float, true>(fin + base, nullptr, p, d, f); });
 }
 
-// Wall-layer kernel: 4 resident blocks per SM whatever the storage (no
-// spills with the six fold variants' address arithmetic; it runs beside the
-// interior kernel, which keeps the SMs' other slots; measured +1 % on the
-// whole FP32 step against the interior kernel's cap).
-template <typename S, typename Real, int K>
-__global__ void __launch_bounds__(KBounds<S, Real, K>::maxt, KBounds<S, Real, K>::minb < 4 ? KBounds<S, Real, K>::minb : 4)
-    k_step_edge(const S* __restrict__ fin, S* __restrict__ fout, GeoDev<Real> geo,
-                const InstParams<Real>* __restrict__ inst, Dims d, int* __restrict__ flag) {
-  const uint32_t layer = uint32_t(d.nt) * uint32_t(d.n3);
-  const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= 6u * layer) return;
-  const uint32_t cell = e < 3u * layer ? e : e + uint32_t(d.nr - 6) * layer;
-  const int b = int(blockIdx.y);
-  const CellPos p = locate_cell(d, b, cell);
-  const size_t base = size_t(b) * Q * uint32_t(d.ncell);
-  const float* ref = ref_of(d, b);
-  Real f[Q];
-  gather_edge<K, S, Real, Codec<S, Real>::uses_ref>(fin + base, ref, p, d, f);
-  collide_store<S, Real, K>(f, fout + base, ref, geo, inst[b], d, p, flag);
-}
-
 // One instance of a batch whose instances differ in geometry and size: its
 // dimensions (batch 1), geometry tables, parameters, two state blocks and
 // the flag that records a non-finite density.
@@ -304,26 +269,18 @@ struct ListInst {
 };
 
 // Work-list step over instances of one metric kind. Work item j = (instance,
-// first, count) covers `count` nodes of one instance: at most blockDim.x,
-// one per thread, or with MULTI a tile of several blocks' worth (thread t
-// takes nodes t, t + blockDim.x, ...; a separate instantiation, because the
-// loop costs the one-block tiles ~5 % on the four-wall ellipsoid): with
-// WALLS = 0 the interior nodes first .. first + count - 1 (no wall within 3
-// nodes: the far-from-wall gather alone); otherwise the wall nodes
-// cells[first .. first + count - 1] of one class, each in its own
-// instantiation -- WALLS = 3: within 3 layers of an r-wall only (the r
-// folds), 4: of an x3-wall only (the x3 folds), 1: the rest (corners,
-// equilibrium walls, short axes: the general wall rule). Splitting them
-// keeps each kernel's code small (instruction fetch is what binds a kernel
-// carrying every wall variant).
+// first, count) covers the nodes first .. first + count - 1 of one instance:
+// at most blockDim.x, one per thread, or with MULTI a tile of several blocks'
+// worth (thread t takes nodes t, t + blockDim.x, ...; a separate
+// instantiation, because the loop costs the one-block tiles ~5 % on the
+// four-wall ellipsoid).
 // Blocks take items j = blockIdx.x, blockIdx.x + gridDim.x, ... (a
 // persistent grid when gridDim.x < nwork). `parity` 0 reads f0 and writes f1,
 // 1 the reverse. The instance record is staged once per item in shared
 // memory.
-template <typename S, typename Real, int K, int WALLS, bool MULTI>
+template <typename S, typename Real, int K, bool MULTI>
 __global__ void __launch_bounds__(KBounds<S, Real, K>::maxt, KBounds<S, Real, K>::minb)
-    k_step_list(const ListInst<S, Real>* __restrict__ insts, const int4* __restrict__ work, int nwork,
-                const int* __restrict__ cells, int parity) {
+    k_step_list(const ListInst<S, Real>* __restrict__ insts, const int4* __restrict__ work, int nwork, int parity) {
   constexpr int kWords = sizeof(ListInst<S, Real>) / 4;
   static_assert(sizeof(ListInst<S, Real>) % 4 == 0, "record must be whole words");
   static_assert(kWords <= 64, "the smallest block (64 threads) copies the record");
@@ -340,12 +297,11 @@ __global__ void __launch_bounds__(KBounds<S, Real, K>::maxt, KBounds<S, Real, K>
     __syncthreads();
     const ListInst<S, Real>& I = sh.rec;
     auto node = [&](int i) {
-      const uint32_t t = WALLS == 0 ? uint32_t(w.y + i) : uint32_t(cells[w.y + i]);
       const Dims d = I.d;
-      const CellPos p = locate(d, t);
+      const CellPos p = locate_cell(d, 0, uint32_t(w.y + i));
       const S* fin = parity ? I.f1 : I.f0;
       S* fout = const_cast<S*>(parity ? I.f0 : I.f1);
-      step_node<S, Real, K, WALLS>(fin, fout, d.ref, I.geo, *I.ip, d, p, I.flag);
+      step_node<S, Real, K>(fin, fout, d.ref, I.geo, *I.ip, d, p, I.flag);
     };
     if constexpr (MULTI) {
       for (int i = int(threadIdx.x); i < w.z; i += int(blockDim.x)) node(i);

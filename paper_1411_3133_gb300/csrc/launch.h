@@ -35,13 +35,8 @@ cudaError_t launch_step_shift_f32(int K, const float* fin, float* fout, const Ge
                                   const InstParams<float>* inst, const Dims& d, int* flag, int threads,
                                   cudaStream_t s);
 
-// Region-split step (periodic x3): wall layers on stream se, interior on s.
-cudaError_t launch_step_split_f64(int K, const double* fin, double* fout, const GeoDev<double>& geo,
-                                  const InstParams<double>* inst, const Dims& d, int* flag, int threads,
-                                  cudaStream_t s, cudaStream_t se);
-cudaError_t launch_step_split_f32(int K, const float* fin, float* fout, const GeoDev<float>& geo,
-                                  const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                                  cudaStream_t s, cudaStream_t se);
+// Region-split step of 2-byte storage (periodic x3): wall layers on stream se,
+// interior on s.
 cudaError_t launch_step_split_h16(int K, const __half* fin, __half* fout, const GeoDev<float>& geo,
                                   const InstParams<float>* inst, const Dims& d, int* flag, int threads,
                                   cudaStream_t s, cudaStream_t se);
@@ -50,23 +45,21 @@ cudaError_t launch_step_split_b16(int K, const __nv_bfloat16* fin, __nv_bfloat16
                                   cudaStream_t s, cudaStream_t se);
 
 // Work-list step over instances of different geometry (ListInst<S, R> array);
-// walls bits 0-1: 0 interior tiles, 1 r-layer wall nodes, 2 x3-layer wall
-// nodes, 3 other wall nodes (1..3 over `cells`); bit 2: interior tiles
-// longer than one block; grid 0 launches one block per work item.
-cudaError_t launch_step_list_f64(int K, int walls, const void* insts, const int4* work, int nwork,
-                                 const int* cells, int threads, int grid, int parity, cudaStream_t s);
+// multi: items longer than one block; grid 0 launches one block per item.
+cudaError_t launch_step_list_f64(int K, bool multi, const void* insts, const int4* work, int nwork,
+                                 int threads, int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_f64(int K, int threads, int* blocks_per_sm);
 int step_list_max_threads_f64();
-cudaError_t launch_step_list_f32(int K, int walls, const void* insts, const int4* work, int nwork,
-                                 const int* cells, int threads, int grid, int parity, cudaStream_t s);
+cudaError_t launch_step_list_f32(int K, bool multi, const void* insts, const int4* work, int nwork,
+                                 int threads, int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_f32(int K, int threads, int* blocks_per_sm);
 int step_list_max_threads_f32();
-cudaError_t launch_step_list_h16(int K, int walls, const void* insts, const int4* work, int nwork,
-                                 const int* cells, int threads, int grid, int parity, cudaStream_t s);
+cudaError_t launch_step_list_h16(int K, bool multi, const void* insts, const int4* work, int nwork,
+                                 int threads, int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_h16(int K, int threads, int* blocks_per_sm);
 int step_list_max_threads_h16();
-cudaError_t launch_step_list_b16(int K, int walls, const void* insts, const int4* work, int nwork,
-                                 const int* cells, int threads, int grid, int parity, cudaStream_t s);
+cudaError_t launch_step_list_b16(int K, bool multi, const void* insts, const int4* work, int nwork,
+                                 int threads, int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_b16(int K, int threads, int* blocks_per_sm);
 int step_list_max_threads_b16();
 
@@ -105,6 +98,10 @@ cudaError_t launch_ref_table(int K, float* ref, const GeoDev<float>& geo, const 
 // and the instances' omega; prec 2 (FP16) or 3 (BF16), fin any state block.
 cudaError_t launch_stream_table(int prec, int K, float4* st, const float* ref, const InstParams<float>* inst,
                                 const void* fin, const Dims& d, cudaStream_t s);
+
+// Source table of a channel (k_source_table): keys * SRC_ROW int4 at tab; any
+// device address as fin.
+cudaError_t launch_source_table(int4* tab, const void* fin, const Dims& d, cudaStream_t s);
 
 // Observables: NQ sums per instance written to out[batch * DIAG_NQ].
 constexpr int DIAG_NQ = 9;

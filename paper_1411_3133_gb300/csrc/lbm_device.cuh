@@ -56,7 +56,22 @@ struct Dims {
   const float4* st;
   int st_rows3;    // n3 (ellipsoid), 1 (periodic x3), 7 (walls on x3)
   int geo_theta;   // 1: geometry rows (and observable weights) per node
+  // source table (gather_table): SRC_ROW offsets per key of node classes
+  const int4* src;
+  int src_nt, src_n3;  // theta and x3 classes (the key's radices)
 };
+
+// Node class along an axis of n nodes: which of a node's sources lie beyond
+// an end of the axis depends only on its distance to the ends, up to 3 nodes
+// -- 0, 1, 2 (first nodes), 3 (inside), 4, 5, 6 (last nodes); every node is
+// its own class on an axis shorter than 7.
+__host__ __device__ __forceinline__ int axis_classes(int n) { return n < 7 ? n : 7; }
+__host__ __device__ __forceinline__ int axis_class(int i, int n) {
+  return n < 7 || i < 3 ? i : (i > n - 4 ? i - n + 7 : 3);
+}
+// A node of class c.
+__host__ __device__ __forceinline__ int axis_class_node(int c, int n) { return n < 7 || c <= 3 ? c : n - 7 + c; }
+constexpr int SRC_ROW = 11;  // int4 per key: 41 offsets, padded
 
 // Index of reference population l of geometry row r in an instance's table:
 // row-major [r][l] where rows are i_r only (cylinder, flat: a warp shares
@@ -557,6 +572,44 @@ __device__ __forceinline__ void gather(const S* __restrict__ fin, const float* r
     }
   }
   for_each_source<K, S, WALLS>(fin, p, d, GatherPut<K, S, R, RAW>::make(f, ref, d));
+}
+
+// The streamed populations of node p through the source table: entry L of the
+// node's key is (stored population * ncell + source node) - node, so one
+// 32-bit addition forms the address whatever the walls do to the path --
+// folds along r, along x3, corner reflections, equilibrium walls' clamping and
+// every periodic wrap. One code path for all of them keeps the step kernels
+// small: with a compile-time variant per wall layer they were bound by
+// instruction fetch (7 to 19 cycles per issue at the walls).
+template <int K, class S, class R, bool RAW>
+__device__ __forceinline__ void gather_table(const S* __restrict__ fin, const float* ref, const CellPos& p,
+                                             const Dims& d, R (&f)[Q]) {
+  const int key = (axis_class(p.ir, d.nr) * d.src_nt + axis_class(p.it, d.nt)) * d.src_n3 + axis_class(p.i3, d.n3);
+  const int4* __restrict__ row = d.src + key * SRC_ROW;
+  auto put = GatherPut<K, S, R, RAW>::make(f, ref, d);
+  static_for<0, SRC_ROW>([&](auto J_) {
+    constexpr int J = decltype(J_)::value;
+    const int4 o = __ldg(row + J);
+    put(std::integral_constant<int, 4 * J>{}, fin + uint32_t(p.cell + o.x), 0, 0);
+    if constexpr (4 * J + 1 < Q) {
+      put(std::integral_constant<int, 4 * J + 1>{}, fin + uint32_t(p.cell + o.y), 0, 0);
+      put(std::integral_constant<int, 4 * J + 2>{}, fin + uint32_t(p.cell + o.z), 0, 0);
+      put(std::integral_constant<int, 4 * J + 3>{}, fin + uint32_t(p.cell + o.w), 0, 0);
+    }
+  });
+}
+
+// The step's gather: nodes at least 3 nodes from every wall take their sources
+// from the node's own neighbours, computed; a warp that holds any other node
+// reads the source table for all its nodes, so it runs one of the two paths.
+template <int K, class S, class R>
+__device__ __forceinline__ void gather_step(const S* __restrict__ fin, const CellPos& p, const Dims& d, R (&f)[Q]) {
+  constexpr bool RAW = Codec<S, R>::uses_ref;
+  if (__any_sync(__activemask(), near_wall(p, d))) {
+    gather_table<K, S, R, RAW>(fin, nullptr, p, d, f);
+  } else {
+    for_each_source<K, S, 0>(fin, p, d, GatherPut<K, S, R, RAW>::make(f, nullptr, d));
+  }
 }
 
 // Store the 41 post-collision deviations g of node p (2-byte storage).

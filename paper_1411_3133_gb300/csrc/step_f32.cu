@@ -10,21 +10,15 @@ cudaError_t launch_step_f32(int K, const float* fin, float* fout, const GeoDev<f
   return launch_step_t<float, float>(K, fin, fout, geo, inst, d, flag, threads, s);
 }
 
-cudaError_t launch_step_list_f32(int K, int walls, const void* insts, const int4* work, int nwork,
-                                 const int* cells, int threads, int grid, int parity, cudaStream_t s) {
-  return launch_step_list_t<float, float>(K, walls, insts, work, nwork, cells, threads, grid, parity, s);
+cudaError_t launch_step_list_f32(int K, bool multi, const void* insts, const int4* work, int nwork,
+                                 int threads, int grid, int parity, cudaStream_t s) {
+  return launch_step_list_t<float, float>(K, multi, insts, work, nwork, threads, grid, parity, s);
 }
 
 int step_list_max_threads_f32() { return step_list_max_threads_t<float, float>(); }
 
 cudaError_t step_list_occupancy_f32(int K, int threads, int* blocks_per_sm) {
   return step_list_occupancy_t<float, float>(K, threads, blocks_per_sm);
-}
-
-cudaError_t launch_step_split_f32(int K, const float* fin, float* fout, const GeoDev<float>& geo,
-                                  const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                                  cudaStream_t s, cudaStream_t se) {
-  return launch_step_split_t<float, float>(K, fin, fout, geo, inst, d, flag, threads, s, se);
 }
 
 }  // namespace lbgm
