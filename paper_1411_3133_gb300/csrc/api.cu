@@ -3,7 +3,6 @@
 // point. All numerical work runs in the kernels of kernels.cuh / aux.cu.
 #include <cuda_runtime.h>
 
-#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -221,66 +220,17 @@ std::string check_sparsity(const std::vector<double>& rows, const lb_geometry_de
   return "";
 }
 
-bool use_tma(const lb_ctx* c) { return c->prec == LB_FP32 && c->tma_ok && c->step_kernel == 2; }
-
-
-// Region-split step: the wall layers run on the context's second stream,
-// concurrently with the interior on the main stream (fork and join by events,
-// which a graph capture records as branches).
-cudaError_t launch_split(lb_ctx* c, int src, int dst) {
-  cudaError_t e = cudaSuccess;
-  if (!c->aux) {
-    e = cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
-    if (e != cudaSuccess) return e;
-  }
-  e = cudaEventRecord(c->ev_fork, c->stream);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(c->aux, c->ev_fork, 0);
-  if (e != cudaSuccess) return e;
-  switch (c->prec) {
-    case LB_FP16_SHIFTED:
-      e = launch_step_split_h16(c->K, static_cast<const __half*>(c->f[src]), static_cast<__half*>(c->f[dst]),
-                                c->geo_f, static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag,
-                                c->block_threads, c->stream, c->aux);
-      break;
-    default:
-      e = launch_step_split_b16(c->K, static_cast<const __nv_bfloat16*>(c->f[src]),
-                                static_cast<__nv_bfloat16*>(c->f[dst]), c->geo_f,
-                                static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag,
-                                c->block_threads, c->stream, c->aux);
-      break;
-  }
-  cudaError_t e2 = cudaEventRecord(c->ev_join, c->aux);  // join even after a failed launch
-  if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(c->stream, c->ev_join, 0);
-  return e != cudaSuccess ? e : e2;
-}
-
-// The step kernel of the context: the TMA kernel (2) where it was asked for;
-// the region split (4) of 2-byte storage where it applies -- flat and
-// cylinder, periodic x3, bounce-back walls, blocks within an i_r layer -- and
-// neither kernel 1 nor the work list (5) was asked for (measured on 24
-// 64 x 4 x 256 cylinders, FP16: 74.4 us a step against 91.6); else the
-// one-kernel step (1): in FP32 82.4 us against 84.9 for a region split and
-// 103.6 for the work list, 87.0 against 92.1 on 24 four-wall ellipsoids.
-int resolved_kernel(const lb_ctx* c) {
-  if (c->any_shift) return 1;  // the half-force variant runs in the plain kernel only
-  if (use_tma(c)) return 2;
-  const int threads = std::min(c->block_threads, 128);
-  if (c->elem_bytes == 2 && (c->step_kernel == 0 || c->step_kernel == 4) && c->geom.periodic3 &&
-      c->geom.wall == LB_WALL_BOUNCEBACK && (c->K == KFLAT || c->K == KCYL) &&
-      (c->dims.nt * c->dims.n3) % threads == 0)
-    return 4;
-  return 1;
-}
+// The step kernel of the context: the TMA kernel where it was asked for (and
+// no instance uses the half-force variant), else the one-kernel step of the
+// storage type, which also stands for LB_OPT_STEP_KERNEL 4 and 5: on 24
+// 64 x 4 x 256 cylinders in FP32 it takes 82.4 us a step against 84.9 for a
+// region split on two streams and 103.6 for a work list.
+bool use_tma(const lb_ctx* c) { return c->prec == LB_FP32 && c->tma_ok && c->step_kernel == 2 && !c->any_shift; }
 
 lb_status launch_step_once(lb_ctx* c) {
   const int src = c->cur, dst = 1 - c->cur;
-  const int kern = resolved_kernel(c);
   cudaError_t e;
-  if (kern == 4)
-    e = launch_split(c, src, dst);
-  else if (c->any_shift && c->prec == LB_FP64)
+  if (c->any_shift && c->prec == LB_FP64)
     e = launch_step_shift_f64(c->K, static_cast<const double*>(c->f[src]), static_cast<double*>(c->f[dst]),
                               c->geo_d, static_cast<const InstParams<double>*>(c->inst), c->dims, c->flag,
                               c->block_threads, c->stream);
@@ -288,7 +238,7 @@ lb_status launch_step_once(lb_ctx* c) {
     e = launch_step_shift_f32(c->K, static_cast<const float*>(c->f[src]), static_cast<float*>(c->f[dst]),
                               c->geo_f, static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag,
                               c->block_threads, c->stream);
-  else if (kern == 2)
+  else if (use_tma(c))
     e = launch_step_tma_f32(c->K, c->tmap[src], static_cast<const float*>(c->f[src]),
                             static_cast<float*>(c->f[dst]), c->geo_f,
                             static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag, c->stream);
@@ -491,11 +441,15 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
   c->src_tab = static_cast<int4*>(
       dalloc(c, size_t(axis_classes(d.nr)) * d.src_nt * d.src_n3 * SRC_ROW * sizeof(int4)));
   d.src = c->src_tab;
-  d.st_rows3 = c->K == KELL ? d.geo_rows3 : (d.periodic3 ? 1 : 7);
+  const uint32_t np = uint32_t(d.n3 + 1) / 2;
+  d.st_row_r = c->K != KELL && d.periodic3 ? 1 : 0;
+  d.st_rows3 = d.st_row_r ? 1 : int(np);
+  d.div_np = FastDiv::make(np);
+  d.div_wl = FastDiv::make(d.st_row_r ? (uint32_t(d.nt) * np + 31) / 32 : (np + 31) / 32 * uint32_t(d.nt));
   if (c->elem_bytes == 2) {
     c->ref_tab = static_cast<float*>(dalloc(c, size_t(batch) * Q * nrows * sizeof(float)));
     c->st_tab = static_cast<float4*>(
-        dalloc(c, size_t(batch) * ST_K * size_t(geom->nr) * size_t(d.st_rows3) * sizeof(float4)));
+        dalloc(c, size_t(batch) * 2 * ST_K * size_t(geom->nr) * size_t(d.st_rows3) * sizeof(float4)));
     if (!c->ref_tab || !c->st_tab) return bail(LB_ERR_CUDA, "device allocation failed");
     d.ref = c->ref_tab;
     d.st = c->st_tab;
@@ -629,7 +583,7 @@ lb_status lb_step(lb_ctx* c, long long n) {
     }
     // the captured kernels depend on the resolved step kernel and on whether
     // an instance uses the half-force variant (both can change with lb_init)
-    const int gk = 2 * resolved_kernel(c) + (c->any_shift ? 1 : 0);
+    const int gk = use_tma(c) ? 2 : c->any_shift ? 1 : 0;
     if (!c->graph || c->graph_threads != c->block_threads || c->graph_kernel != gk) {
       if (c->graph) cudaGraphExecDestroy(c->graph);
       c->graph = nullptr;
@@ -923,12 +877,6 @@ lb_status lb_autotune(lb_ctx* c, int steps_per_trial, lb_tune* best, lb_tune* tr
 void lb_destroy(lb_ctx* c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
-  if (c->aux) {
-    cudaStreamSynchronize(c->aux);
-    cudaStreamDestroy(c->aux);
-  }
-  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-  if (c->ev_join) cudaEventDestroy(c->ev_join);
   free_all(c);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;

@@ -403,7 +403,7 @@ cudaError_t launch_ref_table(int K, float* ref, const GeoDev<float>& geo, const 
 template <class S>
 cudaError_t launch_stream_table_t(int K, float4* st, const float* ref, const InstParams<float>* inst,
                                   const void* fin, const Dims& d, cudaStream_t s) {
-  const uint32_t n = uint32_t(d.batch) * uint32_t(d.nr) * uint32_t(d.st_rows3);
+  const uint32_t n = uint32_t(d.batch) * uint32_t(d.nr) * uint32_t(d.st_rows3) * 2u;
   const uint32_t nb = (n + 127) / 128;
   const S* f = static_cast<const S*>(fin);
   switch (K) {

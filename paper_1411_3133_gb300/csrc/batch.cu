@@ -18,7 +18,9 @@ using namespace lbgm;
 
 namespace {
 
-constexpr int kMaxGroups = 3;  // flat, cylinder, ellipsoid
+// Flat, cylinder, ellipsoid; in 2-byte storage each metric kind splits into
+// the kernel variants of pair.cuh (parity of n3; rows of i_r alone or not).
+constexpr int kMaxGroups = 10;
 
 struct Group {
   int K = 0;
@@ -27,6 +29,8 @@ struct Group {
   size_t inst_off = 0;     // byte offset of the ListInst records in dmem
   size_t work_off = 0;     // byte offset of the int4 tiles in dmem
   int blocks_per_sm = 0;   // occupancy of the kernel at the built block size
+  Dims d{};                // 2-byte storage: an instance of the group
+  size_t smem = 0;         // 2-byte storage: staged rows of a block, bytes
 };
 
 }  // namespace
@@ -99,7 +103,7 @@ ListInst<S, R> record(const lb_ctx* c, int bi, int cur, const GeoDev<R>& geo) {
   r.d = c->dims;
   r.d.batch = 1;
   if (c->dims.ref) r.d.ref = c->dims.ref + size_t(bi) * Q * size_t(c->dims.nr) * size_t(c->dims.geo_rows3);
-  if (c->dims.st) r.d.st = c->dims.st + size_t(bi) * ST_K * size_t(c->dims.nr) * size_t(c->dims.st_rows3);
+  if (c->dims.st) r.d.st = c->dims.st + size_t(bi) * 2 * ST_K * size_t(c->dims.nr) * size_t(c->dims.st_rows3);
   r.geo = geo;
   r.ip = static_cast<const InstParams<R>*>(c->inst) + bi;
   const size_t off = size_t(bi) * Q * c->ncell;
@@ -109,11 +113,16 @@ ListInst<S, R> record(const lb_ctx* c, int bi, int cur, const GeoDev<R>& geo) {
   return r;
 }
 
+// Kernel variant of a member: its group key.
+int variant(const lb_ctx* c) {
+  return c->K * 4 + (c->elem_bytes == 2 ? (c->dims.n3 % 2) * 2 + (c->dims.st_row_r ? 1 : 0) : 0);
+}
+
 template <class S, class R>
-void append_records(const lb_batch* b, int K, std::vector<unsigned char>& bytes, int* ninst,
+void append_records(const lb_batch* b, int key, std::vector<unsigned char>& bytes, int* ninst,
                     const GeoDev<R> lb_ctx::*geo_member) {
   for (const lb_ctx* c : b->m) {
-    if (c->K != K) continue;
+    if (variant(c) != key) continue;
     for (int bi = 0; bi < c->batch; ++bi) {
       const ListInst<S, R> r = record<S, R>(c, bi, c->cur, c->*geo_member);
       const unsigned char* p = reinterpret_cast<const unsigned char*>(&r);
@@ -123,21 +132,14 @@ void append_records(const lb_batch* b, int K, std::vector<unsigned char>& bytes,
   }
 }
 
-int max_threads(lb_precision p) {
-  switch (p) {
-    case LB_FP64: return step_list_max_threads_f64();
-    case LB_FP32: return step_list_max_threads_f32();
-    case LB_FP16_SHIFTED: return step_list_max_threads_h16();
-    default: return step_list_max_threads_b16();
-  }
-}
+int max_threads(lb_precision p) { return p == LB_FP64 ? 256 : 128; }  // the kernels' launch bounds
 
-cudaError_t occupancy(lb_precision p, int K, int threads, int* out) {
+cudaError_t occupancy(lb_precision p, const Group& g, int threads, int* out) {
   switch (p) {
-    case LB_FP64: return step_list_occupancy_f64(K, threads, out);
-    case LB_FP32: return step_list_occupancy_f32(K, threads, out);
-    case LB_FP16_SHIFTED: return step_list_occupancy_h16(K, threads, out);
-    default: return step_list_occupancy_b16(K, threads, out);
+    case LB_FP64: return step_list_occupancy_f64(g.K, threads, out);
+    case LB_FP32: return step_list_occupancy_f32(g.K, threads, out);
+    case LB_FP16_SHIFTED: return step_list_occupancy_h16(g.K, g.d, g.smem, threads, out);
+    default: return step_list_occupancy_b16(g.K, g.d, g.smem, threads, out);
   }
 }
 
@@ -150,30 +152,38 @@ lb_status build(lb_batch* b) {
   std::vector<unsigned char> recs;
   std::vector<int4> tiles[kMaxGroups];
   b->ngroups = 0;
-  for (int K : {int(KCYL), int(KELL), int(KFLAT)}) {
+  std::vector<int> keys;
+  for (int K : {int(KCYL), int(KELL), int(KFLAT)})
+    for (int v = 0; v < 4; ++v) keys.push_back(K * 4 + v);
+  for (int key : keys) {
     Group gr;
-    gr.K = K;
+    gr.K = key / 4;
     const size_t before = recs.size();
     switch (b->prec) {
-      case LB_FP64: append_records<double, double>(b, K, recs, &gr.ninst, &lb_ctx::geo_d); break;
-      case LB_FP32: append_records<float, float>(b, K, recs, &gr.ninst, &lb_ctx::geo_f); break;
-      case LB_FP16_SHIFTED: append_records<__half, float>(b, K, recs, &gr.ninst, &lb_ctx::geo_f); break;
-      default: append_records<__nv_bfloat16, float>(b, K, recs, &gr.ninst, &lb_ctx::geo_f); break;
+      case LB_FP64: append_records<double, double>(b, key, recs, &gr.ninst, &lb_ctx::geo_d); break;
+      case LB_FP32: append_records<float, float>(b, key, recs, &gr.ninst, &lb_ctx::geo_f); break;
+      case LB_FP16_SHIFTED: append_records<__half, float>(b, key, recs, &gr.ninst, &lb_ctx::geo_f); break;
+      default: append_records<__nv_bfloat16, float>(b, key, recs, &gr.ninst, &lb_ctx::geo_f); break;
     }
     if (gr.ninst == 0) continue;
     gr.inst_off = before;
     // tiles, instance-major; instance ids are local to the group
     std::vector<int4>& t = tiles[b->ngroups];
-    const int tile = b->threads * b->tile_blocks;
+    const bool pairs = b->prec == LB_FP16_SHIFTED || b->prec == LB_BF16_SHIFTED;
+    const int tile = (pairs ? b->threads / 32 : b->threads) * b->tile_blocks;  // warps or nodes
     int local = 0;
     for (const lb_ctx* c : b->m) {
-      if (c->K != K) continue;
-      const int n = c->dims.ncell;
+      if (variant(c) != key) continue;
+      const int n = pairs ? int(pair_warps(c->dims)) : c->dims.ncell;
       for (int bi = 0; bi < c->batch; ++bi, ++local)
         for (int a = 0; a < n; a += tile) t.push_back(make_int4(local, a, std::min(tile, n - a), 0));
+      if (pairs) {
+        gr.d = c->dims;
+        gr.smem = std::max(gr.smem, pair_smem_bytes(c->dims, b->threads / 32));
+      }
     }
     gr.nwork = int(t.size());
-    cudaError_t e = occupancy(b->prec, K, b->threads, &gr.blocks_per_sm);
+    cudaError_t e = occupancy(b->prec, gr, b->threads, &gr.blocks_per_sm);
     if (e != cudaSuccess) return bcuda(b, e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     b->g[b->ngroups++] = gr;
   }
@@ -227,12 +237,13 @@ cudaError_t launch_group(const lb_batch* b, const Group& gr, cudaStream_t s) {
     case LB_FP64: return launch_step_list_f64(gr.K, multi, insts, work, gr.nwork, b->threads, grid, b->parity, s);
     case LB_FP32: return launch_step_list_f32(gr.K, multi, insts, work, gr.nwork, b->threads, grid, b->parity, s);
     case LB_FP16_SHIFTED:
-      return launch_step_list_h16(gr.K, multi, insts, work, gr.nwork, b->threads, grid, b->parity, s);
-    default: return launch_step_list_b16(gr.K, multi, insts, work, gr.nwork, b->threads, grid, b->parity, s);
+      return launch_step_list_h16(gr.K, gr.d, gr.smem, insts, work, gr.nwork, b->threads, grid, b->parity, s);
+    default:
+      return launch_step_list_b16(gr.K, gr.d, gr.smem, insts, work, gr.nwork, b->threads, grid, b->parity, s);
   }
 }
 
-// One batch step. The metric kinds read the same buffers and write disjoint
+// One batch step. The groups read the same buffers and write disjoint
 // nodes, so they run side by side: the first on the batch stream, the others
 // forked before it and joined back.
 lb_status step_once(lb_batch* b) {

@@ -111,6 +111,18 @@ __device__ __forceinline__ Moments<V> moments(const V (&f)[Q]) {
   return m;
 }
 
+// The 41 populations (or stored deviations) of a node as moments_shells and
+// collide_shells see them: get<L> reads one, put<L> takes its post-collision
+// value, each L once and after its get. PopArray holds them in an array.
+template <typename V>
+struct PopArray {
+  V (&f)[Q];
+  template <int L>
+  __device__ __forceinline__ V get() const { return f[L]; }
+  template <int L>
+  __device__ __forceinline__ void put(const V& v) const { f[L] = v; }
+};
+
 // acc + (C w) x of a shell: with W the shell's weight is part of the
 // coefficient (2-byte storage, whose populations are deviations over their
 // weight), else the coefficient is C alone.
@@ -142,35 +154,35 @@ struct Had4 {
 // populations are stored deviations g, f_l = w_l g_l + rho_l, and m0 holds the
 // streamed references' moments; without it f are the populations and m0 is
 // not read.
-template <bool W, typename V>
-__device__ __forceinline__ Moments<V> moments_shells(const V (&f)[Q], const Moments<V>& m0) {
+template <bool W, typename V, class Pop>
+__device__ __forceinline__ Moments<V> moments_shells(const Pop& f, const Moments<V>& m0) {
   Moments<V> m;
-  auto S = [&](int P) { return f[2 * P + 1] + f[2 * P + 2]; };
-  auto D = [&](int P) { return f[2 * P + 1] - f[2 * P + 2]; };
+#define LB_S(P) (f.template get<2 * (P) + 1>() + f.template get<2 * (P) + 2>())
+#define LB_D(P) (f.template get<2 * (P) + 1>() - f.template get<2 * (P) + 2>())
   // |c| = 1 along an axis
-  const V s0 = S(0), s1 = S(1), s2 = S(2);
+  const V s0 = LB_S(0), s1 = LB_S(1), s2 = LB_S(2);
   if constexpr (W) {
     m = m0;
-    m.rho = fmav(V(W_REST), f[0], m.rho);
+    m.rho = fmav(V(W_REST), f.template get<0>(), m.rho);
     m.sxx = acc_shell<W, 1, 0>(m.sxx, s0);
     m.syy = acc_shell<W, 1, 0>(m.syy, s1);
     m.szz = acc_shell<W, 1, 0>(m.szz, s2);
-    m.jx = acc_shell<W, 1, 0>(m.jx, D(0));
-    m.jy = acc_shell<W, 1, 0>(m.jy, D(1));
-    m.jz = acc_shell<W, 1, 0>(m.jz, D(2));
+    m.jx = acc_shell<W, 1, 0>(m.jx, LB_D(0));
+    m.jy = acc_shell<W, 1, 0>(m.jy, LB_D(1));
+    m.jz = acc_shell<W, 1, 0>(m.jz, LB_D(2));
   } else {
-    m.rho = f[0];
+    m.rho = f.template get<0>();
     m.sxx = s0;
     m.syy = s1;
     m.szz = s2;
-    m.jx = D(0);
-    m.jy = D(1);
-    m.jz = D(2);
+    m.jx = LB_D(0);
+    m.jy = LB_D(1);
+    m.jz = LB_D(2);
   }
   m.rho = acc_shell<W, 1, 0>(m.rho, s0 + s1 + s2);
   // (+-1, +-1, 0) faces
   {
-    const V axy = S(3), bxy = S(4), axz = S(5), bxz = S(6), ayz = S(7), byz = S(8);
+    const V axy = LB_S(3), bxy = LB_S(4), axz = LB_S(5), bxz = LB_S(6), ayz = LB_S(7), byz = LB_S(8);
     const V pxy = axy + bxy, pxz = axz + bxz, pyz = ayz + byz;
     m.rho = acc_shell<W, 1, 3>(m.rho, pxy + pxz + pyz);
     m.sxx = acc_shell<W, 1, 3>(m.sxx, pxy + pxz);
@@ -185,24 +197,24 @@ __device__ __forceinline__ Moments<V> moments_shells(const V (&f)[Q], const Mome
       m.sxz = axz - bxz;
       m.syz = ayz - byz;
     }
-    const V dxy = D(3), exy = D(4), dxz = D(5), exz = D(6), dyz = D(7), eyz = D(8);
+    const V dxy = LB_D(3), exy = LB_D(4), dxz = LB_D(5), exz = LB_D(6), dyz = LB_D(7), eyz = LB_D(8);
     m.jx = acc_shell<W, 1, 3>(m.jx, (dxy + exy) + (dxz + exz));
     m.jy = acc_shell<W, 1, 3>(m.jy, (dxy - exy) + (dyz + eyz));
     m.jz = acc_shell<W, 1, 3>(m.jz, (dxz - exz) + (dyz - eyz));
   }
   // 3 along an axis
   {
-    const V t0 = S(13), t1 = S(14), t2 = S(15);
+    const V t0 = LB_S(13), t1 = LB_S(14), t2 = LB_S(15);
     m.rho = acc_shell<W, 1, 13>(m.rho, t0 + t1 + t2);
     m.sxx = acc_shell<W, 9, 13>(m.sxx, t0);
     m.syy = acc_shell<W, 9, 13>(m.syy, t1);
     m.szz = acc_shell<W, 9, 13>(m.szz, t2);
-    m.jx = acc_shell<W, 3, 13>(m.jx, D(13));
-    m.jy = acc_shell<W, 3, 13>(m.jy, D(14));
-    m.jz = acc_shell<W, 3, 13>(m.jz, D(15));
+    m.jx = acc_shell<W, 3, 13>(m.jx, LB_D(13));
+    m.jy = acc_shell<W, 3, 13>(m.jy, LB_D(14));
+    m.jz = acc_shell<W, 3, 13>(m.jz, LB_D(15));
   }
   // (+-1, +-1, +-1) and (+-3, +-3, +-3)
-  const Had4<V> b1(S(9), S(10), S(11), S(12)), b3(S(16), S(17), S(18), S(19));
+  const Had4<V> b1(LB_S(9), LB_S(10), LB_S(11), LB_S(12)), b3(LB_S(16), LB_S(17), LB_S(18), LB_S(19));
   m.rho = acc_shell<W, 1, 16>(acc_shell<W, 1, 9>(m.rho, b1.t), b3.t);
   V T;
   if constexpr (W) T = acc_shell<W, 9, 16>(V(Pair<9>::w) * b1.t, b3.t);
@@ -213,16 +225,18 @@ __device__ __forceinline__ Moments<V> moments_shells(const V (&f)[Q], const Mome
   m.sxy = acc_shell<W, 9, 16>(acc_shell<W, 1, 9>(m.sxy, b1.xy), b3.xy);
   m.sxz = acc_shell<W, 9, 16>(acc_shell<W, 1, 9>(m.sxz, b1.xz), b3.xz);
   m.syz = acc_shell<W, 9, 16>(acc_shell<W, 1, 9>(m.syz, b1.yz), b3.yz);
-  const Had4<V> e1(D(9), D(10), D(11), D(12)), e3(D(16), D(17), D(18), D(19));
+  const Had4<V> e1(LB_D(9), LB_D(10), LB_D(11), LB_D(12)), e3(LB_D(16), LB_D(17), LB_D(18), LB_D(19));
   m.jx = acc_shell<W, 3, 16>(acc_shell<W, 1, 9>(m.jx, e1.t), e3.t);
   m.jy = acc_shell<W, 3, 16>(acc_shell<W, 1, 9>(m.jy, e1.xy), e3.xy);
   m.jz = acc_shell<W, 3, 16>(acc_shell<W, 1, 9>(m.jz, e1.xz), e3.xz);
+#undef LB_S
+#undef LB_D
   return m;
 }
 
 template <typename V>
-__device__ __forceinline__ Moments<V> step_moments(const V (&f)[Q]) {
-  return moments_shells<false>(f, Moments<V>{});
+__device__ __forceinline__ Moments<V> step_moments(V (&f)[Q]) {
+  return moments_shells<false, V>(PopArray<V>{f}, Moments<V>{});
 }
 
 // Geometry of one node, read for the metric kind K. The Christoffel symbols
@@ -286,7 +300,7 @@ __device__ __forceinline__ Coef<V> coefficients(const Moments<V>& m, const NodeG
   c.uy = uy;
   c.uz = uz;
   const V uu = fmav(uz, uz, fmav(uy, uy, ux * ux));
-  V trD = g.dtt;
+  V trD = K == KFLAT ? V(0.0) : g.dtt;
   if constexpr (K == KELL || K == KELT) trD = trD + g.dpp;
   if constexpr (K == KELT) trD = trD + g.drr;
   c.rho = rho;
@@ -345,8 +359,11 @@ __device__ __forceinline__ Coef<V> coefficients(const Moments<V>& m, const NodeG
     c.naxz = fmav(rk, ux * uz, kn * m.sxz);
     c.nayz = fmav(rk, uy * uz, kn * m.syz);
   }
-  c.nayy = fmav(rk, fmav(cs2, g.dtt, uy * uy), kn * (m.syy - rc));
-  c.nazz = fmav(rk, fmav(cs2, g.dpp, uz * uz), kn * (m.szz - rc));
+  V yy = uy * uy, zz = uz * uz;
+  if constexpr (K != KFLAT) yy = fmav(cs2, g.dtt, yy);
+  if constexpr (K == KELL || K == KELT) zz = fmav(cs2, g.dpp, zz);
+  c.nayy = fmav(rk, yy, kn * (m.syy - rc));
+  c.nazz = fmav(rk, zz, kn * (m.szz - rc));
   c.t0 = fmav(V(0.5), c.naxx + c.nayy + c.nazz, rho * inv_cs2);
   c.fext_t = G * g.fth;
   if constexpr (K == KELT) {
@@ -362,25 +379,24 @@ __device__ __forceinline__ Coef<V> coefficients(const Moments<V>& m, const NodeG
 // or, with DEV, for the stored deviations g = (f - r) / w of 2-byte storage
 //   g* = (1 - omega) g + a +- B
 // (a and B then include the stream table's t, see collide_shells).
-template <int P, bool DEV, typename V>
-__device__ __forceinline__ void update_pair(V (&f)[Q], const V& om1, const V& a, const V& B) {
-  V& fp = f[2 * P + 1];
-  V& fm = f[2 * P + 2];
+template <int P, bool DEV, typename V, class Pop>
+__device__ __forceinline__ void update_pair(const Pop& f, const V& om1, const V& a, const V& B) {
+  const V fp = f.template get<2 * P + 1>(), fm = f.template get<2 * P + 2>();
   if constexpr (DEV) {
-    fp = fmav(om1, fp, a + B);
-    fm = fmav(om1, fm, a - B);
+    f.template put<2 * P + 1>(fmav(om1, fp, a + B));
+    f.template put<2 * P + 2>(fmav(om1, fm, a - B));
   } else {
     const V w = V(Pair<P>::w);
     const V Bw = B * w;
-    fp = fmav(om1, fp, fmav(a, w, Bw));
-    fm = fmav(om1, fm, fmav(a, w, -Bw));
+    f.template put<2 * P + 1>(fmav(om1, fp, fmav(a, w, Bw)));
+    f.template put<2 * P + 2>(fmav(om1, fm, fmav(a, w, -Bw)));
   }
 }
 
 // The two pairs P, P + 1 of a face shell, c = s_i e_i +- s_j e_j: even part
 // base +- x, odd part bi s_i + bj s_j.
-template <int P, bool DEV, typename V>
-__device__ __forceinline__ void update_face(V (&f)[Q], const V& om1, const V& base, const V& x, const V& bi,
+template <int P, bool DEV, typename V, class Pop>
+__device__ __forceinline__ void update_face(const Pop& f, const V& om1, const V& base, const V& x, const V& bi,
                                             const V& bj) {
   update_pair<P, DEV>(f, om1, base + x, bi + bj);
   update_pair<P + 1, DEV>(f, om1, base - x, bi - bj);
@@ -389,8 +405,8 @@ __device__ __forceinline__ void update_face(V (&f)[Q], const V& om1, const V& ba
 // The four pairs P .. P + 3 of a (1, +-1, +-1)-type shell: even part
 // base + xy s_x s_y + xz s_x s_z + yz s_y s_z, odd part bx s_x + by s_y + bz s_z
 // + d s_x s_y s_z, each a 4-point Hadamard transform.
-template <int P, bool DEV, typename V>
-__device__ __forceinline__ void update_body(V (&f)[Q], const V& om1, const V& base, const V& xy, const V& xz,
+template <int P, bool DEV, typename V, class Pop>
+__device__ __forceinline__ void update_body(const Pop& f, const V& om1, const V& base, const V& xy, const V& xz,
                                             const V& yz, const V& bx, const V& by, const V& bz, const V& d) {
   const V ep = base + xy, em = base - xy, eq = xz + yz, er = xz - yz;
   const V op = bx + by, om = bx - by, oq = bz + d, orr = bz - d;
@@ -423,17 +439,21 @@ struct NoTab {};
 // Starting values of a shell's coefficients: with 2-byte storage the stream
 // table's t, transformed to the shells' coefficient space (k_stream_table),
 // else nothing. E and O of slot P live in entry 3 + P / 2.
+template <typename V>
+struct TabEntry {
+  V x, y, z, w;
+};
 template <bool DEV, typename V>
 struct Start {
-  float4 t;
+  TabEntry<V> t;
   template <int P>
   __device__ __forceinline__ V e(const V& x) const {
-    if constexpr (DEV) return x + V(P % 2 == 0 ? t.x : t.z);
+    if constexpr (DEV) return x + (P % 2 == 0 ? t.x : t.z);
     else return x;
   }
   template <int P>
   __device__ __forceinline__ V o(const V& x) const {
-    if constexpr (DEV) return x + V(P % 2 == 0 ? t.y : t.w);
+    if constexpr (DEV) return x + (P % 2 == 0 ? t.y : t.w);
     else return x;
   }
 };
@@ -467,8 +487,8 @@ struct Start {
 // with te, to the even and odd parts of t = ((1 - omega) rho - r) / w from the
 // stream table `tab`, in coefficient space: they are added to the shells'
 // coefficients instead of to every pair.
-template <typename V, int K, class Tab = NoTab>
-__device__ __forceinline__ void collide_shells(V (&f)[Q], const Coef<V>& k, const NodeGeo<V, K>& g, const V& omega,
+template <typename V, int K, class Pop, class Tab = NoTab>
+__device__ __forceinline__ void collide_shells(const Pop& f, const Coef<V>& k, const NodeGeo<V, K>& g, const V& omega,
                                                const Tab& tab, const V& t_rest) {
   constexpr bool DEV = !std::is_same<Tab, NoTab>::value;
   constexpr bool curv = K != KFLAT;
@@ -579,8 +599,8 @@ __device__ __forceinline__ void collide_shells(V (&f)[Q], const Coef<V>& k, cons
   const V h2 = V(1.0 - 1.0 / CS2);  // 1 + 2 h
 
   // rest velocity
-  if constexpr (DEV) f[0] = fmav(om1, f[0], a0 + t_rest);
-  else f[0] = fmav(om1, f[0], a0 * V(REST_WEIGHT<V>));
+  if constexpr (DEV) f.template put<0>(fmav(om1, f.template get<0>(), a0 + t_rest));
+  else f.template put<0>(fmav(om1, f.template get<0>(), a0 * V(REST_WEIGHT<V>)));
 
   // axes, |c| = 1 and 3: even a0 + m^2 M_ii, odd m L_i + m^3 C_i
   {
@@ -761,7 +781,7 @@ __device__ __forceinline__ void collide_shells(V (&f)[Q], const Coef<V>& k, cons
 
 template <typename V, int K>
 __device__ __forceinline__ void collide(V (&f)[Q], const Coef<V>& k, const NodeGeo<V, K>& g, const V& omega) {
-  collide_shells<V, K>(f, k, g, omega, NoTab{}, V(0.0));
+  collide_shells<V, K>(PopArray<V>{f}, k, g, omega, NoTab{}, V(0.0));
 }
 
 // f^eq(rho, u) for all 41 velocities (initial state, Sec. II).

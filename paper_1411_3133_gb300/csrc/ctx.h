@@ -64,11 +64,9 @@ struct lb_ctx {
   int use_graph = 0;
   cudaGraphExec_t graph = nullptr;   // two steps, buffer 0 -> 1 -> 0
   int graph_threads = 0;
-  int graph_kernel = -1;             // 2 x resolved step kernel + any_shift of the captured graph
+  int graph_kernel = -1;             // captured graph: 0 the step, 1 with the half-force variant, 2 TMA
   int step_kernel = 0;               // LB_OPT_STEP_KERNEL
   bool any_shift = false;            // an instance uses the half-force velocity (old_forcing 2)
-  cudaStream_t aux = nullptr;        // second stream of the region-split step
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool tma_ok = false;               // tensor maps built for both buffers
   alignas(64) unsigned char tmap[2][128];
 };

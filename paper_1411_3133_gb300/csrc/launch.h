@@ -35,33 +35,23 @@ cudaError_t launch_step_shift_f32(int K, const float* fin, float* fout, const Ge
                                   const InstParams<float>* inst, const Dims& d, int* flag, int threads,
                                   cudaStream_t s);
 
-// Region-split step of 2-byte storage (periodic x3): wall layers on stream se,
-// interior on s.
-cudaError_t launch_step_split_h16(int K, const __half* fin, __half* fout, const GeoDev<float>& geo,
-                                  const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                                  cudaStream_t s, cudaStream_t se);
-cudaError_t launch_step_split_b16(int K, const __nv_bfloat16* fin, __nv_bfloat16* fout, const GeoDev<float>& geo,
-                                  const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                                  cudaStream_t s, cudaStream_t se);
-
-// Work-list step over instances of different geometry (ListInst<S, R> array);
-// multi: items longer than one block; grid 0 launches one block per item.
-cudaError_t launch_step_list_f64(int K, bool multi, const void* insts, const int4* work, int nwork,
-                                 int threads, int grid, int parity, cudaStream_t s);
+// Work-list step over instances of different geometry (ListInst array); multi:
+// items longer than one block; grid 0 launches one block per item. FP32, FP64:
+// item (instance, first node, nodes). 2-byte storage: item (instance, first
+// warp, warps) over a group of one metric kind, row kind and parity of n3 --
+// d any of its instances, smem the bytes of staged rows a block needs.
+cudaError_t launch_step_list_f64(int K, bool multi, const void* insts, const int4* work, int nwork, int threads,
+                                 int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_f64(int K, int threads, int* blocks_per_sm);
-int step_list_max_threads_f64();
-cudaError_t launch_step_list_f32(int K, bool multi, const void* insts, const int4* work, int nwork,
-                                 int threads, int grid, int parity, cudaStream_t s);
+cudaError_t launch_step_list_f32(int K, bool multi, const void* insts, const int4* work, int nwork, int threads,
+                                 int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_f32(int K, int threads, int* blocks_per_sm);
-int step_list_max_threads_f32();
-cudaError_t launch_step_list_h16(int K, bool multi, const void* insts, const int4* work, int nwork,
-                                 int threads, int grid, int parity, cudaStream_t s);
-cudaError_t step_list_occupancy_h16(int K, int threads, int* blocks_per_sm);
-int step_list_max_threads_h16();
-cudaError_t launch_step_list_b16(int K, bool multi, const void* insts, const int4* work, int nwork,
-                                 int threads, int grid, int parity, cudaStream_t s);
-cudaError_t step_list_occupancy_b16(int K, int threads, int* blocks_per_sm);
-int step_list_max_threads_b16();
+cudaError_t launch_step_list_h16(int K, const Dims& d, size_t smem, const void* insts, const int4* work,
+                                 int nwork, int threads, int grid, int parity, cudaStream_t s);
+cudaError_t step_list_occupancy_h16(int K, const Dims& d, size_t smem, int threads, int* blocks_per_sm);
+cudaError_t launch_step_list_b16(int K, const Dims& d, size_t smem, const void* insts, const int4* work,
+                                 int nwork, int threads, int grid, int parity, cudaStream_t s);
+cudaError_t step_list_occupancy_b16(int K, const Dims& d, size_t smem, int threads, int* blocks_per_sm);
 
 // TMA-pipelined FP32 step (n3 in {128, 256}); map is a CUtensorMap over the
 // input state (make_state_tensor_map).

@@ -51,10 +51,13 @@ struct Dims {
   // rows, per instance (ref_index; NULL for FP32 / FP64 storage)
   const float* ref;
   int wall_eq;     // 1: equilibrium (Dirichlet) walls on the end nodes
-  // 2-byte storage: the stream table of each instance (stream_index; NULL
-  // for FP32 / FP64 storage) over nr * st_rows3 stream rows
+  // 2-byte storage: the stream table of each instance (stream_of; NULL for
+  // FP32 / FP64 storage) over nr * st_rows3 stream rows, and the divisors of
+  // the pair kernels' node numbering
   const float4* st;
-  int st_rows3;    // n3 (ellipsoid), 1 (periodic x3), 7 (walls on x3)
+  int st_rows3;    // rows per i_r: 1, or the x3 pairs (n3 + 1) / 2
+  int st_row_r;    // 1: rows of i_r alone (flat and cylinder, periodic x3)
+  FastDiv div_np, div_wl;  // x3 pairs per line, warps per i_r layer
   int geo_theta;   // 1: geometry rows (and observable weights) per node
   // source table (gather_table): SRC_ROW offsets per key of node classes
   const int4* src;
@@ -106,28 +109,17 @@ __device__ __forceinline__ const float* ref_of(const Dims& d, int b) {
   return d.ref ? d.ref + size_t(b) * 41 * size_t(d.nr) * size_t(d.geo_rows3) : nullptr;
 }
 
-// Stream rows of 2-byte storage. Which stored population (and whose
-// geometry row's reference) a node receives in streaming depends on its
-// position only through i_r and, with walls on x3, through its distance to
-// them; theta is periodic and the references do not depend on it. A stream
-// row groups the nodes that receive alike: (i_r, i_3) for the ellipsoid
-// (its references vary along x3), i_r for a periodic x3, and (i_r, class of
-// i_3) with classes 0, 1, 2 (first layers), 3 (inside), 4, 5, 6 (last
-// layers) for walls on x3.
-template <int K>
-__device__ __forceinline__ int stream_row(const Dims& d, int ir, int i3) {
-  if constexpr (K == KELL) return ir * d.geo_rows3 + i3;
-  if (d.st_rows3 == 1) return ir;
-  const int c = i3 < 3 ? i3 : (i3 > d.n3 - 4 ? i3 - d.n3 + 7 : 3);
-  return ir * 7 + c;
-}
-
-// Stream table of instance b: 13 float4 per stream row, stored [k][row]
-// (consecutive rows are consecutive float4, so a warp of consecutive i_3
-// reads coalesced). Entry k of row s (f_l = w_l g_l + rho_l: g the stored
-// deviation, rho_l the reference population of the stored value a node of
-// row s receives as population l, t_l = ((1 - omega) rho_l - r_l) / w_l with
-// r_l the node's own reference):
+// Stream table of instance b (2-byte storage). Which stored population (and
+// whose geometry row's reference) a node receives in streaming does not
+// depend on theta, and for the flat channel and the cylinder with a periodic
+// x3 not on x3 either: a stream row is an i_r layer there, else the pair
+// (i_3 = 2 p, 2 p + 1) of an (i_r, x3) line. A row holds 13 entries of 4
+// values for both nodes of the pair, stored [2 k + half][row] as float4 (x of
+// both nodes, y of both) and (z of both, w of both): consecutive pairs are
+// consecutive float4. Entry k (f_l = w_l g_l + rho_l: g the stored deviation,
+// rho_l the reference population of the stored value the node receives as
+// population l, t_l = ((1 - omega) rho_l - r_l) / w_l with r_l the node's own
+// reference):
 //   k = 0: sum rho_l, sum c^x rho_l, sum c^y rho_l, sum c^z rho_l
 //   k = 1: sum c^x c^x rho_l, c^y c^y, c^z c^z, c^x c^y
 //   k = 2: sum c^x c^z rho_l, sum c^y c^z rho_l, t_0, 0
@@ -139,7 +131,7 @@ __device__ __forceinline__ int stream_row(const Dims& d, int ir, int i3) {
 //           4-point Hadamard transform over 4 of a body shell's four
 constexpr int ST_K = 13;
 __device__ __forceinline__ const float4* stream_of(const Dims& d, int b) {
-  return d.st + size_t(b) * ST_K * size_t(d.nr) * size_t(d.st_rows3);
+  return d.st + size_t(b) * 2 * ST_K * size_t(d.nr) * size_t(d.st_rows3);
 }
 
 // Geometry rows in the compute precision. A row is i_r * geo_rows3 + i_3 (or
@@ -242,17 +234,6 @@ struct Codec<__nv_bfloat16, float> {
     return __float2bfloat16_rn((f - __ldg(ref)) * iw);
   }
 };
-
-// The stored number itself (2-byte storage: the deviation g) in FP32 and
-// back, round to nearest.
-__device__ __forceinline__ float raw_dec(__half v) { return __half2float(v); }
-__device__ __forceinline__ float raw_dec(__nv_bfloat16 v) { return __bfloat162float(v); }
-template <class S>
-__device__ __forceinline__ S raw_enc(float x);
-template <>
-__device__ __forceinline__ __half raw_enc<__half>(float x) { return __float2half_rn(x); }
-template <>
-__device__ __forceinline__ __nv_bfloat16 raw_enc<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
 
 // ---------------------------------------------------------------------------
 // pull streaming
@@ -420,43 +401,32 @@ __device__ __forceinline__ void for_each_source_wall(const S* __restrict__ fin, 
   });
 }
 
-// WALLS selects the code paths compiled in: 0 far from every wall only, 1
-// near a wall only, 2 both (the node decides).
-template <int K, class S, int WALLS = 2, class Fn>
+template <int K, class S, class Fn>
 __device__ __forceinline__ void for_each_source(const S* __restrict__ fin, const CellPos& p, const Dims& d,
                                                 Fn&& fn) {
   fn(std::integral_constant<int, 0>{}, fin + uint32_t(p.cell), 0, geo_row<K>(d, p.ir, p.i3));
-  if constexpr (WALLS == 0) {
+  if (!near_wall(p, d))
     for_each_source_far<K>(fin, p, d, fn);
-  } else if constexpr (WALLS == 1) {
+  else
     for_each_source_wall<K>(fin, p, d, fn);
-  } else {
-    if (!near_wall(p, d))
-      for_each_source_far<K>(fin, p, d, fn);
-    else
-      for_each_source_wall<K>(fin, p, d, fn);
-  }
 }
 
-// Sources for a node J = 0, 1, 2 layers from the wall on side SIDE (0: low,
-// 1: high) of axis AX (0: r, 2: x3), at least 3 layers from the walls of
-// the other axis (or with that axis periodic), the walled axis at least 7
-// nodes long: only that wall can lie on a population's one-step path, so the
-// wall rule of src_wall reduces to constants. A population whose backward
-// path (along -c, length s = |c|_inf) meets the wall 2 J + 1 half-nodes away
-// folds once: its source is x + (s - 1 - 2 J) sigma (sigma = c / s) and it
-// arrives flipped; every other population comes from x - c as away from
-// walls.
-template <int AX, int SIDE, int J, int CX, int CY, int CZ, int S>
+// Sources for a node J = 0, 1, 2 layers from the r-wall on side SIDE (0: low,
+// 1: high), at least 3 layers from the x3-walls (or x3 periodic), nr >= 7:
+// only that wall can lie on a population's one-step path, so the wall rule of
+// src_wall reduces to constants. A population whose backward path (along -c,
+// length s = |c|_inf) meets the wall 2 J + 1 half-nodes away folds once: its
+// source is x + (s - 1 - 2 J) sigma (sigma = c / s) and it arrives flipped;
+// every other population comes from x - c as away from walls.
+template <int SIDE, int J, int CX, int CY, int CZ, int S>
 struct LayerFold {
   static constexpr int sx = (CX > 0) - (CX < 0), sy = (CY > 0) - (CY < 0), sz = (CZ > 0) - (CZ < 0);
-  static constexpr int sa = AX == 0 ? sx : sz;
-  static constexpr bool hit = ((SIDE == 0 && sa > 0) || (SIDE == 1 && sa < 0)) && (2 * S > 1 + 2 * J);
+  static constexpr bool hit = ((SIDE == 0 && sx > 0) || (SIDE == 1 && sx < 0)) && (2 * S > 1 + 2 * J);
   static constexpr int q = hit ? S - 1 - 2 * J : -S;
   static constexpr int dx = q * sx, dy = q * sy, dz = q * sz;  // source - node
 };
 
-template <int K, int AX, int SIDE, int J, class S, class Fn>
+template <int K, int SIDE, int J, class S, class Fn>
 __device__ __forceinline__ void for_each_source_layer(const S* __restrict__ fin, const CellPos& p,
                                                       const Dims& d, Fn&& fn) {
   const uint32_t N = uint32_t(d.ncell);
@@ -465,8 +435,8 @@ __device__ __forceinline__ void for_each_source_layer(const S* __restrict__ fin,
   static_for<0, NPAIR>([&](auto P_) {
     constexpr int P = decltype(P_)::value;
     using C = Pair<P>;
-    using Fp = LayerFold<AX, SIDE, J, C::x, C::y, C::z, C::s>;
-    using Fm = LayerFold<AX, SIDE, J, -C::x, -C::y, -C::z, C::s>;
+    using Fp = LayerFold<SIDE, J, C::x, C::y, C::z, C::s>;
+    using Fm = LayerFold<SIDE, J, -C::x, -C::y, -C::z, C::s>;
     const uint32_t sp = uint32_t((nb.rrow[3 - Fp::dx] + nb.tcol[3 - Fp::dy]) * d.n3 + nb.zcol[3 - Fp::dz]);
     const uint32_t sm = uint32_t((nb.rrow[3 - Fm::dx] + nb.tcol[3 - Fm::dy]) * d.n3 + nb.zcol[3 - Fm::dz]);
     constexpr int lp = Fp::hit ? 2 * P + 2 : 2 * P + 1, lm = Fm::hit ? 2 * P + 1 : 2 * P + 2;
@@ -494,84 +464,41 @@ struct DecodeInto {
   }
 };
 
-// Raw visitor of 2-byte storage: f[L] holds the stored deviation g itself
-// (the step works on deviations; see collide_store).
-template <class S>
-struct RawInto {
-  float (&f)[Q];
-  template <class LC>
-  __device__ __forceinline__ void operator()(LC, const S* src, int, int) const {
-    f[LC::value] = raw_dec(__ldg(src));
-  }
-};
-
-// Streamed populations of a node within 3 layers of a wall of axis AX (0:
-// an r-wall, with x3 periodic or the node at least 3 layers from the
-// x3-walls, nr >= 7; 2: an x3-wall, the node at least 3 layers from the
-// r-walls, n3 >= 7), through the per-layer constant folds, into the visitor
-// put (DecodeInto or RawInto).
-template <int K, int AX, class S, class Put>
-__device__ __forceinline__ void gather_edge_v(const S* __restrict__ fin, const CellPos& p, const Dims& d,
-                                              const Put& put) {
+// Streamed populations of a node within 3 layers of an r-wall (x3 periodic or
+// the node at least 3 layers from the x3-walls, nr >= 7) through the
+// per-layer constant folds.
+template <int K, class S, class Put>
+__device__ __forceinline__ void gather_edge(const S* __restrict__ fin, const CellPos& p, const Dims& d,
+                                            const Put& put) {
   put(std::integral_constant<int, 0>{}, fin + uint32_t(p.cell), 0, geo_row<K>(d, p.ir, p.i3));
-  const int i = AX == 0 ? p.ir : p.i3, n = AX == 0 ? d.nr : d.n3;
-  const int side = i < 3 ? 0 : 1;
-  const int j = side == 0 ? i : n - 1 - i;
+  const int side = p.ir < 3 ? 0 : 1;
+  const int j = side == 0 ? p.ir : d.nr - 1 - p.ir;
   switch (side * 3 + j) {
-    case 0: for_each_source_layer<K, AX, 0, 0>(fin, p, d, put); break;
-    case 1: for_each_source_layer<K, AX, 0, 1>(fin, p, d, put); break;
-    case 2: for_each_source_layer<K, AX, 0, 2>(fin, p, d, put); break;
-    case 3: for_each_source_layer<K, AX, 1, 0>(fin, p, d, put); break;
-    case 4: for_each_source_layer<K, AX, 1, 1>(fin, p, d, put); break;
-    default: for_each_source_layer<K, AX, 1, 2>(fin, p, d, put); break;
+    case 0: for_each_source_layer<K, 0, 0>(fin, p, d, put); break;
+    case 1: for_each_source_layer<K, 0, 1>(fin, p, d, put); break;
+    case 2: for_each_source_layer<K, 0, 2>(fin, p, d, put); break;
+    case 3: for_each_source_layer<K, 1, 0>(fin, p, d, put); break;
+    case 4: for_each_source_layer<K, 1, 1>(fin, p, d, put); break;
+    default: for_each_source_layer<K, 1, 2>(fin, p, d, put); break;
   }
-}
-
-// The visitor of a gather: decoded populations f, or with RAW (2-byte
-// storage only) the stored deviations.
-template <int K, class S, class R, bool RAW>
-struct GatherPut {
-  using type = DecodeInto<K, S, R>;
-  __device__ static __forceinline__ type make(R (&f)[Q], const float* ref, const Dims& d) { return {f, ref, d}; }
-};
-template <int K, class S>
-struct GatherPut<K, S, float, true> {
-  using type = RawInto<S>;
-  __device__ static __forceinline__ type make(float (&f)[Q], const float*, const Dims&) { return {f}; }
-};
-
-template <int K, class S, class R, bool RAW = false, int AX = 0>
-__device__ __forceinline__ void gather_edge(const S* __restrict__ fin, const float* ref, const CellPos& p,
-                                            const Dims& d, R (&f)[Q]) {
-  gather_edge_v<K, AX>(fin, p, d, GatherPut<K, S, R, RAW>::make(f, ref, d));
 }
 
 // Load the 41 streamed populations of node p from the post-collision state
-// (instance block fin, reference table ref). WALLS selects the paths
-// compiled in: 0 far from every wall; 1 the general wall rule; 2 the node
-// decides among far, the r-layer folds and the general rule; 3 the r-layer
-// folds alone (gather_edge, AX 0); 4 the x3-layer folds alone (AX 2).
-// WALLS = 2: near an r-wall with bounce-back walls, at least 3 nodes away
-// from any x3 wall, only the r-wall can lie on a population's path, and the
-// compile-time folds of gather_edge replace the general wall rule (the same
-// sources, fewer instructions).
-// RAW (2-byte storage only): f receives the stored deviations g instead of
-// the decoded populations.
-template <int K, class S, class R, int WALLS = 2, bool RAW = false>
+// (instance block fin, reference table ref), decoded (the observables and the
+// half-force variant's step). Near an r-wall with bounce-back walls, at least
+// 3 nodes away from any x3 wall, only the r-wall can lie on a population's
+// path, and the compile-time folds of gather_edge replace the general wall
+// rule (the same sources, fewer instructions).
+template <int K, class S, class R>
 __device__ __forceinline__ void gather(const S* __restrict__ fin, const float* ref, const CellPos& p,
                                        const Dims& d, R (&f)[Q]) {
-  if constexpr (WALLS == 3 || WALLS == 4) {
-    gather_edge<K, S, R, RAW, WALLS == 3 ? 0 : 2>(fin, ref, p, d, f);
+  const DecodeInto<K, S, R> put{f, ref, d};
+  const bool x3_clear = d.periodic3 || (p.i3 >= 3 && p.i3 <= d.n3 - 4);
+  if (!d.wall_eq && d.nr >= 7 && x3_clear && (p.ir < 3 || p.ir > d.nr - 4)) {
+    gather_edge<K>(fin, p, d, put);
     return;
   }
-  if constexpr (WALLS == 2) {
-    const bool x3_clear = d.periodic3 || (p.i3 >= 3 && p.i3 <= d.n3 - 4);
-    if (!d.wall_eq && d.nr >= 7 && x3_clear && (p.ir < 3 || p.ir > d.nr - 4)) {
-      gather_edge<K, S, R, RAW>(fin, ref, p, d, f);
-      return;
-    }
-  }
-  for_each_source<K, S, WALLS>(fin, p, d, GatherPut<K, S, R, RAW>::make(f, ref, d));
+  for_each_source<K>(fin, p, d, put);
 }
 
 // The streamed populations of node p through the source table: entry L of the
@@ -581,20 +508,19 @@ __device__ __forceinline__ void gather(const S* __restrict__ fin, const float* r
 // every periodic wrap. One code path for all of them keeps the step kernels
 // small: with a compile-time variant per wall layer they were bound by
 // instruction fetch (7 to 19 cycles per issue at the walls).
-template <int K, class S, class R, bool RAW>
-__device__ __forceinline__ void gather_table(const S* __restrict__ fin, const float* ref, const CellPos& p,
-                                             const Dims& d, R (&f)[Q]) {
+template <class S>
+__device__ __forceinline__ void gather_table(const S* __restrict__ fin, const CellPos& p, const Dims& d,
+                                             S (&f)[Q]) {
   const int key = (axis_class(p.ir, d.nr) * d.src_nt + axis_class(p.it, d.nt)) * d.src_n3 + axis_class(p.i3, d.n3);
   const int4* __restrict__ row = d.src + key * SRC_ROW;
-  auto put = GatherPut<K, S, R, RAW>::make(f, ref, d);
   static_for<0, SRC_ROW>([&](auto J_) {
     constexpr int J = decltype(J_)::value;
     const int4 o = __ldg(row + J);
-    put(std::integral_constant<int, 4 * J>{}, fin + uint32_t(p.cell + o.x), 0, 0);
+    f[4 * J] = __ldg(fin + uint32_t(p.cell + o.x));
     if constexpr (4 * J + 1 < Q) {
-      put(std::integral_constant<int, 4 * J + 1>{}, fin + uint32_t(p.cell + o.y), 0, 0);
-      put(std::integral_constant<int, 4 * J + 2>{}, fin + uint32_t(p.cell + o.z), 0, 0);
-      put(std::integral_constant<int, 4 * J + 3>{}, fin + uint32_t(p.cell + o.w), 0, 0);
+      f[4 * J + 1] = __ldg(fin + uint32_t(p.cell + o.y));
+      f[4 * J + 2] = __ldg(fin + uint32_t(p.cell + o.z));
+      f[4 * J + 3] = __ldg(fin + uint32_t(p.cell + o.w));
     }
   });
 }
@@ -602,25 +528,14 @@ __device__ __forceinline__ void gather_table(const S* __restrict__ fin, const fl
 // The step's gather: nodes at least 3 nodes from every wall take their sources
 // from the node's own neighbours, computed; a warp that holds any other node
 // reads the source table for all its nodes, so it runs one of the two paths.
-template <int K, class S, class R>
-__device__ __forceinline__ void gather_step(const S* __restrict__ fin, const CellPos& p, const Dims& d, R (&f)[Q]) {
-  constexpr bool RAW = Codec<S, R>::uses_ref;
-  if (__any_sync(__activemask(), near_wall(p, d))) {
-    gather_table<K, S, R, RAW>(fin, nullptr, p, d, f);
-  } else {
-    for_each_source<K, S, 0>(fin, p, d, GatherPut<K, S, R, RAW>::make(f, nullptr, d));
-  }
-}
-
-// Store the 41 post-collision deviations g of node p (2-byte storage).
 template <class S>
-__device__ __forceinline__ void store_raw(S* __restrict__ out, const CellPos& p, const Dims& d,
-                                          const float (&g)[Q]) {
-  const uint32_t N = uint32_t(d.ncell), cell = uint32_t(p.cell);
-  static_for<0, Q>([&](auto L_) {
-    constexpr int L = decltype(L_)::value;
-    out[uint32_t(L) * N + cell] = raw_enc<S>(g[L]);
-  });
+__device__ __forceinline__ void gather_step(const S* __restrict__ fin, const CellPos& p, const Dims& d, S (&f)[Q]) {
+  if (__any_sync(__activemask(), near_wall(p, d))) {
+    gather_table(fin, p, d, f);
+  } else {
+    f[0] = __ldg(fin + uint32_t(p.cell));
+    for_each_source_far<KFLAT>(fin, p, d, [&](auto L_, const S* src, int, int) { f[decltype(L_)::value] = __ldg(src); });
+  }
 }
 
 // Store the 41 post-collision populations of node p into the instance block
@@ -671,59 +586,21 @@ __device__ __forceinline__ NodeGeo<Real, K> load_geo(const GeoDev<Real>& g, int 
   return n;
 }
 
-// A node's stream-table row: entry k of the table in global memory (st the
-// k = 0 entry, stride the table's rows), or of a block's shared-memory copy
-// of one row.
-struct TabGlobal {
-  const float4* __restrict__ st;
-  uint32_t stride;
-  __device__ __forceinline__ float4 at(int k) const { return __ldg(st + k * stride); }
-};
-struct TabShared {
-  const float4* st;
-  __device__ __forceinline__ float4 at(int k) const { return st[k]; }
-};
+// ---------------------------------------------------------------------------
+// work division of the pair kernels (2-byte storage, pair.cuh)
+// ---------------------------------------------------------------------------
+// Warps of one instance. A stream-table row belongs to i_r alone (st_row_r) or
+// to a pair of the (i_r, x3) cross-section. In the first case a warp takes 32
+// consecutive pairs of an i_r layer and holds one row; else 32 consecutive
+// pairs of one (i_r, i_theta) line, warps of consecutive theta next to each
+// other, so that a block whose warps share (i_r, chunk) -- ntheta a multiple
+// of its warps -- holds their rows once.
+__host__ __device__ __forceinline__ uint32_t pair_warps(const Dims& d) { return uint32_t(d.nr) * d.div_wl.d; }
 
-// A node's stream-table row staged in shared memory by its own thread
-// (stage_table): entry k at st[k * stride], stride the block's threads.
-struct TabStaged {
-  const float4* st;
-  int stride;
-  __device__ __forceinline__ float4 at(int k) const { return st[k * stride]; }
-};
-
-// Copy the ST_K entries of stream-table row `row` (table st0 of rows
-// `stride` apart) into this thread's shared-memory slots dst[k * step] by
-// cp.async (16-byte copies that hold no registers while in flight), so
-// their latency runs under the node's gather. The caller waits with
-// stage_wait before reading them.
-__device__ __forceinline__ void stage_table(float4* dst, int step, const float4* __restrict__ st0, uint32_t stride) {
-#pragma unroll
-  for (int k = 0; k < ST_K; ++k) {
-    const uint32_t sa = static_cast<uint32_t>(__cvta_generic_to_shared(dst + k * step));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(st0 + k * stride) : "memory");
-  }
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Moments of the streamed populations f_l = w_l g_l + rho_l from the stored
-// deviations g of 2-byte storage: the streamed references' moments (stream
-// table entries a, b, c) start the sums, and every weight is folded into the
-// multiply-add that accumulates it.
-template <typename V>
-__device__ __forceinline__ Moments<V> moments_dev(const V (&g)[Q], const float4& a, const float4& b,
-                                                  const float4& c) {
-  const Moments<V> m0 = {V(a.x), V(a.y), V(a.z), V(a.w), V(b.x), V(b.y), V(b.z), V(b.w), V(c.x), V(c.y)};
-  return moments_shells<true>(g, m0);
-}
-
-// BGK collision with forcing on the stored deviations g of 2-byte storage,
-// in place, with the node's stream-table row tab.
-template <int K, class Tab>
-__device__ __forceinline__ void collide_dev(float (&g)[Q], const Coef<float>& k, const NodeGeo<float, K>& geo,
-                                            float omega, const Tab& tab, float t0) {
-  collide_shells<float, K>(g, k, geo, omega, tab, t0);
+// Bytes of staged table rows in a block of `warps` warps.
+__host__ __device__ __forceinline__ size_t pair_smem_bytes(const Dims& d, int warps) {
+  const int rows = d.st_row_r ? warps : (d.nt % warps == 0 ? 32 : 32 * warps);
+  return size_t(2 * ST_K) * size_t(rows) * sizeof(float4);
 }
 
 }  // namespace lbgm

@@ -1,5 +1,5 @@
-// Fused time-step kernel, BF16 population deviations, FP32 arithmetic: instantiations for the flat,
-// cylindrical and ellipsoidal metrics.
+// Fused time-step kernels, BF16 deviation storage with FP32 arithmetic:
+// instantiations for the flat, cylindrical and ellipsoidal metrics.
 #include "step_launch.cuh"
 
 namespace lbgm {
@@ -7,24 +7,16 @@ namespace lbgm {
 cudaError_t launch_step_b16(int K, const __nv_bfloat16* fin, __nv_bfloat16* fout, const GeoDev<float>& geo,
                             const InstParams<float>* inst, const Dims& d, int* flag, int threads,
                             cudaStream_t s) {
-  return launch_step_t<__nv_bfloat16, float>(K, fin, fout, geo, inst, d, flag, threads, s);
+  return launch_pair_t<__nv_bfloat16>(K, fin, fout, geo, inst, d, flag, threads, s);
 }
 
-cudaError_t launch_step_list_b16(int K, bool multi, const void* insts, const int4* work, int nwork,
-                                 int threads, int grid, int parity, cudaStream_t s) {
-  return launch_step_list_t<__nv_bfloat16, float>(K, multi, insts, work, nwork, threads, grid, parity, s);
+cudaError_t launch_step_list_b16(int K, const Dims& d, size_t smem, const void* insts, const int4* work,
+                                 int nwork, int threads, int grid, int parity, cudaStream_t s) {
+  return launch_pair_list_t<__nv_bfloat16>(K, d, smem, insts, work, nwork, threads, grid, parity, s);
 }
 
-int step_list_max_threads_b16() { return step_list_max_threads_t<__nv_bfloat16, float>(); }
-
-cudaError_t step_list_occupancy_b16(int K, int threads, int* blocks_per_sm) {
-  return step_list_occupancy_t<__nv_bfloat16, float>(K, threads, blocks_per_sm);
-}
-
-cudaError_t launch_step_split_b16(int K, const __nv_bfloat16* fin, __nv_bfloat16* fout, const GeoDev<float>& geo,
-                                  const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                                  cudaStream_t s, cudaStream_t se) {
-  return launch_step_split_t(K, fin, fout, geo, inst, d, flag, threads, s, se);
+cudaError_t step_list_occupancy_b16(int K, const Dims& d, size_t smem, int threads, int* blocks_per_sm) {
+  return pair_list_occupancy_t<__nv_bfloat16>(K, d, smem, threads, blocks_per_sm);
 }
 
 }  // namespace lbgm

@@ -1,5 +1,5 @@
-// Fused time-step kernel, FP32 populations and arithmetic: instantiations for the flat,
-// cylindrical and ellipsoidal metrics.
+// Fused time-step kernel, FP32 populations and arithmetic: instantiations for
+// every metric.
 #include "step_launch.cuh"
 
 namespace lbgm {
@@ -7,18 +7,16 @@ namespace lbgm {
 cudaError_t launch_step_f32(int K, const float* fin, float* fout, const GeoDev<float>& geo,
                             const InstParams<float>* inst, const Dims& d, int* flag, int threads,
                             cudaStream_t s) {
-  return launch_step_t<float, float>(K, fin, fout, geo, inst, d, flag, threads, s);
+  return launch_step_t<float>(K, fin, fout, geo, inst, d, flag, threads, s);
 }
 
-cudaError_t launch_step_list_f32(int K, bool multi, const void* insts, const int4* work, int nwork,
-                                 int threads, int grid, int parity, cudaStream_t s) {
-  return launch_step_list_t<float, float>(K, multi, insts, work, nwork, threads, grid, parity, s);
+cudaError_t launch_step_list_f32(int K, bool multi, const void* insts, const int4* work, int nwork, int threads,
+                                 int grid, int parity, cudaStream_t s) {
+  return launch_step_list_t<float>(K, multi, insts, work, nwork, threads, grid, parity, s);
 }
-
-int step_list_max_threads_f32() { return step_list_max_threads_t<float, float>(); }
 
 cudaError_t step_list_occupancy_f32(int K, int threads, int* blocks_per_sm) {
-  return step_list_occupancy_t<float, float>(K, threads, blocks_per_sm);
+  return step_list_occupancy_t<float>(K, threads, blocks_per_sm);
 }
 
 }  // namespace lbgm

@@ -1,75 +1,97 @@
-// Launcher of the fused step kernel for one storage/compute type pair; each
-// step_*.cu translation unit instantiates one pair so that the large unrolled
-// kernel bodies compile in parallel.
+// Launchers of the fused step kernel for one storage type; each step_*.cu
+// translation unit instantiates one so that the large unrolled kernel bodies
+// compile in parallel.
 #pragma once
 
-#include "kernels.cuh"
 #include "launch.h"
+#include "pair.cuh"
 
 namespace lbgm {
 
-template <class S, class R>
-cudaError_t launch_step_t(int K, const S* fin, S* fout, const GeoDev<R>& geo, const InstParams<R>* inst,
+// Largest block of the step kernels (their launch bounds).
+template <class S>
+constexpr int step_max_threads() {
+  return std::is_same<S, double>::value ? KBounds<double, KCYL>::maxt : 128;
+}
+
+template <class R>
+cudaError_t launch_step_t(int K, const R* fin, R* fout, const GeoDev<R>& geo, const InstParams<R>* inst,
                           const Dims& d, int* flag, int threads, cudaStream_t s) {
   if (d.batch < 1 || d.batch > 65535) return cudaErrorInvalidValue;
-  threads = threads < StepBounds<S, R>::maxt ? threads : StepBounds<S, R>::maxt;
+  threads = threads < step_max_threads<R>() ? threads : step_max_threads<R>();
   const dim3 blocks((uint32_t(d.ncell) + threads - 1) / threads, uint32_t(d.batch));
   switch (K) {
-    case KFLAT: k_step<S, R, KFLAT><<<blocks, threads, 0, s>>>(fin, fout, geo, inst, d, flag); break;
-    case KCYL: k_step<S, R, KCYL><<<blocks, threads, 0, s>>>(fin, fout, geo, inst, d, flag); break;
-    case KELL: k_step<S, R, KELL><<<blocks, threads, 0, s>>>(fin, fout, geo, inst, d, flag); break;
-    case KELT:  // the theta-resolved ellipsoid: FP64 / FP32 storage, this kernel only
-      if constexpr (!Codec<S, R>::uses_ref) {
-        k_step<S, R, KELT><<<blocks, threads, 0, s>>>(fin, fout, geo, inst, d, flag);
-        break;
-      }
-      return cudaErrorInvalidValue;
+    case KFLAT: k_step<R, KFLAT><<<blocks, threads, 0, s>>>(fin, fout, geo, inst, d, flag); break;
+    case KCYL: k_step<R, KCYL><<<blocks, threads, 0, s>>>(fin, fout, geo, inst, d, flag); break;
+    case KELL: k_step<R, KELL><<<blocks, threads, 0, s>>>(fin, fout, geo, inst, d, flag); break;
+    case KELT: k_step<R, KELT><<<blocks, threads, 0, s>>>(fin, fout, geo, inst, d, flag); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
-// Region-split step of 2-byte storage (flat and cylinder, periodic x3,
-// bounce-back walls): the interior on stream s, then the 6 wall layers on
-// stream se (the caller orders the two streams around the step). Launched
-// second, the small wall-layer kernel takes SMs as interior blocks retire.
-// Blocks must not straddle an i_r layer (split_supported).
-template <class S>
-cudaError_t launch_step_split_t(int K, const S* fin, S* fout, const GeoDev<float>& geo,
-                                const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                                cudaStream_t s, cudaStream_t se) {
-  if (d.batch < 1 || d.batch > 65535 || !d.periodic3 || d.nr < 7) return cudaErrorInvalidValue;
-  threads = threads < StepBounds<S, float>::maxt ? threads : StepBounds<S, float>::maxt;
-  const uint32_t layer = uint32_t(d.nt) * uint32_t(d.n3);
-  if (layer % uint32_t(threads)) return cudaErrorInvalidValue;
-  const dim3 ge(6u * layer / threads, uint32_t(d.batch));
-  const dim3 gb(uint32_t(d.nr - 6) * layer / threads, uint32_t(d.batch));
-  switch (K) {
-    case KFLAT:
-      k_step_bulk_rowsm<S, KFLAT><<<gb, threads, 0, s>>>(fin, fout, geo, inst, d, flag);
-      k_step_edge_rowsm<S, KFLAT><<<ge, threads, 0, se>>>(fin, fout, geo, inst, d, flag);
-      break;
-    case KCYL:
-      k_step_bulk_rowsm<S, KCYL><<<gb, threads, 0, s>>>(fin, fout, geo, inst, d, flag);
-      k_step_edge_rowsm<S, KCYL><<<ge, threads, 0, se>>>(fin, fout, geo, inst, d, flag);
-      break;
-    default:
-      return cudaErrorInvalidValue;
+// Warps per block of the pair kernels and whether its warps share their
+// staged rows: as many warps as asked for where they all lie in one
+// (i_r, chunk) (ntheta a multiple of them) or need one row each, else pairs of
+// warps (26.6 KB of staged rows a block unless they share them).
+inline int pair_block(const Dims& d, int threads, bool* shared) {
+  int w = threads < 128 ? threads / 32 : 4;
+  *shared = false;
+  if (d.st_row_r) return w;
+  if (d.nt % w != 0) w = 2;
+  *shared = d.nt % w == 0;
+  return w;
+}
+
+// f(EVEN, ROW1) with the dispatch's compile-time choices for d.
+template <int K, class F>
+cudaError_t pair_dispatch(const Dims& d, F&& f) {
+  const bool even = d.n3 % 2 == 0;
+  if constexpr (K != KELL) {
+    if (d.st_row_r)
+      return even ? f(std::true_type{}, std::true_type{}) : f(std::false_type{}, std::true_type{});
   }
-  return cudaGetLastError();
+  return even ? f(std::true_type{}, std::false_type{}) : f(std::false_type{}, std::false_type{});
+}
+
+template <class S, int K>
+cudaError_t launch_pair_k(const S* fin, S* fout, const GeoDev<float>& geo, const InstParams<float>* inst,
+                          const Dims& d, int* flag, int threads, cudaStream_t s) {
+  return pair_dispatch<K>(d, [&](auto even, auto row1) {
+    constexpr bool EVEN = decltype(even)::value, ROW1 = decltype(row1)::value;
+    bool shared;
+    const int w = pair_block(d, threads, &shared);
+    const uint32_t warps = pair_warps(d);
+    const dim3 grid((warps + w - 1) / w, uint32_t(d.batch));
+    const size_t smem = pair_smem_bytes(d, w);
+    k_step_pair<S, K, EVEN, ROW1><<<grid, w * 32, smem, s>>>(fin, fout, geo, inst, d, flag, warps, shared);
+    return cudaGetLastError();
+  });
+}
+
+template <class S>
+cudaError_t launch_pair_t(int K, const S* fin, S* fout, const GeoDev<float>& geo, const InstParams<float>* inst,
+                          const Dims& d, int* flag, int threads, cudaStream_t s) {
+  if (d.batch < 1 || d.batch > 65535) return cudaErrorInvalidValue;
+  switch (K) {
+    case KFLAT: return launch_pair_k<S, KFLAT>(fin, fout, geo, inst, d, flag, threads, s);
+    case KCYL: return launch_pair_k<S, KCYL>(fin, fout, geo, inst, d, flag, threads, s);
+    case KELL: return launch_pair_k<S, KELL>(fin, fout, geo, inst, d, flag, threads, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 // grid 0: one block per work item; otherwise `grid` persistent blocks. multi:
 // the items are longer than one block.
-template <class S, class R>
+template <class R>
 cudaError_t launch_step_list_t(int K, bool multi, const void* insts, const int4* work, int nwork, int threads,
                                int grid, int parity, cudaStream_t s) {
   if (nwork == 0) return cudaSuccess;
-  const auto* I = static_cast<const ListInst<S, R>*>(insts);
+  const auto* I = static_cast<const ListInst<R, R>*>(insts);
   const int g = grid > 0 && grid < nwork ? grid : nwork;
-#define LB_LIST(KK)                                                                      \
-  if (multi) k_step_list<S, R, KK, true><<<g, threads, 0, s>>>(I, work, nwork, parity); \
-  else k_step_list<S, R, KK, false><<<g, threads, 0, s>>>(I, work, nwork, parity)
+#define LB_LIST(KK)                                                                   \
+  if (multi) k_step_list<R, KK, true><<<g, threads, 0, s>>>(I, work, nwork, parity); \
+  else k_step_list<R, KK, false><<<g, threads, 0, s>>>(I, work, nwork, parity)
   switch (K) {
     case KFLAT: LB_LIST(KFLAT); break;
     case KCYL: LB_LIST(KCYL); break;
@@ -80,24 +102,62 @@ cudaError_t launch_step_list_t(int K, bool multi, const void* insts, const int4*
   return cudaGetLastError();
 }
 
-// Largest block of the work-list kernel (its launch bounds).
-template <class S, class R>
-int step_list_max_threads_t() {
-  return StepBounds<S, R>::maxt;
+// The same for 2-byte storage; `d` is any instance of the group (one metric
+// kind, row kind and parity of n3), smem the group's staged rows in bytes.
+template <class S, int K>
+cudaError_t launch_pair_list_k(const Dims& d, size_t smem, const void* insts, const int4* work, int nwork,
+                               int threads, int g, int parity, cudaStream_t s) {
+  const auto* I = static_cast<const ListInst<S, float>*>(insts);
+  return pair_dispatch<K>(d, [&](auto even, auto row1) {
+    constexpr bool EVEN = decltype(even)::value, ROW1 = decltype(row1)::value;
+    auto kern = k_step_pair_list<S, K, EVEN, ROW1>;
+    if (smem > 40 * 1024) {
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+      if (e != cudaSuccess) return e;
+    }
+    kern<<<g, threads, smem, s>>>(I, work, nwork, parity);
+    return cudaGetLastError();
+  });
+}
+
+template <class S>
+cudaError_t launch_pair_list_t(int K, const Dims& d, size_t smem, const void* insts, const int4* work,
+                               int nwork, int threads, int grid, int parity, cudaStream_t s) {
+  if (nwork == 0) return cudaSuccess;
+  const int g = grid > 0 && grid < nwork ? grid : nwork;
+  switch (K) {
+    case KFLAT: return launch_pair_list_k<S, KFLAT>(d, smem, insts, work, nwork, threads, g, parity, s);
+    case KCYL: return launch_pair_list_k<S, KCYL>(d, smem, insts, work, nwork, threads, g, parity, s);
+    case KELL: return launch_pair_list_k<S, KELL>(d, smem, insts, work, nwork, threads, g, parity, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 // Resident blocks per SM of the work-list kernel at `threads` per block.
-template <class S, class R>
-cudaError_t step_list_occupancy_t(int K, int threads, int* blocks_per_sm) {
+template <class R>
+cudaError_t step_list_occupancy_t(int K, int threads, int* out) {
   switch (K) {
-    case KFLAT:
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_step_list<S, R, KFLAT, false>, threads, 0);
-    case KCYL:
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_step_list<S, R, KCYL, false>, threads, 0);
-    case KELL:
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_step_list<S, R, KELL, false>, threads, 0);
-    default:
-      return cudaErrorInvalidValue;
+    case KFLAT: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_step_list<R, KFLAT, false>, threads, 0);
+    case KCYL: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_step_list<R, KCYL, false>, threads, 0);
+    case KELL: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_step_list<R, KELL, false>, threads, 0);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <class S>
+cudaError_t pair_list_occupancy_t(int K, const Dims& d, size_t smem, int threads, int* out) {
+  auto occ = [&](auto kk) {
+    constexpr int KK = decltype(kk)::value;
+    return pair_dispatch<KK>(d, [&](auto even, auto row1) {
+      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          out, k_step_pair_list<S, KK, decltype(even)::value, decltype(row1)::value>, threads, smem);
+    });
+  };
+  switch (K) {
+    case KFLAT: return occ(std::integral_constant<int, KFLAT>{});
+    case KCYL: return occ(std::integral_constant<int, KCYL>{});
+    case KELL: return occ(std::integral_constant<int, KELL>{});
+    default: return cudaErrorInvalidValue;
   }
 }
 

@@ -83,7 +83,7 @@ __device__ __forceinline__ Coef<V> shifted_coefficients(const Moments<V>& m, con
 // One node: pull streaming + walls, then the collision of its instance's
 // variant (the same wall-node rule and store as the literal step).
 template <typename S, typename Real, int K>
-__global__ void __launch_bounds__(KBounds<S, Real, K>::maxt, KBounds<S, Real, K>::minb)
+__global__ void __launch_bounds__(KBounds<Real, K>::maxt, KBounds<Real, K>::minb)
     k_step_shift(const S* __restrict__ fin, S* __restrict__ fout, GeoDev<Real> geo,
                  const InstParams<Real>* __restrict__ inst, Dims d, int* __restrict__ flag) {
   const uint32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(KBounds<S, Real, K>::maxt, KBounds<S, Real, K>
   const float* ref = ref_of(d, b);
   const InstParams<Real>& ip = inst[b];
   Real f[Q];
-  gather<K, S, Real, 2>(fin + base, ref, p, d, f);
+  gather<K>(fin + base, ref, p, d, f);
   const Moments<Real> m = step_moments(f);
   if (!finite_v(m.rho)) {
     if (*flag == 0) atomicExch(flag, 1);
@@ -116,7 +116,7 @@ template <class S, class R>
 cudaError_t launch_shift_t(int K, const S* fin, S* fout, const GeoDev<R>& geo, const InstParams<R>* inst,
                            const Dims& d, int* flag, int threads, cudaStream_t s) {
   if (d.batch < 1 || d.batch > 65535) return cudaErrorInvalidValue;
-  threads = threads < StepBounds<S, R>::maxt ? threads : StepBounds<S, R>::maxt;
+  threads = threads < step_max_threads<R>() ? threads : step_max_threads<R>();
   const dim3 blocks((uint32_t(d.ncell) + threads - 1) / threads, uint32_t(d.batch));
   switch (K) {
     case KFLAT: k_step_shift<S, R, KFLAT><<<blocks, threads, 0, s>>>(fin, fout, geo, inst, d, flag); break;
