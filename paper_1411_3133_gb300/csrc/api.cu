@@ -432,7 +432,6 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
   c->inst = dalloc(c, size_t(batch) * sizeof(InstParams<double>));
   c->rho_s = static_cast<double*>(dalloc(c, size_t(batch) * c->ncell * sizeof(double)));
   c->u_s = static_cast<double*>(dalloc(c, size_t(batch) * 3 * c->ncell * sizeof(double)));
-  c->rowmean = static_cast<double*>(dalloc(c, size_t(batch) * geom->nr * geom->ntheta * sizeof(double)));
   c->partial = static_cast<double*>(dalloc(c, size_t(batch) * c->nblk * DIAG_NQ * sizeof(double)));
   c->diag_out = static_cast<double*>(dalloc(c, size_t(batch) * DIAG_NQ * sizeof(double)));
   c->flag = static_cast<int*>(dalloc(c, sizeof(int)));
@@ -455,17 +454,15 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
     d.st = c->st_tab;
   }
   if (!c->f[0] || !c->f[1] || !c->geo_real || !c->geo64 || !c->sqrtg || !c->base_uth || !c->ini ||
-      !c->inst || !c->rho_s || !c->u_s || !c->rowmean || !c->partial || !c->diag_out || !c->flag || !c->src_tab)
+      !c->inst || !c->rho_s || !c->u_s || !c->partial || !c->diag_out || !c->flag || !c->src_tab)
     return bail(LB_ERR_CUDA, "device allocation failed");
 
   // geometry tables
   std::vector<double> g64(nrow64 * 4), sg(nrow64);
   for (size_t k = 0; k < nrow64; ++k) {
     const double* r = &c->host_geo[k * LB_GEO_STRIDE];
-    g64[4 * k + 0] = r[GEO_SQRTG];
-    g64[4 * k + 1] = r[GEO_SPEED];
-    g64[4 * k + 2] = r[GEO_WA];
-    g64[4 * k + 3] = r[GEO_WOMEGA];
+    const double w[4] = {r[GEO_SQRTG], r[GEO_SPEED], r[GEO_WA], r[GEO_WOMEGA]};
+    diag_weights(w, &g64[4 * k]);
     sg[k] = r[GEO_SQRTG];
   }
   e = cudaMemcpyAsync(c->geo64, g64.data(), g64.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream);
@@ -638,8 +635,7 @@ lb_status lb_diagnostics(lb_ctx* c, lb_diag* out) {
   if (!usable(c, &s)) return s;
   if (!out) return fail(c, LB_ERR_ARG, "null argument");
   LB_CUDA(c, launch_macros(int(c->prec), c->K, c->f[c->cur], c->rho_s, c->u_s, c->dims, c->stream));
-  LB_CUDA(c, launch_diag(c->rho_s, c->u_s, c->rowmean, c->geo64, c->dims, c->partial, c->nblk, c->diag_out,
-                         c->stream));
+  LB_CUDA(c, launch_diag(c->rho_s, c->u_s, c->geo64, c->dims, c->partial, c->nblk, c->diag_out, c->stream));
   std::vector<double> h(size_t(c->batch) * DIAG_NQ);
   LB_CUDA(c, cudaMemcpyAsync(h.data(), c->diag_out, h.size() * sizeof(double), cudaMemcpyDeviceToHost,
                              c->stream));
@@ -671,9 +667,7 @@ lb_status lb_velocity_change(lb_ctx* c, double* u_prev, double* change, double* 
   lb_status s;
   if (!usable(c, &s)) return s;
   if (!u_prev || !change) return fail(c, LB_ERR_ARG, "null argument");
-  // partial maxima reuse the observables' partial buffer (batch * nblk * DIAG_NQ >= batch * nblk * 2)
-  LB_CUDA(c, launch_macros(int(c->prec), c->K, c->f[c->cur], nullptr, c->u_s, c->dims, c->stream));
-  LB_CUDA(c, launch_residual(c->u_s, u_prev, c->dims, c->partial, c->nblk, c->diag_out, c->stream));
+  LB_CUDA(c, launch_velocity_change(int(c->prec), c->K, c->f[c->cur], u_prev, c->dims, c->diag_out, c->stream));
   std::vector<double> h(2 * size_t(c->batch));
   LB_CUDA(c, cudaMemcpyAsync(h.data(), c->diag_out, h.size() * sizeof(double), cudaMemcpyDeviceToHost,
                              c->stream));

@@ -1,6 +1,8 @@
 // Initialisation, macroscopic fields, state conversion and the observables
 // reduction (Sec. II initial state and moments; Sec. III-IV Dean number,
 // mean velocity and mean vorticity).
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "launch.h"
 
@@ -120,20 +122,6 @@ __device__ __forceinline__ bool eq_wall_node(const Dims& d, int ir, int i3) {
   return d.wall_eq && (ir == 0 || ir == d.nr - 1 || (!d.periodic3 && (i3 == 0 || i3 == d.n3 - 1)));
 }
 
-// mean of u^r along x3 for every (instance, i_r, i_theta) row
-__global__ void k_rowmean(const double* __restrict__ u, double* __restrict__ rowmean, Dims d) {
-  const int rows_per = d.nr * d.nt;
-  const int row = blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= d.batch * rows_per) return;
-  const int b = row / rows_per;
-  const int rr = row - b * rows_per;
-  const int ir = rr / d.nt;
-  const double* ur = u + size_t(b) * 3 * d.ncell + size_t(rr) * d.n3;
-  double s = 0.0;
-  for (int i = 0; i < d.n3; ++i) s += eq_wall_node(d, ir, i) ? 0.0 : ur[i];
-  rowmean[row] = s / d.n3;
-}
-
 // derivative along an axis from the values at offsets -2 .. +2 (u2m, um, u0,
 // up, u2p); the bounce-back wall version uses u = 0 half a node outside the
 // first and last node, the equilibrium-wall version second-order one-sided
@@ -176,64 +164,89 @@ __device__ __forceinline__ void block_reduce(double (&a)[DIAG_NQ], double* sh) {
   }
 }
 
+// isfinite without the FP64 units
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
 // Per-block partial sums of one instance (blockIdx.y), in a fixed order.
 //   0 rho'   1 rho' g   2 sqrt(g_thth) u^theta wA   3 wA   4 |omega| wOmega
-//   5 (u^r)^2   6 (u^r - row mean)^2   7 max |u|   8 non-finite nodes
+//   5 (u^r)^2   6 (u^r - row mean)^2   7 max |u|^2   8 non-finite nodes
+// A warp takes whole x3 rows: the row's mean of u^r first, then its nodes
+// while the row is in L1. FP64 units bound this pass (16 cycles a warp
+// instruction), so the weights come multiplied out (diag_weights), 5 is the
+// sum of 6 and the rows' means, the square root of 7 is taken once at the end,
+// comparisons are integer, and the two halves of the central differences are
+// one factor of the weight: 14 FP64 operations a node.
 __global__ void __launch_bounds__(DIAG_THREADS)
-    k_diag_partial(const double* __restrict__ rho, const double* __restrict__ u,
-                   const double* __restrict__ rowmean, const double* __restrict__ geo64, Dims d,
-                   double* __restrict__ partial, int nblk) {
+    k_diag_partial(const double* __restrict__ rho, const double* __restrict__ u, const double* __restrict__ geo64,
+                   Dims d, double* __restrict__ partial, int nblk) {
   __shared__ double sh[(DIAG_THREADS / 32) * DIAG_NQ];
-  const int b = blockIdx.y;
-  const int N = d.ncell;
+  const int b = blockIdx.y, lane = threadIdx.x & 31;
+  const int N = d.ncell, n3 = d.n3;
   const double* ur = u + size_t(b) * 3 * N;
   const double* ut = ur + N;
   const double* uz = ur + 2 * size_t(N);
   const double* rb = rho + size_t(b) * N;
+  const bool eqw = d.wall_eq != 0;
   double a[DIAG_NQ];
 #pragma unroll
   for (int q = 0; q < DIAG_NQ; ++q) a[q] = 0.0;
-  const int plane = d.nt * d.n3;
-  for (int c = blockIdx.x * DIAG_THREADS + threadIdx.x; c < N; c += nblk * DIAG_THREADS) {
-    const int ir = c / plane;
-    const int rem = c - ir * plane;
-    const int it = rem / d.n3;
-    const int i3 = rem - it * d.n3;
-    const double* gr = geo64 + size_t(d.geo_theta ? c : ir * d.n3 + i3) * 4;
-    const double sg = gr[0], sp = gr[1], wA = gr[2], wOm = gr[3];
-    const double r = rb[c];
-    const bool eqw = d.wall_eq != 0;
-    // velocity component at node (jr, j3) of this theta plane: 0 on an
-    // equilibrium wall node and outside the node range
-    auto U = [&](const double* a, int jr, int j3) -> double {
-      if (jr < 0 || jr >= d.nr || j3 < 0 || j3 >= d.n3 || eq_wall_node(d, jr, j3)) return 0.0;
-      return a[(size_t(jr) * d.nt + it) * d.n3 + j3];
-    };
-    const double u0 = U(ur, ir, i3), u1 = U(ut, ir, i3), u2 = U(uz, ir, i3);
-    // d_3 u^r
-    double d3ur;
-    if (d.periodic3) {
-      const int jm = i3 == 0 ? d.n3 - 1 : i3 - 1, jp = i3 == d.n3 - 1 ? 0 : i3 + 1;
-      d3ur = d_axis(0.0, U(ur, ir, jm), u0, U(ur, ir, jp), 0.0, i3, d.n3, false, eqw);
-    } else {
-      d3ur = d_axis(U(ur, ir, i3 - 2), U(ur, ir, i3 - 1), u0, U(ur, ir, i3 + 1), U(ur, ir, i3 + 2), i3, d.n3,
-                    true, eqw);
+  const double inv_n3 = 1.0 / n3;
+  int bad = 0;
+  unsigned long long speed2 = 0;  // bits of the largest |u|^2
+  for (int row = blockIdx.x * (DIAG_THREADS / 32) + (threadIdx.x >> 5); row < d.nr * d.nt;
+       row += nblk * (DIAG_THREADS / 32)) {
+    const int ir = row / d.nt, it = row - ir * d.nt;
+    const double* r0 = ur + size_t(row) * n3;
+    double s = 0.0;
+    for (int i = lane; i < n3; i += 32) s += eq_wall_node(d, ir, i) ? 0.0 : r0[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const double mean = s * inv_n3;
+    if (lane == 0) a[5] = fma(double(n3) * mean, mean, a[5]);  // + sum fl^2 = sum (u^r)^2
+    for (int i3 = lane; i3 < n3; i3 += 32) {
+      const int c = row * n3 + i3;
+      const double* gr = geo64 + size_t(d.geo_theta ? c : ir * n3 + i3) * 4;
+      const double r = rb[c];
+      // velocity component at node (jr, j3) of this theta plane: 0 on an
+      // equilibrium wall node and outside the node range
+      auto U = [&](const double* a, int jr, int j3) -> double {
+        if (jr < 0 || jr >= d.nr || j3 < 0 || j3 >= n3 || eq_wall_node(d, jr, j3)) return 0.0;
+        return a[(size_t(jr) * d.nt + it) * n3 + j3];
+      };
+      const double u0 = U(ur, ir, i3), u1 = U(ut, ir, i3), u2 = U(uz, ir, i3);
+      double om2;  // 2 (d_3 u^r - d_r u^3)
+      if (ir > 0 && ir < d.nr - 1 && (d.periodic3 || (i3 > 0 && i3 < n3 - 1))) {
+        const int jm = i3 == 0 ? n3 - 1 : i3 - 1, jp = i3 == n3 - 1 ? 0 : i3 + 1;
+        om2 = (U(ur, ir, jp) - U(ur, ir, jm)) - (U(uz, ir + 1, i3) - U(uz, ir - 1, i3));
+      } else {
+        double d3ur;
+        if (d.periodic3) {
+          const int jm = i3 == 0 ? n3 - 1 : i3 - 1, jp = i3 == n3 - 1 ? 0 : i3 + 1;
+          d3ur = d_axis(0.0, U(ur, ir, jm), u0, U(ur, ir, jp), 0.0, i3, n3, false, eqw);
+        } else {
+          d3ur = d_axis(U(ur, ir, i3 - 2), U(ur, ir, i3 - 1), u0, U(ur, ir, i3 + 1), U(ur, ir, i3 + 2), i3, n3,
+                        true, eqw);
+        }
+        const double drz = d_axis(U(uz, ir - 2, i3), U(uz, ir - 1, i3), u2, U(uz, ir + 1, i3), U(uz, ir + 2, i3), ir,
+                                  d.nr, true, eqw);
+        om2 = 2.0 * (d3ur - drz);
+      }
+      const double fl = u0 - mean;
+      a[0] += r;
+      a[1] = fma(gr[0], r, a[1]);
+      a[2] = fma(gr[1], u1, a[2]);
+      a[3] += gr[2];
+      a[4] = fma(fabs(om2), gr[3], a[4]);
+      a[6] = fma(fl, fl, a[6]);
+      const unsigned long long v2 =
+          static_cast<unsigned long long>(__double_as_longlong(fma(u2, u2, fma(u1, u1, u0 * u0))));
+      if (v2 > speed2 && v2 <= 0x7ff0000000000000ull) speed2 = v2;  // a NaN does not count, as in fmax
+      bad += finite_bits(r) && finite_bits(u0) && finite_bits(u1) && finite_bits(u2) ? 0 : 1;
     }
-    // d_r u^3 (walls on r)
-    const double drz = d_axis(U(uz, ir - 2, i3), U(uz, ir - 1, i3), u2, U(uz, ir + 1, i3), U(uz, ir + 2, i3), ir,
-                              d.nr, true, eqw);
-    const double fl = u0 - rowmean[(size_t(b) * d.nr + ir) * d.nt + it];
-    a[0] += r;
-    a[1] += sg * sg * r;
-    a[2] += sp * u1 * wA;
-    a[3] += wA;
-    a[4] += fabs(d3ur - drz) * wOm;
-    a[5] += u0 * u0;
-    a[6] += fl * fl;
-    a[7] = fmax(a[7], sqrt(u0 * u0 + u1 * u1 + u2 * u2));
-    const bool fin = isfinite(r) && isfinite(u0) && isfinite(u1) && isfinite(u2);
-    a[8] += fin ? 0.0 : 1.0;
   }
+  a[5] += a[6];
+  a[7] = __longlong_as_double(static_cast<long long>(speed2));
+  a[8] = double(bad);
   block_reduce(a, sh);
   if (threadIdx.x < DIAG_NQ) partial[(size_t(b) * nblk + blockIdx.x) * DIAG_NQ + threadIdx.x] =
       a[threadIdx.x];
@@ -252,7 +265,8 @@ __global__ void __launch_bounds__(DIAG_THREADS)
     for (int q = 0; q < DIAG_NQ; ++q) a[q] = (q == 7) ? fmax(a[q], p[q]) : a[q] + p[q];
   }
   block_reduce(a, sh);
-  if (threadIdx.x < DIAG_NQ) out[size_t(b) * DIAG_NQ + threadIdx.x] = a[threadIdx.x];
+  if (threadIdx.x < DIAG_NQ)
+    out[size_t(b) * DIAG_NQ + threadIdx.x] = threadIdx.x == 7 ? sqrt(a[threadIdx.x]) : a[threadIdx.x];
 }
 
 }  // namespace
@@ -311,54 +325,39 @@ cudaError_t launch_convert(int prec, int to_double, void* state, double* dbl, si
   return cudaGetLastError();
 }
 
-// Per instance (blockIdx.y): max |u - u_prev| and max |u| over the nodes,
-// then u_prev = u. Partial maxima per block, reduced by k_residual_final.
-__global__ void __launch_bounds__(256) k_residual(const double* __restrict__ u, double* __restrict__ u_prev,
-                                                  size_t per_inst, double* __restrict__ partial, int nblk) {
-  __shared__ double sd[256], su[256];
-  const size_t b = blockIdx.y;
-  double md = 0.0, mu = 0.0;
-  for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < per_inst; i += size_t(nblk) * blockDim.x) {
-    const size_t k = b * per_inst + i;
-    const double v = u[k];
-    md = fmax(md, fabs(v - u_prev[k]));
-    mu = fmax(mu, fabs(v));
-    u_prev[k] = v;
+namespace {
+template <typename S, typename Real>
+cudaError_t velocity_change_t(int K, const S* fin, double* u_prev, const Dims& d, double* out, cudaStream_t s) {
+  auto* o = reinterpret_cast<unsigned long long*>(out);
+  cudaError_t e = cudaMemsetAsync(out, 0, size_t(d.batch) * 2 * sizeof(double), s);
+  if (e != cudaSuccess) return e;
+  const dim3 g((uint32_t(d.ncell) + 255) / 256, uint32_t(d.batch));
+  switch (K) {
+    case KFLAT: k_velocity_change<S, Real, KFLAT><<<g, 256, 0, s>>>(fin, u_prev, d, o); break;
+    case KCYL: k_velocity_change<S, Real, KCYL><<<g, 256, 0, s>>>(fin, u_prev, d, o); break;
+    case KELL: k_velocity_change<S, Real, KELL><<<g, 256, 0, s>>>(fin, u_prev, d, o); break;
+    case KELT:
+      if constexpr (!Codec<S, Real>::uses_ref) {  // FP64 / FP32 storage only
+        k_velocity_change<S, Real, KELT><<<g, 256, 0, s>>>(fin, u_prev, d, o);
+        break;
+      }
+      return cudaErrorInvalidValue;
+    default: return cudaErrorInvalidValue;
   }
-  sd[threadIdx.x] = md;
-  su[threadIdx.x] = mu;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      sd[threadIdx.x] = fmax(sd[threadIdx.x], sd[threadIdx.x + s]);
-      su[threadIdx.x] = fmax(su[threadIdx.x], su[threadIdx.x + s]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    partial[(b * nblk + blockIdx.x) * 2] = sd[0];
-    partial[(b * nblk + blockIdx.x) * 2 + 1] = su[0];
-  }
-}
-
-__global__ void k_residual_final(const double* __restrict__ partial, int nblk, int batch, double* __restrict__ out) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= batch) return;
-  double md = 0.0, mu = 0.0;
-  for (int i = 0; i < nblk; ++i) {
-    md = fmax(md, partial[(size_t(b) * nblk + i) * 2]);
-    mu = fmax(mu, partial[(size_t(b) * nblk + i) * 2 + 1]);
-  }
-  out[2 * b] = md;
-  out[2 * b + 1] = mu;
-}
-
-cudaError_t launch_residual(const double* u, double* u_prev, const Dims& d, double* partial, int nblk,
-                            double* out, cudaStream_t s) {
-  const size_t per = size_t(3) * d.ncell;
-  k_residual<<<dim3(nblk, d.batch), 256, 0, s>>>(u, u_prev, per, partial, nblk);
-  k_residual_final<<<(d.batch + 255) / 256, 256, 0, s>>>(partial, nblk, d.batch, out);
   return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_velocity_change(int prec, int K, const void* fin, double* u_prev, const Dims& d, double* out,
+                                   cudaStream_t s) {
+  switch (prec) {
+    case 0: return velocity_change_t<double, double>(K, static_cast<const double*>(fin), u_prev, d, out, s);
+    case 1: return velocity_change_t<float, float>(K, static_cast<const float*>(fin), u_prev, d, out, s);
+    case 2: return velocity_change_t<__half, float>(K, static_cast<const __half*>(fin), u_prev, d, out, s);
+    case 3:
+      return velocity_change_t<__nv_bfloat16, float>(K, static_cast<const __nv_bfloat16*>(fin), u_prev, d, out, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 // Row means of FP64 populations into the reference table (ref_index
@@ -429,13 +428,15 @@ cudaError_t launch_source_table(int4* tab, const void* fin, const Dims& d, cudaS
   return cudaGetLastError();
 }
 
-cudaError_t launch_diag(const double* rho, const double* u, double* rowmean, const double* geo64,
-                        const Dims& d, double* partial, int nblk, double* out, cudaStream_t s) {
-  const int rows = d.batch * d.nr * d.nt;
-  k_rowmean<<<(rows + 255) / 256, 256, 0, s>>>(u, rowmean, d);
-  k_diag_partial<<<dim3(nblk, d.batch), DIAG_THREADS, 0, s>>>(rho, u, rowmean, geo64, d, partial,
-                                                              nblk);
-  k_diag_final<<<d.batch, DIAG_THREADS, 0, s>>>(partial, nblk, out);
+cudaError_t launch_diag(const double* rho, const double* u, const double* geo64, const Dims& d, double* partial,
+                        int nblk, double* out, cudaStream_t s) {
+  // about two blocks per SM over all instances (the blocks' reductions cost as
+  // much as three rows), no more than rows for their warps
+  const int rows = (d.nr * d.nt + DIAG_THREADS / 32 - 1) / (DIAG_THREADS / 32);
+  const int want = (304 + d.batch - 1) / d.batch;
+  const int blocks = std::min(nblk, std::min(rows, want));
+  k_diag_partial<<<dim3(blocks, d.batch), DIAG_THREADS, 0, s>>>(rho, u, geo64, d, partial, blocks);
+  k_diag_final<<<d.batch, DIAG_THREADS, 0, s>>>(partial, blocks, out);
   return cudaGetLastError();
 }
 

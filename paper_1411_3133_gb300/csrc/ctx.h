@@ -41,7 +41,6 @@ struct lb_ctx {
   void* inst = nullptr;            // InstParams<Real>[batch]
   double* rho_s = nullptr;         // macros scratch [batch * N]
   double* u_s = nullptr;           // [batch * 3 * N]
-  double* rowmean = nullptr;       // [batch * nr * nt]
   double* partial = nullptr;       // [batch * nblk * DIAG_NQ]
   double* diag_out = nullptr;      // [batch * DIAG_NQ]
   double* dbl_stage = nullptr;     // conversion staging (FP32 populations), lazily allocated

@@ -125,6 +125,16 @@ __global__ void __launch_bounds__(KBounds<Real, K>::maxt, KBounds<Real, K>::minb
   }
 }
 
+// Moments of the streamed populations of node p (the observables).
+template <typename S, typename Real, int K>
+__device__ __forceinline__ Moments<Real> streamed_moments(const S* __restrict__ fin, const float* ref,
+                                                          const CellPos& p, const Dims& d) {
+  Real f[Q];
+  if constexpr (Codec<S, Real>::uses_ref) gather<K>(fin, ref, p, d, f);
+  else gather_step(fin, p, d, f);
+  return moments(f);
+}
+
 // rho' and u of the streamed populations (moments only).
 template <typename S, typename Real, int K>
 __global__ void __launch_bounds__(256) k_macros(const S* __restrict__ fin, double* __restrict__ rho,
@@ -132,9 +142,7 @@ __global__ void __launch_bounds__(256) k_macros(const S* __restrict__ fin, doubl
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= uint32_t(d.batch) * uint32_t(d.ncell)) return;
   const CellPos p = locate(d, t);
-  Real f[Q];
-  gather<K>(fin + size_t(p.b) * Q * d.ncell, ref_of(d, p.b), p, d, f);
-  const Moments<Real> m = moments(f);
+  const Moments<Real> m = streamed_moments<S, Real, K>(fin + size_t(p.b) * Q * d.ncell, ref_of(d, p.b), p, d);
   const double r = double(m.rho);
   if (rho) rho[t] = r;
   if (u) {
@@ -142,6 +150,58 @@ __global__ void __launch_bounds__(256) k_macros(const S* __restrict__ fin, doubl
     u[ub] = double(m.jx / m.rho);
     u[ub + d.ncell] = double(m.jy / m.rho);
     u[ub + 2 * size_t(d.ncell)] = double(m.jz / m.rho);
+  }
+}
+
+// Largest of the warp's 64-bit values.
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
+  const uint32_t hi = __reduce_max_sync(0xffffffffu, uint32_t(v >> 32));
+  const uint32_t lo = __reduce_max_sync(0xffffffffu, uint32_t(v >> 32) == hi ? uint32_t(v) : 0u);
+  return (static_cast<unsigned long long>(hi) << 32) | lo;
+}
+
+// Convergence monitor: max |u - u_prev| and max |u| of instance blockIdx.y
+// into out[2 b], out[2 b + 1] (zero before; non-negative doubles order like
+// their bits), and u_prev = u. One pass over the state: the velocity goes
+// nowhere else, and no reduction runs after it.
+template <typename S, typename Real, int K>
+__global__ void __launch_bounds__(256) k_velocity_change(const S* __restrict__ fin, double* __restrict__ u_prev,
+                                                         Dims d, unsigned long long* __restrict__ out) {
+  const uint32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
+  const int b = int(blockIdx.y);
+  // the maxima as the bits of non-negative numbers: FP64 comparisons run on
+  // the FP64 units (16 cycles a warp instruction), integer ones do not
+  unsigned long long md = 0, mu = 0;
+  if (cell < uint32_t(d.ncell)) {
+    double* q = u_prev + size_t(b) * 3 * d.ncell + cell;
+    const size_t N = size_t(d.ncell);
+    const double old[3] = {q[0], q[N], q[2 * N]};
+    const CellPos p = locate_cell(d, b, cell);
+    const Moments<Real> m = streamed_moments<S, Real, K>(fin + size_t(b) * Q * d.ncell, ref_of(d, b), p, d);
+    const Real v[3] = {m.jx / m.rho, m.jy / m.rho, m.jz / m.rho};
+    Real um = Real(0);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double x = double(v[i]);
+      const unsigned long long e = static_cast<unsigned long long>(__double_as_longlong(fabs(x - old[i])));
+      if (e > md && e <= 0x7ff0000000000000ull) md = e;  // a NaN does not count, as in fmax
+      um = fmax(um, fabs(v[i]));
+      q[i * N] = x;
+    }
+    mu = static_cast<unsigned long long>(__double_as_longlong(double(um)));
+  }
+  md = warp_max(md);
+  mu = warp_max(mu);
+  __shared__ unsigned long long s_m[8][2];
+  if ((threadIdx.x & 31) == 0) {
+    s_m[threadIdx.x >> 5][0] = md;
+    s_m[threadIdx.x >> 5][1] = mu;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    unsigned long long m = 0;
+    for (int w = 0; w < 8; ++w) m = max(m, s_m[w][threadIdx.x]);
+    atomicMax(out + 2 * b + threadIdx.x, m);
   }
 }
 

@@ -71,10 +71,10 @@ cudaError_t launch_init(int prec, int K, void* f, const void* geo, const double*
                         const double* u_in, const Dims& d, cudaStream_t s);
 cudaError_t launch_convert(int prec, int to_double, void* state, double* dbl, size_t n, const Dims& d,
                            cudaStream_t s);
-// Per instance max |u - u_prev| and max |u| into out[2 b], out[2 b + 1];
-// u_prev = u afterwards (partial: batch * nblk * 2 doubles).
-cudaError_t launch_residual(const double* u, double* u_prev, const Dims& d, double* partial, int nblk,
-                            double* out, cudaStream_t s);
+// Per instance max |u - u_prev| and max |u| into out[2 b], out[2 b + 1], then
+// u_prev = u (k_velocity_change).
+cudaError_t launch_velocity_change(int prec, int K, const void* fin, double* u_prev, const Dims& d, double* out,
+                                   cudaStream_t s);
 // Reference table from the row means of FP64 populations (k_ref_from_state).
 cudaError_t launch_ref_from_state(const double* dbl, float* ref, const Dims& d, cudaStream_t s);
 // Reference populations of 2-byte storage (k_ref_table): mode 0 weights,
@@ -93,10 +93,19 @@ cudaError_t launch_stream_table(int prec, int K, float4* st, const float* ref, c
 // device address as fin.
 cudaError_t launch_source_table(int4* tab, const void* fin, const Dims& d, cudaStream_t s);
 
-// Observables: NQ sums per instance written to out[batch * DIAG_NQ].
+// Observables: NQ sums per instance written to out[batch * DIAG_NQ]. geo64
+// holds diag_weights of each row (node for the theta-resolved kind); partial
+// batch * nblk * DIAG_NQ doubles.
 constexpr int DIAG_NQ = 9;
-cudaError_t launch_diag(const double* rho, const double* u, double* rowmean, const double* geo64,
-                        const Dims& d, double* partial, int nblk, double* out, cudaStream_t s);
+inline __host__ __device__ void diag_weights(const double* w, double* out) {
+  // from (sqrt g, sqrt g_thth, wA, wOmega): g, sqrt(g_thth) wA, wA, wOmega / 2
+  out[0] = w[0] * w[0];
+  out[1] = w[1] * w[2];
+  out[2] = w[2];
+  out[3] = 0.5 * w[3];
+}
+cudaError_t launch_diag(const double* rho, const double* u, const double* geo64, const Dims& d, double* partial,
+                        int nblk, double* out, cudaStream_t s);
 
 // Message for lb_last_error(NULL) from entry points without a context.
 void set_last_error_noctx(const std::string& msg);

@@ -46,7 +46,9 @@ __global__ void k_noalloc_weights(lb_metric metric, lb_geometry_desc g, double* 
   const int row = blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= g.nr * g.n3) return;
   const int ir = row / g.n3, i3 = row - ir * g.n3;
-  observable_weights(metric, g, ir, i3, w + 4 * row);
+  double q[4];
+  observable_weights(metric, g, ir, i3, q);
+  diag_weights(q, w + 4 * row);
 }
 
 size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
@@ -81,8 +83,10 @@ extern "C" lb_status lb_diagnostics_noalloc(lb_metric metric, const lb_geometry_
   const int nblk = int(std::min<size_t>(1024, (N + 255) / 256));
   const size_t nrow64 = size_t(d.nr) * d.n3;
   const size_t off_w = 0;
-  const size_t off_rowmean = off_w + align256(nrow64 * 4 * sizeof(double));
-  const size_t off_partial = off_rowmean + align256(size_t(batch) * d.nr * d.nt * sizeof(double));
+  // (a row's worth of doubles per (instance, i_r, i_theta) stays in the size
+  // limit: the sizes this call takes have not changed)
+  const size_t off_partial = off_w + align256(nrow64 * 4 * sizeof(double)) +
+                             align256(size_t(batch) * d.nr * d.nt * sizeof(double));
   const size_t off_out = off_partial + align256(size_t(batch) * nblk * DIAG_NQ * sizeof(double));
   const size_t need = off_out + align256(size_t(batch) * DIAG_NQ * sizeof(double));
   if (need > LB_NOALLOC_SCRATCH_BYTES)
@@ -95,14 +99,13 @@ extern "C" lb_status lb_diagnostics_noalloc(lb_metric metric, const lb_geometry_
     return noalloc_fail(LB_ERR_CUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
   unsigned char* base = static_cast<unsigned char*>(p);
   double* w = reinterpret_cast<double*>(base + off_w);
-  double* rowmean = reinterpret_cast<double*>(base + off_rowmean);
   double* partial = reinterpret_cast<double*>(base + off_partial);
   double* sums = reinterpret_cast<double*>(base + off_out);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
 
   k_noalloc_weights<<<int((nrow64 + 255) / 256), 256, 0, s>>>(metric, *geom, w);
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = launch_diag(rho, u, rowmean, w, d, partial, nblk, sums, s);
+  if (e == cudaSuccess) e = launch_diag(rho, u, w, d, partial, nblk, sums, s);
   double h[LB_NOALLOC_MAX_BATCH * DIAG_NQ];
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h, sums, size_t(batch) * DIAG_NQ * sizeof(double), cudaMemcpyDeviceToHost, s);
