@@ -1,9 +1,10 @@
 // Batches of contexts of different geometry (lb_batch_* of include/lbgm.h).
 //
 // Every instance of every member becomes one ListInst record; instances are
-// grouped by metric kind and each group gets one work list, tiles (instance,
-// first node, count) over all its nodes. One batch step is one k_step_list
-// launch per kind, the kinds after the first on forked streams.
+// grouped by kernel variant (metric kind; in 2-byte storage also the parity of
+// n3 and the row kind). One batch step is one work-list launch over the tiles
+// of a group's nodes per LIST_MAX of its instances, the launches after the
+// first on forked streams.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -18,19 +19,16 @@ using namespace lbgm;
 
 namespace {
 
-// Flat, cylinder, ellipsoid; in 2-byte storage each metric kind splits into
-// the kernel variants of pair.cuh (parity of n3; rows of i_r alone or not).
-constexpr int kMaxGroups = 10;
+constexpr int kLanes = 6;  // concurrent streams of a batch step
 
 struct Group {
   int K = 0;
   int ninst = 0;
-  int nwork = 0;
-  size_t inst_off = 0;     // byte offset of the ListInst records in dmem
-  size_t work_off = 0;     // byte offset of the int4 tiles in dmem
-  int blocks_per_sm = 0;   // occupancy of the kernel at the built block size
-  Dims d{};                // 2-byte storage: an instance of the group
-  size_t smem = 0;         // 2-byte storage: staged rows of a block, bytes
+  std::vector<unsigned char> recs;  // ListInst records
+  std::vector<int> items;           // work items of each instance
+  int blocks_per_sm = 0;            // occupancy of the kernel at the built block size
+  Dims d{};                         // 2-byte storage: an instance of the group
+  size_t smem = 0;                  // 2-byte storage: staged rows of a block, bytes
 };
 
 }  // namespace
@@ -49,14 +47,12 @@ struct lb_batch {
   int built_tile_blocks = 0;
   std::vector<int> base_cur;  // member buffer parity when the records were written
   int parity = 0;             // batch steps since then, mod 2
-  Group g[kMaxGroups];
-  int ngroups = 0;
-  void* dmem = nullptr;
-  size_t dmem_bytes = 0;
+  std::vector<Group> g;
+  int tile = 0;               // nodes (FP32, FP64) or warps (2-byte storage) of a work item
 
-  cudaStream_t aux[kMaxGroups - 1] = {};
+  cudaStream_t aux[kLanes - 1] = {};
   cudaEvent_t ev_fork = nullptr;
-  cudaEvent_t ev_join[kMaxGroups - 1] = {};
+  cudaEvent_t ev_join[kLanes - 1] = {};
 
   int threads = 128;
   int tile_blocks = 1;  // LB_OPT_TILE_BLOCKS: nodes per tile = tile_blocks x threads
@@ -144,70 +140,40 @@ cudaError_t occupancy(lb_precision p, const Group& g, int threads, int* out) {
 }
 
 // Write the instance records (with the members' current buffer parity) and
-// the tile lists for block size b->threads (tiles of b->tile_blocks blocks'
-// worth of nodes), and upload them.
+// count their work items for block size b->threads (tiles of b->tile_blocks
+// blocks' worth of nodes). Host only: the launches carry the records.
 lb_status build(lb_batch* b) {
   drop_graph(b);
   b->built = false;
-  std::vector<unsigned char> recs;
-  std::vector<int4> tiles[kMaxGroups];
-  b->ngroups = 0;
+  b->g.clear();
+  const bool pairs = b->prec == LB_FP16_SHIFTED || b->prec == LB_BF16_SHIFTED;
+  b->tile = (pairs ? b->threads / 32 : b->threads) * b->tile_blocks;
   std::vector<int> keys;
   for (int K : {int(KCYL), int(KELL), int(KFLAT)})
     for (int v = 0; v < 4; ++v) keys.push_back(K * 4 + v);
   for (int key : keys) {
     Group gr;
     gr.K = key / 4;
-    const size_t before = recs.size();
     switch (b->prec) {
-      case LB_FP64: append_records<double, double>(b, key, recs, &gr.ninst, &lb_ctx::geo_d); break;
-      case LB_FP32: append_records<float, float>(b, key, recs, &gr.ninst, &lb_ctx::geo_f); break;
-      case LB_FP16_SHIFTED: append_records<__half, float>(b, key, recs, &gr.ninst, &lb_ctx::geo_f); break;
-      default: append_records<__nv_bfloat16, float>(b, key, recs, &gr.ninst, &lb_ctx::geo_f); break;
+      case LB_FP64: append_records<double, double>(b, key, gr.recs, &gr.ninst, &lb_ctx::geo_d); break;
+      case LB_FP32: append_records<float, float>(b, key, gr.recs, &gr.ninst, &lb_ctx::geo_f); break;
+      case LB_FP16_SHIFTED: append_records<__half, float>(b, key, gr.recs, &gr.ninst, &lb_ctx::geo_f); break;
+      default: append_records<__nv_bfloat16, float>(b, key, gr.recs, &gr.ninst, &lb_ctx::geo_f); break;
     }
     if (gr.ninst == 0) continue;
-    gr.inst_off = before;
-    // tiles, instance-major; instance ids are local to the group
-    std::vector<int4>& t = tiles[b->ngroups];
-    const bool pairs = b->prec == LB_FP16_SHIFTED || b->prec == LB_BF16_SHIFTED;
-    const int tile = (pairs ? b->threads / 32 : b->threads) * b->tile_blocks;  // warps or nodes
-    int local = 0;
     for (const lb_ctx* c : b->m) {
       if (variant(c) != key) continue;
       const int n = pairs ? int(pair_warps(c->dims)) : c->dims.ncell;
-      for (int bi = 0; bi < c->batch; ++bi, ++local)
-        for (int a = 0; a < n; a += tile) t.push_back(make_int4(local, a, std::min(tile, n - a), 0));
+      for (int bi = 0; bi < c->batch; ++bi) gr.items.push_back((n + b->tile - 1) / b->tile);
       if (pairs) {
         gr.d = c->dims;
         gr.smem = std::max(gr.smem, pair_smem_bytes(c->dims, b->threads / 32));
       }
     }
-    gr.nwork = int(t.size());
     cudaError_t e = occupancy(b->prec, gr, b->threads, &gr.blocks_per_sm);
     if (e != cudaSuccess) return bcuda(b, e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-    b->g[b->ngroups++] = gr;
+    b->g.push_back(std::move(gr));
   }
-  // layout: records | tiles per group
-  auto al = [](size_t x) { return (x + 255) / 256 * 256; };
-  size_t off = al(recs.size());
-  for (int i = 0; i < b->ngroups; ++i) {
-    b->g[i].work_off = off;
-    off = al(off + tiles[i].size() * sizeof(int4));
-  }
-  const size_t need = off;
-  if (need > b->dmem_bytes) {
-    if (b->dmem) cudaFree(b->dmem);
-    b->dmem = nullptr;
-    b->dmem_bytes = 0;
-    LB_BCUDA(b, cudaMalloc(&b->dmem, need));
-    b->dmem_bytes = need;
-  }
-  unsigned char* base = static_cast<unsigned char*>(b->dmem);
-  LB_BCUDA(b, cudaMemcpyAsync(base, recs.data(), recs.size(), cudaMemcpyHostToDevice, b->stream));
-  for (int i = 0; i < b->ngroups; ++i)
-    LB_BCUDA(b, cudaMemcpyAsync(base + b->g[i].work_off, tiles[i].data(), tiles[i].size() * sizeof(int4),
-                                cudaMemcpyHostToDevice, b->stream));
-  LB_BCUDA(b, cudaStreamSynchronize(b->stream));  // the host vectors go out of scope
   b->base_cur.resize(b->m.size());
   for (size_t i = 0; i < b->m.size(); ++i) b->base_cur[i] = b->m[i]->cur;
   b->parity = 0;
@@ -226,36 +192,43 @@ bool records_current(const lb_batch* b) {
   return true;
 }
 
-// The work list of one group on stream s.
-cudaError_t launch_group(const lb_batch* b, const Group& gr, cudaStream_t s) {
-  const unsigned char* base = static_cast<const unsigned char*>(b->dmem);
-  const void* insts = base + gr.inst_off;
+// The work list of instances i0 .. i0 + n - 1 of one group on stream s.
+cudaError_t launch_part(const lb_batch* b, const Group& gr, int i0, int n, cudaStream_t s) {
   const int grid = b->schedule == 1 ? std::max(1, gr.blocks_per_sm) * b->nsm : 0;
-  const int4* work = reinterpret_cast<const int4*>(base + gr.work_off);
-  const bool multi = b->built_tile_blocks > 1;
+  const void* recs = gr.recs.data() + gr.recs.size() / size_t(gr.ninst) * size_t(i0);
+  const int* items = gr.items.data() + i0;
   switch (b->prec) {
-    case LB_FP64: return launch_step_list_f64(gr.K, multi, insts, work, gr.nwork, b->threads, grid, b->parity, s);
-    case LB_FP32: return launch_step_list_f32(gr.K, multi, insts, work, gr.nwork, b->threads, grid, b->parity, s);
+    case LB_FP64: return launch_step_list_f64(gr.K, recs, n, items, b->tile, b->threads, grid, b->parity, s);
+    case LB_FP32: return launch_step_list_f32(gr.K, recs, n, items, b->tile, b->threads, grid, b->parity, s);
     case LB_FP16_SHIFTED:
-      return launch_step_list_h16(gr.K, gr.d, gr.smem, insts, work, gr.nwork, b->threads, grid, b->parity, s);
+      return launch_step_list_h16(gr.K, gr.d, gr.smem, recs, n, items, b->tile, b->threads, grid, b->parity, s);
     default:
-      return launch_step_list_b16(gr.K, gr.d, gr.smem, insts, work, gr.nwork, b->threads, grid, b->parity, s);
+      return launch_step_list_b16(gr.K, gr.d, gr.smem, recs, n, items, b->tile, b->threads, grid, b->parity, s);
   }
 }
 
-// One batch step. The groups read the same buffers and write disjoint
-// nodes, so they run side by side: the first on the batch stream, the others
-// forked before it and joined back.
+// One batch step. The launches read the same buffers and write disjoint nodes,
+// so they run side by side: the first on the batch stream, the others on
+// streams forked before it and joined back.
 lb_status step_once(lb_batch* b) {
-  const int n = b->ngroups;
+  struct Part {
+    const Group* g;
+    int i0, n;
+  };
+  std::vector<Part> parts;
+  for (const Group& g : b->g)
+    for (int i = 0; i < g.ninst; i += LIST_MAX) parts.push_back({&g, i, std::min(LIST_MAX, g.ninst - i)});
+  const int n = int(parts.size()), lanes = std::min(n, kLanes);
   if (n > 1) LB_BCUDA(b, cudaEventRecord(b->ev_fork, b->stream));
-  if (n > 0) LB_BCUDA(b, launch_group(b, b->g[0], b->stream));
-  for (int k = 1; k < n; ++k) {
-    LB_BCUDA(b, cudaStreamWaitEvent(b->aux[k - 1], b->ev_fork, 0));
-    LB_BCUDA(b, launch_group(b, b->g[k], b->aux[k - 1]));
-    LB_BCUDA(b, cudaEventRecord(b->ev_join[k - 1], b->aux[k - 1]));
+  for (int k = 0; k < n; ++k) {
+    const int lane = k % kLanes;
+    if (k > 0 && k < kLanes) LB_BCUDA(b, cudaStreamWaitEvent(b->aux[k - 1], b->ev_fork, 0));
+    LB_BCUDA(b, launch_part(b, *parts[k].g, parts[k].i0, parts[k].n, lane == 0 ? b->stream : b->aux[lane - 1]));
   }
-  for (int k = 1; k < n; ++k) LB_BCUDA(b, cudaStreamWaitEvent(b->stream, b->ev_join[k - 1], 0));
+  for (int k = 1; k < lanes; ++k) {
+    LB_BCUDA(b, cudaEventRecord(b->ev_join[k - 1], b->aux[k - 1]));
+    LB_BCUDA(b, cudaStreamWaitEvent(b->stream, b->ev_join[k - 1], 0));
+  }
   b->parity ^= 1;
   return LB_OK;
 }
@@ -384,7 +357,7 @@ lb_status lb_batch_create(lb_ctx* const* members, int count, lb_batch** out) {
   if (e == cudaSuccess && cur_dev != b->device) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, b->device);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
-  for (int i = 0; i < kMaxGroups - 1 && e == cudaSuccess; ++i) {
+  for (int i = 0; i < kLanes - 1 && e == cudaSuccess; ++i) {
     e = cudaStreamCreateWithFlags(&b->aux[i], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_join[i], cudaEventDisableTiming);
   }
@@ -497,8 +470,7 @@ void lb_batch_destroy(lb_batch* b) {
   if (!b) return;
   if (b->stream) cudaStreamSynchronize(b->stream);
   drop_graph(b);
-  if (b->dmem) cudaFree(b->dmem);
-  for (int i = 0; i < kMaxGroups - 1; ++i) {
+  for (int i = 0; i < kLanes - 1; ++i) {
     if (b->aux[i]) cudaStreamDestroy(b->aux[i]);
     if (b->ev_join[i]) cudaEventDestroy(b->ev_join[i]);
   }

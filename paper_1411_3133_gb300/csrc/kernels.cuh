@@ -84,44 +84,56 @@ struct ListInst {
   int* flag;
 };
 
-// Work-list step over instances of one metric kind. Work item j = (instance,
-// first, count) covers the nodes first .. first + count - 1 of one instance:
-// at most blockDim.x, one per thread, or with MULTI a tile of several blocks'
-// worth (thread t takes nodes t, t + blockDim.x, ...; a separate
-// instantiation, because the loop costs the one-block tiles ~5 % on the
-// four-wall ellipsoid).
-// Blocks take items j = blockIdx.x, blockIdx.x + gridDim.x, ... (a
-// persistent grid when gridDim.x < nwork). `parity` 0 reads f0 and writes f1,
-// 1 the reverse. The instance record is staged once per item in shared
-// memory.
-template <typename Real, int K, bool MULTI>
+// Arguments of a work-list launch: up to N instances and the first work item
+// of each (tile_start[count] items in all). They travel in the kernel's
+// parameters, so a block reads its instance's record through the constant
+// cache with a block-uniform index, as the uniform-batch kernels read theirs:
+// staged in shared memory the record took the step's registers (184 bytes
+// spilled on the cylinder: 103.6 us a step against 82.4 for k_step on 24
+// 64 x 4 x 256 cylinders in FP32).
+template <typename S, typename Real>
+struct ListArgs {
+  static constexpr int N = 64;  // LIST_MAX
+  ListInst<S, Real> rec[N];
+  int tile_start[N + 1];
+  int count, tile, parity;
+
+  // Instance of work item j.
+  __device__ __forceinline__ int instance(int j) const {
+    int i = 0;
+#pragma unroll
+    for (int s = N / 2; s > 0; s >>= 1)
+      if (i + s < count && tile_start[i + s] <= j) i += s;
+    return i;
+  }
+};
+
+// Work-list step over instances of one metric kind: item j is the j-th tile of
+// `tile` consecutive nodes over all instances. One block per item of at most
+// one block's worth of nodes, or with LOOP items of several blocks' worth and
+// blocks that take items blockIdx.x, blockIdx.x + gridDim.x, ... (the loops
+// cost registers: a separate instantiation). `parity` 0 reads f0 and writes
+// f1, 1 the reverse.
+template <typename Real, int K, bool LOOP>
 __global__ void __launch_bounds__(KBounds<Real, K>::maxt, KBounds<Real, K>::minb)
-    k_step_list(const ListInst<Real, Real>* __restrict__ insts, const int4* __restrict__ work, int nwork, int parity) {
-  constexpr int kWords = sizeof(ListInst<Real, Real>) / 4;
-  static_assert(sizeof(ListInst<Real, Real>) % 4 == 0, "record must be whole words");
-  __shared__ union {
-    ListInst<Real, Real> rec;
-    uint32_t w[kWords];
-  } sh;
-  for (int j = blockIdx.x; j < nwork; j += gridDim.x) {
-    const int4 w = work[j];
-    __syncthreads();  // the previous item's readers are done
-    for (int i = int(threadIdx.x); i < kWords; i += int(blockDim.x))
-      sh.w[i] = reinterpret_cast<const uint32_t*>(insts + w.x)[i];
-    __syncthreads();
-    const ListInst<Real, Real>& I = sh.rec;
-    auto node = [&](int i) {
-      const Dims d = I.d;
-      const CellPos p = locate_cell(d, 0, uint32_t(w.y + i));
-      const Real* fin = parity ? I.f1 : I.f0;
-      Real* fout = const_cast<Real*>(parity ? I.f0 : I.f1);
-      step_node<Real, K>(fin, fout, I.geo, *I.ip, d, p, I.flag);
-    };
-    if constexpr (MULTI) {
-      for (int i = int(threadIdx.x); i < w.z; i += int(blockDim.x)) node(i);
-    } else {
-      if (int(threadIdx.x) < w.z) node(int(threadIdx.x));
-    }
+    k_step_list(const __grid_constant__ ListArgs<Real, Real> a) {
+  auto item = [&](int j) {
+    const int i = a.instance(j);
+    const ListInst<Real, Real>& I = a.rec[i];
+    const Real* fin = a.parity ? I.f1 : I.f0;
+    Real* fout = const_cast<Real*>(a.parity ? I.f0 : I.f1);
+    const int first = (j - a.tile_start[i]) * a.tile, end = min(first + a.tile, I.d.ncell);
+    int c = first + int(threadIdx.x);
+    if (c >= end) return;
+    do {
+      step_node<Real, K>(fin, fout, I.geo, *I.ip, I.d, locate_cell(I.d, 0, uint32_t(c)), I.flag);
+      c += int(blockDim.x);
+    } while (LOOP && c < end);
+  };
+  if constexpr (LOOP) {
+    for (int j = blockIdx.x; j < a.tile_start[a.count]; j += gridDim.x) item(j);
+  } else {
+    item(int(blockIdx.x));
   }
 }
 

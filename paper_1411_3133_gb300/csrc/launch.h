@@ -35,22 +35,24 @@ cudaError_t launch_step_shift_f32(int K, const float* fin, float* fout, const Ge
                                   const InstParams<float>* inst, const Dims& d, int* flag, int threads,
                                   cudaStream_t s);
 
-// Work-list step over instances of different geometry (ListInst array); multi:
-// items longer than one block; grid 0 launches one block per item. FP32, FP64:
-// item (instance, first node, nodes). 2-byte storage: item (instance, first
-// warp, warps) over a group of one metric kind, row kind and parity of n3 --
-// d any of its instances, smem the bytes of staged rows a block needs.
-cudaError_t launch_step_list_f64(int K, bool multi, const void* insts, const int4* work, int nwork, int threads,
+// Work-list step over `count` (at most LIST_MAX) instances of different
+// geometry: their host records (ListInst), the work items of each and the
+// tile, the nodes (FP32, FP64) or warps (2-byte storage) of an item; grid 0
+// launches one block per item. 2-byte storage: a group of one metric kind, row
+// kind and parity of n3 -- d any of its instances, smem the bytes of staged
+// rows a block needs.
+constexpr int LIST_MAX = 64;
+cudaError_t launch_step_list_f64(int K, const void* recs, int count, const int* items, int tile, int threads,
                                  int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_f64(int K, int threads, int* blocks_per_sm);
-cudaError_t launch_step_list_f32(int K, bool multi, const void* insts, const int4* work, int nwork, int threads,
+cudaError_t launch_step_list_f32(int K, const void* recs, int count, const int* items, int tile, int threads,
                                  int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_f32(int K, int threads, int* blocks_per_sm);
-cudaError_t launch_step_list_h16(int K, const Dims& d, size_t smem, const void* insts, const int4* work,
-                                 int nwork, int threads, int grid, int parity, cudaStream_t s);
+cudaError_t launch_step_list_h16(int K, const Dims& d, size_t smem, const void* recs, int count, const int* items,
+                                 int tile, int threads, int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_h16(int K, const Dims& d, size_t smem, int threads, int* blocks_per_sm);
-cudaError_t launch_step_list_b16(int K, const Dims& d, size_t smem, const void* insts, const int4* work,
-                                 int nwork, int threads, int grid, int parity, cudaStream_t s);
+cudaError_t launch_step_list_b16(int K, const Dims& d, size_t smem, const void* recs, int count, const int* items,
+                                 int tile, int threads, int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_b16(int K, const Dims& d, size_t smem, int threads, int* blocks_per_sm);
 
 // TMA-pipelined FP32 step (n3 in {128, 256}); map is a CUtensorMap over the

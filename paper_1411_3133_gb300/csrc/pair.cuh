@@ -320,34 +320,25 @@ __global__ void __launch_bounds__(128, LBGM_PAIR_MINB)
                               w < warps, shared != 0, sm, flag);
 }
 
-// Work list over instances of one metric kind and row parity: item (instance,
-// first warp, warps), one or several blocks' worth.
+// Work list over instances of one metric kind and row parity (ListArgs; a tile
+// is a number of warps).
 template <typename S, int K, bool EVEN, bool ROW1>
 __global__ void __launch_bounds__(128, LBGM_PAIR_MINB)
-    k_step_pair_list(const ListInst<S, float>* __restrict__ insts, const int4* __restrict__ work, int nwork,
-                     int parity) {
-  constexpr int kWords = sizeof(ListInst<S, float>) / 4;
+    k_step_pair_list(const __grid_constant__ ListArgs<S, float> a) {
   extern __shared__ float4 sm[];
-  __shared__ union {
-    ListInst<S, float> rec;
-    uint32_t w[kWords];
-  } sh;
   const int wpb = int(blockDim.x >> 5);
-  for (int j = blockIdx.x; j < nwork; j += gridDim.x) {
-    const int4 item = work[j];
-    __syncthreads();  // the previous item's readers are done
-    for (int i = int(threadIdx.x); i < kWords; i += int(blockDim.x))
-      sh.w[i] = reinterpret_cast<const uint32_t*>(insts + item.x)[i];
-    __syncthreads();
-    const Dims d = sh.rec.d;
-    const S* fin = parity ? sh.rec.f1 : sh.rec.f0;
-    S* fout = const_cast<S*>(parity ? sh.rec.f0 : sh.rec.f1);
-    const bool shared = !ROW1 && d.nt % wpb == 0;
-    for (int i = 0; i < item.z; i += wpb) {
-      if (i > 0) __syncthreads();  // the staged rows of the previous warps have been read
-      const int w = i + int(threadIdx.x >> 5);
-      step_pair<S, K, EVEN, ROW1>(fin, fout, d.ref, d.st, sh.rec.geo, sh.rec.ip, d, uint32_t(item.y + w), w < item.z,
-                                  shared, sm, sh.rec.flag);
+  for (int j = blockIdx.x; j < a.tile_start[a.count]; j += gridDim.x) {
+    const int i = a.instance(j);
+    const ListInst<S, float>& I = a.rec[i];
+    const S* fin = a.parity ? I.f1 : I.f0;
+    S* fout = const_cast<S*>(a.parity ? I.f0 : I.f1);
+    const int warps = int(pair_warps(I.d)), first = (j - a.tile_start[i]) * a.tile;
+    const bool shared = !ROW1 && I.d.nt % wpb == 0;
+    for (int w0 = first; w0 < min(first + a.tile, warps); w0 += wpb) {
+      if (j != int(blockIdx.x) || w0 != first) __syncthreads();  // the rows staged before have been read
+      const int w = w0 + int(threadIdx.x >> 5);
+      step_pair<S, K, EVEN, ROW1>(fin, fout, I.d.ref, I.d.st, I.geo, I.ip, I.d, uint32_t(w), w < warps, shared, sm,
+                                  I.flag);
     }
   }
 }

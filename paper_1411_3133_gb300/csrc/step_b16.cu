@@ -10,9 +10,9 @@ cudaError_t launch_step_b16(int K, const __nv_bfloat16* fin, __nv_bfloat16* fout
   return launch_pair_t<__nv_bfloat16>(K, fin, fout, geo, inst, d, flag, threads, s);
 }
 
-cudaError_t launch_step_list_b16(int K, const Dims& d, size_t smem, const void* insts, const int4* work,
-                                 int nwork, int threads, int grid, int parity, cudaStream_t s) {
-  return launch_pair_list_t<__nv_bfloat16>(K, d, smem, insts, work, nwork, threads, grid, parity, s);
+cudaError_t launch_step_list_b16(int K, const Dims& d, size_t smem, const void* recs, int count, const int* items,
+                                 int tile, int threads, int grid, int parity, cudaStream_t s) {
+  return launch_pair_list_t<__nv_bfloat16>(K, d, smem, recs, count, items, tile, threads, grid, parity, s);
 }
 
 cudaError_t step_list_occupancy_b16(int K, const Dims& d, size_t smem, int threads, int* blocks_per_sm) {

@@ -10,9 +10,9 @@ cudaError_t launch_step_f32(int K, const float* fin, float* fout, const GeoDev<f
   return launch_step_t<float>(K, fin, fout, geo, inst, d, flag, threads, s);
 }
 
-cudaError_t launch_step_list_f32(int K, bool multi, const void* insts, const int4* work, int nwork, int threads,
+cudaError_t launch_step_list_f32(int K, const void* recs, int count, const int* items, int tile, int threads,
                                  int grid, int parity, cudaStream_t s) {
-  return launch_step_list_t<float>(K, multi, insts, work, nwork, threads, grid, parity, s);
+  return launch_step_list_t<float>(K, recs, count, items, tile, threads, grid, parity, s);
 }
 
 cudaError_t step_list_occupancy_f32(int K, int threads, int* blocks_per_sm) {

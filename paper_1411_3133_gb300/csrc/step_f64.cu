@@ -10,9 +10,9 @@ cudaError_t launch_step_f64(int K, const double* fin, double* fout, const GeoDev
   return launch_step_t<double>(K, fin, fout, geo, inst, d, flag, threads, s);
 }
 
-cudaError_t launch_step_list_f64(int K, bool multi, const void* insts, const int4* work, int nwork, int threads,
+cudaError_t launch_step_list_f64(int K, const void* recs, int count, const int* items, int tile, int threads,
                                  int grid, int parity, cudaStream_t s) {
-  return launch_step_list_t<double>(K, multi, insts, work, nwork, threads, grid, parity, s);
+  return launch_step_list_t<double>(K, recs, count, items, tile, threads, grid, parity, s);
 }
 
 cudaError_t step_list_occupancy_f64(int K, int threads, int* blocks_per_sm) {

@@ -10,9 +10,9 @@ cudaError_t launch_step_h16(int K, const __half* fin, __half* fout, const GeoDev
   return launch_pair_t<__half>(K, fin, fout, geo, inst, d, flag, threads, s);
 }
 
-cudaError_t launch_step_list_h16(int K, const Dims& d, size_t smem, const void* insts, const int4* work,
-                                 int nwork, int threads, int grid, int parity, cudaStream_t s) {
-  return launch_pair_list_t<__half>(K, d, smem, insts, work, nwork, threads, grid, parity, s);
+cudaError_t launch_step_list_h16(int K, const Dims& d, size_t smem, const void* recs, int count, const int* items,
+                                 int tile, int threads, int grid, int parity, cudaStream_t s) {
+  return launch_pair_list_t<__half>(K, d, smem, recs, count, items, tile, threads, grid, parity, s);
 }
 
 cudaError_t step_list_occupancy_h16(int K, const Dims& d, size_t smem, int threads, int* blocks_per_sm) {

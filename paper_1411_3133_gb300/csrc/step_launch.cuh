@@ -3,6 +3,8 @@
 // compile in parallel.
 #pragma once
 
+#include <cstring>
+
 #include "launch.h"
 #include "pair.cuh"
 
@@ -81,17 +83,30 @@ cudaError_t launch_pair_t(int K, const S* fin, S* fout, const GeoDev<float>& geo
   }
 }
 
-// grid 0: one block per work item; otherwise `grid` persistent blocks. multi:
-// the items are longer than one block.
+// The arguments of one work-list launch over `count` records (at most
+// ListArgs::N) of `items` tiles each.
+template <class S, class R>
+ListArgs<S, R> list_args(const void* recs, int count, const int* items, int tile, int parity) {
+  ListArgs<S, R> a;
+  std::memcpy(a.rec, recs, size_t(count) * sizeof(a.rec[0]));
+  a.tile_start[0] = 0;
+  for (int i = 0; i < count; ++i) a.tile_start[i + 1] = a.tile_start[i] + items[i];
+  a.count = count;
+  a.tile = tile;
+  a.parity = parity;
+  return a;
+}
+
+// grid 0: one block per work item; otherwise `grid` persistent blocks.
 template <class R>
-cudaError_t launch_step_list_t(int K, bool multi, const void* insts, const int4* work, int nwork, int threads,
-                               int grid, int parity, cudaStream_t s) {
-  if (nwork == 0) return cudaSuccess;
-  const auto* I = static_cast<const ListInst<R, R>*>(insts);
-  const int g = grid > 0 && grid < nwork ? grid : nwork;
-#define LB_LIST(KK)                                                                   \
-  if (multi) k_step_list<R, KK, true><<<g, threads, 0, s>>>(I, work, nwork, parity); \
-  else k_step_list<R, KK, false><<<g, threads, 0, s>>>(I, work, nwork, parity)
+cudaError_t launch_step_list_t(int K, const void* recs, int count, const int* items, int tile, int threads, int grid,
+                               int parity, cudaStream_t s) {
+  const ListArgs<R, R> a = list_args<R, R>(recs, count, items, tile, parity);
+  const int n = a.tile_start[count], g = grid > 0 && grid < n ? grid : n;
+  const bool loop = g < n || tile > threads;
+#define LB_LIST(KK)                                              \
+  if (loop) k_step_list<R, KK, true><<<g, threads, 0, s>>>(a); \
+  else k_step_list<R, KK, false><<<g, threads, 0, s>>>(a)
   switch (K) {
     case KFLAT: LB_LIST(KFLAT); break;
     case KCYL: LB_LIST(KCYL); break;
@@ -105,9 +120,9 @@ cudaError_t launch_step_list_t(int K, bool multi, const void* insts, const int4*
 // The same for 2-byte storage; `d` is any instance of the group (one metric
 // kind, row kind and parity of n3), smem the group's staged rows in bytes.
 template <class S, int K>
-cudaError_t launch_pair_list_k(const Dims& d, size_t smem, const void* insts, const int4* work, int nwork,
-                               int threads, int g, int parity, cudaStream_t s) {
-  const auto* I = static_cast<const ListInst<S, float>*>(insts);
+cudaError_t launch_pair_list_k(const Dims& d, size_t smem, const ListArgs<S, float>& a, int threads, int grid,
+                               cudaStream_t s) {
+  const int n = a.tile_start[a.count], g = grid > 0 && grid < n ? grid : n;
   return pair_dispatch<K>(d, [&](auto even, auto row1) {
     constexpr bool EVEN = decltype(even)::value, ROW1 = decltype(row1)::value;
     auto kern = k_step_pair_list<S, K, EVEN, ROW1>;
@@ -115,20 +130,19 @@ cudaError_t launch_pair_list_k(const Dims& d, size_t smem, const void* insts, co
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
       if (e != cudaSuccess) return e;
     }
-    kern<<<g, threads, smem, s>>>(I, work, nwork, parity);
+    kern<<<g, threads, smem, s>>>(a);
     return cudaGetLastError();
   });
 }
 
 template <class S>
-cudaError_t launch_pair_list_t(int K, const Dims& d, size_t smem, const void* insts, const int4* work,
-                               int nwork, int threads, int grid, int parity, cudaStream_t s) {
-  if (nwork == 0) return cudaSuccess;
-  const int g = grid > 0 && grid < nwork ? grid : nwork;
+cudaError_t launch_pair_list_t(int K, const Dims& d, size_t smem, const void* recs, int count, const int* items,
+                               int tile, int threads, int grid, int parity, cudaStream_t s) {
+  const ListArgs<S, float> a = list_args<S, float>(recs, count, items, tile, parity);
   switch (K) {
-    case KFLAT: return launch_pair_list_k<S, KFLAT>(d, smem, insts, work, nwork, threads, g, parity, s);
-    case KCYL: return launch_pair_list_k<S, KCYL>(d, smem, insts, work, nwork, threads, g, parity, s);
-    case KELL: return launch_pair_list_k<S, KELL>(d, smem, insts, work, nwork, threads, g, parity, s);
+    case KFLAT: return launch_pair_list_k<S, KFLAT>(d, smem, a, threads, grid, s);
+    case KCYL: return launch_pair_list_k<S, KCYL>(d, smem, a, threads, grid, s);
+    case KELL: return launch_pair_list_k<S, KELL>(d, smem, a, threads, grid, s);
     default: return cudaErrorInvalidValue;
   }
 }
