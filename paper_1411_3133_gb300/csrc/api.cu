@@ -3,10 +3,12 @@
 // point. All numerical work runs in the kernels of kernels.cuh / aux.cu.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -227,40 +229,49 @@ std::string check_sparsity(const std::vector<double>& rows, const lb_geometry_de
 // region split on two streams and 103.6 for a work list.
 bool use_tma(const lb_ctx* c) { return c->prec == LB_FP32 && c->tma_ok && c->step_kernel == 2 && !c->any_shift; }
 
+// One time step of instances i0 .. i0 + count - 1 from buffer src into 1 - src.
+cudaError_t launch_step(lb_ctx* c, int src, int i0, int count, cudaStream_t s) {
+  Dims d = c->dims;
+  d.batch = count;
+  if (d.ref) d.ref += size_t(i0) * Q * size_t(d.nr) * size_t(d.geo_rows3);
+  if (d.st) d.st += size_t(i0) * 2 * ST_K * size_t(d.nr) * size_t(d.st_rows3);
+  const size_t off = size_t(i0) * Q * c->ncell;
+  auto go = [&](auto fn, auto* elem, const auto& geo) {
+    using S = std::remove_pointer_t<decltype(elem)>;
+    using R = std::conditional_t<std::is_same<S, double>::value, double, float>;
+    return fn(c->K, static_cast<const S*>(c->f[src]) + off, static_cast<S*>(c->f[1 - src]) + off, geo,
+              static_cast<const InstParams<R>*>(c->inst) + i0, d, c->flag, c->block_threads, s);
+  };
+  switch (c->prec) {
+    case LB_FP64:
+      return go(c->any_shift ? launch_step_shift_f64 : launch_step_f64, static_cast<double*>(nullptr), c->geo_d);
+    case LB_FP32:
+      if (use_tma(c))  // every instance, on the context's stream
+        return launch_step_tma_f32(c->K, c->tmap[src], static_cast<const float*>(c->f[src]),
+                                   static_cast<float*>(c->f[1 - src]), c->geo_f,
+                                   static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag, s);
+      return go(c->any_shift ? launch_step_shift_f32 : launch_step_f32, static_cast<float*>(nullptr), c->geo_f);
+    case LB_FP16_SHIFTED: return go(launch_step_h16, static_cast<__half*>(nullptr), c->geo_f);
+    default: return go(launch_step_b16, static_cast<__nv_bfloat16*>(nullptr), c->geo_f);
+  }
+}
+
 lb_status launch_step_once(lb_ctx* c) {
-  const int src = c->cur, dst = 1 - c->cur;
-  cudaError_t e;
-  if (c->any_shift && c->prec == LB_FP64)
-    e = launch_step_shift_f64(c->K, static_cast<const double*>(c->f[src]), static_cast<double*>(c->f[dst]),
-                              c->geo_d, static_cast<const InstParams<double>*>(c->inst), c->dims, c->flag,
-                              c->block_threads, c->stream);
-  else if (c->any_shift)
-    e = launch_step_shift_f32(c->K, static_cast<const float*>(c->f[src]), static_cast<float*>(c->f[dst]),
-                              c->geo_f, static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag,
-                              c->block_threads, c->stream);
-  else if (use_tma(c))
-    e = launch_step_tma_f32(c->K, c->tmap[src], static_cast<const float*>(c->f[src]),
-                            static_cast<float*>(c->f[dst]), c->geo_f,
-                            static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag, c->stream);
-  else if (c->prec == LB_FP64)
-    e = launch_step_f64(c->K, static_cast<const double*>(c->f[src]), static_cast<double*>(c->f[dst]),
-                        c->geo_d, static_cast<const InstParams<double>*>(c->inst), c->dims, c->flag,
-                        c->block_threads, c->stream);
-  else if (c->prec == LB_FP32)
-    e = launch_step_f32(c->K, static_cast<const float*>(c->f[src]), static_cast<float*>(c->f[dst]),
-                        c->geo_f, static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag,
-                        c->block_threads, c->stream);
-  else if (c->prec == LB_FP16_SHIFTED)
-    e = launch_step_h16(c->K, static_cast<const __half*>(c->f[src]), static_cast<__half*>(c->f[dst]),
-                        c->geo_f, static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag,
-                        c->block_threads, c->stream);
-  else
-    e = launch_step_b16(c->K, static_cast<const __nv_bfloat16*>(c->f[src]),
-                        static_cast<__nv_bfloat16*>(c->f[dst]), c->geo_f,
-                        static_cast<const InstParams<float>*>(c->inst), c->dims, c->flag,
-                        c->block_threads, c->stream);
+  cudaError_t e = launch_step(c, c->cur, 0, c->batch, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
-  c->cur = dst;
+  c->cur = 1 - c->cur;
+  return LB_OK;
+}
+
+// n steps with the instances taken in chunks (lanes.h).
+lb_status launch_steps_chunked(lb_ctx* c, long long n) {
+  const int cur = c->cur;
+  cudaError_t e = run_lanes(c->lanes, c->plan, n, c->stream, [&](const LaneChunk& ch, long long i, cudaStream_t s) {
+    return launch_step(c, int(cur ^ (i & 1)), ch.first, ch.count, s);
+  });
+  if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
+  c->cur = int(cur ^ (n & 1));
+  c->step += n;
   return LB_OK;
 }
 
@@ -489,6 +500,7 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
       tensor_map_bytes() <= sizeof(c->tmap[0]))
     c->tma_ok = make_state_tensor_map(c->tmap[0], static_cast<const float*>(c->f[0]), d) == cudaSuccess &&
                 make_state_tensor_map(c->tmap[1], static_cast<const float*>(c->f[1]), d) == cudaSuccess;
+  c->plan = plan_lanes(std::vector<LaneInst>(size_t(batch), {0, c->ncell, 2 * Q * c->ncell * c->elem_bytes}), batch);
   *out = c;
   return LB_OK;
 }
@@ -571,6 +583,16 @@ lb_status lb_step(lb_ctx* c, long long n) {
   lb_status s;
   if (!usable(c, &s)) return s;
   if (n < 0) return fail(c, LB_ERR_ARG, "need n >= 0");
+  while (n >= LANE_MIN_STEPS && !c->plan.empty() && !use_tma(c)) {
+    const long long to_check = c->check_every > 0 ? c->check_every - c->step % c->check_every : n;
+    const long long k = std::min(n, to_check);
+    if (k < LANE_MIN_STEPS) break;
+    s = launch_steps_chunked(c, k);
+    if (s != LB_OK) return s;
+    n -= k;
+    if (c->check_every > 0 && c->step % c->check_every == 0 && (s = check_flag(c)) != LB_OK) return s;
+  }
+  if (n == 0) return LB_OK;
   if (c->use_graph && c->check_every == 0 && n >= 3) {
     if (c->cur != 0) {  // the captured pair starts from buffer 0
       s = launch_step_once(c);
@@ -871,6 +893,7 @@ lb_status lb_autotune(lb_ctx* c, int steps_per_trial, lb_tune* best, lb_tune* tr
 void lb_destroy(lb_ctx* c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
+  c->lanes.destroy();
   free_all(c);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;

@@ -19,9 +19,9 @@ using namespace lbgm;
 
 namespace {
 
-constexpr int kLanes = 6;  // concurrent streams of a batch step
 
 struct Group {
+  int key = 0;  // variant()
   int K = 0;
   int ninst = 0;
   std::vector<unsigned char> recs;  // ListInst records
@@ -50,9 +50,9 @@ struct lb_batch {
   std::vector<Group> g;
   int tile = 0;               // nodes (FP32, FP64) or warps (2-byte storage) of a work item
 
-  cudaStream_t aux[kLanes - 1] = {};
-  cudaEvent_t ev_fork = nullptr;
-  cudaEvent_t ev_join[kLanes - 1] = {};
+  LaneStreams lanes;
+  std::vector<LaneChunk> plan;  // a call of several steps: chunks of the groups' instances
+  std::vector<LaneChunk> flat;  // one step: every instance, LIST_MAX to a launch
 
   int threads = 128;
   int tile_blocks = 1;  // LB_OPT_TILE_BLOCKS: nodes per tile = tile_blocks x threads
@@ -153,6 +153,7 @@ lb_status build(lb_batch* b) {
     for (int v = 0; v < 4; ++v) keys.push_back(K * 4 + v);
   for (int key : keys) {
     Group gr;
+    gr.key = key;
     gr.K = key / 4;
     switch (b->prec) {
       case LB_FP64: append_records<double, double>(b, key, gr.recs, &gr.ninst, &lb_ctx::geo_d); break;
@@ -174,6 +175,20 @@ lb_status build(lb_batch* b) {
     if (e != cudaSuccess) return bcuda(b, e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     b->g.push_back(std::move(gr));
   }
+  // chunk indices count within their group
+  b->flat.clear();
+  std::vector<LaneInst> inst;
+  std::vector<int> first;
+  for (size_t gi = 0; gi < b->g.size(); ++gi) {
+    first.push_back(int(inst.size()));
+    for (const lb_ctx* c : b->m)
+      if (variant(c) == b->g[gi].key)
+        inst.insert(inst.end(), size_t(c->batch), {int(gi), c->ncell, 2 * Q * c->ncell * c->elem_bytes});
+    for (int i = 0; i < b->g[gi].ninst; i += LIST_MAX)
+      b->flat.push_back({int(gi), i, std::min(LIST_MAX, b->g[gi].ninst - i), int(b->flat.size()) % LANES});
+  }
+  b->plan = plan_lanes(inst, LIST_MAX);
+  for (LaneChunk& c : b->plan) c.first -= first[size_t(c.group)];
   b->base_cur.resize(b->m.size());
   for (size_t i = 0; i < b->m.size(); ++i) b->base_cur[i] = b->m[i]->cur;
   b->parity = 0;
@@ -192,46 +207,43 @@ bool records_current(const lb_batch* b) {
   return true;
 }
 
-// The work list of instances i0 .. i0 + n - 1 of one group on stream s.
-cudaError_t launch_part(const lb_batch* b, const Group& gr, int i0, int n, cudaStream_t s) {
+// One step of a chunk of one group's instances on stream s, at parity `par`.
+cudaError_t launch_chunk(const lb_batch* b, const LaneChunk& c, int par, cudaStream_t s) {
+  const Group& gr = b->g[size_t(c.group)];
   const int grid = b->schedule == 1 ? std::max(1, gr.blocks_per_sm) * b->nsm : 0;
-  const void* recs = gr.recs.data() + gr.recs.size() / size_t(gr.ninst) * size_t(i0);
-  const int* items = gr.items.data() + i0;
+  const void* recs = gr.recs.data() + gr.recs.size() / size_t(gr.ninst) * size_t(c.first);
+  const int* items = gr.items.data() + c.first;
   switch (b->prec) {
-    case LB_FP64: return launch_step_list_f64(gr.K, recs, n, items, b->tile, b->threads, grid, b->parity, s);
-    case LB_FP32: return launch_step_list_f32(gr.K, recs, n, items, b->tile, b->threads, grid, b->parity, s);
+    case LB_FP64: return launch_step_list_f64(gr.K, recs, c.count, items, b->tile, b->threads, grid, par, s);
+    case LB_FP32: return launch_step_list_f32(gr.K, recs, c.count, items, b->tile, b->threads, grid, par, s);
     case LB_FP16_SHIFTED:
-      return launch_step_list_h16(gr.K, gr.d, gr.smem, recs, n, items, b->tile, b->threads, grid, b->parity, s);
+      return launch_step_list_h16(gr.K, gr.d, gr.smem, recs, c.count, items, b->tile, b->threads, grid, par, s);
     default:
-      return launch_step_list_b16(gr.K, gr.d, gr.smem, recs, n, items, b->tile, b->threads, grid, b->parity, s);
+      return launch_step_list_b16(gr.K, gr.d, gr.smem, recs, c.count, items, b->tile, b->threads, grid, par, s);
   }
 }
 
-// One batch step. The launches read the same buffers and write disjoint nodes,
-// so they run side by side: the first on the batch stream, the others on
-// streams forked before it and joined back.
-lb_status step_once(lb_batch* b) {
-  struct Part {
-    const Group* g;
-    int i0, n;
-  };
-  std::vector<Part> parts;
-  for (const Group& g : b->g)
-    for (int i = 0; i < g.ninst; i += LIST_MAX) parts.push_back({&g, i, std::min(LIST_MAX, g.ninst - i)});
-  const int n = int(parts.size()), lanes = std::min(n, kLanes);
-  if (n > 1) LB_BCUDA(b, cudaEventRecord(b->ev_fork, b->stream));
-  for (int k = 0; k < n; ++k) {
-    const int lane = k % kLanes;
-    if (k > 0 && k < kLanes) LB_BCUDA(b, cudaStreamWaitEvent(b->aux[k - 1], b->ev_fork, 0));
-    LB_BCUDA(b, launch_part(b, *parts[k].g, parts[k].i0, parts[k].n, lane == 0 ? b->stream : b->aux[lane - 1]));
+// n batch steps: the chunks read the same buffers and write disjoint nodes, so
+// they run side by side on the lanes; several steps in the order of lanes.h.
+lb_status steps(lb_batch* b, long long n) {
+  const std::vector<LaneChunk>& plan = n >= LANE_MIN_STEPS && !b->plan.empty() ? b->plan : b->flat;
+  const int par = b->parity;
+  cudaError_t e = cudaSuccess;
+  if (plan.size() == 1) {
+    for (long long i = 0; i < n && e == cudaSuccess; ++i) e = launch_chunk(b, plan[0], int(par ^ (i & 1)), b->stream);
+  } else {
+    const long long each = &plan == &b->flat ? 1 : n;
+    for (long long i0 = 0; i0 < n && e == cudaSuccess; i0 += each)
+      e = run_lanes(b->lanes, plan, each, b->stream, [&](const LaneChunk& c, long long i, cudaStream_t s) {
+        return launch_chunk(b, c, int(par ^ ((i0 + i) & 1)), s);
+      });
   }
-  for (int k = 1; k < lanes; ++k) {
-    LB_BCUDA(b, cudaEventRecord(b->ev_join[k - 1], b->aux[k - 1]));
-    LB_BCUDA(b, cudaStreamWaitEvent(b->stream, b->ev_join[k - 1], 0));
-  }
-  b->parity ^= 1;
+  if (e != cudaSuccess) return bcuda(b, e, "step kernel launch");
+  b->parity = int(par ^ (n & 1));
   return LB_OK;
 }
+
+lb_status step_once(lb_batch* b) { return steps(b, 1); }
 
 void advance_members(lb_batch* b, long long n) {
   for (lb_ctx* c : b->m) {
@@ -281,6 +293,17 @@ lb_status run(lb_batch* b, long long n, bool graph) {
     lb_status s = build(b);
     if (s != LB_OK) return s;
   }
+  while (n >= LANE_MIN_STEPS && !b->plan.empty()) {
+    const long long to_check = b->check_every > 0 ? b->check_every - b->step % b->check_every : n;
+    const long long k = std::min(n, to_check);
+    if (k < LANE_MIN_STEPS) break;
+    lb_status s = steps(b, k);
+    if (s != LB_OK) return s;
+    advance_members(b, k);
+    n -= k;
+    if (b->check_every > 0 && b->step % b->check_every == 0 && (s = check_members(b)) != LB_OK) return s;
+  }
+  if (n == 0) return LB_OK;
   if (graph && b->use_graph && b->check_every == 0 && n >= 3) {
     if (b->parity != 0) {  // the captured pair starts at parity 0
       lb_status s = step_once(b);
@@ -356,11 +379,7 @@ lb_status lb_batch_create(lb_ctx* const* members, int count, lb_batch** out) {
   cudaError_t e = cudaGetDevice(&cur_dev);
   if (e == cudaSuccess && cur_dev != b->device) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, b->device);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
-  for (int i = 0; i < kLanes - 1 && e == cudaSuccess; ++i) {
-    e = cudaStreamCreateWithFlags(&b->aux[i], cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_join[i], cudaEventDisableTiming);
-  }
+  if (e == cudaSuccess) e = b->lanes.create();
   if (e != cudaSuccess) return bail(LB_ERR_CUDA, std::string("batch setup: ") + cudaGetErrorString(e));
   *out = b;
   return LB_OK;
@@ -470,11 +489,7 @@ void lb_batch_destroy(lb_batch* b) {
   if (!b) return;
   if (b->stream) cudaStreamSynchronize(b->stream);
   drop_graph(b);
-  for (int i = 0; i < kLanes - 1; ++i) {
-    if (b->aux[i]) cudaStreamDestroy(b->aux[i]);
-    if (b->ev_join[i]) cudaEventDestroy(b->ev_join[i]);
-  }
-  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
+  b->lanes.destroy();
   delete b;
 }
 

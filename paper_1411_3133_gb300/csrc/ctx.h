@@ -10,6 +10,7 @@
 
 #include "../../include/lbgm.h"
 #include "kernels.cuh"
+#include "lanes.h"
 
 struct lb_ctx {
   lb_metric metric;
@@ -66,6 +67,8 @@ struct lb_ctx {
   int graph_kernel = -1;             // captured graph: 0 the step, 1 with the half-force variant, 2 TMA
   int step_kernel = 0;               // LB_OPT_STEP_KERNEL
   bool any_shift = false;            // an instance uses the half-force velocity (old_forcing 2)
+  std::vector<lbgm::LaneChunk> plan; // order of the instances in a call of several steps
+  lbgm::LaneStreams lanes;
   bool tma_ok = false;               // tensor maps built for both buffers
   alignas(64) unsigned char tmap[2][128];
 };

@@ -19,38 +19,44 @@ __device__ __forceinline__ void step_node(const Real* __restrict__ fin, Real* __
                                           const GeoDev<Real>& geo, const InstParams<Real>& ip, const Dims& d,
                                           const CellPos& p, int* __restrict__ flag) {
   Real f[Q];
+  const int row = geo_row_node<K>(d, p.ir, p.it, p.i3);
+  NodeGeo<Real, K> g;
+  // the theta-resolved ellipsoid's 15 values per node come from HBM: asked for
+  // before the gather (2 x 65 x 64 x 128, FP32: 74.6 -> 69.8 us a step); rows
+  // shared by nodes come from L1 and L2 and would only hold registers
+  if constexpr (K == KELT) g = load_geo<Real, K>(geo, row);
   gather_step(fin, p, d, f);
   const Moments<Real> m = step_moments(f);
   if (!finite_v(m.rho)) {  // NaN or Inf
     if (*flag == 0) atomicExch(flag, 1);
   }
-  const int row = geo_row_node<K>(d, p.ir, p.it, p.i3);
-  const NodeGeo<Real, K> g = load_geo<Real, K>(geo, row);
+  if constexpr (K != KELT) g = load_geo<Real, K>(geo, row);
   if (d.wall_eq && (p.ir == 0 || p.ir == d.nr - 1 || (!d.periodic3 && (p.i3 == 0 || p.i3 == d.n3 - 1)))) {
     equilibrium<Real, K>(m.rho, Real(0.0), Real(0.0), Real(0.0), g, f);
-  } else {
-    const Coef<Real> k = coefficients<Real, K>(m, g, ip.kappa, ip.G);
-    collide<Real, K>(f, k, g, ip.omega);
+    store_node<K>(fout, nullptr, p, d, f);
+    return;
   }
+  const Coef<Real> k = coefficients<Real, K>(m, g, ip.kappa, ip.G);
+  collide<Real, K>(f, k, g, ip.omega);
   store_node<K>(fout, nullptr, p, d, f);
 }
 
 // Launch bounds of the one-node-per-thread step. FP32: at most 128 threads per
-// block and 6 resident blocks per SM (80 registers; the kernel is bound by
-// latency as much as by HBM, measured best of 5..8), 5 for the ellipsoids,
-// whose geometry rows and extra Christoffel terms need more registers. FP64
-// keeps its registers (bound by the FP64 units). LBGM_STEP32_MAXT /
-// LBGM_STEP32_MINB override the FP32 values for tuning builds.
+// block and 5 resident blocks per SM (96 registers). Measured at 8 / 7 / 6 / 5 /
+// 4 blocks with the instances held in L2 (lanes.h), us a step: 24 cylinders of
+// 64 x 4 x 256 88 / 79 / 72 / 66 / -, 24 four-wall ellipsoids - / - / 80 / 68 /
+// 69, the theta-resolved ellipsoid - / - / 83 / 75 / 78. FP64 keeps its
+// registers (bound by the FP64 units). LBGM_STEP32_MAXT / LBGM_STEP32_MINB
+// override the FP32 values for tuning builds.
 #ifndef LBGM_STEP32_MAXT
 #define LBGM_STEP32_MAXT 128
 #endif
 #ifndef LBGM_STEP32_MINB
-#define LBGM_STEP32_MINB 6
+#define LBGM_STEP32_MINB 5
 #endif
 template <class Real, int K>
 struct KBounds {
-  static constexpr int maxt = LBGM_STEP32_MAXT;
-  static constexpr int minb = (K == KELL || K == KELT) && LBGM_STEP32_MINB > 1 ? LBGM_STEP32_MINB - 1 : LBGM_STEP32_MINB;
+  static constexpr int maxt = LBGM_STEP32_MAXT, minb = LBGM_STEP32_MINB;
 };
 template <int K>
 struct KBounds<double, K> {
@@ -93,7 +99,7 @@ struct ListInst {
 // 64 x 4 x 256 cylinders in FP32).
 template <typename S, typename Real>
 struct ListArgs {
-  static constexpr int N = 64;  // LIST_MAX
+  static constexpr int N = 16;  // LIST_MAX
   ListInst<S, Real> rec[N];
   int tile_start[N + 1];
   int count, tile, parity;

@@ -41,7 +41,7 @@ cudaError_t launch_step_shift_f32(int K, const float* fin, float* fout, const Ge
 // launches one block per item. 2-byte storage: a group of one metric kind, row
 // kind and parity of n3 -- d any of its instances, smem the bytes of staged
 // rows a block needs.
-constexpr int LIST_MAX = 64;
+constexpr int LIST_MAX = 16;
 cudaError_t launch_step_list_f64(int K, const void* recs, int count, const int* items, int tile, int threads,
                                  int grid, int parity, cudaStream_t s);
 cudaError_t step_list_occupancy_f64(int K, int threads, int* blocks_per_sm);
