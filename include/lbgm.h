@@ -179,31 +179,31 @@ typedef enum {
                                steps (k >= 0; 0: never; default 0) */
   LB_OPT_BLOCK_THREADS = 1, /* threads per block of the step kernel
                                (64..256, multiple of 32; default 128). The
-                               one-node-per-thread kernel with FP32
-                               arithmetic runs at most 128 per block (its
-                               register cap); larger values run as 128 */
-  LB_OPT_USE_GRAPH = 2,     /* 1: lb_step replays a captured CUDA graph of
-                               pairs of steps (default 0) */
-  LB_OPT_STEP_KERNEL = 3,   /* 0: automatic (default): FP64 arithmetic 1,
-                               else 4 where x3 is periodic with bounce-back
-                               walls, else 5;
-                               1: the one-node-per-thread kernel, gathering
-                               from global memory; 2: the TMA-pipelined
-                               kernel (FP32, bounce-back walls and n3 in
-                               {128, 256} only);
-                               4: the region split (periodic x3 and
-                               bounce-back walls only): one
-                               kernel for the 3 node layers next to each
-                               r-wall, one for the interior without any
-                               wall code; 5: tiled: runs of interior nodes
-                               and the wall nodes in two kernels (the
-                               lb_batch work-list kernels over this context
-                               alone), for any geometry. With instances
-                               of the half-force velocity variant
-                               (lb_params.old_forcing 2) the context runs
-                               kernel 1 whatever is set here.
-                               Unsupported choices return LB_ERR_ARG. All
-                               give bitwise identical states. */
+                               kernels with FP32 arithmetic run at most 128
+                               per block (their register cap); larger
+                               values run as 128 */
+  LB_OPT_USE_GRAPH = 2,     /* 1: replay a captured CUDA graph of pairs of
+                               steps (default 0) where that is the faster
+                               way: lb_step with the TMA kernel or the
+                               half-force variant, and lb_batch_step of
+                               fewer than 4 steps or of channels too small
+                               to be taken in groups. Elsewhere the steps
+                               are launched one by one, each kernel
+                               starting under the end of the one before,
+                               which is faster than a replay */
+  LB_OPT_STEP_KERNEL = 3,   /* 0: automatic (default), 1, 4, 5: the
+                               one-kernel step of the storage type (4 and
+                               5 named a region split and a tiled step
+                               that it has replaced; 4 still needs a
+                               periodic x3 and bounce-back walls);
+                               2: the TMA-pipelined kernel (FP32,
+                               bounce-back walls and n3 in {128, 256}
+                               only). With instances of the half-force
+                               velocity variant (lb_params.old_forcing 2)
+                               the context runs that variant's kernel
+                               whatever is set here. Unsupported choices
+                               return LB_ERR_ARG. All give bitwise
+                               identical states. */
   LB_OPT_SCHEDULE = 4,      /* batches only (lb_batch_set_option): 0: one
                                block per tile of block_threads nodes
                                (default); 1: a persistent grid of (resident
@@ -300,7 +300,10 @@ lb_status lb_init_fields(lb_ctx* ctx, const lb_params* params, const double* rho
 
 /* n >= 0 time steps (Eq. LB): pull streaming with full bounce-back at the
  * walls, moments, f^eq, non-equilibrium stress, forcing term with the
- * Christoffel symbols and the body force, BGK collision. Asynchronous unless
+ * Christoffel symbols and the body force, BGK collision. With n >= 4 and
+ * several instances that fit L2 in groups, a group takes all n steps before
+ * the next one starts, four groups side by side on streams of the context's
+ * own, joined to its stream before the call returns. Asynchronous unless
  * LB_OPT_CHECK_EVERY is set; then returns LB_ERR_NONFINITE when a check
  * finds a non-finite density. */
 lb_status lb_step(lb_ctx* ctx, long long n);
@@ -393,9 +396,9 @@ lb_status lb_fma_peak(lb_precision precision, void* cuda_stream, double* flops_p
 
 /* Autotuner of the step launch. Runs steps_per_trial (>= 1) time steps in
  * each configuration -- block_threads in {64, 96, 128} (FP64: {64, 128, 192,
- * 256}) with the plain step kernel, {64, 96, 128} with the region split
- * where x3 is periodic and with the tiled step, and the TMA kernel where the
- * context supports it -- timed with
+ * 256}) for LB_OPT_STEP_KERNEL 1, {64, 96, 128} for 4 where x3 is periodic
+ * with bounce-back walls and for 5 (the same kernel), and the TMA kernel where
+ * the context supports it -- timed with
  * CUDA events on the context's stream, then keeps the fastest. Every
  * configuration computes bitwise the same states, so the trial steps are
  * real time steps: they advance the simulation and the step count. best
@@ -418,15 +421,14 @@ const char* lb_last_error(const lb_ctx* ctx);
  * A sweep over Dean numbers, radii and grid sizes (Sec. III and IV vary
  * the driving force, the radii ratio and the cross-section) has instances
  * of different metric kind and size. lb_batch_step advances every instance
- * of every member context by one time step per step with two launches of a
- * work-list kernel per metric kind present: one over tiles of up to
- * block_threads consecutive interior nodes (instance, first node, count),
- * one over tiles of the nodes within three nodes of a wall (instance, first
- * index into a list of wall nodes, count), so instances of any size share
- * the grid. All these launches run concurrently on forked streams (they
- * read one buffer and write disjoint nodes). The update is the one of
- * lb_step (Eq. LB), node for node, and the resulting states are bitwise
- * those of lb_step on each member.
+ * of every member context by one time step per step with work-list launches:
+ * one kernel over tiles of up to block_threads consecutive nodes of up to 16
+ * instances of one metric kind (2-byte storage: and one parity of n3), so
+ * instances of any size share the grid. With n >= 4 the instances are taken
+ * through the steps in L2-sized groups as by lb_step. The launches run
+ * concurrently on the batch's own streams (they read one buffer and write
+ * disjoint nodes). The update is the one of lb_step (Eq. LB), node for node,
+ * and the resulting states are bitwise those of lb_step on each member.
  *
  * Members stay owned by the caller and usable with every lb_* call
  * (lb_init, lb_diagnostics, lb_get_state, ...) between batch steps; they
@@ -437,7 +439,7 @@ const char* lb_last_error(const lb_ctx* ctx);
 typedef struct lb_batch lb_batch;
 
 /* members: host array [count] of initialised or not-yet-initialised
- * contexts. No device work; the work list is built on the first step. */
+ * contexts. No device work. */
 lb_status lb_batch_create(lb_ctx* const* members, int count, lb_batch** out);
 
 /* n >= 0 time steps of every member (each must be initialised). Options:
@@ -462,7 +464,7 @@ long long lb_batch_nodes(const lb_batch* batch);
 /* Batch steps taken since creation. */
 long long lb_batch_step_count(const lb_batch* batch);
 
-/* Release the batch's work list, streams and graph (not the members). */
+/* Release the batch's streams and graph (not the members). */
 void lb_batch_destroy(lb_batch* batch);
 
 /* Message of the last failure on the batch (NULL: as lb_last_error(NULL)). */
@@ -478,7 +480,7 @@ const char* lb_batch_last_error(const lb_batch* batch);
  * 1..n_fourier) feed depth - 1 hidden layers of `width` SiLU units and a
  * linear layer of 4 outputs, which predicts (y - mean)/std per field
  * (lb_mlp_set_output_scale). Weights: FP32 master copy and Adam moments,
- * BF16 in every product, FP32 accumulation; He-uniform initial weights from
+ * BF16 in every product, FP32 activations and accumulation; He-uniform initial weights from
  * a SplitMix64 stream seeded with `seed`, zero biases. Parameters are laid
  * out layer by layer as W (fan_out x fan_in, row-major) then b. All x, y
  * arrays are device FP32, row-major ([n][n_plain + 1], [n][4]); calls are

@@ -229,8 +229,9 @@ std::string check_sparsity(const std::vector<double>& rows, const lb_geometry_de
 // region split on two streams and 103.6 for a work list.
 bool use_tma(const lb_ctx* c) { return c->prec == LB_FP32 && c->tma_ok && c->step_kernel == 2 && !c->any_shift; }
 
-// One time step of instances i0 .. i0 + count - 1 from buffer src into 1 - src.
-cudaError_t launch_step(lb_ctx* c, int src, int i0, int count, cudaStream_t s) {
+// One time step of instances i0 .. i0 + count - 1 from buffer src into 1 - src;
+// chained: see launch_chained.
+cudaError_t launch_step(lb_ctx* c, int src, int i0, int count, bool chained, cudaStream_t s) {
   Dims d = c->dims;
   d.batch = count;
   if (d.ref) d.ref += size_t(i0) * Q * size_t(d.nr) * size_t(d.geo_rows3);
@@ -240,7 +241,7 @@ cudaError_t launch_step(lb_ctx* c, int src, int i0, int count, cudaStream_t s) {
     using S = std::remove_pointer_t<decltype(elem)>;
     using R = std::conditional_t<std::is_same<S, double>::value, double, float>;
     return fn(c->K, static_cast<const S*>(c->f[src]) + off, static_cast<S*>(c->f[1 - src]) + off, geo,
-              static_cast<const InstParams<R>*>(c->inst) + i0, d, c->flag, c->block_threads, s);
+              static_cast<const InstParams<R>*>(c->inst) + i0, d, c->flag, c->block_threads, chained, s);
   };
   switch (c->prec) {
     case LB_FP64:
@@ -257,7 +258,7 @@ cudaError_t launch_step(lb_ctx* c, int src, int i0, int count, cudaStream_t s) {
 }
 
 lb_status launch_step_once(lb_ctx* c) {
-  cudaError_t e = launch_step(c, c->cur, 0, c->batch, c->stream);
+  cudaError_t e = launch_step(c, c->cur, 0, c->batch, true, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
   c->cur = 1 - c->cur;
   return LB_OK;
@@ -267,7 +268,7 @@ lb_status launch_step_once(lb_ctx* c) {
 lb_status launch_steps_chunked(lb_ctx* c, long long n) {
   const int cur = c->cur;
   cudaError_t e = run_lanes(c->lanes, c->plan, n, c->stream, [&](const LaneChunk& ch, long long i, cudaStream_t s) {
-    return launch_step(c, int(cur ^ (i & 1)), ch.first, ch.count, s);
+    return launch_step(c, int(cur ^ (i & 1)), ch.first, ch.count, false, s);
   });
   if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
   c->cur = int(cur ^ (n & 1));
@@ -593,7 +594,9 @@ lb_status lb_step(lb_ctx* c, long long n) {
     if (c->check_every > 0 && c->step % c->check_every == 0 && (s = check_flag(c)) != LB_OK) return s;
   }
   if (n == 0) return LB_OK;
-  if (c->use_graph && c->check_every == 0 && n >= 3) {
+  // chained launches (launch_chained) are faster than replaying a graph of
+  // them; the TMA kernel and the half-force variant have none
+  if (c->use_graph && c->check_every == 0 && n >= 3 && (use_tma(c) || c->any_shift)) {
     if (c->cur != 0) {  // the captured pair starts from buffer 0
       s = launch_step_once(c);
       if (s != LB_OK) return s;
@@ -602,7 +605,7 @@ lb_status lb_step(lb_ctx* c, long long n) {
     }
     // the captured kernels depend on the resolved step kernel and on whether
     // an instance uses the half-force variant (both can change with lb_init)
-    const int gk = use_tma(c) ? 2 : c->any_shift ? 1 : 0;
+    const int gk = use_tma(c) ? 2 : 1;
     if (!c->graph || c->graph_threads != c->block_threads || c->graph_kernel != gk) {
       if (c->graph) cudaGraphExecDestroy(c->graph);
       c->graph = nullptr;

@@ -207,19 +207,20 @@ bool records_current(const lb_batch* b) {
   return true;
 }
 
-// One step of a chunk of one group's instances on stream s, at parity `par`.
-cudaError_t launch_chunk(const lb_batch* b, const LaneChunk& c, int par, cudaStream_t s) {
+// One step of a chunk of one group's instances on stream s, at parity `par`;
+// chained: see launch_chained.
+cudaError_t launch_chunk(const lb_batch* b, const LaneChunk& c, int par, bool chained, cudaStream_t s) {
   const Group& gr = b->g[size_t(c.group)];
   const int grid = b->schedule == 1 ? std::max(1, gr.blocks_per_sm) * b->nsm : 0;
   const void* recs = gr.recs.data() + gr.recs.size() / size_t(gr.ninst) * size_t(c.first);
   const int* items = gr.items.data() + c.first;
   switch (b->prec) {
-    case LB_FP64: return launch_step_list_f64(gr.K, recs, c.count, items, b->tile, b->threads, grid, par, s);
-    case LB_FP32: return launch_step_list_f32(gr.K, recs, c.count, items, b->tile, b->threads, grid, par, s);
+    case LB_FP64: return launch_step_list_f64(gr.K, recs, c.count, items, b->tile, b->threads, grid, par, chained, s);
+    case LB_FP32: return launch_step_list_f32(gr.K, recs, c.count, items, b->tile, b->threads, grid, par, chained, s);
     case LB_FP16_SHIFTED:
-      return launch_step_list_h16(gr.K, gr.d, gr.smem, recs, c.count, items, b->tile, b->threads, grid, par, s);
+      return launch_step_list_h16(gr.K, gr.d, gr.smem, recs, c.count, items, b->tile, b->threads, grid, par, chained, s);
     default:
-      return launch_step_list_b16(gr.K, gr.d, gr.smem, recs, c.count, items, b->tile, b->threads, grid, par, s);
+      return launch_step_list_b16(gr.K, gr.d, gr.smem, recs, c.count, items, b->tile, b->threads, grid, par, chained, s);
   }
 }
 
@@ -230,12 +231,12 @@ lb_status steps(lb_batch* b, long long n) {
   const int par = b->parity;
   cudaError_t e = cudaSuccess;
   if (plan.size() == 1) {
-    for (long long i = 0; i < n && e == cudaSuccess; ++i) e = launch_chunk(b, plan[0], int(par ^ (i & 1)), b->stream);
+    for (long long i = 0; i < n && e == cudaSuccess; ++i) e = launch_chunk(b, plan[0], int(par ^ (i & 1)), true, b->stream);
   } else {
     const long long each = &plan == &b->flat ? 1 : n;
     for (long long i0 = 0; i0 < n && e == cudaSuccess; i0 += each)
       e = run_lanes(b->lanes, plan, each, b->stream, [&](const LaneChunk& c, long long i, cudaStream_t s) {
-        return launch_chunk(b, c, int(par ^ ((i0 + i) & 1)), s);
+        return launch_chunk(b, c, int(par ^ ((i0 + i) & 1)), false, s);
       });
   }
   if (e != cudaSuccess) return bcuda(b, e, "step kernel launch");
@@ -304,7 +305,7 @@ lb_status run(lb_batch* b, long long n, bool graph) {
     if (b->check_every > 0 && b->step % b->check_every == 0 && (s = check_members(b)) != LB_OK) return s;
   }
   if (n == 0) return LB_OK;
-  if (graph && b->use_graph && b->check_every == 0 && n >= 3) {
+  if (graph && b->use_graph && b->check_every == 0 && n >= 3 && b->flat.size() > 1) {
     if (b->parity != 0) {  // the captured pair starts at parity 0
       lb_status s = step_once(b);
       if (s != LB_OK) return s;

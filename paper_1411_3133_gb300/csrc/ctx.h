@@ -64,7 +64,7 @@ struct lb_ctx {
   int use_graph = 0;
   cudaGraphExec_t graph = nullptr;   // two steps, buffer 0 -> 1 -> 0
   int graph_threads = 0;
-  int graph_kernel = -1;             // captured graph: 0 the step, 1 with the half-force variant, 2 TMA
+  int graph_kernel = -1;             // captured graph: 1 the half-force variant, 2 TMA
   int step_kernel = 0;               // LB_OPT_STEP_KERNEL
   bool any_shift = false;            // an instance uses the half-force velocity (old_forcing 2)
   std::vector<lbgm::LaneChunk> plan; // order of the instances in a call of several steps

@@ -7,6 +7,14 @@
 
 namespace lbgm {
 
+// Programmatic dependent launch between the steps of a chain (launch_chained):
+// a step's blocks may start while the step before still runs -- they find
+// their nodes, source-table rows and geometry -- and wait for its end and its
+// memory before they touch the state. Without the launch attribute both are
+// no-ops.
+__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Fused time step (Eq. LB) of one node p of one instance whose state blocks
 // start at fin and fout: pull streaming + walls (gather_step), moments,
 // equilibrium, non-equilibrium stress, forcing, BGK, store. flag is set to 1
@@ -25,6 +33,7 @@ __device__ __forceinline__ void step_node(const Real* __restrict__ fin, Real* __
   // before the gather (2 x 65 x 64 x 128, FP32: 74.6 -> 69.8 us a step); rows
   // shared by nodes come from L1 and L2 and would only hold registers
   if constexpr (K == KELT) g = load_geo<Real, K>(geo, row);
+  chain_wait();
   gather_step(fin, p, d, f);
   const Moments<Real> m = step_moments(f);
   if (!finite_v(m.rho)) {  // NaN or Inf
@@ -69,6 +78,7 @@ template <typename Real, int K>
 __global__ void __launch_bounds__(KBounds<Real, K>::maxt, KBounds<Real, K>::minb)
     k_step(const Real* __restrict__ fin, Real* __restrict__ fout, GeoDev<Real> geo,
            const InstParams<Real>* __restrict__ inst, Dims d, int* __restrict__ flag) {
+  chain_start();
   const uint32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= uint32_t(d.ncell)) return;
   const int b = int(blockIdx.y);
@@ -123,6 +133,7 @@ struct ListArgs {
 template <typename Real, int K, bool LOOP>
 __global__ void __launch_bounds__(KBounds<Real, K>::maxt, KBounds<Real, K>::minb)
     k_step_list(const __grid_constant__ ListArgs<Real, Real> a) {
+  chain_start();
   auto item = [&](int j) {
     const int i = a.instance(j);
     const ListInst<Real, Real>& I = a.rec[i];

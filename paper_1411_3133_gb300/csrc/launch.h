@@ -13,27 +13,28 @@ namespace lbgm {
 
 struct InitInst;
 
+// chained: see launch_chained.
 cudaError_t launch_step_f64(int K, const double* fin, double* fout, const GeoDev<double>& geo,
                             const InstParams<double>* inst, const Dims& d, int* flag, int threads,
-                            cudaStream_t s);
+                            bool chained, cudaStream_t s);
 cudaError_t launch_step_f32(int K, const float* fin, float* fout, const GeoDev<float>& geo,
                             const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                            cudaStream_t s);
+                            bool chained, cudaStream_t s);
 cudaError_t launch_step_h16(int K, const __half* fin, __half* fout, const GeoDev<float>& geo,
                             const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                            cudaStream_t s);
+                            bool chained, cudaStream_t s);
 cudaError_t launch_step_b16(int K, const __nv_bfloat16* fin, __nv_bfloat16* fout, const GeoDev<float>& geo,
                             const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                            cudaStream_t s);
+                            bool chained, cudaStream_t s);
 
 // Plain step whose instances may use the half-force velocity variant
 // (InstParams::pad = 1); see step_shift.cu.
 cudaError_t launch_step_shift_f64(int K, const double* fin, double* fout, const GeoDev<double>& geo,
                                   const InstParams<double>* inst, const Dims& d, int* flag, int threads,
-                                  cudaStream_t s);
+                                  bool chained, cudaStream_t s);
 cudaError_t launch_step_shift_f32(int K, const float* fin, float* fout, const GeoDev<float>& geo,
                                   const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                                  cudaStream_t s);
+                                  bool chained, cudaStream_t s);
 
 // Work-list step over `count` (at most LIST_MAX) instances of different
 // geometry: their host records (ListInst), the work items of each and the
@@ -43,16 +44,16 @@ cudaError_t launch_step_shift_f32(int K, const float* fin, float* fout, const Ge
 // rows a block needs.
 constexpr int LIST_MAX = 16;
 cudaError_t launch_step_list_f64(int K, const void* recs, int count, const int* items, int tile, int threads,
-                                 int grid, int parity, cudaStream_t s);
+                                 int grid, int parity, bool chained, cudaStream_t s);
 cudaError_t step_list_occupancy_f64(int K, int threads, int* blocks_per_sm);
 cudaError_t launch_step_list_f32(int K, const void* recs, int count, const int* items, int tile, int threads,
-                                 int grid, int parity, cudaStream_t s);
+                                 int grid, int parity, bool chained, cudaStream_t s);
 cudaError_t step_list_occupancy_f32(int K, int threads, int* blocks_per_sm);
 cudaError_t launch_step_list_h16(int K, const Dims& d, size_t smem, const void* recs, int count, const int* items,
-                                 int tile, int threads, int grid, int parity, cudaStream_t s);
+                                 int tile, int threads, int grid, int parity, bool chained, cudaStream_t s);
 cudaError_t step_list_occupancy_h16(int K, const Dims& d, size_t smem, int threads, int* blocks_per_sm);
 cudaError_t launch_step_list_b16(int K, const Dims& d, size_t smem, const void* recs, int count, const int* items,
-                                 int tile, int threads, int grid, int parity, cudaStream_t s);
+                                 int tile, int threads, int grid, int parity, bool chained, cudaStream_t s);
 cudaError_t step_list_occupancy_b16(int K, const Dims& d, size_t smem, int threads, int* blocks_per_sm);
 
 // TMA-pipelined FP32 step (n3 in {128, 256}); map is a CUtensorMap over the

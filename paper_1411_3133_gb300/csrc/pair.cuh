@@ -261,6 +261,7 @@ __device__ __forceinline__ void step_pair(const S* __restrict__ fin, S* __restri
   uint32_t raw[Q];
   bool near = near_wall(p, d);
   if constexpr (!ROW1) near = near || (!d.periodic3 && p.i3 + 1 > d.n3 - 4);
+  chain_wait();
   if (__any_sync(0xffffffffu, near)) gather_pair_table<S>(fin, p, pair, d, raw);
   else gather_pair_far<S, EVEN>(fin, p, pair, d, raw);
   const InstParams<float> ip = *inst;
@@ -299,21 +300,26 @@ __device__ __forceinline__ void step_pair(const S* __restrict__ fin, S* __restri
   }
 }
 
-// Resident blocks of 128 threads per SM: 3 (168 registers, no spills; 24
-// 64 x 4 x 256 channels in FP16, cylinder / four-wall ellipsoid: 65 / 78 us a
-// step, at 4 blocks 68 / 97 with 200 bytes spilled, at 5 88 / 145). Parking the
-// gathered values in shared memory to fit 4 measured slower (109 / 126).
+// Largest block and resident blocks per SM (168 registers, no spills).
+// Measured on 24 64 x 4 x 256 channels in FP16, cylinder / four-wall ellipsoid,
+// one launch a step: blocks of 128 threads, 3 / 4 / 5 of them 65 / 78, 68 / 97
+// and 88 / 145 us a step (the last two spill); parking the gathered values in
+// shared memory to fit 4 measured slower (109 / 126).
+#ifndef LBGM_PAIR_MAXT
+#define LBGM_PAIR_MAXT 128
+#endif
 #ifndef LBGM_PAIR_MINB
 #define LBGM_PAIR_MINB 3
 #endif
 
 // Uniform batch: fin, fout are whole states, grid row y is instance y.
 template <typename S, int K, bool EVEN, bool ROW1>
-__global__ void __launch_bounds__(128, LBGM_PAIR_MINB)
+__global__ void __launch_bounds__(LBGM_PAIR_MAXT, LBGM_PAIR_MINB)
     k_step_pair(const S* __restrict__ fin, S* __restrict__ fout, GeoDev<float> geo,
                 const InstParams<float>* __restrict__ inst, Dims d, int* __restrict__ flag, uint32_t warps,
                 int shared) {
   extern __shared__ float4 sm[];
+  chain_start();
   const uint32_t b = blockIdx.y, w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const size_t base = size_t(b) * Q * uint32_t(d.ncell);
   step_pair<S, K, EVEN, ROW1>(fin + base, fout + base, ref_of(d, int(b)), stream_of(d, int(b)), geo, inst + b, d, w,
@@ -323,9 +329,10 @@ __global__ void __launch_bounds__(128, LBGM_PAIR_MINB)
 // Work list over instances of one metric kind and row parity (ListArgs; a tile
 // is a number of warps).
 template <typename S, int K, bool EVEN, bool ROW1>
-__global__ void __launch_bounds__(128, LBGM_PAIR_MINB)
+__global__ void __launch_bounds__(LBGM_PAIR_MAXT, LBGM_PAIR_MINB)
     k_step_pair_list(const __grid_constant__ ListArgs<S, float> a) {
   extern __shared__ float4 sm[];
+  chain_start();
   const int wpb = int(blockDim.x >> 5);
   for (int j = blockIdx.x; j < a.tile_start[a.count]; j += gridDim.x) {
     const int i = a.instance(j);

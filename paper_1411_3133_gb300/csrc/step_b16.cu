@@ -6,13 +6,13 @@ namespace lbgm {
 
 cudaError_t launch_step_b16(int K, const __nv_bfloat16* fin, __nv_bfloat16* fout, const GeoDev<float>& geo,
                             const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                            cudaStream_t s) {
-  return launch_pair_t<__nv_bfloat16>(K, fin, fout, geo, inst, d, flag, threads, s);
+                            bool chained, cudaStream_t s) {
+  return launch_pair_t<__nv_bfloat16>(K, fin, fout, geo, inst, d, flag, threads, chained, s);
 }
 
 cudaError_t launch_step_list_b16(int K, const Dims& d, size_t smem, const void* recs, int count, const int* items,
-                                 int tile, int threads, int grid, int parity, cudaStream_t s) {
-  return launch_pair_list_t<__nv_bfloat16>(K, d, smem, recs, count, items, tile, threads, grid, parity, s);
+                                 int tile, int threads, int grid, int parity, bool chained, cudaStream_t s) {
+  return launch_pair_list_t<__nv_bfloat16>(K, d, smem, recs, count, items, tile, threads, grid, parity, chained, s);
 }
 
 cudaError_t step_list_occupancy_b16(int K, const Dims& d, size_t smem, int threads, int* blocks_per_sm) {

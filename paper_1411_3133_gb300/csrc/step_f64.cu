@@ -6,13 +6,13 @@ namespace lbgm {
 
 cudaError_t launch_step_f64(int K, const double* fin, double* fout, const GeoDev<double>& geo,
                             const InstParams<double>* inst, const Dims& d, int* flag, int threads,
-                            cudaStream_t s) {
-  return launch_step_t<double>(K, fin, fout, geo, inst, d, flag, threads, s);
+                            bool chained, cudaStream_t s) {
+  return launch_step_t<double>(K, fin, fout, geo, inst, d, flag, threads, chained, s);
 }
 
 cudaError_t launch_step_list_f64(int K, const void* recs, int count, const int* items, int tile, int threads,
-                                 int grid, int parity, cudaStream_t s) {
-  return launch_step_list_t<double>(K, recs, count, items, tile, threads, grid, parity, s);
+                                 int grid, int parity, bool chained, cudaStream_t s) {
+  return launch_step_list_t<double>(K, recs, count, items, tile, threads, grid, parity, chained, s);
 }
 
 cudaError_t step_list_occupancy_f64(int K, int threads, int* blocks_per_sm) {

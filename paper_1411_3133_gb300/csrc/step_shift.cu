@@ -131,13 +131,13 @@ cudaError_t launch_shift_t(int K, const S* fin, S* fout, const GeoDev<R>& geo, c
 
 cudaError_t launch_step_shift_f64(int K, const double* fin, double* fout, const GeoDev<double>& geo,
                                   const InstParams<double>* inst, const Dims& d, int* flag, int threads,
-                                  cudaStream_t s) {
+                                  bool /*chained*/, cudaStream_t s) {
   return launch_shift_t<double, double>(K, fin, fout, geo, inst, d, flag, threads, s);
 }
 
 cudaError_t launch_step_shift_f32(int K, const float* fin, float* fout, const GeoDev<float>& geo,
                                   const InstParams<float>* inst, const Dims& d, int* flag, int threads,
-                                  cudaStream_t s) {
+                                  bool /*chained*/, cudaStream_t s) {
   return launch_shift_t<float, float>(K, fin, fout, geo, inst, d, flag, threads, s);
 }
 
