@@ -493,7 +493,7 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
       geo_arrays(static_cast<float*>(c->geo_real), nrows, c->geo_f);
     }
   }
-  if (e == cudaSuccess) e = launch_source_table(c->src_tab, c->f[0], d, c->stream);
+  if (e == cudaSuccess) e = launch_source_table(c->src_tab, d, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return bail(LB_ERR_CUDA, std::string("geometry upload: ") + cudaGetErrorString(e));

@@ -53,12 +53,30 @@ cudaError_t init_t(int K, S* f, const GeoDev<Real>& geo, const double* sqrtg, co
   return cudaGetLastError();
 }
 
-// Source table (gather_table): one thread per key, from the general source
-// rule at a node of the key's classes. fin is any address: the sources'
-// addresses are formed, never read.
-__global__ void __launch_bounds__(64) k_source_table(int* __restrict__ tab, const float* fin, Dims d) {
+// Velocities by population index, for code that loops over them.
+struct VelTable {
+  signed char c[Q][4];  // x, y, z, |c|_inf
+};
+constexpr VelTable make_velocities() {
+  VelTable t{};
+  for (int l = 1; l < Q; ++l) {
+    int s = 0;
+    for (int a = 0; a < 3; ++a) {
+      const int v = vel(l, a);
+      t.c[l][a] = static_cast<signed char>(v);
+      s = v > s ? v : -v > s ? -v : s;
+    }
+    t.c[l][3] = static_cast<signed char>(s);
+  }
+  return t;
+}
+__constant__ VelTable c_vel = make_velocities();
+
+// Source table (gather_table): one thread per key and entry, from the general
+// source rule at a node of the key's classes.
+__global__ void __launch_bounds__(256) k_source_table(int* __restrict__ tab, Dims d) {
   const int keys = axis_classes(d.nr) * d.src_nt * d.src_n3;
-  const int k = int(blockIdx.x * blockDim.x + threadIdx.x);
+  const int t = int(blockIdx.x * blockDim.x + threadIdx.x), k = t / (4 * SRC_ROW), l = t - k * 4 * SRC_ROW;
   if (k >= keys) return;
   const int c3 = k % d.src_n3, ct = (k / d.src_n3) % d.src_nt, cr = k / (d.src_n3 * d.src_nt);
   CellPos p;
@@ -67,12 +85,23 @@ __global__ void __launch_bounds__(64) k_source_table(int* __restrict__ tab, cons
   p.it = axis_class_node(ct, d.nt);
   p.i3 = axis_class_node(c3, d.n3);
   p.cell = (p.ir * d.nt + p.it) * d.n3 + p.i3;
-  int* row = tab + k * 4 * SRC_ROW;
-  auto put = [&](auto L_, const float* src, int, int) { row[decltype(L_)::value] = int(src - fin) - p.cell; };
-  put(std::integral_constant<int, 0>{}, fin + p.cell, 0, 0);
-  if (near_wall(p, d)) for_each_source_wall<KFLAT, float>(fin, p, d, put);
-  else for_each_source_far<KFLAT, float>(fin, p, d, put);
-  for (int j = Q; j < 4 * SRC_ROW; ++j) row[j] = 0;
+  int off = 0;
+  if (l > 0 && l < Q) {
+    const int cx = c_vel.c[l][0], cy = c_vel.c[l][1], cz = c_vel.c[l][2];
+    int yr, yz, src, from = l;
+    if (d.wall_eq) {  // the source clamped onto the wall layers
+      yr = min(max(p.ir - cx, 0), d.nr - 1);
+      yz = p.i3 - cz;
+      yz = d.periodic3 ? wrap_small(yz, d.n3) : min(max(yz, 0), d.n3 - 1);
+      src = (yr * d.nt + wrap_small(p.it - cy, d.nt)) * d.n3 + yz;
+    } else {
+      bool flip;
+      src = src_wall(cx, cy, cz, c_vel.c[l][3], p, d, flip, yr, yz);
+      if (flip) from = ((l - 1) ^ 1) + 1;  // the opposite of l
+    }
+    off = from * d.ncell + src - p.cell;
+  }
+  tab[t] = off;
 }
 
 // weights by population index, for the element-wise conversions
@@ -422,9 +451,9 @@ cudaError_t launch_stream_table(int prec, int K, float4* st, const float* ref, c
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_source_table(int4* tab, const void* fin, const Dims& d, cudaStream_t s) {
-  const int keys = axis_classes(d.nr) * d.src_nt * d.src_n3;
-  k_source_table<<<(keys + 63) / 64, 64, 0, s>>>(reinterpret_cast<int*>(tab), static_cast<const float*>(fin), d);
+cudaError_t launch_source_table(int4* tab, const Dims& d, cudaStream_t s) {
+  const int n = axis_classes(d.nr) * d.src_nt * d.src_n3 * 4 * SRC_ROW;
+  k_source_table<<<(n + 255) / 256, 256, 0, s>>>(reinterpret_cast<int*>(tab), d);
   return cudaGetLastError();
 }
 

@@ -92,9 +92,8 @@ cudaError_t launch_ref_table(int K, float* ref, const GeoDev<float>& geo, const 
 cudaError_t launch_stream_table(int prec, int K, float4* st, const float* ref, const InstParams<float>* inst,
                                 const void* fin, const Dims& d, cudaStream_t s);
 
-// Source table of a channel (k_source_table): keys * SRC_ROW int4 at tab; any
-// device address as fin.
-cudaError_t launch_source_table(int4* tab, const void* fin, const Dims& d, cudaStream_t s);
+// Source table of a channel (k_source_table): keys * SRC_ROW int4 at tab.
+cudaError_t launch_source_table(int4* tab, const Dims& d, cudaStream_t s);
 
 // Observables: NQ sums per instance written to out[batch * DIAG_NQ]. geo64
 // holds diag_weights of each row (node for the theta-resolved kind); partial

@@ -279,25 +279,23 @@ __device__ __forceinline__ int src_far(const Neighbours& n, const Dims& d) {
 // half-node units Q = 2 q the walls are odd integers lo < 0 < hi. Going back
 // one time step means moving 2 s towards negative Q; each fold flips the
 // population to its opposite.
-template <int CX, int CY, int CZ, int S>
-__device__ __forceinline__ int src_wall(const CellPos& p, const Dims& d, bool& flip, int& src_ir, int& src_i3) {
-  constexpr int sx = (CX > 0) - (CX < 0), sy = (CY > 0) - (CY < 0), sz = (CZ > 0) - (CZ < 0);
+__device__ __forceinline__ int src_wall(int cx, int cy, int cz, int s, const CellPos& p, const Dims& d, bool& flip,
+                                        int& src_ir, int& src_i3) {
+  const int sx = (cx > 0) - (cx < 0), sy = (cy > 0) - (cy < 0), sz = (cz > 0) - (cz < 0);
   int lo = -(1 << 30), hi = (1 << 30);
-  if constexpr (sx != 0) {
+  if (sx != 0) {
     const int l_ = sx > 0 ? -1 - 2 * p.ir : 2 * p.ir + 1 - 2 * d.nr;
     const int h_ = sx > 0 ? 2 * d.nr - 1 - 2 * p.ir : 2 * p.ir + 1;
     lo = max(lo, l_);
     hi = min(hi, h_);
   }
-  if constexpr (sz != 0) {
-    if (!d.periodic3) {
-      const int l_ = sz > 0 ? -1 - 2 * p.i3 : 2 * p.i3 + 1 - 2 * d.n3;
-      const int h_ = sz > 0 ? 2 * d.n3 - 1 - 2 * p.i3 : 2 * p.i3 + 1;
-      lo = max(lo, l_);
-      hi = min(hi, h_);
-    }
+  if (sz != 0 && !d.periodic3) {
+    const int l_ = sz > 0 ? -1 - 2 * p.i3 : 2 * p.i3 + 1 - 2 * d.n3;
+    const int h_ = sz > 0 ? 2 * d.n3 - 1 - 2 * p.i3 : 2 * p.i3 + 1;
+    lo = max(lo, l_);
+    hi = min(hi, h_);
   }
-  constexpr int D = 2 * S;
+  const int D = 2 * s;
   int Qe;
   flip = false;
   if (-D >= lo) {
@@ -393,8 +391,8 @@ __device__ __forceinline__ void for_each_source_wall(const S* __restrict__ fin, 
     using C = Pair<P>;
     bool fp, fm;
     int rp, zp, rm, zm;
-    const uint32_t sp = uint32_t(src_wall<C::x, C::y, C::z, C::s>(p, d, fp, rp, zp));
-    const uint32_t sm = uint32_t(src_wall<-C::x, -C::y, -C::z, C::s>(p, d, fm, rm, zm));
+    const uint32_t sp = uint32_t(src_wall(C::x, C::y, C::z, C::s, p, d, fp, rp, zp));
+    const uint32_t sm = uint32_t(src_wall(-C::x, -C::y, -C::z, C::s, p, d, fm, rm, zm));
     const int lp = fp ? 2 * P + 2 : 2 * P + 1, lm = fm ? 2 * P + 1 : 2 * P + 2;
     fn(std::integral_constant<int, 2 * P + 1>{}, fin + (lp * N + sp), lp, geo_row<K>(d, rp, zp));
     fn(std::integral_constant<int, 2 * P + 2>{}, fin + (lm * N + sm), lm, geo_row<K>(d, rm, zm));
