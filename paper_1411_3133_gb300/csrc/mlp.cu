@@ -14,12 +14,10 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
-#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <string>
-#include <type_traits>
 #include <vector>
 
 #include "../../include/lbgm.h"
@@ -51,222 +49,138 @@ __global__ void k_features(const float* __restrict__ x, int n, int np, int nf, f
 
 __device__ __forceinline__ float sigmoidf(float z) { return 1.0f / (1.0f + expf(-z)); }
 
-// Products C = A B on the tensor cores (mma.sync m16n8k16, BF16 operands, FP32
-// accumulation) with FP32 operands taken apart into three BF16 terms: a = h +
-// m + l, each term the rounding of what the ones before left, holds all 24 bits
-// of a, so against a BF16 weight the three products are exact and against
-// another FP32 operand the six largest of the nine leave out 2^-26 of the
-// product. 64 x 64 output tiles, 8 warps of 16 x 32; 32-deep k slices go
-// through registers (loaded while the slice before is multiplied, as 16-byte
-// words where the operand allows it, VEC) and are taken apart on their way to
-// shared memory. A 4096 x 256 x 256 layer: 28 us as multiply-adds on the FP32
-// pipes with the same tiles (33 % busy, 14 warps an SM), 30 us before that.
-constexpr int TM = 64, TN = 64, TK = 32;
-// A slice in shared memory: 64 columns of 32 k (KC, rows padded to 40) or 32 k
-// of 64 columns (padded to 72); both are free of ldmatrix bank conflicts.
-constexpr int PLANE = 64 * 40;
-constexpr int ROW_KC = 40, ROW_CK = 72;
+// Products C = A B on the FP32 pipes. Every output is one chain of FP32
+// multiply-adds in ascending k, whatever the tile: training amplifies rounding
+// (a weight that rounds to the other BF16 neighbour changes the gradients by
+// 1e-3 of their rms), so the kernels' sums keep one order. Tensor cores with
+// the FP32 operands split into three BF16 terms ran the four steps below in
+// 0.72 ms, but with sums of their own order.
+// 64 x 64 output tiles, 128 threads with 8 x 4 outputs each: 26 us for 4096 x
+// 256 x 256 (20 TFLOP/s), as 4 x 4 outputs of 256 threads take, which read 8
+// values of shared memory for 16 multiply-adds; 8 x 8 leave three warps on an
+// SM and take 34 us. 32-deep k slices, loaded as 16-byte words where the operand
+// allows it (VEC) into registers while the slice before is multiplied, double
+// buffered in shared memory. Column groups of 4 are swizzled by k / 4, so that
+// stores along k and reads along the columns meet no bank conflicts.
+constexpr int TL = 64, TK = 32, LTHREADS = 128, QUADS = TL * TK / 4 / LTHREADS;
+struct Tiles {
+  float A[2][TK][TL];
+  float B[2][TK][TL];
+};
 
 __device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ uint2 load4(const __nv_bfloat16* p) { return *reinterpret_cast<const uint2*>(p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 r = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
+                     __uint_as_float(r.y & 0xffff0000u));
+}
 __device__ __forceinline__ float load1(const float* p) { return *p; }
 __device__ __forceinline__ float load1(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 
-// 4 consecutive elements of an operand in registers.
-template <class T>
-struct Quad;
-template <>
-struct Quad<float> {
-  float4 v;
-  static constexpr int planes = 3;
-};
-template <>
-struct Quad<__nv_bfloat16> {
-  uint2 v;
-  static constexpr int planes = 1;
-};
-__device__ __forceinline__ uint32_t bf16x2(float lo, float hi) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
-__device__ __forceinline__ float lo_f(uint32_t r) { return __uint_as_float(r << 16); }
-__device__ __forceinline__ float hi_f(uint32_t r) { return __uint_as_float(r & 0xffff0000u); }
-// what a term leaves of x; nothing of an infinity or NaN, which the term holds
-__device__ __forceinline__ float rest(float x, float term) { return fabsf(term) <= 3.4e38f ? x - term : 0.0f; }
-
-// One thread's two quads of a slice [k0, k0 + TK) x [c0, c0 + 64). Operand with
+// One thread's i-th quad of a slice [k0, k0 + TK) x [c0, c0 + 64). Operand with
 // k contiguous (KC): element (k, c) at p[c * ld + k], a quad is 4 k of one c;
 // else at p[k * ld + c], 4 c of one k. Zero outside k < K, c < C.
 template <bool KC>
 __device__ __forceinline__ void quad_at(int i, int& k, int& c) {
-  const int x = int(threadIdx.x) + i * 256;
+  const int x = int(threadIdx.x) + i * LTHREADS;
   k = KC ? (x & 7) * 4 : x >> 4;
   c = KC ? x >> 3 : (x & 15) * 4;
 }
-template <bool KC, bool VEC, class T>
-__device__ __forceinline__ Quad<T> slice_load(int i, const T* __restrict__ p, size_t ld, int k0, int c0, int K, int C) {
+template <bool KC, bool VEC, class E>
+__device__ __forceinline__ float4 slice_load(int i, const E* __restrict__ p, size_t ld, int k0, int c0, int K, int C) {
   int k, c;
   quad_at<KC>(i, k, c);
   k += k0;
   c += c0;
-  Quad<T> r;
-  r.v = {};
+  float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
   if (k >= K || c >= C) return r;
-  const T* q = KC ? p + size_t(c) * ld + k : p + size_t(k) * ld + c;
-  if constexpr (VEC) {  // K (KC) or C is a multiple of 4: whole words
-    r.v = load4(q);
-  } else {
-    const int left = KC ? K - k : C - c;
-    float e[4] = {load1(q), 0.f, 0.f, 0.f};
-    for (int j = 1; j < 4; ++j)
-      if (j < left) e[j] = load1(q + j);
-    if constexpr (std::is_same<T, float>::value) r.v = make_float4(e[0], e[1], e[2], e[3]);
-    else r.v = make_uint2(bf16x2(e[0], e[1]), bf16x2(e[2], e[3]));
-  }
+  const E* q = KC ? p + size_t(c) * ld + k : p + size_t(k) * ld + c;
+  if constexpr (VEC) return load4(q);  // K (KC) or C is a multiple of 4: whole words
+  const int left = KC ? K - k : C - c;
+  r.x = load1(q);
+  if (left > 1) r.y = load1(q + 1);
+  if (left > 2) r.z = load1(q + 2);
+  if (left > 3) r.w = load1(q + 3);
   return r;
 }
-template <bool KC, class T>
-__device__ __forceinline__ void slice_store(int i, __nv_bfloat16* s, const Quad<T>& r) {
+__device__ __forceinline__ int swizzled(int k, int group) { return (group ^ (k >> 2)) * 4; }
+template <bool KC>
+__device__ __forceinline__ void slice_store(int i, float (&s)[TK][TL], const float4& r) {
   int k, c;
   quad_at<KC>(i, k, c);
-  __nv_bfloat16* at = s + (KC ? c * ROW_KC + k : k * ROW_CK + c);
-  if constexpr (std::is_same<T, float>::value) {
-    float4 x = r.v;
-#pragma unroll
-    for (int t = 0; t < 3; ++t) {
-      const uint32_t a = bf16x2(x.x, x.y), b = bf16x2(x.z, x.w);
-      *reinterpret_cast<uint2*>(at + t * PLANE) = make_uint2(a, b);
-      x = make_float4(rest(x.x, lo_f(a)), rest(x.y, hi_f(a)), rest(x.z, lo_f(b)), rest(x.w, hi_f(b)));
-    }
+  if constexpr (KC) {
+    const int at = swizzled(k, c >> 2) + (c & 3);  // k / 4 is the same for all four
+    s[k][at] = r.x;
+    s[k + 1][at] = r.y;
+    s[k + 2][at] = r.z;
+    s[k + 3][at] = r.w;
   } else {
-    *reinterpret_cast<uint2*>(at) = r.v;
+    *reinterpret_cast<float4*>(&s[k][swizzled(k, c >> 2)]) = r;
   }
 }
 
-template <bool TRANS>
-__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const __nv_bfloat16* p) {
-  const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
-  if constexpr (TRANS)
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(a)
-                 : "memory");
-  else
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(a)
-                 : "memory");
-}
-__device__ __forceinline__ void mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-      "{%0, %1, %2, %3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// The warp's 16 x 32 outputs: acc[j] holds columns 8 j .. 8 j + 7 of its 32, in
-// the layout of mma's accumulator: rows lane / 4 and lane / 4 + 8, columns
-// 2 (lane % 4) and the next. f(row, column, value) for each, in the tile.
-template <class F>
-__device__ __forceinline__ void for_outputs(const float (&acc)[4][4], F&& f) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int r = (w >> 1) * 16 + lane / 4, c = (w & 1) * 32 + 2 * (lane & 3);
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) f(r + (e >> 1) * 8, c + 8 * j + (e & 1), acc[j][e]);
-}
-
-// acc += the 64 x 64 tile at (m0, n0) of A B over k in [kb, ke); colsum (A not
-// KC; NULL: none) += the sums over the thread's k of its 4 columns of A.
+// acc += the 64 x 64 tile at (m0, n0) of A B over k in [0, K): the thread's rows
+// are 4 ty .. and 32 + 4 ty .., its columns 4 tx ..
 template <bool AKC, bool BKC, bool VEC, class TA, class TB>
-__device__ __forceinline__ void tile_product(__nv_bfloat16* sm, const TA* __restrict__ A, size_t lda, int M,
-                                             const TB* __restrict__ B, size_t ldb, int N, int kb, int ke, int m0,
-                                             int n0, float (&acc)[4][4], float4* colsum) {
-  constexpr int PA = Quad<TA>::planes, PB = Quad<TB>::planes;
-  __nv_bfloat16* sa = sm;
-  __nv_bfloat16* sb = sm + PA * PLANE;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int mw = (w >> 1) * 16, nw = (w & 1) * 32, q = lane >> 3, r = lane & 7;
-  Quad<TA> ra[2];
-  Quad<TB> rb[2];
+__device__ __forceinline__ void tile_product(Tiles& sh, const TA* __restrict__ A, size_t lda, int M,
+                                             const TB* __restrict__ B, size_t ldb, int N, int K, int m0, int n0,
+                                             float (&acc)[8][4]) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  float4 ra[QUADS], rb[QUADS];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    ra[i] = slice_load<AKC, VEC>(i, A, lda, kb, m0, ke, M);
-    rb[i] = slice_load<BKC, VEC>(i, B, ldb, kb, n0, ke, N);
+  for (int i = 0; i < QUADS; ++i) {
+    ra[i] = slice_load<AKC, VEC>(i, A, lda, 0, m0, K, M);
+    rb[i] = slice_load<BKC, VEC>(i, B, ldb, 0, n0, K, N);
   }
-  for (int k0 = kb; k0 < ke; k0 += TK) {
-    if (k0 > kb) __syncthreads();  // every warp is done with the slice before
+  int buf = 0;
+  for (int k0 = 0; k0 < K; k0 += TK, buf ^= 1) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      slice_store<AKC>(i, sa, ra[i]);
-      slice_store<BKC>(i, sb, rb[i]);
-      if constexpr (!AKC) {
-        if (colsum) {
-          colsum->x += ra[i].v.x;
-          colsum->y += ra[i].v.y;
-          colsum->z += ra[i].v.z;
-          colsum->w += ra[i].v.w;
-        }
-      }
+    for (int i = 0; i < QUADS; ++i) {
+      slice_store<AKC>(i, sh.A[buf], ra[i]);
+      slice_store<BKC>(i, sh.B[buf], rb[i]);
     }
-    __syncthreads();
-    if (k0 + TK < ke) {
+    __syncthreads();  // also: every warp is done with the slice that used this buffer
+    if (k0 + TK < K) {
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        ra[i] = slice_load<AKC, VEC>(i, A, lda, k0 + TK, m0, ke, M);
-        rb[i] = slice_load<BKC, VEC>(i, B, ldb, k0 + TK, n0, ke, N);
+      for (int i = 0; i < QUADS; ++i) {
+        ra[i] = slice_load<AKC, VEC>(i, A, lda, k0 + TK, m0, K, M);
+        rb[i] = slice_load<BKC, VEC>(i, B, ldb, k0 + TK, n0, K, N);
       }
     }
 #pragma unroll
-    for (int kk = 0; kk < TK; kk += 16) {
-      uint32_t a[PA][4], b[PB][2][4];
+    for (int kk = 0; kk < TK; ++kk) {
+      float av[8], bv[4];
+      *reinterpret_cast<float4*>(av) = load4(&sh.A[buf][kk][swizzled(kk, ty)]);
+      *reinterpret_cast<float4*>(av + 4) = load4(&sh.A[buf][kk][swizzled(kk, ty + 8)]);
+      *reinterpret_cast<float4*>(bv) = load4(&sh.B[buf][kk][swizzled(kk, tx)]);
 #pragma unroll
-      for (int t = 0; t < PA; ++t) {
-        const __nv_bfloat16* s = sa + t * PLANE;
-        if constexpr (AKC) ldmatrix4<false>(a[t], s + (mw + (lane & 15)) * ROW_KC + kk + (lane >> 4) * 8);
-        else ldmatrix4<true>(a[t], s + (kk + (q >> 1) * 8 + r) * ROW_CK + mw + (q & 1) * 8);
-      }
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int t = 0; t < PB; ++t)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const __nv_bfloat16* s = sb + t * PLANE;
-          const int n = nw + 16 * h;
-          if constexpr (BKC) ldmatrix4<false>(b[t][h], s + (n + (q >> 1) * 8 + r) * ROW_KC + kk + (q & 1) * 8);
-          else ldmatrix4<true>(b[t][h], s + (kk + (q & 1) * 8 + r) * ROW_CK + n + (q >> 1) * 8);
-        }
-      // the sum over 16 k from zero, smallest terms first, then added to the
-      // accumulators by FP32 additions: mma cuts its sum off instead of
-      // rounding it, and over a chain of them the cuts add up (error of the
-      // gradients against FP64 4.9e-6 where the FP32 pipes give 7e-7)
-      float part[4][4] = {};
-#pragma unroll
-      for (int ta = PA - 1; ta >= 0; --ta)
-#pragma unroll
-        for (int tb = PB - 1; tb >= 0; --tb) {
-          if (ta + tb > 2) continue;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) mma(part[j], a[ta], b[tb][j >> 1][(j & 1) * 2], b[tb][j >> 1][(j & 1) * 2 + 1]);
-        }
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[j][e] += part[j][e];
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
     }
   }
+}
+
+// f(row, column, value) for the thread's outputs, in the tile.
+template <class F>
+__device__ __forceinline__ void for_outputs(const float (&acc)[8][4], F&& f) {
+  const int r = (threadIdx.x >> 4) * 4, c = (threadIdx.x & 15) * 4;
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) f(r + (i & 3) + 32 * (i >> 2), c + j, acc[i][j]);
 }
 
 // Hidden layer: Z = in W^T + b, H = SiLU(Z); in n x fi, W fo x fi.
 template <bool VEC>
-__global__ void __launch_bounds__(256) k_layer(int n, int fo, int fi, const float* __restrict__ in,
-                                               const __nv_bfloat16* __restrict__ W, const float* __restrict__ bias,
-                                               float* __restrict__ Z, float* __restrict__ H) {
-  __shared__ __align__(16) __nv_bfloat16 sm[4 * PLANE];
-  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
-  float acc[4][4] = {};
-  tile_product<true, true, VEC>(sm, in, fi, n, W, fi, fo, 0, fi, m0, n0, acc, nullptr);
+__global__ void __launch_bounds__(LTHREADS) k_layer(int n, int fo, int fi, const float* __restrict__ in,
+                                                       const __nv_bfloat16* __restrict__ W,
+                                                       const float* __restrict__ bias, float* __restrict__ Z,
+                                                       float* __restrict__ H) {
+  __shared__ Tiles sh;
+  const int m0 = blockIdx.x * TL, n0 = blockIdx.y * TL;
+  float acc[8][4] = {};
+  tile_product<true, true, VEC>(sh, in, fi, n, W, fi, fo, fi, m0, n0, acc);
   for_outputs(acc, [&](int r, int c, float v) {
     if (m0 + r >= n || n0 + c >= fo) return;
     const size_t at = size_t(m0 + r) * fo + n0 + c;
@@ -279,12 +193,13 @@ __global__ void __launch_bounds__(256) k_layer(int n, int fo, int fi, const floa
 // Backward through a hidden layer: Z = (dZ_next W) SiLU'(Z), in place; dZ_next
 // n x fo, W fo x fi, Z n x fi.
 template <bool VEC>
-__global__ void __launch_bounds__(256) k_layer_back(int n, int fo, int fi, const float* __restrict__ dZn,
-                                                    const __nv_bfloat16* __restrict__ W, float* __restrict__ Z) {
-  __shared__ __align__(16) __nv_bfloat16 sm[4 * PLANE];
-  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
-  float acc[4][4] = {};
-  tile_product<true, false, VEC>(sm, dZn, fo, n, W, fi, fi, 0, fo, m0, n0, acc, nullptr);
+__global__ void __launch_bounds__(LTHREADS) k_layer_back(int n, int fo, int fi, const float* __restrict__ dZn,
+                                                            const __nv_bfloat16* __restrict__ W,
+                                                            float* __restrict__ Z) {
+  __shared__ Tiles sh;
+  const int m0 = blockIdx.x * TL, n0 = blockIdx.y * TL;
+  float acc[8][4] = {};
+  tile_product<true, false, VEC>(sh, dZn, fo, n, W, fi, fi, fo, m0, n0, acc);
   for_outputs(acc, [&](int r, int c, float v) {
     if (m0 + r >= n || n0 + c >= fi) return;
     const size_t at = size_t(m0 + r) * fi + n0 + c;
@@ -293,131 +208,195 @@ __global__ void __launch_bounds__(256) k_layer_back(int n, int fo, int fi, const
   });
 }
 
-// Output layer, one warp per row: Y = H W^T + b (4 outputs). Training (y not
-// NULL): the gradient of the mean squared error of normalised outputs dY =
-// 2 (Y - T) / (n NOUT), T = (y - mean) istd, its way back through the last
-// hidden layer Z = (dY W) SiLU'(Z) (in place), and per-block partial sums of
-// the squared error; else pred = Y std + mean.
+// Output layer of OUT_ROWS rows: Y = H W^T + b (4 outputs, one thread each, H
+// and W staged in shared memory 256 columns at a time: 15 us for 4096 rows, 24
+// with H read where it is used). Training (y not NULL):
+// the gradient of the mean squared error of normalised outputs dY = 2 (Y - T) /
+// (n NOUT), T = (y - mean) istd, its way back through the last hidden layer Z =
+// (dY W) SiLU'(Z) (in place), and the block's partial sum of the squared error;
+// else pred = Y std + mean.
+constexpr int OUT_ROWS = 16, OUT_COLS = 256;
 __global__ void __launch_bounds__(256) k_output(int n, int fi, const float* __restrict__ H,
                                                 const __nv_bfloat16* __restrict__ W, const float* __restrict__ bias,
                                                 const float* __restrict__ scale, const float* __restrict__ y,
                                                 float* __restrict__ dY, float* __restrict__ Z,
                                                 float* __restrict__ partial, float* __restrict__ pred) {
-  __shared__ float s_e[8];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int row = blockIdx.x * 8 + wib;
-  float e2 = 0.0f;
-  if (row < n) {
-    float o[NOUT] = {};
-    const float* h = H + size_t(row) * fi;
-    for (int k = lane; k < fi; k += 32) {
-      const float hv = h[k];
+  __shared__ float s_d[OUT_ROWS][NOUT], s_e[OUT_ROWS * NOUT];
+  __shared__ float s_h[OUT_ROWS][OUT_COLS + 1], s_w[NOUT][OUT_COLS + 1];
+  const int row0 = blockIdx.x * OUT_ROWS;
+  const int r = threadIdx.x / NOUT, q = threadIdx.x % NOUT, row = row0 + r;
+  float o = 0.0f;
+  for (int k0 = 0; k0 < fi; k0 += OUT_COLS) {
+    const int k = k0 + int(threadIdx.x), ke = min(OUT_COLS, fi - k0);
+    if (k < fi) {
 #pragma unroll
-      for (int q = 0; q < NOUT; ++q) o[q] = fmaf(hv, load1(W + size_t(q) * fi + k), o[q]);
+      for (int i = 0; i < OUT_ROWS; ++i) s_h[i][threadIdx.x] = row0 + i < n ? H[size_t(row0 + i) * fi + k] : 0.0f;
+#pragma unroll
+      for (int i = 0; i < NOUT; ++i) s_w[i][threadIdx.x] = load1(W + size_t(i) * fi + k);
     }
-#pragma unroll
-    for (int q = 0; q < NOUT; ++q) {
-#pragma unroll
-      for (int s = 16; s > 0; s >>= 1) o[q] += __shfl_xor_sync(0xffffffffu, o[q], s);
-      o[q] += bias[q];
+    __syncthreads();
+    if (threadIdx.x < OUT_ROWS * NOUT) {
+#pragma unroll 16
+      for (int j = 0; j < ke; ++j) o = fmaf(s_h[r][j], s_w[q][j], o);
     }
-    const float* mean = scale;
-    const float* istd = scale + NOUT;
-    const float* sd = scale + 2 * NOUT;
-    if (y) {
-      float d[NOUT];
-#pragma unroll
-      for (int q = 0; q < NOUT; ++q) {
-        const float t = (y[size_t(row) * NOUT + q] - mean[q]) * istd[q];
-        const float e = o[q] - t;
-        d[q] = 2.0f * e / float(n * NOUT);
-        e2 += e * e;
-        if (lane == q) dY[size_t(row) * NOUT + q] = d[q];
+    __syncthreads();
+  }
+  if (threadIdx.x < OUT_ROWS * NOUT) {
+    float d = 0.0f, e2 = 0.0f;
+    if (row < n) {
+      o += bias[q];
+      if (y) {
+        const float t = (y[size_t(row) * NOUT + q] - scale[q]) * scale[NOUT + q];
+        const float e = o - t;
+        d = 2.0f * e / float(n * NOUT);
+        e2 = e * e;
+        dY[size_t(row) * NOUT + q] = d;
+      } else {
+        pred[size_t(row) * NOUT + q] = o * scale[2 * NOUT + q] + scale[q];
       }
-      float* zr = Z + size_t(row) * fi;
-      for (int k = lane; k < fi; k += 32) {
-        float g = 0.0f;
-#pragma unroll
-        for (int q = 0; q < NOUT; ++q) g = fmaf(d[q], load1(W + size_t(q) * fi + k), g);
-        const float z = zr[k], s = sigmoidf(z);
-        zr[k] = g * (s * (1.0f + z * (1.0f - s)));
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < NOUT; ++q)
-        if (lane == q) pred[size_t(row) * NOUT + q] = o[q] * sd[q] + mean[q];
     }
+    s_d[r][q] = d;
+    s_e[threadIdx.x] = e2;
   }
   if (!y) return;
-  if (lane == 0) s_e[wib] = e2;
   __syncthreads();
+  const int rows = min(OUT_ROWS, n - row0);
+  for (int k = threadIdx.x; k < fi; k += 256) {
+    float w[NOUT];
+#pragma unroll
+    for (int q = 0; q < NOUT; ++q) w[q] = load1(W + size_t(q) * fi + k);
+    for (int r = 0; r < rows; ++r) {
+      float g = 0.0f;
+#pragma unroll
+      for (int q = 0; q < NOUT; ++q) g = fmaf(s_d[r][q], w[q], g);
+      float* zr = Z + size_t(row0 + r) * fi + k;
+      const float z = *zr, s = sigmoidf(z);
+      *zr = g * (s * (1.0f + z * (1.0f - s)));
+    }
+  }
   if (threadIdx.x == 0) {
     float t = 0.0f;
-    for (int w = 0; w < 8; ++w) t += s_e[w];
+    for (int i = 0; i < OUT_ROWS * NOUT; ++i) t += s_e[i];
     partial[blockIdx.x] = t;
   }
 }
 
-// Weight gradients of every layer in one launch: dW[o][k] = sum_i dZ[i][o]
-// in[i][k], db[o] = sum_i dZ[i][o]. Grid x: 64 x 64 tiles of all layers, grid
-// y: chunks of rows, each with its own copy of the gradient (part + y *
-// nparam), summed by k_adam in a fixed order -- one chunk alone would leave
-// the 16 tiles of a 256 x 256 layer on 16 SMs.
+__device__ __forceinline__ void copy_async(void* dst, const float* src, int bytes, bool valid) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  const int n = valid ? bytes : 0;  // the rest is filled with zeros
+  if (bytes == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+// Gradients of every layer in one launch: dW[o][k] = sum_i dZ[i][o] in[i][k] by
+// 32 x 32 tiles of 128 threads with 4 x 2 outputs (a 256 x 256 layer alone is 64
+// blocks; the sums over the rows stay one chain, so smaller tiles are what
+// spreads them over the SMs). A further block per 32 rows of dW sums the bias'
+// gradient db[o] = sum_i dZ[i][o]. Too few warps to hide a load behind another's
+// arithmetic: the slices of 32 rows arrive by cp.async, three of them in
+// flight. 105 us for the 5 x 256 network on 4096 rows; 157 us with the next
+// slice in registers and db summed from global memory.
 constexpr int MAX_DEPTH = 16;
+constexpr int TG = 32, GTHREADS = 128, GROWS = 32, GSTAGES = 4;
 struct WeightJobs {
   int layers;
   struct {
     const float* dZ;
     const float* in;
-    int fo, fi, tile0, vec;
+    int fo, fi, tile0;
+    bool vec_z, vec_in;  // rows are whole 16-byte words
     size_t w_off, b_off;
   } job[MAX_DEPTH];
 };
-__global__ void __launch_bounds__(256) k_weight_grads(WeightJobs jobs, int n, int chunk, float* __restrict__ part,
-                                                      size_t nparam) {
-  __shared__ __align__(16) __nv_bfloat16 sm[6 * PLANE];
+__global__ void __launch_bounds__(GTHREADS) k_weight_grads(const __grid_constant__ WeightJobs jobs, int n,
+                                                           float* __restrict__ g) {
+  __shared__ float4 st[GSTAGES][2][GROWS][TG / 4];
   int l = 0;
   while (l + 1 < jobs.layers && int(blockIdx.x) >= jobs.job[l + 1].tile0) ++l;
   const auto& J = jobs.job[l];
-  const int tiles_n = (J.fi + TN - 1) / TN, tile = int(blockIdx.x) - J.tile0;
-  const int m0 = tile / tiles_n * TM, n0 = tile % tiles_n * TN;
-  const int kb = int(blockIdx.y) * chunk, ke = min(n, kb + chunk);
-  float acc[4][4] = {};
-  float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
-  float4* csp = n0 == 0 ? &cs : nullptr;
-  if (J.vec) tile_product<false, false, true>(sm, J.dZ, J.fo, J.fo, J.in, J.fi, J.fi, kb, ke, m0, n0, acc, csp);
-  else tile_product<false, false, false>(sm, J.dZ, J.fo, J.fo, J.in, J.fi, J.fi, kb, ke, m0, n0, acc, csp);
-  float* g = part + size_t(blockIdx.y) * nparam;
-  for_outputs(acc, [&](int r, int c, float v) {
-    if (m0 + r < J.fo && n0 + c < J.fi) g[J.w_off + size_t(m0 + r) * J.fi + n0 + c] = v;
-  });
-  if (csp) {  // thread t holds the sums of columns 4 (t % 16) .. over its k: add the 16 threads'
-    float* s = reinterpret_cast<float*>(sm);
-    __syncthreads();
-    *reinterpret_cast<float4*>(s + (threadIdx.x >> 4) * TM + (threadIdx.x & 15) * 4) = cs;
-    __syncthreads();
-    if (threadIdx.x < TM && m0 + int(threadIdx.x) < J.fo) {
-      float t = 0.0f;
+  const int fo = J.fo, fi = J.fi;
+  const float* __restrict__ dZ = J.dZ;
+  const float* __restrict__ in = J.in;
+  const int tiles_n = (fi + TG - 1) / TG + 1, tile = int(blockIdx.x) - J.tile0;
+  const int m0 = tile / tiles_n * TG, n0 = tile % tiles_n * TG;
+  const bool bias = tile % tiles_n == tiles_n - 1;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  // rows [k0, k0 + 32) of columns [c0, c0 + 32) of an operand
+  auto fetch_one = [&](float4 (&dst)[GROWS][TG / 4], const float* __restrict__ p, int cols, bool vec, int c0, int k0) {
+    if (vec) {
+      const int c = c0 + (threadIdx.x & 7) * 4;
 #pragma unroll
-      for (int k = 0; k < 16; ++k) t += s[k * TM + threadIdx.x];
-      g[J.b_off + m0 + threadIdx.x] = t;
+      for (int i = 0; i < GROWS * TG / 4 / GTHREADS; ++i) {
+        const int k = (threadIdx.x >> 3) + i * (GTHREADS / 8), row = k0 + k;
+        const bool ok = row < n && c < cols;
+        copy_async(&dst[k][threadIdx.x & 7], ok ? p + size_t(row) * cols + c : p, 16, ok);
+      }
+    } else {
+      const int c = c0 + (threadIdx.x & 31);
+#pragma unroll
+      for (int i = 0; i < GROWS * TG / GTHREADS; ++i) {
+        const int k = (threadIdx.x >> 5) + i * (GTHREADS / 32), row = k0 + k;
+        const bool ok = row < n && c < cols;
+        copy_async(reinterpret_cast<float*>(dst[k]) + (threadIdx.x & 31), ok ? p + size_t(row) * cols + c : p, 4, ok);
+      }
+    }
+  };
+  auto fetch = [&](int s, int k0) {
+    fetch_one(st[s][0], dZ, fo, J.vec_z, m0, k0);
+    if (!bias) fetch_one(st[s][1], in, fi, J.vec_in, n0, k0);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int s = 0; s < GSTAGES - 1; ++s) fetch(s, s * GROWS);
+  float acc[4][2] = {};
+  float col = 0.0f;
+  int s = 0;
+  for (int k0 = 0; k0 < n; k0 += GROWS, s = (s + 1) % GSTAGES) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(GSTAGES - 2) : "memory");
+    __syncthreads();  // the slice is there, and the one before has been read
+    fetch((s + GSTAGES - 1) % GSTAGES, k0 + (GSTAGES - 1) * GROWS);
+    if (bias) {
+      if (threadIdx.x < TG) {
+        const float* z = reinterpret_cast<const float*>(st[s][0]) + threadIdx.x;
+#pragma unroll
+        for (int kk = 0; kk < GROWS; ++kk) col += z[kk * TG];
+      }
+      continue;
+    }
+#pragma unroll
+    for (int kk = 0; kk < GROWS; ++kk) {
+      const float4 a = st[s][0][kk][ty];
+      const float2 b = reinterpret_cast<const float2*>(st[s][1][kk])[tx];
+      const float av[4] = {a.x, a.y, a.z, a.w}, bv[2] = {b.x, b.y};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
     }
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (bias) {
+    if (threadIdx.x < TG && m0 + int(threadIdx.x) < fo) g[J.b_off + m0 + threadIdx.x] = col;
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      if (m0 + ty * 4 + i < fo && n0 + tx * 2 + j < fi)
+        g[J.w_off + size_t(m0 + ty * 4 + i) * fi + n0 + tx * 2 + j] = acc[i][j];
 }
 
-// Sum of the chunks' gradients, then Adam on the FP32 master parameters and
-// their BF16 copy. Block 0 also sums the loss.
-__global__ void __launch_bounds__(256) k_adam(float* __restrict__ w, float* __restrict__ g,
-                                              const float* __restrict__ part, int chunks, float* __restrict__ m,
-                                              float* __restrict__ v, __nv_bfloat16* __restrict__ wb, size_t count,
-                                              float lr, float b1, float b2, float c1, float c2, float eps,
+// Adam on the FP32 master parameters; refreshes their BF16 copy. Block 0 also
+// sums the loss.
+__global__ void __launch_bounds__(256) k_adam(float* __restrict__ w, const float* __restrict__ g,
+                                              float* __restrict__ m, float* __restrict__ v,
+                                              __nv_bfloat16* __restrict__ wb, size_t count, float lr, float b1,
+                                              float b2, float c1, float c2, float eps,
                                               const float* __restrict__ loss_part, int nloss, float denom,
                                               float* __restrict__ loss) {
   const size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x;
   if (i < count) {
-    float gi = part[i];
-    for (int c = 1; c < chunks; ++c) gi += part[size_t(c) * count + i];
-    g[i] = gi;
+    const float gi = g[i];
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
     const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
     m[i] = mi;
@@ -459,8 +438,6 @@ struct lb_mlp {
   __nv_bfloat16* wb = nullptr;
   float *phi = nullptr, *dY = nullptr, *partial = nullptr, *loss = nullptr;
   std::vector<float*> Z, H;                // per hidden layer [max_batch][width]; Z becomes dZ backwards
-  float* part = nullptr;                   // [max_chunks][nparam] weight gradients of row chunks
-  int max_chunks = 1;
   float* scale = nullptr;                  // mean[4], istd[4], std[4]
   long long steps = 0;
   std::string err;
@@ -507,9 +484,9 @@ cudaError_t forward(lb_mlp* net, const float* x, int n) {
   for (int l = 0; l < net->depth - 1; ++l) {
     const int fi = net->fan_in[l], fo = net->fan_out[l];
     const __nv_bfloat16* W = net->wb + net->w_off[l];
-    const dim3 grid((n + TM - 1) / TM, (fo + TN - 1) / TN);
+    const dim3 grid((n + TL - 1) / TL, (fo + TL - 1) / TL);
     const bool vec = words(in, 4, fi) && words(W, 2, fi);
-    (vec ? k_layer<true> : k_layer<false>)<<<grid, 256, 0, s>>>(n, fo, fi, in, W, net->w + net->b_off[l], net->Z[l],
+    (vec ? k_layer<true> : k_layer<false>)<<<grid, LTHREADS, 0, s>>>(n, fo, fi, in, W, net->w + net->b_off[l], net->Z[l],
                                                                 net->H[l]);
     in = net->H[l];
   }
@@ -519,7 +496,7 @@ cudaError_t forward(lb_mlp* net, const float* x, int n) {
 // The output layer (k_output): training on y, or the fields pred.
 cudaError_t output(lb_mlp* net, int n, const float* y, float* pred) {
   const int l = net->depth - 1;
-  k_output<<<nblk(n, 8), 256, 0, net->stream>>>(n, net->fan_in[l], net->H[l - 1], net->wb + net->w_off[l],
+  k_output<<<nblk(n, OUT_ROWS), 256, 0, net->stream>>>(n, net->fan_in[l], net->H[l - 1], net->wb + net->w_off[l],
                                                 net->w + net->b_off[l], net->scale, y, net->dY, net->Z[l - 1],
                                                 net->partial, pred);
   return cudaGetLastError();
@@ -566,12 +543,9 @@ lb_status lb_mlp_create(int n_plain, int n_fourier, int width, int depth, int ma
   if (e == cudaSuccess) e = alloc(n, &n->wb, n->nparam);
   if (e == cudaSuccess) e = alloc(n, &n->phi, size_t(max_batch) * n->nin);
   if (e == cudaSuccess) e = alloc(n, &n->dY, size_t(max_batch) * NOUT);
-  if (e == cudaSuccess) e = alloc(n, &n->partial, nblk(max_batch, 8));
+  if (e == cudaSuccess) e = alloc(n, &n->partial, nblk(max_batch, OUT_ROWS));
   if (e == cudaSuccess) e = alloc(n, &n->loss, 1);
   if (e == cudaSuccess) e = alloc(n, &n->scale, 3 * NOUT);
-  // row chunks of 256 for the weight gradients, as many as 64 MB of copies hold
-  n->max_chunks = int(std::min<size_t>((size_t(max_batch) + 255) / 256, std::max<size_t>(1, (size_t(64) << 20) / (4 * n->nparam))));
-  if (e == cudaSuccess) e = alloc(n, &n->part, n->max_chunks * n->nparam);
   n->Z.assign(depth - 1, nullptr);
   n->H.assign(depth - 1, nullptr);
   for (int l = 0; l < depth - 1 && e == cudaSuccess; ++l) {
@@ -662,9 +636,9 @@ lb_status lb_mlp_train_step(lb_mlp* n, const float* x, const float* y, int count
   for (int l = n->depth - 2; l > 0; --l) {
     const int fi = n->fan_in[l], fo = n->fan_out[l];
     const __nv_bfloat16* W = n->wb + n->w_off[l];
-    const dim3 grid((count + TM - 1) / TM, (fi + TN - 1) / TN);
+    const dim3 grid((count + TL - 1) / TL, (fi + TL - 1) / TL);
     const bool vec = words(n->Z[l], 4, fo) && words(W, 2, fi);
-    (vec ? k_layer_back<true> : k_layer_back<false>)<<<grid, 256, 0, s>>>(count, fo, fi, n->Z[l], W, n->Z[l - 1]);
+    (vec ? k_layer_back<true> : k_layer_back<false>)<<<grid, LTHREADS, 0, s>>>(count, fo, fi, n->Z[l], W, n->Z[l - 1]);
   }
   LB_MCUDA(n, cudaGetLastError());
   WeightJobs jobs;
@@ -676,22 +650,20 @@ lb_status lb_mlp_train_step(lb_mlp* n, const float* x, const float* y, int count
     J.fo = n->fan_out[l];
     J.dZ = l == n->depth - 1 ? n->dY : n->Z[l];
     J.in = l == 0 ? n->phi : n->H[l - 1];
-    J.vec = words(J.dZ, 4, J.fo) && words(J.in, 4, J.fi);
+    J.vec_z = words(J.dZ, 4, J.fo);
+    J.vec_in = words(J.in, 4, J.fi);
     J.tile0 = tiles;
     J.w_off = n->w_off[l];
     J.b_off = n->b_off[l];
-    tiles += ((J.fo + TM - 1) / TM) * ((J.fi + TN - 1) / TN);
+    tiles += ((J.fo + TG - 1) / TG) * ((J.fi + TG - 1) / TG + 1);
   }
-  int chunks = std::min(n->max_chunks, (count + 255) / 256);
-  const int chunk = ((count + chunks - 1) / chunks + TK - 1) / TK * TK;
-  chunks = (count + chunk - 1) / chunk;
-  k_weight_grads<<<dim3(tiles, chunks), 256, 0, s>>>(jobs, count, chunk, n->part, n->nparam);
+  k_weight_grads<<<unsigned(tiles), GTHREADS, 0, s>>>(jobs, count, n->g);
   LB_MCUDA(n, cudaGetLastError());
   ++n->steps;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.0f - std::pow(b1, float(n->steps)), c2 = 1.0f - std::pow(b2, float(n->steps));
-  k_adam<<<nblk(n->nparam), 256, 0, s>>>(n->w, n->g, n->part, chunks, n->m, n->v, n->wb, n->nparam, lr, b1, b2, c1,
-                                         c2, 1e-8f, n->partial, int(nblk(count, 8)), float(count * NOUT), n->loss);
+  k_adam<<<nblk(n->nparam), 256, 0, s>>>(n->w, n->g, n->m, n->v, n->wb, n->nparam, lr, b1, b2, c1, c2, 1e-8f,
+                                         n->partial, int(nblk(count, OUT_ROWS)), float(count * NOUT), n->loss);
   LB_MCUDA(n, cudaGetLastError());
   if (loss) {
     LB_MCUDA(n, cudaMemcpyAsync(loss, n->loss, sizeof(float), cudaMemcpyDeviceToHost, s));
