@@ -35,20 +35,18 @@ BYTES_PER_UPDATE = {"fp64": 2 * 41 * 8, "fp32": 2 * 41 * 4, "fp16_shifted": 2 * 
                     "bf16_shifted": 2 * 41 * 2}
 DTYPE = {"fp64": "f64", "fp32": "f32", "fp16_shifted": "f16 storage / f32 math",
          "bf16_shifted": "bf16 storage / f32 math"}
-PROFILE_FILE = os.path.join(ROOT, "profiles", "k_step_split_fp32_cyl64x4x256_b24.md")
-KERNEL_SOURCES = ["paper_1411_3133_gb300/csrc/collision.cuh", "paper_1411_3133_gb300/csrc/lbm_device.cuh",
-                  "paper_1411_3133_gb300/csrc/kernels.cuh",
-                  "paper_1411_3133_gb300/csrc/step_launch.cuh", "paper_1411_3133_gb300/csrc/step_f32.cu",
-                  "paper_1411_3133_gb300/csrc/lattice.cuh"]
+PROFILE_FILE = os.path.join(ROOT, "profiles", "k_step_fp32_cyl64x4x256_b24.md")
+BODY_SOURCES = [f"paper_1411_3133_gb300/csrc/{f}" for f in
+                ("collision.cuh", "lbm_device.cuh", "kernels.cuh", "lattice.cuh")]
+KERNEL_SOURCES = BODY_SOURCES + [f"paper_1411_3133_gb300/csrc/{f}" for f in
+                                 ("step_launch.cuh", "lanes.h", "step_f32.cu")]
 METRIC = "MLUPS and % of HBM roofline at 1 GB300"
 
 
 FP64_PROFILE_FILE = os.path.join(ROOT, "profiles", "k_step_fp64_cyl64x4x256_b24.md")
 # the FP64 step is the plain k_step; its instruction counts depend on the
 # kernel body alone
-FP64_KERNEL_SOURCES = ["paper_1411_3133_gb300/csrc/collision.cuh", "paper_1411_3133_gb300/csrc/lbm_device.cuh",
-                  "paper_1411_3133_gb300/csrc/kernels.cuh",
-                       "paper_1411_3133_gb300/csrc/step_f64.cu", "paper_1411_3133_gb300/csrc/lattice.cuh"]
+FP64_KERNEL_SOURCES = BODY_SOURCES + ["paper_1411_3133_gb300/csrc/step_f64.cu"]
 
 
 def kernel_source_hash(sources=None) -> str:
@@ -74,21 +72,18 @@ def profile_value(path, key, sources=None):
 
 
 def measured_traffic():
-    """DRAM bytes per launch of the FP32 split step (committed ncu summary)."""
+    """DRAM bytes per step of the FP32 sweep (committed ncu summary)."""
     return profile_value(PROFILE_FILE, "dram_bytes_per_launch")
 
 
 # ncu summaries of the other timed configurations: DRAM bytes of one whole
 # step (all its kernels), valid for the step sources of that storage type
-STEP_SOURCES = {p: ["paper_1411_3133_gb300/csrc/collision.cuh", "paper_1411_3133_gb300/csrc/lbm_device.cuh",
-                  "paper_1411_3133_gb300/csrc/kernels.cuh",
-                    "paper_1411_3133_gb300/csrc/step_launch.cuh", f"paper_1411_3133_gb300/csrc/step_{t}.cu",
-                    "paper_1411_3133_gb300/csrc/lattice.cuh"]
+STEP_SOURCES = {p: BODY_SOURCES + [f"paper_1411_3133_gb300/csrc/{f}" for f in
+                                   ("pair.cuh", "step_launch.cuh", "lanes.h", f"step_{t}.cu")]
                 for p, t in (("fp32", "f32"), ("fp16_shifted", "h16"), ("bf16_shifted", "b16"))}
-STEP_PROFILES = {("sweep", "fp16_shifted"): "k_step_split_fp16_cyl64x4x256_b24.md",
-                 ("ellipsoid", "fp16_shifted"): "k_step_list_fp16_ell64x4x256_b24.md",
-                 ("ellipsoid", "fp32"): "k_step_list_fp32_ell64x4x256_b24.md",
-                 ("mixed", "fp32"): "k_step_list_fp32_mixed128.md"}
+STEP_PROFILES = {("sweep", "fp16_shifted"): "k_step_pair_fp16_cyl64x4x256_b24.md",
+                 ("ellipsoid", "fp16_shifted"): "k_step_pair_fp16_ell64x4x256_b24.md",
+                 ("ellipsoid", "fp32"): "k_step_fp32_ell64x4x256_b24.md"}
 
 
 def step_traffic(workload, precision):
@@ -100,9 +95,8 @@ def step_traffic(workload, precision):
 
 
 def measured_fp32_flops():
-    """FP32 flops per lattice update of the region-split FP32 step, both
-    kernels (ncu FFMA, FADD, FMUL thread-instruction counts, committed
-    summary)."""
+    """FP32 flops per lattice update of the FP32 step (ncu FFMA, FADD, FMUL
+    thread-instruction counts, committed summary)."""
     return profile_value(PROFILE_FILE, "fp32_flops_per_update")
 
 
@@ -283,7 +277,6 @@ def timed_windows(runner, stream, steps: int, min_seconds: float, min_windows: i
 class SweepRunner:
     """24 instances of the 64 x 4 x 256 cylinder in one context (k_step)."""
     profiled = True
-    launches_per_step = 1
 
     def __init__(self, args, L, rank):
         self.args, self.L = args, L
@@ -304,18 +297,10 @@ class SweepRunner:
         self.ctx.lb_init(params)
         self.cells = wl.batch * wl.ncells
         self.stream = self.ctx.stream
-        if args.step_kernel == "auto":      # the library's automatic choice for this workload
-            args.step_kernel = "plain" if args.precision == "fp64" else "split"
-        # 2-byte storage: the split kernels that keep the block's row in shared
-        # memory (blocks within one i_r layer: nt n3 a multiple of the block)
-        rowsm = "_rowsm" if (args.precision.endswith("_shifted")
-                             and (wl.ntheta * wl.n3) % args.threads == 0) else ""
-        self.kernel = {"tma": "k_step_tma<KCYL,256>",
-                       "split": f"k_step_bulk{rowsm}<{args.precision},KCYL> + k_step_edge{rowsm} "
-                                f"({args.threads} threads)"}.get(
-            args.step_kernel, f"k_step<{args.precision},KCYL> ({args.threads} threads)")
-        self.profiled = args.precision == "fp32" and args.step_kernel == "split"
-        self.launches_per_step = 2 if args.step_kernel == "split" else 1
+        self.kernel = step_kernel_name(args, "KCYL")
+        self.profiled = args.precision == "fp32" and args.step_kernel != "tma"
+        self.launches_per_step = 1 if args.step_kernel == "tma" else step_launches([wl] * wl.batch, args.precision,
+                                                                                   args.steps)
 
     def warmup(self, n):
         self.ctx.lb_step(n)
@@ -348,7 +333,8 @@ class SweepRunner:
                             f"eta=0.975, {wl.batch} instances (12 De in 25..60 x tau 0.55/0.6), "
                             f"D3Q41, {wl.precision}",
                 "cells_per_instance": wl.ncells, "instances": wl.batch, "precision": wl.precision,
-                "l2": f"inputs larger than L2: state {2 * self.state_bytes / 1e6:.0f} MB, no flush"}
+                "l2": f"inputs larger than L2: state {2 * self.state_bytes / 1e6:.0f} MB, no flush; the library takes "
+                      "the instances in groups that fit L2 through a call's steps"}
 
     def extra(self):
         return {}
@@ -382,12 +368,9 @@ class EllipsoidRunner(SweepRunner):
         self.ctx.lb_init(params)
         self.cells = 24 * wl.ncells
         self.stream = self.ctx.stream
-        if args.step_kernel == "auto":
-            args.step_kernel = "plain" if args.precision == "fp64" else "tiled"
-        self.kernel = {"tiled": f"k_step_list<{args.precision},KELL> interior + wall tiles ({args.threads} threads)"
-                       }.get(args.step_kernel, f"k_step<{args.precision},KELL> ({args.threads} threads)")
+        self.kernel = step_kernel_name(args, "KELL")
         self.profiled = False
-        self.launches_per_step = work_lists([wl] * 24) if args.step_kernel == "tiled" else 1
+        self.launches_per_step = step_launches([wl] * 24, args.precision, args.steps)
 
     def config(self):
         wl = self.wl
@@ -395,15 +378,15 @@ class EllipsoidRunner(SweepRunner):
                             f"{wl.nr}x{wl.ntheta}x{wl.n3}, walls on r and phi, 24 instances (De 20..150), "
                             f"D3Q41, {self.args.precision}",
                 "cells_per_instance": wl.ncells, "instances": 24, "precision": self.args.precision,
-                "l2": f"inputs larger than L2: state {2 * self.state_bytes / 1e6:.0f} MB, no flush"}
+                "l2": f"inputs larger than L2: state {2 * self.state_bytes / 1e6:.0f} MB, no flush; the library takes "
+                      "the instances in groups that fit L2 through a call's steps"}
 
 
 def work_lists(channels):
-    """Work-list launches of one tiled or batch step over `channels` (objects
-    with metric, nr, n3, periodic3 and wall): per metric kind the interior
-    tiles and each non-empty wall-node class the library builds -- nodes
-    near an r-wall only, near an x3-wall only, and the rest (corners and
-    equilibrium walls)."""
+    """Classes of nodes that the gather tells apart in `channels` (objects with
+    metric, nr, n3, periodic3 and wall): per metric kind the interior and each
+    non-empty class of wall nodes -- near an r-wall only, near an x3-wall only,
+    and the rest (corners and equilibrium walls)."""
     kinds = {}
     for ch in channels:
         lists = kinds.setdefault(ch.metric, set())
@@ -419,11 +402,54 @@ def work_lists(channels):
     return sum(len(v) for v in kinds.values())
 
 
+def step_kernel_name(args, kind):
+    """The kernel a context's step launches."""
+    if args.step_kernel == "tma":
+        return f"k_step_tma<{kind},256>"
+    pair = "_pair" if args.precision.endswith("_shifted") else ""
+    return f"k_step{pair}<{args.precision},{kind}> ({args.threads} threads)"
+
+
+def step_launches(channels, precision, steps, list_max=None):
+    """Kernel launches per step of a call of `steps` steps over `channels`
+    (objects with metric, ncells and n3), in the chunks the library takes them in
+    (csrc/lanes.h): one launch a step and chunk. list_max: a batch, whose
+    instances are grouped by metric (2-byte storage: and parity of n3), at most
+    list_max to a launch; None: one context."""
+    two_byte = precision.endswith("_shifted")
+    if list_max is None:
+        groups = [list(channels)]
+    else:
+        keyed = {}
+        for c in channels:
+            keyed.setdefault((c.metric, c.n3 % 2 if two_byte else 0), []).append(c)
+        groups = list(keyed.values())
+    flat = sum(-(-len(g) // (list_max or len(g))) for g in groups)
+    if steps < 4:
+        return flat
+    hold, per_node = 90 << 20, BYTES_PER_UPDATE[precision]
+    target = min(hold // 4, sum(c.ncells * per_node for g in groups for c in g) // 4)
+    chunks = 0
+    for g in groups:
+        i = 0
+        while i < len(g):
+            b, n, k = g[i].ncells * per_node, g[i].ncells, 1
+            i += 1
+            while i < len(g) and (list_max is None or k < list_max):
+                more = b + g[i].ncells * per_node
+                if more > target and (n >= 60000 or more > hold // 2):
+                    break
+                b, n, k, i = more, n + g[i].ncells, k + 1, i + 1
+            if b > hold // 2:
+                return flat
+            chunks += 1
+    return chunks if chunks > 1 else flat
+
+
 class MixedRunner:
     """128 channels of mixed metric and size (cylinders and double-curved
     channels, N_r in {32, 48, 64}, N_3 in 128..512, De in 20..150) in one
-    lb_batch: per metric kind and step, one k_step_list launch over the
-    interior tiles and one per wall-node class; autotuned."""
+    lb_batch: work-list launches over groups of the instances; autotuned."""
     profiled = False
 
     def __init__(self, args, L, rank):
@@ -431,12 +457,13 @@ class MixedRunner:
         from paper_1411_3133_gb300.workloads import mixed_batch
         self.args, self.L = args, L
         self.insts = mixed_batch(seed=rank_seed(20241111, rank))
-        self.launches_per_step = work_lists(self.insts)
+        self.launches_per_step = step_launches(self.insts, args.precision, args.steps, 16)
         self.ctxs, self.batch = mixed_contexts(self.insts, args.precision)
         self.batch.lb_batch_set_option(L.LB_OPT_USE_GRAPH, 1)
         self.cells = self.batch.lb_batch_nodes()
         self.stream = self.ctxs[0].stream
-        self.kernel = f"k_step_list<{args.precision},KCYL|KELL>"
+        pair = "_pair" if args.precision.endswith("_shifted") else ""
+        self.kernel = f"k_step{pair}_list<{args.precision},KCYL|KELL>"
         self.tune = None
 
     def warmup(self, n):
@@ -475,7 +502,8 @@ class MixedRunner:
                             "{32,48,64} x 4 x N_3 in 128..512, De in 20..150, tau 0.55, D3Q41, "
                             f"{self.args.precision}, one lb_batch",
                 "nodes": self.cells, "instances": len(self.insts), "precision": self.args.precision,
-                "l2": f"inputs larger than L2: state {2 * self.state_bytes / 1e6:.0f} MB, no flush"}
+                "l2": f"inputs larger than L2: state {2 * self.state_bytes / 1e6:.0f} MB, no flush; the library takes "
+                      "the instances in groups that fit L2 through a call's steps"}
 
     def extra(self):
         best, trials = self.tune
@@ -579,7 +607,7 @@ def main():
         roofline["alu"] = {"achieved": round(alu, 3), "peak": round(alu_peak, 3), "unit": "TFLOP/s",
                            "frac": round(alu / alu_peak, 4), "fp32_flops_per_update": fpu32,
                            "peak_source": "measured (lb_fma_peak, FP32 FMA chains on this GPU)"}
-    fpu = measured_fp64_flops() if (args.precision == "fp64" and args.step_kernel == "plain"
+    fpu = measured_fp64_flops() if (args.precision == "fp64" and args.step_kernel != "tma"
                                     and args.workload == "sweep") else None
     if fpu is not None:
         # the FP64 step is bound by the FP64 units: report it against the
