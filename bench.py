@@ -412,7 +412,7 @@ def step_kernel_name(args, kind):
 
 def step_launches(channels, precision, steps, list_max=None):
     """Kernel launches per step of a call of `steps` steps over `channels`
-    (objects with metric, ncells and n3), in the chunks the library takes them in
+    (objects with metric, ncells, nr, n3 and periodic3), in the chunks the library takes them in
     (csrc/lanes.h): one launch a step and chunk. list_max: a batch, whose
     instances are grouped by metric (2-byte storage: and parity of n3), at most
     list_max to a launch; None: one context."""
@@ -427,16 +427,20 @@ def step_launches(channels, precision, steps, list_max=None):
     flat = sum(-(-len(g) // (list_max or len(g))) for g in groups)
     if steps < 4:
         return flat
-    hold, per_node = 90 << 20, BYTES_PER_UPDATE[precision]
-    target = min(hold // 4, sum(c.ncells * per_node for g in groups for c in g) // 4)
+    def held(c):  # two buffers and the 2-byte storage's stream table
+        rows3 = 1 if c.periodic3 and c.metric != "ellipsoidal" else (c.n3 + 1) // 2
+        return c.ncells * BYTES_PER_UPDATE[precision] + (26 * 16 * c.nr * rows3 if two_byte else 0)
+
+    hold = 90 << 20
+    target = min(hold // 4, sum(held(c) for g in groups for c in g) // 4)
     chunks = 0
     for g in groups:
         i = 0
         while i < len(g):
-            b, n, k = g[i].ncells * per_node, g[i].ncells, 1
+            b, n, k = held(g[i]), g[i].ncells, 1
             i += 1
             while i < len(g) and (list_max is None or k < list_max):
-                more = b + g[i].ncells * per_node
+                more = b + held(g[i])
                 if more > target and (n >= 60000 or more > hold // 2):
                     break
                 b, n, k, i = more, n + g[i].ncells, k + 1, i + 1

@@ -501,7 +501,9 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
       tensor_map_bytes() <= sizeof(c->tmap[0]))
     c->tma_ok = make_state_tensor_map(c->tmap[0], static_cast<const float*>(c->f[0]), d) == cudaSuccess &&
                 make_state_tensor_map(c->tmap[1], static_cast<const float*>(c->f[1]), d) == cudaSuccess;
-  c->plan = plan_lanes(std::vector<LaneInst>(size_t(batch), {0, c->ncell, 2 * Q * c->ncell * c->elem_bytes}), batch);
+  c->step_bytes = 2 * Q * c->ncell * c->elem_bytes;
+  if (c->st_tab) c->step_bytes += 2 * ST_K * size_t(geom->nr) * size_t(d.st_rows3) * sizeof(float4);
+  c->plan = plan_lanes(std::vector<LaneInst>(size_t(batch), {0, c->ncell, c->step_bytes}), batch);
   *out = c;
   return LB_OK;
 }

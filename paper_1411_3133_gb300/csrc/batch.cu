@@ -183,7 +183,7 @@ lb_status build(lb_batch* b) {
     first.push_back(int(inst.size()));
     for (const lb_ctx* c : b->m)
       if (variant(c) == b->g[gi].key)
-        inst.insert(inst.end(), size_t(c->batch), {int(gi), c->ncell, 2 * Q * c->ncell * c->elem_bytes});
+        inst.insert(inst.end(), size_t(c->batch), {int(gi), c->ncell, c->step_bytes});
     for (int i = 0; i < b->g[gi].ninst; i += LIST_MAX)
       b->flat.push_back({int(gi), i, std::min(LIST_MAX, b->g[gi].ninst - i), int(b->flat.size()) % LANES});
   }

@@ -67,6 +67,7 @@ struct lb_ctx {
   int graph_kernel = -1;             // captured graph: 1 the half-force variant, 2 TMA
   int step_kernel = 0;               // LB_OPT_STEP_KERNEL
   bool any_shift = false;            // an instance uses the half-force velocity (old_forcing 2)
+  size_t step_bytes = 0;             // what an instance's steps use: two buffers and its stream table
   std::vector<lbgm::LaneChunk> plan; // order of the instances in a call of several steps
   lbgm::LaneStreams lanes;
   bool tma_ok = false;               // tensor maps built for both buffers

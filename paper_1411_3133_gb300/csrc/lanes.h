@@ -10,7 +10,10 @@
 // cylinder FP32 19.5 / 22.7, FP16 23.0 / 29.0; four-wall ellipsoid FP32 18.1 /
 // 22.7, FP16 20.3 / 25.3. The line: what the streams hold at once stays below
 // 90 MB (four streams of 43 MB fall back to 19.8), and a launch is long enough
-// to be issued while the others run (about 2 us, 60 000 nodes).
+// to be issued while the others run (about 2 us, 60 000 nodes). The 2-byte
+// storage's stream table counts as held: with the state alone the ellipsoid ran
+// in groups of two whose tables (3.4 MB an instance) went to HBM, 68.7 us a step
+// of the 24 in FP16 against 63.8.
 #pragma once
 
 #include <algorithm>
@@ -27,7 +30,7 @@ struct LaneChunk {
 };
 
 // One instance: its group (only instances of one group share a launch), nodes
-// and the bytes of its two buffers.
+// and the bytes its steps use.
 struct LaneInst {
   int group;
   size_t nodes, bytes;
