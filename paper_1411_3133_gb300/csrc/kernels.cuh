@@ -10,8 +10,8 @@ namespace lbgm {
 // Programmatic dependent launch between the steps of a chain (launch_chained):
 // a step's blocks may start while the step before still runs -- they find
 // their nodes, source-table rows and geometry -- and wait for its end and its
-// memory before they touch the state. Without the launch attribute both are
-// no-ops.
+// memory before they touch the state (gather_table says how they may read it).
+// Without the launch attribute both are no-ops.
 __device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -23,7 +23,7 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 // density and metric (Sec. III). FP32 and FP64 storage (2-byte storage:
 // pair.cuh).
 template <typename Real, int K>
-__device__ __forceinline__ void step_node(const Real* __restrict__ fin, Real* __restrict__ fout,
+__device__ __forceinline__ void step_node(const Real* fin, Real* __restrict__ fout,
                                           const GeoDev<Real>& geo, const InstParams<Real>& ip, const Dims& d,
                                           const CellPos& p, int* __restrict__ flag) {
   Real f[Q];
@@ -76,7 +76,7 @@ struct KBounds<double, K> {
 // the instance's block base is uniform across the thread block.
 template <typename Real, int K>
 __global__ void __launch_bounds__(KBounds<Real, K>::maxt, KBounds<Real, K>::minb)
-    k_step(const Real* __restrict__ fin, Real* __restrict__ fout, GeoDev<Real> geo,
+    k_step(const Real* fin, Real* __restrict__ fout, GeoDev<Real> geo,
            const InstParams<Real>* __restrict__ inst, Dims d, int* __restrict__ flag) {
   chain_start();
   const uint32_t cell = blockIdx.x * blockDim.x + threadIdx.x;

@@ -337,8 +337,7 @@ __device__ __forceinline__ bool near_wall(const CellPos& p, const Dims& d) {
 // 32-bit: an instance block holds fewer than 2^32 bytes (checked when the
 // context is created).
 template <int K, class S, class Fn>
-__device__ __forceinline__ void for_each_source_far(const S* __restrict__ fin, const CellPos& p, const Dims& d,
-                                                    Fn&& fn) {
+__device__ __forceinline__ void for_each_source_far(const S* fin, const CellPos& p, const Dims& d, Fn&& fn) {
   const uint32_t N = uint32_t(d.ncell);
   Neighbours nb;
   make_neighbours(p, d, nb);
@@ -506,19 +505,24 @@ __device__ __forceinline__ void gather(const S* __restrict__ fin, const float* r
 // every periodic wrap. One code path for all of them keeps the step kernels
 // small: with a compile-time variant per wall layer they were bound by
 // instruction fetch (7 to 19 cycles per issue at the walls).
+//
+// The state is read by ordinary loads, through pointers that promise nothing:
+// a chained step (launch_chained) starts while the step that writes its input
+// still runs, so its input is not read-only for the kernel's lifetime as the
+// non-coherent path needs (__ldg, const __restrict__ arguments), and only
+// ordinary loads are ordered after chain_wait.
 template <class S>
-__device__ __forceinline__ void gather_table(const S* __restrict__ fin, const CellPos& p, const Dims& d,
-                                             S (&f)[Q]) {
+__device__ __forceinline__ void gather_table(const S* fin, const CellPos& p, const Dims& d, S (&f)[Q]) {
   const int key = (axis_class(p.ir, d.nr) * d.src_nt + axis_class(p.it, d.nt)) * d.src_n3 + axis_class(p.i3, d.n3);
   const int4* __restrict__ row = d.src + key * SRC_ROW;
   static_for<0, SRC_ROW>([&](auto J_) {
     constexpr int J = decltype(J_)::value;
     const int4 o = __ldg(row + J);
-    f[4 * J] = __ldg(fin + uint32_t(p.cell + o.x));
+    f[4 * J] = fin[uint32_t(p.cell + o.x)];
     if constexpr (4 * J + 1 < Q) {
-      f[4 * J + 1] = __ldg(fin + uint32_t(p.cell + o.y));
-      f[4 * J + 2] = __ldg(fin + uint32_t(p.cell + o.z));
-      f[4 * J + 3] = __ldg(fin + uint32_t(p.cell + o.w));
+      f[4 * J + 1] = fin[uint32_t(p.cell + o.y)];
+      f[4 * J + 2] = fin[uint32_t(p.cell + o.z)];
+      f[4 * J + 3] = fin[uint32_t(p.cell + o.w)];
     }
   });
 }
@@ -527,12 +531,12 @@ __device__ __forceinline__ void gather_table(const S* __restrict__ fin, const Ce
 // from the node's own neighbours, computed; a warp that holds any other node
 // reads the source table for all its nodes, so it runs one of the two paths.
 template <class S>
-__device__ __forceinline__ void gather_step(const S* __restrict__ fin, const CellPos& p, const Dims& d, S (&f)[Q]) {
+__device__ __forceinline__ void gather_step(const S* fin, const CellPos& p, const Dims& d, S (&f)[Q]) {
   if (__any_sync(__activemask(), near_wall(p, d))) {
     gather_table(fin, p, d, f);
   } else {
-    f[0] = __ldg(fin + uint32_t(p.cell));
-    for_each_source_far<KFLAT>(fin, p, d, [&](auto L_, const S* src, int, int) { f[decltype(L_)::value] = __ldg(src); });
+    f[0] = fin[uint32_t(p.cell)];
+    for_each_source_far<KFLAT>(fin, p, d, [&](auto L_, const S* src, int, int) { f[decltype(L_)::value] = *src; });
   }
 }
 

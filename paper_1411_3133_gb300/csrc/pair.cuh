@@ -63,9 +63,9 @@ struct Pack2<__nv_bfloat16> {
   }
 };
 
-__device__ __forceinline__ uint32_t ld16(const void* p) {
-  return uint32_t(__ldg(static_cast<const unsigned short*>(p)));
-}
+// State reads: ordinary loads (gather_table).
+__device__ __forceinline__ uint32_t ld16(const void* p) { return *static_cast<const unsigned short*>(p); }
+__device__ __forceinline__ uint32_t ld32(const void* p) { return *static_cast<const uint32_t*>(p); }
 __device__ __forceinline__ uint32_t join16(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x5410); }
 
 // The gathered pair as the shell functions see it: reads unpack, results go
@@ -121,8 +121,8 @@ __device__ __forceinline__ void copy_async_wait() {
 // ---------------------------------------------------------------------------
 // Streamed values of the pair far from every wall.
 template <class S, bool EVEN>
-__device__ __forceinline__ void gather_pair_far(const S* __restrict__ fin, const CellPos& p, bool second,
-                                                const Dims& d, uint32_t (&raw)[Q]) {
+__device__ __forceinline__ void gather_pair_far(const S* fin, const CellPos& p, bool second, const Dims& d,
+                                                uint32_t (&raw)[Q]) {
   const uint32_t N = uint32_t(d.ncell);
   int rrow[7], tcol[7], zc[8];
 #pragma unroll
@@ -135,7 +135,7 @@ __device__ __forceinline__ void gather_pair_far(const S* __restrict__ fin, const
     const int z = p.i3 + k;
     zc[k + 3] = d.periodic3 ? wrap_small(z, d.n3) : z;
   }
-  raw[0] = EVEN ? __ldg(reinterpret_cast<const uint32_t*>(fin + p.cell))
+  raw[0] = EVEN ? ld32(fin + p.cell)
                 : join16(ld16(fin + p.cell), ld16(fin + p.cell + (second ? 1 : 0)));
   static_for<0, 2 * NPAIR>([&](auto I_) {
     constexpr int I = decltype(I_)::value, P = I / 2, sg = I % 2 ? -1 : 1;
@@ -143,7 +143,7 @@ __device__ __forceinline__ void gather_pair_far(const S* __restrict__ fin, const
     constexpr int cx = sg * C::x, cy = sg * C::y, cz = sg * C::z, L = I + 1;
     const uint32_t row = uint32_t(L) * N + uint32_t((rrow[cx + 3] + tcol[cy + 3]) * d.n3);
     if constexpr (cz == 0 && EVEN) {
-      raw[L] = __ldg(reinterpret_cast<const uint32_t*>(fin + (row + uint32_t(p.i3))));
+      raw[L] = ld32(fin + (row + uint32_t(p.i3)));
     } else {
       const int z0 = zc[3 - cz], z1 = EVEN || second ? zc[4 - cz] : z0;
       raw[L] = join16(ld16(fin + (row + uint32_t(z0))), ld16(fin + (row + uint32_t(z1))));
@@ -154,8 +154,8 @@ __device__ __forceinline__ void gather_pair_far(const S* __restrict__ fin, const
 // Streamed values of the pair through the source table (gather_table), each
 // node by its own key.
 template <class S>
-__device__ __forceinline__ void gather_pair_table(const S* __restrict__ fin, const CellPos& p, bool second,
-                                                  const Dims& d, uint32_t (&raw)[Q]) {
+__device__ __forceinline__ void gather_pair_table(const S* fin, const CellPos& p, bool second, const Dims& d,
+                                                  uint32_t (&raw)[Q]) {
   const int key = (axis_class(p.ir, d.nr) * d.src_nt + axis_class(p.it, d.nt)) * d.src_n3;
   const int one = second ? 1 : 0;
   const int4* __restrict__ r0 = d.src + (key + axis_class(p.i3, d.n3)) * SRC_ROW;
@@ -212,7 +212,7 @@ __device__ __forceinline__ NodeGeo<PF2, K> load_geo_pair(const GeoDev<float>& g,
 // (not ROW1) the block's warps lie in one (i_r, chunk) and stage its rows
 // together.
 template <typename S, int K, bool EVEN, bool ROW1>
-__device__ __forceinline__ void step_pair(const S* __restrict__ fin, S* __restrict__ fout, const float* ref,
+__device__ __forceinline__ void step_pair(const S* fin, S* __restrict__ fout, const float* ref,
                                           const float4* __restrict__ st, const GeoDev<float>& geo,
                                           const InstParams<float>* __restrict__ inst, const Dims& d, uint32_t wrp,
                                           bool active, bool shared, float4* sm, int* __restrict__ flag) {
@@ -315,7 +315,7 @@ __device__ __forceinline__ void step_pair(const S* __restrict__ fin, S* __restri
 // Uniform batch: fin, fout are whole states, grid row y is instance y.
 template <typename S, int K, bool EVEN, bool ROW1>
 __global__ void __launch_bounds__(LBGM_PAIR_MAXT, LBGM_PAIR_MINB)
-    k_step_pair(const S* __restrict__ fin, S* __restrict__ fout, GeoDev<float> geo,
+    k_step_pair(const S* fin, S* __restrict__ fout, GeoDev<float> geo,
                 const InstParams<float>* __restrict__ inst, Dims d, int* __restrict__ flag, uint32_t warps,
                 int shared) {
   extern __shared__ float4 sm[];
