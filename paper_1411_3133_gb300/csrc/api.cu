@@ -276,6 +276,52 @@ lb_status launch_steps_chunked(lb_ctx* c, long long n) {
   return LB_OK;
 }
 
+// n > 0 steps without a check: in groups where that pays (lanes.h), else one launch a step.
+lb_status advance(lb_ctx* c, long long n) {
+  lb_status s;
+  if (n >= LANE_MIN_STEPS && !c->plan.empty() && !use_tma(c)) return launch_steps_chunked(c, n);
+  // chained launches (launch_chained) are faster than replaying a graph of
+  // them; the TMA kernel and the half-force variant have none
+  if (c->use_graph && c->check_every == 0 && n >= 3 && (use_tma(c) || c->any_shift)) {
+    if (c->cur != 0) {  // the captured pair starts from buffer 0
+      s = launch_step_once(c);
+      if (s != LB_OK) return s;
+      ++c->step;
+      --n;
+    }
+    // the captured kernels depend on the resolved step kernel and on whether
+    // an instance uses the half-force variant (both can change with lb_init)
+    const int gk = use_tma(c) ? 2 : 1;
+    if (!c->graph || c->graph_threads != c->block_threads || c->graph_kernel != gk) {
+      if (c->graph) cudaGraphExecDestroy(c->graph);
+      c->graph = nullptr;
+      cudaGraph_t g = nullptr;
+      LB_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
+      lb_status s1 = launch_step_once(c);
+      lb_status s2 = s1 == LB_OK ? launch_step_once(c) : s1;
+      cudaError_t e = cudaStreamEndCapture(c->stream, &g);
+      if (s2 != LB_OK) return s2;
+      if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamEndCapture");
+      e = cudaGraphInstantiate(&c->graph, g, 0);
+      cudaGraphDestroy(g);
+      if (e != cudaSuccess) return cuda_fail(c, e, "cudaGraphInstantiate");
+      c->graph_threads = c->block_threads;
+      c->graph_kernel = gk;
+    }
+    for (long long i = 0; i + 1 < n; i += 2) {
+      LB_CUDA(c, cudaGraphLaunch(c->graph, c->stream));
+      c->step += 2;
+    }
+    n &= 1;
+  }
+  for (long long i = 0; i < n; ++i) {
+    s = launch_step_once(c);
+    if (s != LB_OK) return s;
+    ++c->step;
+  }
+  return LB_OK;
+}
+
 lb_status check_flag(lb_ctx* c) {
   int h = 0;
   LB_CUDA(c, cudaMemcpyAsync(&h, c->flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -586,58 +632,11 @@ lb_status lb_step(lb_ctx* c, long long n) {
   lb_status s;
   if (!usable(c, &s)) return s;
   if (n < 0) return fail(c, LB_ERR_ARG, "need n >= 0");
-  while (n >= LANE_MIN_STEPS && !c->plan.empty() && !use_tma(c)) {
-    const long long to_check = c->check_every > 0 ? c->check_every - c->step % c->check_every : n;
-    const long long k = std::min(n, to_check);
-    if (k < LANE_MIN_STEPS) break;
-    s = launch_steps_chunked(c, k);
-    if (s != LB_OK) return s;
+  while (n > 0) {  // from check to check
+    const long long k = c->check_every > 0 ? std::min(n, c->check_every - c->step % c->check_every) : n;
+    if ((s = advance(c, k)) != LB_OK) return s;
     n -= k;
     if (c->check_every > 0 && c->step % c->check_every == 0 && (s = check_flag(c)) != LB_OK) return s;
-  }
-  if (n == 0) return LB_OK;
-  // chained launches (launch_chained) are faster than replaying a graph of
-  // them; the TMA kernel and the half-force variant have none
-  if (c->use_graph && c->check_every == 0 && n >= 3 && (use_tma(c) || c->any_shift)) {
-    if (c->cur != 0) {  // the captured pair starts from buffer 0
-      s = launch_step_once(c);
-      if (s != LB_OK) return s;
-      ++c->step;
-      --n;
-    }
-    // the captured kernels depend on the resolved step kernel and on whether
-    // an instance uses the half-force variant (both can change with lb_init)
-    const int gk = use_tma(c) ? 2 : 1;
-    if (!c->graph || c->graph_threads != c->block_threads || c->graph_kernel != gk) {
-      if (c->graph) cudaGraphExecDestroy(c->graph);
-      c->graph = nullptr;
-      cudaGraph_t g = nullptr;
-      LB_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-      lb_status s1 = launch_step_once(c);
-      lb_status s2 = s1 == LB_OK ? launch_step_once(c) : s1;
-      cudaError_t e = cudaStreamEndCapture(c->stream, &g);
-      if (s2 != LB_OK) return s2;
-      if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamEndCapture");
-      e = cudaGraphInstantiate(&c->graph, g, 0);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) return cuda_fail(c, e, "cudaGraphInstantiate");
-      c->graph_threads = c->block_threads;
-      c->graph_kernel = gk;
-    }
-    for (long long i = 0; i + 1 < n; i += 2) {
-      LB_CUDA(c, cudaGraphLaunch(c->graph, c->stream));
-      c->step += 2;
-    }
-    n &= 1;
-  }
-  for (long long i = 0; i < n; ++i) {
-    s = launch_step_once(c);
-    if (s != LB_OK) return s;
-    ++c->step;
-    if (c->check_every > 0 && (c->step % c->check_every) == 0) {
-      s = check_flag(c);
-      if (s != LB_OK) return s;
-    }
   }
   return LB_OK;
 }

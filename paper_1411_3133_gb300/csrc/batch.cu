@@ -288,23 +288,13 @@ lb_status ready(lb_batch* b) {
   return LB_OK;
 }
 
-// n steps; trials of the autotuner pass graph = false.
-lb_status run(lb_batch* b, long long n, bool graph) {
-  if (!records_current(b)) {
-    lb_status s = build(b);
-    if (s != LB_OK) return s;
+// n > 0 steps without a check: in groups where that pays (lanes.h), else a step at a time.
+lb_status advance(lb_batch* b, long long n, bool graph) {
+  if (n >= LANE_MIN_STEPS && !b->plan.empty()) {
+    lb_status s = steps(b, n);
+    if (s == LB_OK) advance_members(b, n);
+    return s;
   }
-  while (n >= LANE_MIN_STEPS && !b->plan.empty()) {
-    const long long to_check = b->check_every > 0 ? b->check_every - b->step % b->check_every : n;
-    const long long k = std::min(n, to_check);
-    if (k < LANE_MIN_STEPS) break;
-    lb_status s = steps(b, k);
-    if (s != LB_OK) return s;
-    advance_members(b, k);
-    n -= k;
-    if (b->check_every > 0 && b->step % b->check_every == 0 && (s = check_members(b)) != LB_OK) return s;
-  }
-  if (n == 0) return LB_OK;
   if (graph && b->use_graph && b->check_every == 0 && n >= 3 && b->flat.size() > 1) {
     if (b->parity != 0) {  // the captured pair starts at parity 0
       lb_status s = step_once(b);
@@ -338,10 +328,19 @@ lb_status run(lb_batch* b, long long n, bool graph) {
     lb_status s = step_once(b);
     if (s != LB_OK) return s;
     advance_members(b, 1);
-    if (b->check_every > 0 && (b->step % b->check_every) == 0) {
-      s = check_members(b);
-      if (s != LB_OK) return s;
-    }
+  }
+  return LB_OK;
+}
+
+// n steps; trials of the autotuner pass graph = false.
+lb_status run(lb_batch* b, long long n, bool graph) {
+  lb_status s;
+  if (!records_current(b) && (s = build(b)) != LB_OK) return s;
+  while (n > 0) {  // from check to check
+    const long long k = b->check_every > 0 ? std::min(n, b->check_every - b->step % b->check_every) : n;
+    if ((s = advance(b, k, graph)) != LB_OK) return s;
+    n -= k;
+    if (b->check_every > 0 && b->step % b->check_every == 0 && (s = check_members(b)) != LB_OK) return s;
   }
   return LB_OK;
 }

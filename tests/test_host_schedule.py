@@ -1,0 +1,62 @@
+"""Which launches a call makes, and on which streams: the host side over a
+stand-in runtime (host_library.py)."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from host_library import Host, build_host_library, launches, take_log  # noqa: F401
+from paper_1411_3133_gb300 import lbgm as L
+
+SWEEP = ("cylindrical", (64, 4, 256), 5, "fp32")  # five instances of 21.5 MB: groups of one
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return build_host_library(str(tmp_path_factory.mktemp("host")))
+
+
+class Batch:
+    def __init__(self, lib, members):
+        self.lib, self.members, self.h = lib, members, ctypes.c_void_p()
+        arr = (ctypes.c_void_p * len(members))(*[m.ctx for m in members])
+        assert lib.lb_batch_create(arr, len(members), ctypes.byref(self.h)) == L.LB_OK
+
+    def option(self, opt, value):
+        assert self.lib.lb_batch_set_option(self.h, opt, value) == L.LB_OK
+
+    def step(self, n):
+        assert self.lib.lb_batch_step(self.h, n) == L.LB_OK, self.lib.lb_batch_last_error(self.h)
+
+    def close(self):
+        self.lib.lb_batch_destroy(self.h)
+
+
+def _whole(log, instances):
+    """Launches that take every instance at once (the steps outside groups)."""
+    return sum(x["count"] == instances for x in log)
+
+
+@pytest.mark.parametrize("batch", [False, True], ids=["context", "batch"])
+@pytest.mark.parametrize("precision", ["fp32", "fp16_shifted"])
+def test_checks_do_not_end_the_groups(lib, precision, batch):
+    """With a check every 100 steps, a call from step 97 takes 3 steps one by
+    one and the others in groups."""
+    c = Host(lib, *SWEEP[:3], precision)
+    b = Batch(lib, [c]) if batch else None
+    for on in filter(None, (c, b)):
+        on.option(L.LB_OPT_CHECK_EVERY, 100)
+    take = b.step if batch else c.step
+    take(97)
+    assert _whole(launches(lib), 5) == 0
+    take(203)
+    log = launches(lib)
+    assert _whole(log, 5) == 3
+    assert sum(x["count"] for x in log) == 203 * 5
+    assert np.array_equal(c.counts(), [300] * 5)
+    take(2)
+    take(1)
+    assert _whole(launches(lib), 5) == 3 and np.array_equal(c.counts(), [303] * 5)
+    if batch:
+        b.close()
+    c.close()
