@@ -398,7 +398,9 @@ lb_status lb_fma_peak(lb_precision precision, void* cuda_stream, double* flops_p
  * each configuration -- block_threads in {64, 96, 128} (FP64: {64, 128, 192,
  * 256}) for LB_OPT_STEP_KERNEL 1, {64, 96, 128} for 4 where x3 is periodic
  * with bounce-back walls and for 5 (the same kernel), and the TMA kernel where
- * the context supports it -- timed with
+ * the context supports it -- after one untimed step as one call of lb_step
+ * takes them (so with steps_per_trial >= 4 and several instances in groups,
+ * which the TMA kernel does not run in), timed with
  * CUDA events on the context's stream, then keeps the fastest. Every
  * configuration computes bitwise the same states, so the trial steps are
  * real time steps: they advance the simulation and the step count. best

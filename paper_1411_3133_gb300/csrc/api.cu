@@ -276,13 +276,14 @@ lb_status launch_steps_chunked(lb_ctx* c, long long n) {
   return LB_OK;
 }
 
-// n > 0 steps without a check: in groups where that pays (lanes.h), else one launch a step.
-lb_status advance(lb_ctx* c, long long n) {
+// n > 0 steps without a check: in groups where that pays (lanes.h), else one
+// launch a step; trials of the autotuner pass graph = false.
+lb_status advance(lb_ctx* c, long long n, bool graph) {
   lb_status s;
   if (n >= LANE_MIN_STEPS && !c->plan.empty() && !use_tma(c)) return launch_steps_chunked(c, n);
   // chained launches (launch_chained) are faster than replaying a graph of
   // them; the TMA kernel and the half-force variant have none
-  if (c->use_graph && c->check_every == 0 && n >= 3 && (use_tma(c) || c->any_shift)) {
+  if (graph && c->use_graph && c->check_every == 0 && n >= 3 && (use_tma(c) || c->any_shift)) {
     if (c->cur != 0) {  // the captured pair starts from buffer 0
       s = launch_step_once(c);
       if (s != LB_OK) return s;
@@ -634,7 +635,7 @@ lb_status lb_step(lb_ctx* c, long long n) {
   if (n < 0) return fail(c, LB_ERR_ARG, "need n >= 0");
   while (n > 0) {  // from check to check
     const long long k = c->check_every > 0 ? std::min(n, c->check_every - c->step % c->check_every) : n;
-    if ((s = advance(c, k)) != LB_OK) return s;
+    if ((s = advance(c, k, true)) != LB_OK) return s;
     n -= k;
     if (c->check_every > 0 && c->step % c->check_every == 0 && (s = check_flag(c)) != LB_OK) return s;
   }
@@ -861,11 +862,10 @@ lb_status lb_autotune(lb_ctx* c, int steps_per_trial, lb_tune* best, lb_tune* tr
   for (lb_tune& k : cand) {
     c->block_threads = k.block_threads > 0 ? k.block_threads : keep_threads;
     c->step_kernel = k.schedule;
-    for (int i = 0; i <= steps_per_trial && st == LB_OK; ++i) {  // step 0 is the untimed warm-up
-      if (i == 1 && (e = cudaEventRecord(e0, c->stream)) != cudaSuccess) st = cuda_fail(c, e, "cudaEventRecord");
-      if (st == LB_OK) st = launch_step_once(c);
-      if (st == LB_OK) ++c->step;
-    }
+    st = advance(c, 1, false);  // untimed
+    if (st == LB_OK && (e = cudaEventRecord(e0, c->stream)) != cudaSuccess) st = cuda_fail(c, e, "cudaEventRecord");
+    // as lb_step takes them: from LANE_MIN_STEPS on in groups
+    if (st == LB_OK) st = advance(c, steps_per_trial, false);
     if (st == LB_OK && (e = cudaEventRecord(e1, c->stream)) != cudaSuccess) st = cuda_fail(c, e, "cudaEventRecord");
     if (st == LB_OK && (e = cudaEventSynchronize(e1)) != cudaSuccess) st = cuda_fail(c, e, "cudaEventSynchronize");
     float ms = 0.f;

@@ -60,3 +60,21 @@ def test_checks_do_not_end_the_groups(lib, precision, batch):
     if batch:
         b.close()
     c.close()
+
+
+@pytest.mark.parametrize("steps,kernel", [(8, 1), (2, 2)])
+def test_autotuner_times_what_a_call_runs(lib, steps, kernel):
+    """Node costs at which one launch over all instances is slower than the TMA
+    kernel and the groups are faster than both: trials of 4 and more steps see
+    the groups, shorter ones (whose calls run without) do not."""
+    lib.fake_set_costs(2.0, 0.5e-4, 1e-4, 50e6, 0.8e-4)
+    c = Host(lib, *SWEEP)
+    best, trials, n = L.lb_tune(), (L.lb_tune * 16)(), ctypes.c_int()
+    c.ok(lib.lb_autotune(c.ctx, steps, ctypes.byref(best), trials, 16, ctypes.byref(n)))
+    take_log(lib)
+    assert n.value == 10 and (best.schedule == 2) == (kernel == 2)
+    assert np.array_equal(c.counts(), [10 * (steps + 1)] * 5)
+    c.step(8)
+    assert {x["kind"] for x in launches(lib)} == {"tma" if kernel == 2 else "f32"}
+    c.close()
+    lib.fake_set_costs(2.0, 1e-4, 1e-4, 1e18, 1e-4)
