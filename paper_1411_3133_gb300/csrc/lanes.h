@@ -8,12 +8,21 @@
 // streams. Measured on one GB300, GLUPS of 64 x 4 x 256 channels, all 24
 // instances a step on one stream against 4 streams of one or two instances:
 // cylinder FP32 19.5 / 22.7, FP16 23.0 / 29.0; four-wall ellipsoid FP32 18.1 /
-// 22.7, FP16 20.3 / 25.3. The line: what the streams hold at once stays below
-// 90 MB (four streams of 43 MB fall back to 19.8), and a launch is long enough
-// to be issued while the others run (about 2 us, 60 000 nodes). The 2-byte
-// storage's stream table counts as held: with the state alone the ellipsoid ran
-// in groups of two whose tables (3.4 MB an instance) went to HBM, 68.7 us a step
-// of the 24 in FP16 against 63.8.
+// 22.7, FP16 20.3 / 25.3. The lines: instances are joined up to a quarter of
+// 90 MiB, so that four streams hold what L2 keeps, and further up to half of it
+// where the launch would be too short to be issued while the others run (about
+// 2 us, 60 000 nodes). An instance of its own may be as large as half of it:
+// four streams then hold up to 180 MiB and much of the state comes from HBM --
+// 12 of 96 x 4 x 340 in FP32 (43 MB each) 78.2 us a step, 79.8 in one launch over
+// all, 69.0 on two streams; 4 of 64 x 4 x 256 in FP64 235, 249, 235. A bound of
+// 90 MiB on what all streams hold together, with two streams for chunks above a
+// quarter of it, costs more than it gives: 24 mixed channels in FP32 3.90 ->
+// 3.72 ms for 40 steps, but 20 of 64 x 4 x 300 (25 MB each) 69.9 -> 80.0 us a
+// step and batches of 4 to 10 unlike channels up to 1.5 times as long. With an
+// instance above half of it the plan is empty. The 2-byte storage's stream table
+// counts as held: with the state alone the ellipsoid ran in groups of two whose
+// tables (3.4 MB an instance) went to HBM, 68.7 us a step of the 24 in FP16
+// against 63.8.
 #pragma once
 
 #include <algorithm>
