@@ -267,9 +267,11 @@ lb_status launch_step_once(lb_ctx* c) {
 // n steps with the instances taken in chunks (lanes.h).
 lb_status launch_steps_chunked(lb_ctx* c, long long n) {
   const int cur = c->cur;
-  cudaError_t e = run_lanes(c->lanes, c->plan, n, c->stream, [&](const LaneChunk& ch, long long i, cudaStream_t s) {
-    return launch_step(c, int(cur ^ (i & 1)), ch.first, ch.count, false, s);
-  });
+  cudaError_t e = c->lanes.create(c->stream, c->device);
+  if (e == cudaSuccess)
+    e = run_lanes(c->lanes, c->plan, n, c->stream, [&](const LaneChunk& ch, long long i, cudaStream_t s) {
+      return launch_step(c, int(cur ^ (i & 1)), ch.first, ch.count, false, s);
+    });
   if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
   c->cur = int(cur ^ (n & 1));
   c->step += n;

@@ -379,7 +379,7 @@ lb_status lb_batch_create(lb_ctx* const* members, int count, lb_batch** out) {
   cudaError_t e = cudaGetDevice(&cur_dev);
   if (e == cudaSuccess && cur_dev != b->device) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, b->device);
-  if (e == cudaSuccess) e = b->lanes.create();
+  if (e == cudaSuccess) e = b->lanes.create(b->stream, b->device);
   if (e != cudaSuccess) return bail(LB_ERR_CUDA, std::string("batch setup: ") + cudaGetErrorString(e));
   *out = b;
   return LB_OK;

@@ -89,14 +89,20 @@ struct LaneStreams {
   cudaStream_t aux[LANES - 1] = {};
   cudaEvent_t fork = nullptr, join[LANES - 1] = {};
 
-  cudaError_t create() {
+  // On `device` and with the priority of the owner's stream, whatever device is
+  // current when the first call needs them.
+  cudaError_t create(cudaStream_t own, int device) {
     if (fork) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
+    int current = device, priority = 0;
+    cudaError_t e = cudaGetDevice(&current);
+    if (e == cudaSuccess && current != device) e = cudaSetDevice(device);
+    if (e == cudaSuccess) e = cudaStreamGetPriority(own, &priority);
     for (int i = 0; i < LANES - 1 && e == cudaSuccess; ++i) {
-      if (!aux[i]) e = cudaStreamCreateWithFlags(&aux[i], cudaStreamNonBlocking);
+      if (!aux[i]) e = cudaStreamCreateWithPriority(&aux[i], cudaStreamNonBlocking, priority);
       if (e == cudaSuccess && !join[i]) e = cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming);
     }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    if (current != device) cudaSetDevice(current);
     return e;
   }
   void destroy() {
@@ -110,13 +116,12 @@ struct LaneStreams {
   cudaStream_t lane(int i, cudaStream_t own) const { return i == 0 ? own : aux[i - 1]; }
 };
 
-// n steps of every chunk: launch(chunk, step, stream) enqueues one step of one
-// chunk. The streams' launches are issued in turn, and every stream is joined
+// n steps of every chunk on created streams: launch(chunk, step, stream)
+// enqueues one step of one chunk. The streams' launches are issued in turn, and every stream is joined
 // back to `own` even after a failed launch.
 template <class F>
 cudaError_t run_lanes(LaneStreams& ls, const std::vector<LaneChunk>& plan, long long n, cudaStream_t own, F&& launch) {
-  cudaError_t e = ls.create();
-  if (e == cudaSuccess) e = cudaEventRecord(ls.fork, own);
+  cudaError_t e = cudaEventRecord(ls.fork, own);
   if (e != cudaSuccess) return e;
   std::vector<const LaneChunk*> todo[LANES];
   for (const LaneChunk& c : plan) todo[c.lane].push_back(&c);

@@ -79,6 +79,7 @@ const char* fake_take_log() {
   return out.c_str();
 }
 void fake_set_device(int d) { g_device = d; }
+int fake_device() { return g_device; }
 // a step of `bytes` costs launch + nodes * (fits or not) microseconds
 void fake_set_costs(double launch, double fits, double not_fits, double fit_bytes, double tma) {
   g_launch_cost = launch;

@@ -78,3 +78,22 @@ def test_autotuner_times_what_a_call_runs(lib, steps, kernel):
     assert {x["kind"] for x in launches(lib)} == {"tma" if kernel == 2 else "f32"}
     c.close()
     lib.fake_set_costs(2.0, 1e-4, 1e-4, 1e18, 1e-4)
+
+
+@pytest.mark.parametrize("batch", [False, True], ids=["context", "batch"])
+def test_streams_of_the_groups_are_like_the_owners(lib, batch):
+    """On the context's device, whatever device is current at the first long
+    call (which stays current), and with its stream's priority."""
+    c = Host(lib, *SWEEP, priority=-3)
+    b = Batch(lib, [c]) if batch else None
+    take = b.step if batch else c.step
+    if not batch:
+        lib.fake_set_device(1)
+    take(4)
+    made = [x for x in take_log(lib) if x["kind"] == "create"]
+    assert len(made) == 3 and {(x["device"], x["priority"]) for x in made} == {(0, -3)}
+    assert lib.fake_device() == (0 if batch else 1)
+    lib.fake_set_device(0)
+    if batch:
+        b.close()
+    c.close()
