@@ -182,15 +182,19 @@ typedef enum {
                                kernels with FP32 arithmetic run at most 128
                                per block (their register cap); larger
                                values run as 128 */
-  LB_OPT_USE_GRAPH = 2,     /* 1: replay a captured CUDA graph of pairs of
-                               steps (default 0) where that is the faster
-                               way: lb_step with the TMA kernel or the
-                               half-force variant, and lb_batch_step of
-                               fewer than 4 steps or of channels too small
-                               to be taken in groups. Elsewhere the steps
+  LB_OPT_USE_GRAPH = 2,     /* 1: replay captured CUDA graphs of steps
+                               (default 0). Calls of 256 and more steps
+                               (between checks) are issued 32 steps of a
+                               group at a time, so that they return long
+                               before the steps are done. Shorter calls
+                               replay pairs of steps where that is the
+                               faster way: lb_step with the TMA kernel or
+                               the half-force variant, and lb_batch_step of
+                               fewer than 4 steps or of channels too large
+                               to be taken in groups; elsewhere the steps
                                are launched one by one, each kernel
                                starting under the end of the one before,
-                               which is faster than a replay */
+                               which is faster than a replay of pairs */
   LB_OPT_STEP_KERNEL = 3,   /* 0: automatic (default), 1, 4, 5: the
                                one-kernel step of the storage type (4 and
                                5 named a region split and a tiled step

@@ -60,6 +60,7 @@ void* dalloc(lb_ctx* c, size_t bytes) {
 void free_all(lb_ctx* c) {
   if (c->graph) cudaGraphExecDestroy(c->graph);
   c->graph = nullptr;
+  c->replays.clear();
   for (auto& a : c->allocations) {
     if (c->has_alloc)
       c->alloc.free(a.first, a.second, c->stream, c->alloc.user);
@@ -264,13 +265,15 @@ lb_status launch_step_once(lb_ctx* c) {
   return LB_OK;
 }
 
-// n steps with the instances taken in chunks (lanes.h).
-lb_status launch_steps_chunked(lb_ctx* c, long long n) {
+// n steps of a plan's chunks (lanes.h): the groups, or every instance in one
+// chunk, whose launches are chained; replays may be NULL.
+lb_status launch_steps_chunked(lb_ctx* c, const std::vector<LaneChunk>& plan, long long n, Replays* replays) {
   const int cur = c->cur;
+  const bool chained = plan.size() == 1;
   cudaError_t e = c->lanes.create(c->stream, c->device);
   if (e == cudaSuccess)
-    e = run_lanes(c->lanes, c->plan, n, c->stream, [&](const LaneChunk& ch, long long i, cudaStream_t s) {
-      return launch_step(c, int(cur ^ (i & 1)), ch.first, ch.count, false, s);
+    e = run_lanes(c->lanes, plan, n, c->stream, replays, cur, [&](const LaneChunk& ch, long long i, cudaStream_t s) {
+      return launch_step(c, int(cur ^ (i & 1)), ch.first, ch.count, chained, s);
     });
   if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
   c->cur = int(cur ^ (n & 1));
@@ -282,9 +285,13 @@ lb_status launch_steps_chunked(lb_ctx* c, long long n) {
 // launch a step; trials of the autotuner pass graph = false.
 lb_status advance(lb_ctx* c, long long n, bool graph) {
   lb_status s;
-  if (n >= LANE_MIN_STEPS && !c->plan.empty() && !use_tma(c)) return launch_steps_chunked(c, n);
-  // chained launches (launch_chained) are faster than replaying a graph of
-  // them; the TMA kernel and the half-force variant have none
+  const bool grouped = n >= LANE_MIN_STEPS && !c->plan.empty() && !use_tma(c);
+  const std::vector<LaneChunk>& plan = grouped ? c->plan : c->whole;
+  // the TMA kernel and the half-force variant have no chained launches: pairs
+  // of their steps are replayed below
+  const bool replay = graph && c->use_graph && (grouped || !(use_tma(c) || c->any_shift)) &&
+                      c->replays.ready(n, plan.size(), 2 * c->block_threads + (c->any_shift ? 1 : 0), c->stream);
+  if (grouped || replay) return launch_steps_chunked(c, plan, n, replay ? &c->replays : nullptr);
   if (graph && c->use_graph && c->check_every == 0 && n >= 3 && (use_tma(c) || c->any_shift)) {
     if (c->cur != 0) {  // the captured pair starts from buffer 0
       s = launch_step_once(c);
@@ -553,6 +560,7 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
   c->step_bytes = 2 * Q * c->ncell * c->elem_bytes;
   if (c->st_tab) c->step_bytes += 2 * ST_K * size_t(geom->nr) * size_t(d.st_rows3) * sizeof(float4);
   c->plan = plan_lanes(std::vector<LaneInst>(size_t(batch), {0, c->ncell, c->step_bytes}), batch);
+  c->whole = {{0, 0, batch, 0}};
   *out = c;
   return LB_OK;
 }

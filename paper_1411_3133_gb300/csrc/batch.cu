@@ -51,6 +51,7 @@ struct lb_batch {
   int tile = 0;               // nodes (FP32, FP64) or warps (2-byte storage) of a work item
 
   LaneStreams lanes;
+  Replays replays;              // of plan's chunks, or of flat's where there is no plan
   std::vector<LaneChunk> plan;  // a call of several steps: chunks of the groups' instances
   std::vector<LaneChunk> flat;  // one step: every instance, LIST_MAX to a launch
 
@@ -91,6 +92,7 @@ lb_status bcuda(lb_batch* b, cudaError_t e, const char* what) {
 void drop_graph(lb_batch* b) {
   if (b->graph) cudaGraphExecDestroy(b->graph);
   b->graph = nullptr;
+  b->replays.clear();
 }
 
 template <class S, class R>
@@ -226,25 +228,23 @@ cudaError_t launch_chunk(const lb_batch* b, const LaneChunk& c, int par, bool ch
 
 // n batch steps: the chunks read the same buffers and write disjoint nodes, so
 // they run side by side on the lanes; several steps in the order of lanes.h.
-lb_status steps(lb_batch* b, long long n) {
+lb_status steps(lb_batch* b, long long n, Replays* replays) {
   const std::vector<LaneChunk>& plan = n >= LANE_MIN_STEPS && !b->plan.empty() ? b->plan : b->flat;
   const int par = b->parity;
+  // one chunk: chained launches; several without a plan meet after every step
+  const bool chained = plan.size() == 1;
+  const long long each = !chained && &plan == &b->flat ? 1 : n;
   cudaError_t e = cudaSuccess;
-  if (plan.size() == 1) {
-    for (long long i = 0; i < n && e == cudaSuccess; ++i) e = launch_chunk(b, plan[0], int(par ^ (i & 1)), true, b->stream);
-  } else {
-    const long long each = &plan == &b->flat ? 1 : n;
-    for (long long i0 = 0; i0 < n && e == cudaSuccess; i0 += each)
-      e = run_lanes(b->lanes, plan, each, b->stream, [&](const LaneChunk& c, long long i, cudaStream_t s) {
-        return launch_chunk(b, c, int(par ^ ((i0 + i) & 1)), false, s);
-      });
-  }
+  for (long long i0 = 0; i0 < n && e == cudaSuccess; i0 += each)
+    e = run_lanes(b->lanes, plan, each, b->stream, replays, par, [&](const LaneChunk& c, long long i, cudaStream_t s) {
+      return launch_chunk(b, c, int(par ^ ((i0 + i) & 1)), chained, s);
+    });
   if (e != cudaSuccess) return bcuda(b, e, "step kernel launch");
   b->parity = int(par ^ (n & 1));
   return LB_OK;
 }
 
-lb_status step_once(lb_batch* b) { return steps(b, 1); }
+lb_status step_once(lb_batch* b) { return steps(b, 1, nullptr); }
 
 void advance_members(lb_batch* b, long long n) {
   for (lb_ctx* c : b->m) {
@@ -290,8 +290,11 @@ lb_status ready(lb_batch* b) {
 
 // n > 0 steps without a check: in groups where that pays (lanes.h), else a step at a time.
 lb_status advance(lb_batch* b, long long n, bool graph) {
-  if (n >= LANE_MIN_STEPS && !b->plan.empty()) {
-    lb_status s = steps(b, n);
+  const bool grouped = n >= LANE_MIN_STEPS && !b->plan.empty();
+  const bool replay = graph && b->use_graph && (grouped || b->flat.size() == 1) &&
+                      b->replays.ready(n, grouped ? b->plan.size() : 1, b->schedule, b->stream);
+  if (grouped || replay) {
+    lb_status s = steps(b, n, replay ? &b->replays : nullptr);
     if (s == LB_OK) advance_members(b, n);
     return s;
   }

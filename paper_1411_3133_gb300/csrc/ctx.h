@@ -69,7 +69,9 @@ struct lb_ctx {
   bool any_shift = false;            // an instance uses the half-force velocity (old_forcing 2)
   size_t step_bytes = 0;             // what an instance's steps use: two buffers and its stream table
   std::vector<lbgm::LaneChunk> plan; // order of the instances in a call of several steps
+  std::vector<lbgm::LaneChunk> whole; // every instance as one chunk
   lbgm::LaneStreams lanes;
+  lbgm::Replays replays;             // of the plan's chunks, or of `whole` where there is no plan
   bool tma_ok = false;               // tensor maps built for both buffers
   alignas(64) unsigned char tmap[2][128];
 };

@@ -116,23 +116,95 @@ struct LaneStreams {
   cudaStream_t lane(int i, cudaStream_t own) const { return i == 0 ? own : aux[i - 1]; }
 };
 
+// Captured steps of the chunks (LB_OPT_USE_GRAPH): a long call is issued
+// REPLAY_STEPS steps of a chunk at a time, so that its caller is free again
+// while the GPU works. Launched one by one, a step of 24 groups takes the caller
+// 40 us of its 66, and once a stream's queue of about 1000 launches is full the
+// call waits for the GPU. Caller's time of 2000 steps, launched / replayed, us a
+// step: 24 cylinders of 64 x 4 x 256 in FP32 60 / 1.1 of 65 / 62, one in FP64
+// 35 / 0.05 of 72. The steps themselves take 0.96 to 1.06 of their time (four-wall
+// ellipsoids FP32 67.7 / 68.9, FP16 62.7 / 60.7; 43 MB instances 77.6 / 82.3), the
+// same with 16 to 128 steps in a graph. A graph is made at a chunk's first long
+// call, under the steps launched before it; shorter calls would not earn it back.
+constexpr int REPLAY_STEPS = 32;
+constexpr long long REPLAY_MIN = 8 * REPLAY_STEPS;
+constexpr size_t REPLAY_CHUNKS = 256;  // more are launched one by one: graphs hold memory
+
+struct Replays {
+  std::vector<cudaGraphExec_t> exec;  // [2 chunk + buffer that the first step reads]
+  long long key = -1;                 // of the captured launches
+
+  void clear() {
+    for (cudaGraphExec_t x : exec)
+      if (x) cudaGraphExecDestroy(x);
+    exec.clear();
+  }
+  // Whether n steps of `chunks` chunks on `own` are replayed; graphs of another
+  // key (or another plan) are dropped. Not while the caller captures `own`.
+  bool ready(long long n, size_t chunks, long long key_, cudaStream_t own) {
+    if (n < REPLAY_MIN || chunks > REPLAY_CHUNKS) return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(own, &st) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (st != cudaStreamCaptureStatusNone) return false;
+    if (key_ != key || exec.size() != 2 * chunks) {
+      clear();
+      exec.assign(2 * chunks, nullptr);
+      key = key_;
+    }
+    return true;
+  }
+  // REPLAY_STEPS steps of a chunk on `on`; step(i, stream) enqueues the i-th one
+  // (for the capture, on `work`).
+  template <class F>
+  cudaError_t launch(size_t at, cudaStream_t work, cudaStream_t on, F&& step) {
+    cudaGraphExec_t& x = exec[at];
+    if (!x) {
+      cudaError_t e = cudaStreamBeginCapture(work, cudaStreamCaptureModeThreadLocal);
+      if (e != cudaSuccess) return e;
+      for (int i = 0; i < REPLAY_STEPS && e == cudaSuccess; ++i) e = step(i, work);
+      cudaGraph_t g = nullptr;
+      const cudaError_t e2 = cudaStreamEndCapture(work, &g);
+      if (e == cudaSuccess) e = e2;
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&x, g, 0);
+      if (g) cudaGraphDestroy(g);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaGraphLaunch(x, on);
+  }
+};
+
 // n steps of every chunk on created streams: launch(chunk, step, stream)
-// enqueues one step of one chunk. The streams' launches are issued in turn, and every stream is joined
-// back to `own` even after a failed launch.
+// enqueues one step of one chunk. The streams' launches are issued in turn, and
+// every stream is joined back to `own` even after a failed launch. With
+// `replays` (ready) all but the first n % REPLAY_STEPS steps are replayed;
+// `buffer` is the buffer that step 0 reads.
 template <class F>
-cudaError_t run_lanes(LaneStreams& ls, const std::vector<LaneChunk>& plan, long long n, cudaStream_t own, F&& launch) {
-  cudaError_t e = cudaEventRecord(ls.fork, own);
-  if (e != cudaSuccess) return e;
+cudaError_t run_lanes(LaneStreams& ls, const std::vector<LaneChunk>& plan, long long n, cudaStream_t own,
+                      Replays* replays, int buffer, F&& launch) {
   std::vector<const LaneChunk*> todo[LANES];
   for (const LaneChunk& c : plan) todo[c.lane].push_back(&c);
+  // (one chunk: no event between its chained launches and those before)
+  cudaError_t e = plan.size() > 1 ? cudaEventRecord(ls.fork, own) : cudaSuccess;
+  if (e != cudaSuccess) return e;
   for (int l = 1; l < LANES && e == cudaSuccess; ++l)
     if (!todo[l].empty()) e = cudaStreamWaitEvent(ls.aux[l - 1], ls.fork, 0);
   size_t longest = 0;
   for (auto& t : todo) longest = std::max(longest, t.size());
+  const long long single = replays ? n % REPLAY_STEPS : n;
   for (size_t k = 0; k < longest; ++k)
-    for (long long i = 0; i < n; ++i)
-      for (int l = 0; l < LANES && e == cudaSuccess; ++l)
-        if (k < todo[l].size()) e = launch(*todo[l][k], i, ls.lane(l, own));
+    for (long long i = 0; i < n; i += i < single ? 1 : REPLAY_STEPS)
+      for (int l = 0; l < LANES && e == cudaSuccess; ++l) {
+        if (k >= todo[l].size()) continue;
+        const LaneChunk& c = *todo[l][k];
+        if (i < single)
+          e = launch(c, i, ls.lane(l, own));
+        else
+          e = replays->launch(2 * size_t(&c - plan.data()) + size_t((buffer ^ i) & 1), ls.aux[0], ls.lane(l, own),
+                              [&](int j, cudaStream_t s) { return launch(c, i + j, s); });
+      }
   for (int l = 1; l < LANES; ++l) {
     if (todo[l].empty()) continue;
     cudaError_t e2 = cudaEventRecord(ls.join[l - 1], ls.aux[l - 1]);

@@ -88,6 +88,7 @@ void fake_set_costs(double launch, double fits, double not_fits, double fit_byte
   g_fit = size_t(fit_bytes);
   g_tma_cost = tma;
 }
+void fake_capture(void* s, int on) { static_cast<Stream*>(s)->capture = on ? new Graph : nullptr; }
 void* fake_stream(int priority) { return new Stream{g_ids++, g_device, priority}; }
 
 // ---- runtime ----
@@ -101,6 +102,7 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cu
   return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) { std::memset(d, v, n); return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
 const char* cudaGetErrorString(cudaError_t) { return "fake error"; }
 
 cudaError_t cudaStreamCreateWithPriority(cudaStream_t* s, unsigned, int priority) {

@@ -37,6 +37,7 @@ def build_host_library(out_dir):
             getattr(lib, name).restype, getattr(lib, name).argtypes = res, args
     lib.fake_take_log.restype = ctypes.c_char_p
     lib.fake_stream.restype = ctypes.c_void_p
+    lib.fake_capture.argtypes = [ctypes.c_void_p, ctypes.c_int]
     lib.fake_set_costs.argtypes = [ctypes.c_double] * 5
     return lib
 

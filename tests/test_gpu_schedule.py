@@ -36,3 +36,63 @@ def test_checks_groups_and_single_steps(call, batch):
     if batch:
         b.close()
     c.close()
+
+
+REPLAYED = CASES + [("cylindrical", True, (16, 4, 32), 70, "bf16_shifted"), ("cylindrical", True, (16, 4, 32), 1, "fp32"),
+                    ("ellipsoidal", False, (16, 4, 33), 2, "fp16_shifted")]
+
+
+@pytest.mark.parametrize("call", REPLAYED, ids=lambda c: f"{c[0]}-{'x'.join(map(str, c[2]))}-b{c[3]}-{c[4]}")
+@pytest.mark.parametrize("batch", [False, True], ids=["context", "batch"])
+def test_replayed_long_calls(call, batch):
+    """From either buffer, twice, and with launched steps in between."""
+    L = lib()
+    c = _context(L, *call)
+    b = L.LBBatch([c]) if batch else None
+    (b.lb_batch_set_option if batch else c.lb_set_option)(L.LB_OPT_USE_GRAPH, 1)
+    for n in (289, 256, 3, 300):
+        b.lb_batch_step(n) if batch else c.lb_step(n)
+    assert np.array_equal(_state(c), _waited_for(L, call, 848))
+    if batch:
+        b.close()
+    c.close()
+
+
+def test_a_callers_capture_takes_a_long_call():
+    """With LB_OPT_USE_GRAPH, on a stream that the caller captures."""
+    import torch
+    L = lib()
+    c = _context(L, *CASES[0])
+    c.lb_set_option(L.LB_OPT_USE_GRAPH, 1)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=c.stream, capture_error_mode="thread_local"):
+        c.lb_step(260)
+    g.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(_state(c), _waited_for(L, CASES[0], 260))
+    c.close()
+
+
+@pytest.mark.parametrize("call", [("cylindrical", True, (64, 4, 256), 8, "fp32"),
+                                  ("cylindrical", True, (64, 4, 256), 1, "fp64")], ids=["groups", "chained"])
+def test_a_long_call_returns_before_its_steps(call):
+    """LB_OPT_USE_GRAPH keeps the caller free: under 0.3 of the steps' time is
+    spent in the call (launched one by one nine tenths in the groups, three
+    quarters in the chained launches, whose queue holds 1000; replayed a few
+    percent)."""
+    import time
+
+    import torch
+    L = lib()
+    c = _context(L, *call)
+    c.lb_set_option(L.LB_OPT_USE_GRAPH, 1)
+    held = []
+    for _ in range(4):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        c.lb_step(4000)
+        h = time.perf_counter() - t
+        torch.cuda.synchronize()
+        held.append(h / (time.perf_counter() - t))
+    assert min(held) < 0.3
+    c.close()

@@ -97,3 +97,64 @@ def test_streams_of_the_groups_are_like_the_owners(lib, batch):
     if batch:
         b.close()
     c.close()
+
+
+# groups of one instance; several instances a group; one chained launch a step
+LONG = [(("cylindrical", (64, 4, 256), 5, "fp32"), 5), (("cylindrical", (16, 4, 32), 70, "fp16_shifted"), 3),
+        (("cylindrical", (64, 4, 256), 1, "fp64"), 1)]
+
+
+@pytest.mark.parametrize("spec,chunks", LONG, ids=["groups", "small", "chained"])
+@pytest.mark.parametrize("batch", [False, True], ids=["context", "batch"])
+def test_long_calls_are_replayed(lib, spec, chunks, batch):
+    """LB_OPT_USE_GRAPH: of a call of 2000 steps a few are launched by the
+    caller, the rest in graphs made once per chunk and first buffer; the graphs
+    follow the launch options, and nobody's capture is interrupted."""
+    c = Host(lib, *spec)
+    b = Batch(lib, [c]) if batch else None
+    on, take = (b, b.step) if batch else (c, c.step)
+    on.option(L.LB_OPT_USE_GRAPH, 1)
+    if batch and spec[2] > 16:
+        chunks = 5  # at most 16 instances a launch
+    total = 0
+
+    def call(n, made, threads=128):
+        nonlocal total
+        take(n)
+        total += n
+        log = take_log(lib)
+        steps = [x for x in log if "count" in x]
+        assert sum(x["count"] for x in steps) == n * spec[2] and {x["threads"] for x in steps} == {threads}
+        assert sum(x["kind"] == "instantiate" for x in log) == made
+        assert np.array_equal(c.counts(), [total] * spec[2])
+        return [x for x in steps if not x["replay"]]
+
+    take_log(lib)
+    assert len(call(2000, chunks)) <= 31 * chunks
+    assert len(call(2000, 0)) <= 31 * chunks
+    call(1001, chunks)     # an odd number of steps first: the other buffer
+    call(333, 0)
+    call(1000, 0)
+    on.option(L.LB_OPT_BLOCK_THREADS, 64)
+    call(320, chunks, 64)
+    assert all(not x["replay"] for x in call(20, 0, 64))       # short calls are launched
+    lib.fake_capture(c.stream, 1)
+    take(2000)             # goes into the caller's own graph
+    lib.fake_capture(c.stream, 0)
+    assert not [x for x in take_log(lib) if x["kind"] == "instantiate"]
+    if batch:
+        b.close()
+    c.close()
+
+
+def test_replays_follow_the_parameters(lib):
+    """lb_init may switch to the half-force kernel and back."""
+    c = Host(lib, *SWEEP)
+    c.option(L.LB_OPT_USE_GRAPH, 1)
+    for old_forcing, kind in ((0, "f32"), (2, "shift32"), (0, "f32")):
+        c.init(old_forcing)
+        take_log(lib)
+        c.step(320)
+        assert {x["kind"] for x in launches(lib)} == {kind}
+        assert np.array_equal(c.counts(), [320] * 5)
+    c.close()
