@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(DIAG_THREADS)
   for (int q = 0; q < DIAG_NQ; ++q) a[q] = 0.0;
   const double inv_n3 = 1.0 / n3;
   int bad = 0;
+  bool direct = false;            // 5 from u^r itself, since a row with an infinity
   unsigned long long speed2 = 0;  // bits of the largest |u|^2
   for (int row = blockIdx.x * (DIAG_THREADS / 32) + (threadIdx.x >> 5); row < d.nr * d.nt;
        row += nblk * (DIAG_THREADS / 32)) {
@@ -231,7 +232,18 @@ __global__ void __launch_bounds__(DIAG_THREADS)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     const double mean = s * inv_n3;
-    if (lane == 0) a[5] = fma(double(n3) * mean, mean, a[5]);  // + sum fl^2 = sum (u^r)^2
+    if (!direct && !finite_bits(mean)) {  // no mean to split (u^r)^2 by, and 6 becomes a NaN
+      a[5] += a[6];
+      direct = true;
+    }
+    if (!direct) {
+      if (lane == 0) a[5] = fma(double(n3) * mean, mean, a[5]);  // + sum fl^2 = sum (u^r)^2
+    } else {
+      for (int i = lane; i < n3; i += 32) {
+        const double v = eq_wall_node(d, ir, i) ? 0.0 : r0[i];
+        a[5] = fma(v, v, a[5]);
+      }
+    }
     for (int i3 = lane; i3 < n3; i3 += 32) {
       const int c = row * n3 + i3;
       const double* gr = geo64 + size_t(d.geo_theta ? c : ir * n3 + i3) * 4;
@@ -273,7 +285,7 @@ __global__ void __launch_bounds__(DIAG_THREADS)
       bad += finite_bits(r) && finite_bits(u0) && finite_bits(u1) && finite_bits(u2) ? 0 : 1;
     }
   }
-  a[5] += a[6];
+  if (!direct) a[5] += a[6];
   a[7] = __longlong_as_double(static_cast<long long>(speed2));
   a[8] = double(bad);
   block_reduce(a, sh);
