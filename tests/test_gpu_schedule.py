@@ -96,3 +96,33 @@ def test_a_long_call_returns_before_its_steps(call):
         held.append(h / (time.perf_counter() - t))
     assert min(held) < 0.3
     c.close()
+
+
+@pytest.mark.parametrize("plan", [False, True], ids=["one", "groups"])
+def test_replayed_pairs_of_the_tma_and_half_force_kernels(plan):
+    """Calls that replay a captured pair of steps -- the TMA kernel, the
+    half-force variant -- from either buffer and across an lb_init that changes
+    the kernel, against single steps that are waited for."""
+    L = lib()
+    spec = L.ChannelSpec("cylindrical", 1.0, 1.0 / 0.975, 48, 4, 256)
+    batch = 6 if plan else 1
+    outs = []
+    for graph in (1, 0):
+        c = L.LBContext(spec, batch=batch, precision="fp32")
+        c.lb_set_option(L.LB_OPT_USE_GRAPH, graph)
+        states = []
+        for forcing, kernel in ((0, 2), (2, 2), (2, 1), (0, 2), (0, 1)):
+            c.lb_set_option(L.LB_OPT_STEP_KERNEL, kernel)
+            c.lb_init([L.make_params(0.6 + 0.05 * i, 1e-5, forcing, 1 + i, 1e-3, False) for i in range(batch)])
+            for n in (1, 37, 8, 3):
+                if graph:
+                    c.lb_step(n)
+                else:
+                    for _ in range(n):
+                        c.lb_step(1)
+                        c.stream.synchronize()
+            states.append(_state(c))
+        outs.append(states)
+        c.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*outs))
+    assert not np.array_equal(outs[0][0], outs[0][1])      # the variant is another step
