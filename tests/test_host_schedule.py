@@ -158,3 +158,34 @@ def test_replays_follow_the_parameters(lib):
         assert {x["kind"] for x in launches(lib)} == {kind}
         assert np.array_equal(c.counts(), [320] * 5)
     c.close()
+
+
+def _channel(metric, nr, ntheta, n3, periodic3=True):
+    from oracle.geometry import Channel
+    return Channel(metric, 1.0, 1.0 / 0.975, nr, ntheta, n3, periodic3=periodic3)
+
+
+@pytest.mark.parametrize("steps", [1, 3, 4, 20])
+@pytest.mark.parametrize("precision", ["fp32", "fp16_shifted", "fp64"])
+def test_bench_counts_the_launches(lib, precision, steps):
+    """bench.step_launches (its gpu_launches) against the launches of the
+    library: uniform contexts, and batches of unlike channels."""
+    import bench
+    for ch, batch in ((_channel("cylindrical", 64, 4, 256), 24), (_channel("ellipsoidal", 64, 4, 256, False), 7),
+                      (_channel("cylindrical", 16, 4, 32), 70), (_channel("cylindrical", 96, 8, 400), 3)):
+        c = Host(lib, ch.metric, (ch.nr, ch.ntheta, ch.n3), batch, precision, ch.periodic3)
+        take_log(lib)
+        c.step(steps)
+        assert len(launches(lib)) == steps * bench.step_launches([ch] * batch, precision, steps)
+        c.close()
+    chs = [_channel("cylindrical", 32 + 16 * (i % 3), 4, 128 + 37 * i) for i in range(7)] + \
+        [_channel("ellipsoidal", 64, 4, 200 + 31 * i, False) for i in range(19)]
+    stream = lib.fake_stream(0)
+    members = [Host(lib, ch.metric, (ch.nr, ch.ntheta, ch.n3), 1, precision, ch.periodic3, stream=stream) for ch in chs]
+    b = Batch(lib, members)
+    take_log(lib)
+    b.step(steps)
+    assert len(launches(lib)) == steps * bench.step_launches(chs, precision, steps, 16)
+    b.close()
+    for m in members:
+        m.close()
