@@ -61,3 +61,26 @@ def test_2byte_against_oracle(kind, size, precision, eps):
     g_max = np.abs((fo - w * rest) / w).max()
     assert max_rel(tw.lib_f() / w, fo / w, 1.0) <= 85 * eps * g_max
     tw.close()
+
+
+@pytest.mark.parametrize("precision,eps", [("fp16_shifted", 2.0 ** -11), ("bf16_shifted", 2.0 ** -8)])
+@pytest.mark.parametrize("size", SIZES, ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("kind", KINDS, ids=lambda k: f"{k[0]}-{'per' if k[1] else 'wall'}-{k[2]}")
+def test_2byte_step_velocity_by_velocity(kind, size, precision, eps):
+    """One step from the stored state itself, deviations g = f / w - 1 from the
+    rest state: every population is off by one rounding of its own g, eps |g|,
+    and by the FP32 arithmetic before it, some 700 operations on numbers of
+    order 1: below 1000 x 2^-24. A population from a wrong node or of the wrong
+    direction is off by the noise's own g, 0.03 and more."""
+    from oracle import lattice as OL
+    L = lib()
+    tw = _twin(kind, size, precision)
+    tw.ctx.lb_set_option(L.LB_OPT_STORAGE_REFERENCE, 0)
+    tw.ctx.lb_init(tw.lparams)
+    for s, f in zip(tw.sims, tw.lib_f()):
+        s.f = f.copy()
+    tw.step(1)
+    w = OL.W[None, :, None]
+    g = np.stack([s.f for s in tw.sims]) / w - 1.0
+    assert (np.abs(tw.lib_f() / w - 1.0 - g) <= eps * np.abs(g) + 1000 * 2.0 ** -24).all()
+    tw.close()
