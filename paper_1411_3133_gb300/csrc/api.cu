@@ -246,6 +246,7 @@ cudaError_t launch_step(lb_ctx* c, int src, int i0, int count, bool chained, cud
   };
   switch (c->prec) {
     case LB_FP64:
+      chained = chained && fp64_chains((long long)((c->ncell + c->block_threads - 1) / c->block_threads) * count);
       return go(c->any_shift ? launch_step_shift_f64 : launch_step_f64, static_cast<double*>(nullptr), c->geo_d);
     case LB_FP32:
       if (use_tma(c))  // every instance, on the context's stream

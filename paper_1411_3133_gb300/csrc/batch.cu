@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <numeric>
 #include <string>
 #include <vector>
 
@@ -216,6 +217,10 @@ cudaError_t launch_chunk(const lb_batch* b, const LaneChunk& c, int par, bool ch
   const int grid = b->schedule == 1 ? std::max(1, gr.blocks_per_sm) * b->nsm : 0;
   const void* recs = gr.recs.data() + gr.recs.size() / size_t(gr.ninst) * size_t(c.first);
   const int* items = gr.items.data() + c.first;
+  if (b->prec == LB_FP64) {
+    const long long n = std::accumulate(items, items + c.count, 0ll);
+    chained = chained && fp64_chains(grid > 0 ? std::min<long long>(grid, n) : n);
+  }
   switch (b->prec) {
     case LB_FP64: return launch_step_list_f64(gr.K, recs, c.count, items, b->tile, b->threads, grid, par, chained, s);
     case LB_FP32: return launch_step_list_f32(gr.K, recs, c.count, items, b->tile, b->threads, grid, par, chained, s);

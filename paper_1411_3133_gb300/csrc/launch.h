@@ -13,6 +13,18 @@ namespace lbgm {
 
 struct InitInst;
 
+constexpr int SMS = 152;  // of a GB300
+
+// Whether an FP64 step of `blocks` blocks is worth chaining. Chained, the blocks
+// of the next two or three steps already sit where an SM has room, and an SM that
+// holds two blocks of one step needs twice as long for it (its FP64 units bound
+// the step); unchained, a step of at most one block per SM has one on each.
+// Flat channels, us a step chained / unchained (graph replay before there were
+// chained launches: 29.1): 49 blocks 18.7 / 20.9, 64 20.2 to 25.7 / 20.9, 96
+// 30.5 / 20.8, 144 32.9 / 20.9, 152 18.9 / 20.9, 160 34.6 / 37.2. FP32 arithmetic
+// is bound by latency there and gains in every size (144 blocks 3.5 / 4.6).
+constexpr bool fp64_chains(long long blocks) { return 3 * blocks <= SMS || blocks >= SMS; }
+
 // chained: see launch_chained.
 cudaError_t launch_step_f64(int K, const double* fin, double* fout, const GeoDev<double>& geo,
                             const InstParams<double>* inst, const Dims& d, int* flag, int threads,

@@ -189,3 +189,24 @@ def test_bench_counts_the_launches(lib, precision, steps):
     b.close()
     for m in members:
         m.close()
+
+
+@pytest.mark.parametrize("batch", [False, True], ids=["context", "batch"])
+@pytest.mark.parametrize("precision,instances,threads,chained",
+                         [("fp64", 3, 128, True), ("fp64", 4, 128, False), ("fp64", 9, 128, False),
+                          ("fp64", 10, 128, True), ("fp64", 9, 64, True), ("fp64", 3, 64, False),
+                          ("fp32", 6, 128, True), ("fp16_shifted", 8, 128, True)])
+def test_fp64_steps_of_one_block_per_sm_are_not_chained(lib, precision, instances, threads, chained, batch):
+    """16 x 4 x 32 nodes: 16 blocks of 128 an instance, 152 SMs. Between a third
+    of them and all, two blocks of a chained FP64 step meet on one SM."""
+    c = Host(lib, "cylindrical", (16, 4, 32), instances, precision)
+    b = Batch(lib, [c]) if batch else None
+    (b or c).option(L.LB_OPT_BLOCK_THREADS, threads)
+    for n in (1, 12):
+        take_log(lib)
+        (b or c).step(n)
+        log = launches(lib)
+        assert len(log) == n and {x["chained"] for x in log} == {int(chained)}
+    if batch:
+        b.close()
+    c.close()
