@@ -164,10 +164,12 @@ __device__ __forceinline__ Moments<Real> streamed_moments(const S* __restrict__ 
   return moments(f);
 }
 
-// rho' and u of the streamed populations (moments only).
+// rho' and u of the streamed populations (moments only). 2-byte storage asks
+// for three blocks per SM: without it the ellipsoid's kernel takes 122 registers
+// for 80, two blocks, and 8 four-wall 64 x 4 x 255 channels 100 us for 78.
 template <typename S, typename Real, int K>
-__global__ void __launch_bounds__(256) k_macros(const S* __restrict__ fin, double* __restrict__ rho,
-                                                double* __restrict__ u, Dims d) {
+__global__ void __launch_bounds__(256, sizeof(S) == 2 ? 3 : 1)
+    k_macros(const S* __restrict__ fin, double* __restrict__ rho, double* __restrict__ u, Dims d) {
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= uint32_t(d.batch) * uint32_t(d.ncell)) return;
   const CellPos p = locate(d, t);
