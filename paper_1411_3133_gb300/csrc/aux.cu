@@ -444,12 +444,12 @@ template <class S>
 cudaError_t launch_stream_table_t(int K, float4* st, const float* ref, const InstParams<float>* inst,
                                   const void* fin, const Dims& d, cudaStream_t s) {
   const uint32_t n = uint32_t(d.batch) * uint32_t(d.nr) * uint32_t(d.st_rows3) * 2u;
-  const uint32_t nb = (n + 127) / 128;
+  const uint32_t nb = (n + ST_THREADS - 1) / ST_THREADS;
   const S* f = static_cast<const S*>(fin);
   switch (K) {
-    case KFLAT: k_stream_table<KFLAT, S><<<nb, 128, 0, s>>>(st, ref, inst, f, d); break;
-    case KCYL: k_stream_table<KCYL, S><<<nb, 128, 0, s>>>(st, ref, inst, f, d); break;
-    case KELL: k_stream_table<KELL, S><<<nb, 128, 0, s>>>(st, ref, inst, f, d); break;
+    case KFLAT: k_stream_table<KFLAT, S><<<nb, ST_THREADS, 0, s>>>(st, ref, inst, f, d); break;
+    case KCYL: k_stream_table<KCYL, S><<<nb, ST_THREADS, 0, s>>>(st, ref, inst, f, d); break;
+    case KELL: k_stream_table<KELL, S><<<nb, ST_THREADS, 0, s>>>(st, ref, inst, f, d); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
