@@ -340,40 +340,20 @@ __global__ void __launch_bounds__(256) k_ref_table(float* __restrict__ ref, GeoD
   for (int l = 0; l < Q; ++l) rb[ref_index<K>(d, l, int(row))] = fe[l];
 }
 
-// Stream table of 2-byte storage (stream_of): one thread per instance, stream
-// row and node of the row's pair (the last pair of an odd line repeats its
-// one node). The sources of the node at theta = 0 give, for every population
-// l, the stored population index and geometry row whose reference rho_l it
-// receives -- the sources of the step's gather. fin is any state block of the
-// context: its addresses are formed, never read. FP64 arithmetic bounds it: the
-// zero products are left out, and a block is one warp, so that a cylinder's few
-// rows are spread over the SMs (lb_init of one 64 x 4 x 256 cylinder in FP16 88 ->
-// 81 us, of 24 four-wall 64 x 4 x 255 ellipsoids 1000 -> 902).
-constexpr int ST_THREADS = 32;
-template <int K, class S>
-__global__ void __launch_bounds__(ST_THREADS) k_stream_table(float4* __restrict__ st,
-                                                             const float* __restrict__ ref,
-                                                             const InstParams<float>* __restrict__ inst,
-                                                             const S* fin, Dims d) {
-  const uint32_t nrows = uint32_t(d.nr) * uint32_t(d.st_rows3);
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= uint32_t(d.batch) * nrows * 2u) return;
-  const uint32_t half = t & 1u;
-  const int b = int((t / 2) / nrows), srow = int(t / 2 - uint32_t(b) * nrows);
-  CellPos p;
-  p.b = b;
-  p.it = 0;
-  p.ir = srow / d.st_rows3;
-  p.i3 = d.st_row_r ? 0 : 2 * (srow - p.ir * d.st_rows3) + int(half);
-  if (p.i3 >= d.n3) p.i3 -= int(half);
-  p.cell = (p.ir * d.nt + p.it) * d.n3 + p.i3;
-  const float* rb = ref + size_t(b) * Q * size_t(d.nr) * size_t(d.geo_rows3);
+// Stream table entries of node p (stream_of): put(k, x, y, z, w). The sources
+// of the node at theta = 0 give, for every population l, the stored population
+// index and geometry row whose reference rho_l it receives -- the sources of the
+// step's gather. rb is the instance's reference table, fin any state block of
+// the context: its addresses are formed, never read.
+template <int K, class S, class Put>
+__device__ __forceinline__ void stream_entries(const float* __restrict__ rb, float omega, const S* fin,
+                                               const CellPos& p, const Dims& d, Put&& put) {
   double rho_l[Q];
   for_each_source<K, S>(fin, p, d, [&](auto L_, const S*, int sl, int row) {
     constexpr int L = decltype(L_)::value;
     rho_l[L] = double(rb[ref_index<K>(d, sl, row)]);
   });
-  const float om1 = 1.0f - inst[b].omega;  // as the step computes it
+  const float om1 = 1.0f - omega;  // as the step computes it
   const int own = geo_row<K>(d, p.ir, p.i3);
   double tl[Q];
   double m[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -398,15 +378,6 @@ __global__ void __launch_bounds__(ST_THREADS) k_stream_table(float4* __restrict_
     add(9, std::integral_constant<int, cy * cz>{});
     tl[L] = (double(om1) * r - double(rb[ref_index<K>(d, L, own)])) / WeightOf<L>::w;
   });
-  float* out = reinterpret_cast<float*>(st + size_t(b) * 2 * ST_K * nrows + uint32_t(srow)) + half;
-  auto put = [&](int k, double x, double y, double z, double w) {
-    float* o = out + size_t(2 * k) * nrows * 4;
-    o[0] = float(x);
-    o[2] = float(y);
-    o += size_t(nrows) * 4;
-    o[0] = float(z);
-    o[2] = float(w);
-  };
   // even and odd parts of t per pair, then each shell's transform to the
   // coefficients its pairs are evaluated from (update_face, update_body)
   double te[NPAIR], to[NPAIR];
@@ -439,6 +410,82 @@ __global__ void __launch_bounds__(ST_THREADS) k_stream_table(float4* __restrict_
   put(2, m[8], m[9], tl[0], 0.0);
 #pragma unroll
   for (int j = 0; j < NPAIR / 2; ++j) put(3 + j, te[2 * j], to[2 * j], te[2 * j + 1], to[2 * j + 1]);
+}
+
+// Stream table of 2-byte storage: one thread per instance, stream row and node
+// of the row's pair (the last pair of an odd line repeats its one node). FP64
+// arithmetic bounds it: the zero products are left out, and a block is one warp,
+// so that a cylinder's few rows are spread over the SMs (lb_init of one 64 x 4 x
+// 256 cylinder in FP16 88 -> 81 us, of 24 four-wall 64 x 4 x 255 ellipsoids 1000
+// -> 902).
+constexpr int ST_THREADS = 32;
+template <int K, class S>
+__global__ void __launch_bounds__(ST_THREADS) k_stream_table(float4* __restrict__ st,
+                                                             const float* __restrict__ ref,
+                                                             const InstParams<float>* __restrict__ inst,
+                                                             const S* fin, Dims d) {
+  const uint32_t nrows = uint32_t(d.nr) * uint32_t(d.st_rows3);
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= uint32_t(d.batch) * nrows * 2u) return;
+  const uint32_t half = t & 1u;
+  const int b = int((t / 2) / nrows), srow = int(t / 2 - uint32_t(b) * nrows);
+  CellPos p;
+  p.b = b;
+  p.it = 0;
+  p.ir = srow / d.st_rows3;
+  p.i3 = d.st_row_r ? 0 : 2 * (srow - p.ir * d.st_rows3) + int(half);
+  if (p.i3 >= d.n3) p.i3 -= int(half);
+  p.cell = (p.ir * d.nt + p.it) * d.n3 + p.i3;
+  float* out = reinterpret_cast<float*>(st + size_t(b) * 2 * ST_K * nrows + uint32_t(srow)) + half;
+  stream_entries<K, S>(ref + size_t(b) * Q * size_t(d.nr) * size_t(d.geo_rows3), inst[b].omega, fin, p, d,
+                       [&](int k, double x, double y, double z, double w) {
+                         float* o = out + size_t(2 * k) * nrows * 4;
+                         o[0] = float(x);
+                         o[2] = float(y);
+                         o += size_t(nrows) * 4;
+                         o[0] = float(z);
+                         o[2] = float(w);
+                       });
+}
+
+// The same where walls on x3 are all that tells the rows of an i_r layer apart
+// (flat channel and cylinder): a block per layer and instance forms the entries
+// of the at most 7 node classes along x3 (axis_class) and copies them to the
+// layer's rows. lb_init of 24 walled 33 x 3 x 101 cylinders in FP16 240 -> 120 us.
+constexpr int ST_CLASS_THREADS = 64;
+template <int K, class S>
+__global__ void __launch_bounds__(ST_CLASS_THREADS) k_stream_table_classes(float4* __restrict__ st,
+                                                                           const float* __restrict__ ref,
+                                                                           const InstParams<float>* __restrict__ inst,
+                                                                           const S* fin, Dims d) {
+  __shared__ float val[7][4 * ST_K];
+  const int b = int(blockIdx.y);
+  CellPos p;
+  p.b = b;
+  p.it = 0;
+  p.ir = int(blockIdx.x);
+  if (int(threadIdx.x) < axis_classes(d.n3)) {
+    p.i3 = axis_class_node(int(threadIdx.x), d.n3);
+    p.cell = p.ir * d.nt * d.n3 + p.i3;
+    float* v = val[threadIdx.x];
+    stream_entries<K, S>(ref + size_t(b) * Q * size_t(d.nr) * size_t(d.geo_rows3), inst[b].omega, fin, p, d,
+                         [&](int k, double x, double y, double z, double w) {
+                           v[4 * k] = float(x);
+                           v[4 * k + 1] = float(y);
+                           v[4 * k + 2] = float(z);
+                           v[4 * k + 3] = float(w);
+                         });
+  }
+  __syncthreads();
+  const size_t nrows = size_t(d.nr) * size_t(d.st_rows3);
+  float4* out = st + size_t(b) * 2 * ST_K * nrows + size_t(p.ir) * size_t(d.st_rows3);
+  for (int i = int(threadIdx.x); i < d.st_rows3; i += ST_CLASS_THREADS) {
+    const float* v0 = val[axis_class(2 * i, d.n3)];
+    const float* v1 = val[axis_class(min(2 * i + 1, d.n3 - 1), d.n3)];
+#pragma unroll
+    for (int k = 0; k < 2 * ST_K; ++k)
+      out[size_t(k) * nrows + size_t(i)] = make_float4(v0[2 * k], v1[2 * k], v0[2 * k + 1], v1[2 * k + 1]);
+  }
 }
 
 }  // namespace lbgm
