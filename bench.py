@@ -428,7 +428,9 @@ def step_launches(channels, precision, steps, list_max=None):
     if steps < 4:
         return flat
     def held(c):  # two buffers and the 2-byte storage's stream table
-        rows3 = 1 if c.periodic3 and c.metric != "ellipsoidal" else (c.n3 + 1) // 2
+        rows3 = (c.n3 + 1) // 2
+        if c.metric != "ellipsoidal":
+            rows3 = 1 if c.periodic3 else min(rows3, 5)
         return c.ncells * BYTES_PER_UPDATE[precision] + (26 * 16 * c.nr * rows3 if two_byte else 0)
 
     hold = 90 << 20

@@ -511,7 +511,7 @@ lb_status lb_create_geometry(lb_metric metric, const lb_geometry_desc* geom, int
   d.src = c->src_tab;
   const uint32_t np = uint32_t(d.n3 + 1) / 2;
   d.st_row_r = c->K != KELL && d.periodic3 ? 1 : 0;
-  d.st_rows3 = d.st_row_r ? 1 : int(np);
+  d.st_rows3 = d.st_row_r ? 1 : c->K == KELL ? int(np) : pair_rows(int(np));
   d.div_np = FastDiv::make(np);
   d.div_wl = FastDiv::make(d.st_row_r ? (uint32_t(d.nt) * np + 31) / 32 : (np + 31) / 32 * uint32_t(d.nt));
   if (c->elem_bytes == 2) {

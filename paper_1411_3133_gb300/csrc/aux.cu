@@ -445,12 +445,9 @@ cudaError_t launch_stream_table_t(int K, float4* st, const float* ref, const Ins
                                   const void* fin, const Dims& d, cudaStream_t s) {
   const uint32_t n = uint32_t(d.batch) * uint32_t(d.nr) * uint32_t(d.st_rows3) * 2u;
   const uint32_t nb = (n + ST_THREADS - 1) / ST_THREADS;
-  const dim3 layers(unsigned(d.nr), unsigned(d.batch));
   const S* f = static_cast<const S*>(fin);
-  if (K == KFLAT && d.st_row_r) k_stream_table<KFLAT, S><<<nb, ST_THREADS, 0, s>>>(st, ref, inst, f, d);
-  else if (K == KFLAT) k_stream_table_classes<KFLAT, S><<<layers, ST_CLASS_THREADS, 0, s>>>(st, ref, inst, f, d);
-  else if (K == KCYL && d.st_row_r) k_stream_table<KCYL, S><<<nb, ST_THREADS, 0, s>>>(st, ref, inst, f, d);
-  else if (K == KCYL) k_stream_table_classes<KCYL, S><<<layers, ST_CLASS_THREADS, 0, s>>>(st, ref, inst, f, d);
+  if (K == KFLAT) k_stream_table<KFLAT, S><<<nb, ST_THREADS, 0, s>>>(st, ref, inst, f, d);
+  else if (K == KCYL) k_stream_table<KCYL, S><<<nb, ST_THREADS, 0, s>>>(st, ref, inst, f, d);
   else if (K == KELL) k_stream_table<KELL, S><<<nb, ST_THREADS, 0, s>>>(st, ref, inst, f, d);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();

@@ -433,7 +433,8 @@ __global__ void __launch_bounds__(ST_THREADS) k_stream_table(float4* __restrict_
   p.b = b;
   p.it = 0;
   p.ir = srow / d.st_rows3;
-  p.i3 = d.st_row_r ? 0 : 2 * (srow - p.ir * d.st_rows3) + int(half);
+  const int r3 = srow - p.ir * d.st_rows3;
+  p.i3 = d.st_row_r ? 0 : 2 * (K == KELL ? r3 : pair_of_row(r3, (d.n3 + 1) / 2)) + int(half);
   if (p.i3 >= d.n3) p.i3 -= int(half);
   p.cell = (p.ir * d.nt + p.it) * d.n3 + p.i3;
   float* out = reinterpret_cast<float*>(st + size_t(b) * 2 * ST_K * nrows + uint32_t(srow)) + half;
@@ -446,46 +447,6 @@ __global__ void __launch_bounds__(ST_THREADS) k_stream_table(float4* __restrict_
                          o[0] = float(z);
                          o[2] = float(w);
                        });
-}
-
-// The same where walls on x3 are all that tells the rows of an i_r layer apart
-// (flat channel and cylinder): a block per layer and instance forms the entries
-// of the at most 7 node classes along x3 (axis_class) and copies them to the
-// layer's rows. lb_init of 24 walled 33 x 3 x 101 cylinders in FP16 240 -> 120 us.
-constexpr int ST_CLASS_THREADS = 64;
-template <int K, class S>
-__global__ void __launch_bounds__(ST_CLASS_THREADS) k_stream_table_classes(float4* __restrict__ st,
-                                                                           const float* __restrict__ ref,
-                                                                           const InstParams<float>* __restrict__ inst,
-                                                                           const S* fin, Dims d) {
-  __shared__ float val[7][4 * ST_K];
-  const int b = int(blockIdx.y);
-  CellPos p;
-  p.b = b;
-  p.it = 0;
-  p.ir = int(blockIdx.x);
-  if (int(threadIdx.x) < axis_classes(d.n3)) {
-    p.i3 = axis_class_node(int(threadIdx.x), d.n3);
-    p.cell = p.ir * d.nt * d.n3 + p.i3;
-    float* v = val[threadIdx.x];
-    stream_entries<K, S>(ref + size_t(b) * Q * size_t(d.nr) * size_t(d.geo_rows3), inst[b].omega, fin, p, d,
-                         [&](int k, double x, double y, double z, double w) {
-                           v[4 * k] = float(x);
-                           v[4 * k + 1] = float(y);
-                           v[4 * k + 2] = float(z);
-                           v[4 * k + 3] = float(w);
-                         });
-  }
-  __syncthreads();
-  const size_t nrows = size_t(d.nr) * size_t(d.st_rows3);
-  float4* out = st + size_t(b) * 2 * ST_K * nrows + size_t(p.ir) * size_t(d.st_rows3);
-  for (int i = int(threadIdx.x); i < d.st_rows3; i += ST_CLASS_THREADS) {
-    const float* v0 = val[axis_class(2 * i, d.n3)];
-    const float* v1 = val[axis_class(min(2 * i + 1, d.n3 - 1), d.n3)];
-#pragma unroll
-    for (int k = 0; k < 2 * ST_K; ++k)
-      out[size_t(k) * nrows + size_t(i)] = make_float4(v0[2 * k], v1[2 * k], v0[2 * k + 1], v1[2 * k + 1]);
-  }
 }
 
 }  // namespace lbgm

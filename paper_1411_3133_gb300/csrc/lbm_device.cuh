@@ -55,7 +55,7 @@ struct Dims {
   // FP32 / FP64 storage) over nr * st_rows3 stream rows, and the divisors of
   // the pair kernels' node numbering
   const float4* st;
-  int st_rows3;    // rows per i_r: 1, or the x3 pairs (n3 + 1) / 2
+  int st_rows3;    // rows per i_r: 1, the x3 pairs (n3 + 1) / 2, or their kinds (pair_rows)
   int st_row_r;    // 1: rows of i_r alone (flat and cylinder, periodic x3)
   FastDiv div_np, div_wl;  // x3 pairs per line, warps per i_r layer
   int geo_theta;   // 1: geometry rows (and observable weights) per node
@@ -74,6 +74,18 @@ __host__ __device__ __forceinline__ int axis_class(int i, int n) {
 }
 // A node of class c.
 __host__ __device__ __forceinline__ int axis_class_node(int c, int n) { return n < 7 || c <= 3 ? c : n - 7 + c; }
+// Stream rows of an i_r layer between x3 walls where the metric does not depend
+// on x3 (flat, cylinder; np pairs of nodes along x3): the first two pairs, those
+// whose nodes are all of class 3, the last two. With a row for every pair the
+// table was larger than the state (416 B a pair; 259 MB for 24 cylinders of
+// 130 x 1 x 400, 6.5 MB now), and lb_init of those, which writes it, took 356 us
+// (now 178).
+__host__ __device__ __forceinline__ int pair_rows(int np) { return np < 5 ? np : 5; }
+__host__ __device__ __forceinline__ int pair_row(int i, int np) {
+  return np < 5 || i < 2 ? i : (i >= np - 2 ? i - np + 5 : 2);
+}
+// A pair of row r.
+__host__ __device__ __forceinline__ int pair_of_row(int r, int np) { return np < 5 || r < 3 ? r : np - 5 + r; }
 constexpr int SRC_ROW = 11;  // int4 per key: 41 offsets, padded
 
 // Index of reference population l of geometry row r in an instance's table:
@@ -112,8 +124,9 @@ __device__ __forceinline__ const float* ref_of(const Dims& d, int b) {
 // Stream table of instance b (2-byte storage). Which stored population (and
 // whose geometry row's reference) a node receives in streaming does not
 // depend on theta, and for the flat channel and the cylinder with a periodic
-// x3 not on x3 either: a stream row is an i_r layer there, else the pair
-// (i_3 = 2 p, 2 p + 1) of an (i_r, x3) line. A row holds 13 entries of 4
+// x3 not on x3 either: a stream row is an i_r layer there, between x3 walls a
+// kind of pair of the layer (pair_rows), in the ellipsoid the pair (i_3 = 2 p,
+// 2 p + 1) of an (i_r, x3) line. A row holds 13 entries of 4
 // values for both nodes of the pair, stored [2 k + half][row] as float4 (x of
 // both nodes, y of both) and (z of both, w of both): consecutive pairs are
 // consecutive float4. Entry k (f_l = w_l g_l + rho_l: g the stored deviation,

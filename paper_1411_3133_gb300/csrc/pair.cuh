@@ -248,8 +248,8 @@ __device__ __forceinline__ void step_pair(const S* fin, S* __restrict__ fout, co
       i = np - 1;
     }
     p.i3 = 2 * i;
-    const float4* src = st + (p.ir * np + i);
-    const int stride = d.nr * np;
+    const float4* src = st + (p.ir * d.st_rows3 + (K == KELL ? i : pair_row(i, np)));
+    const int stride = d.nr * d.st_rows3;
     float4* own = shared ? sm : sm + wib * 64 * ST_K;
     const int step = shared ? int(blockDim.x >> 5) : 1;
 #pragma unroll 1

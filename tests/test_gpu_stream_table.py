@@ -2,9 +2,11 @@
 by their distance to the walls on x3 alone."""
 import time
 
+import numpy as np
 import pytest
 
-from gpu_helpers import lib
+from gpu_helpers import Twin, lib
+from oracle.geometry import Channel
 
 pytestmark = pytest.mark.gpu
 
@@ -29,3 +31,29 @@ def test_walled_rows_cost_little_more_than_periodic_ones():
         best[periodic3] = min(times)
         c.close()
     assert best[False] < 1.6 * best[True]
+
+
+@pytest.mark.parametrize("wall", ["bounceback", "equilibrium"])
+@pytest.mark.parametrize("metric", ["cylindrical", "flat"])
+@pytest.mark.parametrize("n3", list(range(7, 14)) + [65, 66, 130])
+def test_step_through_the_kinds_of_pairs(metric, wall, n3):
+    """Two pairs of nodes at each wall on x3 and the kind between them, with the
+    rows of a laminar profile as reference (a wall swaps r of c and -c). One step
+    from the stored state: a population is off by one rounding of g = (f - r) / w,
+    2^-11 |g| with |g| <= |f / w - 1| + |r / w - 1|, and by the FP32 arithmetic
+    before it, some 700 operations on numbers of order 1. A pair read as another
+    kind misses the swap, 0.05 and more."""
+    from oracle import lattice as OL
+    ro = 1.0 if metric == "flat" else 1.05
+    ch = Channel(metric, 0.0 if metric == "flat" else 1.0, ro, 9, 2, n3, periodic3=False, wall=wall)
+    p = dict(tau=0.7, G=2e-4, seed=3, amp=1e-2, base=True)
+    tw = Twin(ch, [p], "fp16_shifted")
+    tw.ctx.lb_init(tw.lparams)
+    for s, f in zip(tw.sims, tw.lib_f()):
+        s.f = f.copy()
+    tw.step(1)
+    w = OL.W[None, :, None]
+    err = np.abs(tw.lib_f() - np.stack([s.f for s in tw.sims])) / w
+    dev = np.abs(tw.lib_f() / w - 1.0).max()
+    assert err.max() <= 2.0 ** -11 * 2 * dev + 1000 * 2.0 ** -24
+    tw.close()

@@ -210,3 +210,30 @@ def test_fp64_steps_of_one_block_per_sm_are_not_chained(lib, precision, instance
     if batch:
         b.close()
     c.close()
+
+
+@pytest.mark.parametrize("metric,n3", [("cylindrical", 401), ("cylindrical", 8), ("flat", 256)])
+def test_walls_on_x3_cost_no_memory(lib, metric, n3):
+    """2-byte storage: a channel walled on x3 holds 5 rows of the stream table an
+    i_r layer instead of one, 4 x 416 bytes, and more source keys (x3 classes);
+    not a row for every pair of nodes, 208 bytes a node of the cross-section."""
+    alloc_t, free_t = (dict(L.lb_allocator._fields_)[k] for k in ("alloc", "free"))
+    libc = ctypes.CDLL(None)
+    libc.malloc.restype, libc.malloc.argtypes = ctypes.c_void_p, [ctypes.c_size_t]
+    libc.free.argtypes = [ctypes.c_void_p]
+    held = {}
+    for periodic3 in (True, False):
+        total = [0]
+
+        def grab(n, stream, user):
+            total[0] += n
+            return libc.malloc(n)
+
+        a = L.lb_allocator(alloc=alloc_t(grab), free=free_t(lambda p, n, stream, user: libc.free(p)))
+        desc = L.make_desc(1.0, 1.0 / 0.975, 130, 1, n3, periodic3=periodic3)
+        c = ctypes.c_void_p()
+        assert lib.lb_create_geometry(L.METRICS[metric], ctypes.byref(desc), 3, L.PRECISIONS["fp16_shifted"],
+                                      ctypes.c_void_p(lib.fake_stream(0)), ctypes.byref(a), ctypes.byref(c)) == L.LB_OK
+        held[periodic3] = total[0]
+        lib.lb_destroy(c)
+    assert held[False] <= held[True] + 3 * 130 * 4 * 416 + 7 * 7 * 7 * 176
