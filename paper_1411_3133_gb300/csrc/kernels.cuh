@@ -12,8 +12,17 @@ namespace lbgm {
 // their nodes, source-table rows and geometry -- and wait for its end and its
 // memory before they touch the state (gather_table says how they may read it).
 // Without the launch attribute both are no-ops.
+// chain_start lets the next step's blocks in. FP32 arithmetic asks for them
+// first of all. An FP64 step asks after its own wait, so that at most the step to
+// come waits on the SMs: asked for at once, blocks of two or three steps sat
+// there, some SMs got two blocks of one step and their FP64 units took twice as
+// long. us a step, asked for at once / after the wait: one cylinder of 49 blocks
+// 28.4 / 20.0; two contexts of 24 blocks side by side 29.1 / 21.7, four 35.5 /
+// 24.7 (32.3 before steps were chained).
 __device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class Real>
+constexpr bool CHAIN_LATE = sizeof(Real) == 8;
 
 // Fused time step (Eq. LB) of one node p of one instance whose state blocks
 // start at fin and fout: pull streaming + walls (gather_step), moments,
@@ -34,6 +43,7 @@ __device__ __forceinline__ void step_node(const Real* fin, Real* __restrict__ fo
   // shared by nodes come from L1 and L2 and would only hold registers
   if constexpr (K == KELT) g = load_geo<Real, K>(geo, row);
   chain_wait();
+  if constexpr (CHAIN_LATE<Real>) chain_start();
   gather_step(fin, p, d, f);
   const Moments<Real> m = step_moments(f);
   if (!finite_v(m.rho)) {  // NaN or Inf
@@ -78,7 +88,7 @@ template <typename Real, int K>
 __global__ void __launch_bounds__(KBounds<Real, K>::maxt, KBounds<Real, K>::minb)
     k_step(const Real* fin, Real* __restrict__ fout, GeoDev<Real> geo,
            const InstParams<Real>* __restrict__ inst, Dims d, int* __restrict__ flag) {
-  chain_start();
+  if constexpr (!CHAIN_LATE<Real>) chain_start();
   const uint32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= uint32_t(d.ncell)) return;
   const int b = int(blockIdx.y);
@@ -133,7 +143,7 @@ struct ListArgs {
 template <typename Real, int K, bool LOOP>
 __global__ void __launch_bounds__(KBounds<Real, K>::maxt, KBounds<Real, K>::minb)
     k_step_list(const __grid_constant__ ListArgs<Real, Real> a) {
-  chain_start();
+  if constexpr (!CHAIN_LATE<Real>) chain_start();
   auto item = [&](int j) {
     const int i = a.instance(j);
     const ListInst<Real, Real>& I = a.rec[i];

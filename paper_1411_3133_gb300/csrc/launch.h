@@ -15,14 +15,15 @@ struct InitInst;
 
 constexpr int SMS = 152;  // of a GB300
 
-// Whether an FP64 step of `blocks` blocks is worth chaining. Chained, the blocks
-// of the next two or three steps already sit where an SM has room, and an SM that
-// holds two blocks of one step needs twice as long for it (its FP64 units bound
-// the step); unchained, a step of at most one block per SM has one on each.
-// Flat channels, us a step chained / unchained (graph replay before there were
-// chained launches: 29.1): 49 blocks 18.7 / 20.9, 64 20.2 to 25.7 / 20.9, 96
-// 30.5 / 20.8, 144 32.9 / 20.9, 152 18.9 / 20.9, 160 34.6 / 37.2. FP32 arithmetic
-// is bound by latency there and gains in every size (144 blocks 3.5 / 4.6).
+// Whether an FP64 step of `blocks` blocks is worth chaining. An SM that holds two
+// blocks of one step needs twice as long for it (its FP64 units bound the step),
+// and the blocks of the next step, which sit on the SMs while they wait, bring
+// that about where the caller's other contexts step beside it. Cylinders, us a
+// step chained / unchained: one context alone 20.0 / 22.6 at 64 to 144 blocks;
+// three of 64 side by side 36.6 / 31.6, two of 96 37.9 / 31.4, four of 96 46.6 /
+// 46.7. Below a third of the SMs the waiting blocks find
+// SMs of their own (two contexts of 49 21.8, four of 24 24.7). FP32 arithmetic is
+// bound by latency there and gains in every size (144 blocks 3.5 / 4.6).
 constexpr bool fp64_chains(long long blocks) { return 3 * blocks <= SMS || blocks >= SMS; }
 
 // chained: see launch_chained.

@@ -126,3 +126,34 @@ def test_replayed_pairs_of_the_tma_and_half_force_kernels(plan):
         c.close()
     assert all(np.array_equal(a, b) for a, b in zip(*outs))
     assert not np.array_equal(outs[0][0], outs[0][1])      # the variant is another step
+
+
+def test_small_fp64_steps_leave_each_other_their_sms():
+    """Contexts whose blocks fit the SMs one by one take about the time of one:
+    1.07 for two of 24 blocks, 1.0 for one of 49 against one of 24 (1.46 and 1.4
+    while the blocks of several steps to come waited on the SMs)."""
+    import time
+
+    import torch
+    L = lib()
+
+    def us(blocks, contexts):
+        cs = [L.LBContext(L.ChannelSpec("cylindrical", 1.0, 1.05, blocks, 1, 128), batch=1, precision="fp64")
+              for _ in range(contexts)]
+        for c in cs:
+            c.lb_init([L.make_params(0.8, 1e-6, False, 1, 1e-4, False)])
+        best = 1e9
+        for _ in range(8):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            for c in cs:
+                c.lb_step(100)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t)
+        for c in cs:
+            c.close()
+        return best * 1e4
+
+    one = us(24, 1)
+    assert us(49, 1) < 1.2 * one
+    assert us(24, 2) < 1.25 * one
