@@ -225,9 +225,8 @@ std::string check_sparsity(const std::vector<double>& rows, const lb_geometry_de
 
 // The step kernel of the context: the TMA kernel where it was asked for (and
 // no instance uses the half-force variant), else the one-kernel step of the
-// storage type, which also stands for LB_OPT_STEP_KERNEL 4 and 5: on 24
-// 64 x 4 x 256 cylinders in FP32 it takes 82.4 us a step against 84.9 for a
-// region split on two streams and 103.6 for a work list.
+// storage type, which LB_OPT_STEP_KERNEL 4 and 5, the names of a region split
+// and a tiled step that it has replaced, select too.
 bool use_tma(const lb_ctx* c) { return c->prec == LB_FP32 && c->tma_ok && c->step_kernel == 2 && !c->any_shift; }
 
 // One time step of instances i0 .. i0 + count - 1 from buffer src into 1 - src;

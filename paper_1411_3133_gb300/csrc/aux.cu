@@ -200,11 +200,12 @@ __device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x
 //   0 rho'   1 rho' g   2 sqrt(g_thth) u^theta wA   3 wA   4 |omega| wOmega
 //   5 (u^r)^2   6 (u^r - row mean)^2   7 max |u|^2   8 non-finite nodes
 // A warp takes whole x3 rows: the row's mean of u^r first, then its nodes
-// while the row is in L1. FP64 units bound this pass (16 cycles a warp
-// instruction), so the weights come multiplied out (diag_weights), 5 is the
-// sum of 6 and the rows' means, the square root of 7 is taken once at the end,
-// comparisons are integer, and the two halves of the central differences are
-// one factor of the weight: 14 FP64 operations a node.
+// while the row is in L1. 89 us for 24 x 64 x 4 x 256 nodes, 42 of them the FP64
+// units' (16 cycles a warp instruction), the rest latency at 16 warps per SM. So
+// the weights come multiplied out (diag_weights), 5 is the sum of 6 and the
+// rows' means, the square root of 7 is taken once at the end, comparisons are
+// integer, and the two halves of the central differences are one factor of the
+// weight: 14 FP64 operations a node.
 __global__ void __launch_bounds__(DIAG_THREADS)
     k_diag_partial(const double* __restrict__ rho, const double* __restrict__ u, const double* __restrict__ geo64,
                    Dims d, double* __restrict__ partial, int nblk) {
