@@ -218,6 +218,8 @@ typedef enum {
                                work-list tile, in blocks' worth: 1
                                (default), 2 or 4; each thread of a tile's
                                block takes every blockDim-th node of it.
+                               Halved in a launch of fewer than two tiles
+                               per SM.
                                Bitwise neutral. */
   LB_OPT_STORAGE_REFERENCE = 6 /* FP16/BF16 storage only: the reference
                                r_l of the stored deviation (f_l - r_l)/w_l.

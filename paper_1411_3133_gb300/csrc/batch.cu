@@ -8,7 +8,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <numeric>
 #include <string>
 #include <vector>
 
@@ -26,7 +25,7 @@ struct Group {
   int K = 0;
   int ninst = 0;
   std::vector<unsigned char> recs;  // ListInst records
-  std::vector<int> items;           // work items of each instance
+  std::vector<int> work;            // nodes (FP32, FP64) or warps (2-byte storage) of each instance
   int blocks_per_sm = 0;            // occupancy of the kernel at the built block size
   Dims d{};                         // 2-byte storage: an instance of the group
   size_t smem = 0;                  // 2-byte storage: staged rows of a block, bytes
@@ -49,7 +48,7 @@ struct lb_batch {
   std::vector<int> base_cur;  // member buffer parity when the records were written
   int parity = 0;             // batch steps since then, mod 2
   std::vector<Group> g;
-  int tile = 0;               // nodes (FP32, FP64) or warps (2-byte storage) of a work item
+  int block_work = 0;         // nodes (FP32, FP64) or warps (2-byte storage) of a block
 
   LaneStreams lanes;
   Replays replays;              // of plan's chunks, or of flat's where there is no plan
@@ -142,15 +141,15 @@ cudaError_t occupancy(lb_precision p, const Group& g, int threads, int* out) {
   }
 }
 
-// Write the instance records (with the members' current buffer parity) and
-// count their work items for block size b->threads (tiles of b->tile_blocks
-// blocks' worth of nodes). Host only: the launches carry the records.
+// Write the instance records (with the members' current buffer parity) and plan
+// their launches for block size b->threads. Host only: the launches carry the
+// records.
 lb_status build(lb_batch* b) {
   drop_graph(b);
   b->built = false;
   b->g.clear();
   const bool pairs = b->prec == LB_FP16_SHIFTED || b->prec == LB_BF16_SHIFTED;
-  b->tile = (pairs ? b->threads / 32 : b->threads) * b->tile_blocks;
+  b->block_work = pairs ? b->threads / 32 : b->threads;
   std::vector<int> keys;
   for (int K : {int(KCYL), int(KELL), int(KFLAT)})
     for (int v = 0; v < 4; ++v) keys.push_back(K * 4 + v);
@@ -167,8 +166,7 @@ lb_status build(lb_batch* b) {
     if (gr.ninst == 0) continue;
     for (const lb_ctx* c : b->m) {
       if (variant(c) != key) continue;
-      const int n = pairs ? int(pair_warps(c->dims)) : c->dims.ncell;
-      for (int bi = 0; bi < c->batch; ++bi) gr.items.push_back((n + b->tile - 1) / b->tile);
+      gr.work.insert(gr.work.end(), size_t(c->batch), pairs ? int(pair_warps(c->dims)) : c->dims.ncell);
       if (pairs) {
         gr.d = c->dims;
         gr.smem = std::max(gr.smem, pair_smem_bytes(c->dims, b->threads / 32));
@@ -211,23 +209,30 @@ bool records_current(const lb_batch* b) {
 }
 
 // One step of a chunk of one group's instances on stream s, at parity `par`;
-// chained: see launch_chained.
+// chained: see launch_chained. A work item is a tile of tile_blocks blocks'
+// worth of nodes, halved while the launch has fewer than two items per SM: the
+// groups of lanes.h are short launches, and with tiles of 4 blocks' worth 18 unlike
+// channels (300 000 nodes) took 68 us a step in BF16, 35 now (49 before there were
+// groups; 35 with tiles of one block's worth).
 cudaError_t launch_chunk(const lb_batch* b, const LaneChunk& c, int par, bool chained, cudaStream_t s) {
   const Group& gr = b->g[size_t(c.group)];
   const int grid = b->schedule == 1 ? std::max(1, gr.blocks_per_sm) * b->nsm : 0;
   const void* recs = gr.recs.data() + gr.recs.size() / size_t(gr.ninst) * size_t(c.first);
-  const int* items = gr.items.data() + c.first;
-  if (b->prec == LB_FP64) {
-    const long long n = std::accumulate(items, items + c.count, 0ll);
-    chained = chained && fp64_chains(grid > 0 ? std::min<long long>(grid, n) : n);
+  int items[LIST_MAX], tile = 0;
+  long long n = 0;
+  for (int blocks = b->tile_blocks; n == 0 || (n < 2 * b->nsm && blocks > 0); blocks /= 2) {
+    tile = b->block_work * blocks;
+    n = 0;
+    for (int i = 0; i < c.count; ++i) n += items[i] = (gr.work[size_t(c.first + i)] + tile - 1) / tile;
   }
+  if (b->prec == LB_FP64) chained = chained && fp64_chains(grid > 0 ? std::min<long long>(grid, n) : n);
   switch (b->prec) {
-    case LB_FP64: return launch_step_list_f64(gr.K, recs, c.count, items, b->tile, b->threads, grid, par, chained, s);
-    case LB_FP32: return launch_step_list_f32(gr.K, recs, c.count, items, b->tile, b->threads, grid, par, chained, s);
+    case LB_FP64: return launch_step_list_f64(gr.K, recs, c.count, items, tile, b->threads, grid, par, chained, s);
+    case LB_FP32: return launch_step_list_f32(gr.K, recs, c.count, items, tile, b->threads, grid, par, chained, s);
     case LB_FP16_SHIFTED:
-      return launch_step_list_h16(gr.K, gr.d, gr.smem, recs, c.count, items, b->tile, b->threads, grid, par, chained, s);
+      return launch_step_list_h16(gr.K, gr.d, gr.smem, recs, c.count, items, tile, b->threads, grid, par, chained, s);
     default:
-      return launch_step_list_b16(gr.K, gr.d, gr.smem, recs, c.count, items, b->tile, b->threads, grid, par, chained, s);
+      return launch_step_list_b16(gr.K, gr.d, gr.smem, recs, c.count, items, tile, b->threads, grid, par, chained, s);
   }
 }
 

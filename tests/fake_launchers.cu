@@ -7,7 +7,8 @@
 #include "../paper_1411_3133_gb300/csrc/launch.h"
 
 using Instances = std::vector<std::pair<const void*, void*>>;
-void fake_step(const char* kind, const Instances& inst, int elem, double nodes, bool chained, int threads, cudaStream_t s);
+void fake_step(const char* kind, const Instances& inst, int elem, double nodes, bool chained, int threads, cudaStream_t s,
+               int tile = 0);
 
 namespace lbgm {
 namespace {
@@ -23,7 +24,7 @@ cudaError_t uniform(const char* kind, const S* fin, S* fout, const Dims& d, bool
 }
 
 template <class S, class R>
-cudaError_t listed(const char* kind, const void* recs, int count, int parity, bool chained, int threads,
+cudaError_t listed(const char* kind, const void* recs, int count, int tile, int parity, bool chained, int threads,
                    cudaStream_t s) {
   Instances inst;
   double nodes = 0;
@@ -32,7 +33,7 @@ cudaError_t listed(const char* kind, const void* recs, int count, int parity, bo
     inst.push_back({parity ? r[i].f1 : r[i].f0, const_cast<S*>(parity ? r[i].f0 : r[i].f1)});
     nodes += r[i].d.ncell;
   }
-  fake_step(kind, inst, sizeof(S), nodes, chained, threads, s);
+  fake_step(kind, inst, sizeof(S), nodes, chained, threads, s, tile);
   return cudaSuccess;
 }
 
@@ -50,19 +51,19 @@ FAKE_STEP(launch_step_b16, "b16", __nv_bfloat16, float)
 FAKE_STEP(launch_step_shift_f64, "shift64", double, double)
 FAKE_STEP(launch_step_shift_f32, "shift32", float, float)
 
-cudaError_t launch_step_list_f64(int, const void* r, int n, const int*, int, int t, int, int par, bool ch, cudaStream_t s) {
-  return listed<double, double>("list64", r, n, par, ch, t, s);
+cudaError_t launch_step_list_f64(int, const void* r, int n, const int*, int tile, int t, int, int par, bool ch, cudaStream_t s) {
+  return listed<double, double>("list64", r, n, tile, par, ch, t, s);
 }
-cudaError_t launch_step_list_f32(int, const void* r, int n, const int*, int, int t, int, int par, bool ch, cudaStream_t s) {
-  return listed<float, float>("list32", r, n, par, ch, t, s);
+cudaError_t launch_step_list_f32(int, const void* r, int n, const int*, int tile, int t, int, int par, bool ch, cudaStream_t s) {
+  return listed<float, float>("list32", r, n, tile, par, ch, t, s);
 }
-cudaError_t launch_step_list_h16(int, const Dims&, size_t, const void* r, int n, const int*, int, int t, int, int par,
+cudaError_t launch_step_list_h16(int, const Dims&, size_t, const void* r, int n, const int*, int tile, int t, int, int par,
                                  bool ch, cudaStream_t s) {
-  return listed<__half, float>("listh16", r, n, par, ch, t, s);
+  return listed<__half, float>("listh16", r, n, tile, par, ch, t, s);
 }
-cudaError_t launch_step_list_b16(int, const Dims&, size_t, const void* r, int n, const int*, int, int t, int, int par,
+cudaError_t launch_step_list_b16(int, const Dims&, size_t, const void* r, int n, const int*, int tile, int t, int, int par,
                                  bool ch, cudaStream_t s) {
-  return listed<__nv_bfloat16, float>("listb16", r, n, par, ch, t, s);
+  return listed<__nv_bfloat16, float>("listb16", r, n, tile, par, ch, t, s);
 }
 cudaError_t step_list_occupancy_f64(int, int, int* o) { *o = 2; return cudaSuccess; }
 cudaError_t step_list_occupancy_f32(int, int, int* o) { *o = 5; return cudaSuccess; }

@@ -50,7 +50,7 @@ void issue(cudaStream_t s, std::function<void(cudaStream_t)> op) {
 
 // One step launch: input and output of each instance, elements of `elem` bytes.
 void fake_step(const char* kind, const std::vector<std::pair<const void*, void*>>& inst, int elem, double nodes,
-               bool chained, int threads, cudaStream_t s) {
+               bool chained, int threads, cudaStream_t s, int tile) {
   const std::string k = kind;
   const size_t bytes = size_t(nodes * 2 * 41 * elem);
   issue(s, [=](cudaStream_t on) {
@@ -63,9 +63,9 @@ void fake_step(const char* kind, const std::vector<std::pair<const void*, void*>
     const double rate = k == "tma" ? g_tma_cost : g_node_cost[bytes > g_fit ? 1 : 0];
     st(on)->clock += g_launch_cost + rate * nodes;
     char line[160];
-    std::snprintf(line, sizeof line, "%s stream=%d first=%llx count=%zu chained=%d threads=%d replay=%d", k.c_str(),
+    std::snprintf(line, sizeof line, "%s stream=%d first=%llx count=%zu chained=%d threads=%d replay=%d tile=%d", k.c_str(),
                   st(on)->id, (unsigned long long)(uintptr_t)inst[0].first, inst.size(), chained ? 1 : 0, threads,
-                  g_replaying ? 1 : 0);
+                  g_replaying ? 1 : 0, tile);
     log(line);
   });
 }

@@ -237,3 +237,18 @@ def test_walls_on_x3_cost_no_memory(lib, metric, n3):
         held[periodic3] = total[0]
         lib.lb_destroy(c)
     assert held[False] <= held[True] + 3 * 130 * 4 * 416 + 7 * 7 * 7 * 176
+
+
+def test_long_tiles_leave_two_blocks_per_sm(lib):
+    """LB_OPT_TILE_BLOCKS 4 in blocks of 128 nodes: 512 an instance of 65536 (64 x 4
+    x 256), so tiles of one block (4 would be 128 of them for 152 SMs); 10 instances
+    of 16384 on their own, one launch of 1280, take tiles of 4 (320)."""
+    for batch, size, n, tile in ((5, (64, 4, 256), 8, 128), (10, (32, 4, 128), 1, 512)):
+        c = Host(lib, "cylindrical", size, batch, "fp32")
+        b = Batch(lib, [c])
+        b.option(L.LB_OPT_TILE_BLOCKS, 4)
+        take_log(lib)
+        b.step(n)
+        assert {x["tile"] for x in launches(lib)} == {tile}
+        b.close()
+        c.close()
